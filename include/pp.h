@@ -75,7 +75,9 @@ typedef struct {
     int32_t placement[PP_MAX_K]; /* n_1 .. n_m;     unused slots are -1 */
 } pp_solution;
 
-/* Device-time breakdown of the last pp_solve_exact / pp_solve_exact_dev of a problem. */
+/* Device-time breakdown of the last pp_solve_exact / pp_solve_exact_dev of a problem.  An ordinary
+ * solve is one launch that has no phases (sweep_launches = total_launches = 1); fast_path and
+ * pair_levels then tell which kernels the dense search of this problem consists of. */
 typedef struct {
     float ms_rank;     /* gamma table, rank compression (Eq. 3) and the base frontier (one node used) */
     float ms_sweep;    /* all popcount levels (two nodes and more) of the (min,max) sweep */
@@ -100,8 +102,8 @@ typedef struct {
  * Validates, builds the uint64 memory prefix sums and the per-node window table (for each
  * node w and segment end c', the earliest segment start that still fits), uploads them.
  * *out receives the handle; free it with pp_problem_destroy.
- * The list of node sets the search walks depends on k only: its device copy (4 * 2^k bytes) is
- * made by the first problem of that k on a device and kept until the process ends.
+ * The list of node sets the dense sweep walks depends on k only: its device copy (4 * 2^k bytes) is
+ * made by the first sweep of that k on a device and kept until the process ends.
  */
 pp_status pp_problem_create(int32_t L, const uint64_t *layer_out_bits,
                             const uint64_t *layer_mem_bytes, int32_t k,
@@ -116,7 +118,10 @@ void pp_problem_destroy(pp_problem *p);
  * later work of this problem.  NULL selects the legacy default stream. */
 pp_status pp_problem_set_stream(pp_problem *p, void *cuda_stream);
 
-/* Bytes of device scratch the exact search needs (state table, gamma and rank tables). */
+/* Bytes of device scratch the exact search needs (state table, gamma and rank tables).  Without a
+ * workspace a synchronous solve takes up to 128 MB plus 12 * k * 2^k bytes from the library's pool, and
+ * allocates the rest only when the dense sweep has to run; an asynchronous one needs room for every
+ * state and allocates it at the first call if that is more. */
 pp_status pp_problem_workspace_bytes(const pp_problem *p, uint64_t *bytes);
 
 /* Hand the library a caller-owned device buffer (256-byte aligned, at least
@@ -127,7 +132,9 @@ pp_status pp_problem_set_workspace(pp_problem *p, void *device_buffer, uint64_t 
 /*
  * Exact search (Eq. 2 minimised over every cut set and every injective placement) by a
  * (min,max) dynamic programme over (used-node mask, last node, last cut layer), swept by
- * popcount of the mask; then the canonical plan by backtracking.
+ * popcount of the mask; then the canonical plan by backtracking.  States that provably lie on no
+ * better plan than one already found are not expanded; where too many remain (a synchronous solve of
+ * 15 nodes and more), the programme is swept densely instead.  The result is the same bit for bit.
  *   beta_ms   host [1]    beta* in milliseconds, +inf if infeasible
  *   m         host [1]    number of segments, 0 if infeasible
  *   cuts      host [k-1]  e_1..e_{m-1}, rest -1   (may be NULL when k == 1)
@@ -345,10 +352,10 @@ pp_status pp_kpath_matching(int32_t n, const uint32_t *bw_kbps, int32_t n_cuts, 
  *   node_speed  host [k]  work units per millisecond of each node; 0 = the node cannot compute
  * c_k = (exact integer sum of the partition's work) / (speed of its node): one IEEE-754 binary64
  * division, in milliseconds, like gamma.  All other arguments, the constraints, the canonical plan
- * and the outputs are those of pp_problem_create + pp_solve_exact.  One call does everything
- * (allocates its tables, runs, frees); synchronous, legacy default stream.  The state table holds
- * doubles (k * 2^k * L * 8 bytes) and every compute time has its own table entry (k * L * L * 8
- * bytes): PP_ERR_LIMIT beyond k = 16 or L = 256, PP_ERR_NOMEM when the device cannot hold them.
+ * and the outputs are those of pp_problem_create + pp_solve_exact.  One call does everything, with
+ * scratch from the library's pool (k * L * L * 4 bytes of compute times and up to 128 MB of states, room
+ * for all of them, k * 2^(k-1) * L * 4 bytes, only when that is not enough); synchronous, legacy default
+ * stream.  PP_ERR_LIMIT beyond k = 16 or L = 256, PP_ERR_NOMEM when the device cannot hold the scratch.
  * With layer_work all zero the result is that of pp_solve_exact.
  */
 #define PP_COMPUTE_MAX_K 16
@@ -359,15 +366,16 @@ pp_status pp_solve_exact_compute(int32_t L, const uint64_t *layer_out_bits, cons
                                  int32_t *cuts, int32_t *placement);
 
 /* Device-time breakdown of the last exact solve of `p`; synchronises the problem's stream.
- * ms_total is always measured.  ms_rank, ms_sweep and ms_finalize need events between the
- * phases, which keep one phase's kernels from being launched under the tail of the previous
- * one: they are recorded only after pp_problem_set_profiling(p, 1) and read 0 otherwise. */
+ * ms_total is always measured.  ms_rank, ms_sweep and ms_finalize are the phases of the dense
+ * search: after pp_problem_set_profiling(p, 1) every solve takes it, with events between the phases
+ * (which keep one phase's kernels from being launched under the tail of the previous one); they
+ * read 0 otherwise. */
 pp_status pp_last_solve_profile(pp_problem *p, pp_profile *out);
 pp_status pp_problem_set_profiling(pp_problem *p, int32_t on);
 
 /* Test hook: after a solve, copy one row of the state table to the host as latencies:
  * row_out[c] = value of state (mask, v, c) in milliseconds (+inf if unreachable), c = 0..L-1.
- * `mask` must contain node v.  Synchronous. */
+ * `mask` must contain node v.  Synchronous; runs the dense sweep first when the last solve did not. */
 pp_status pp_debug_read_state_row(pp_problem *p, uint32_t mask, int32_t v, double *row_out);
 
 /* Test hook (host only, needs no device): the order in which the sweep lists the non-empty node
@@ -395,7 +403,7 @@ pp_status pp_debug_fail_alloc(int32_t nth);
 /* Force (1) or forbid (0) the generic sweep kernel; 2 = automatic choice among the kernels that
  * take one source mask per warp (the two-mask kernel is left out); 3 = the two-mask kernel on every
  * level it can run, however small; -1 restores the automatic choice.  Meant for tests that want
- * every kernel checked on the same instance. */
+ * every kernel checked on the same instance; any mode but -1 takes the dense sweep. */
 pp_status pp_problem_force_generic(pp_problem *p, int32_t mode);
 
 /*

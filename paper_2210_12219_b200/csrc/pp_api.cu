@@ -17,27 +17,39 @@
 using namespace pp;
 
 struct pp_problem {
-    int L = 0, k = 0, Lpad = 0, U = 0, elem = 2;
+    int L = 0, k = 0;
     std::vector<uint64_t> bits, mem, cap, M;
-    std::vector<uint32_t> bw, ubw;
-    std::vector<int16_t> lo, pair_u;
-    unsigned char *d_inputs = nullptr;  // one allocation for all small device arrays
-    unsigned char *d_work = nullptr;    // exact-search scratch (own or caller's)
+    std::vector<uint32_t> bw;
+    std::vector<int16_t> lo;
+    unsigned char *d_inputs = nullptr;  // one allocation: the inputs, the counters, a result record
+    size_t inputs_bytes = 0;
+    bool uploaded = false;              // the inputs have been copied (queued on `stream`)
+    unsigned char *d_sparse = nullptr;  // scratch of the bounded search when there is no workspace
+    unsigned char *d_work = nullptr;    // workspace (own or caller's): either search runs in it
     uint64_t work_bytes = 0;
     bool own_work = false;
+    int sms = 0;                        // multiprocessors of the device the problem lives on
     cudaStream_t stream = nullptr;
-    cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
-    pp_solution h_sol_buf{};       // host copy of the result record
-    int32_t h_err_buf = 0;
-    pp_solution *h_sol = &h_sol_buf;
+    cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};  // of the dense search, created by its first run
     pp_solution *d_sol = nullptr;
-    int32_t *h_err = &h_err_buf;
-    Dev d{};
+    PruneNote *d_note = nullptr;
+    PruneDev prune{};
     bool solved = false, profiled = false;
-    int sweep_launches = 0, total_launches = 0, fast_used = 0, pair_levels = 0;
+    bool sparse_ran = false;            // the last solve ran the bounded search
+    bool table_whole = false;           // ... the dense one: its table holds every state
+    PruneNote note{};                   // of the last synchronous bounded search
+    bool note_on_device = false;
     int force_generic = -1;
     bool profiling = false;             // record events between the phases of a solve
-    bool mask_swaps = false;            // the mask list pairs up (see mask_list)
+
+    // what only the dense search needs, prepared by its first run
+    bool dense_dims = false, dense_ready = false;
+    int Lpad = 0, U = 0, elem = 2;
+    std::vector<uint32_t> ubw;
+    std::vector<int16_t> pair_u;
+    unsigned char *d_dense = nullptr;
+    Dev d{};
+    int sweep_launches = 0, total_launches = 0, fast_used = 0, pair_levels = 0;
     std::vector<signed char> pair_lvl;  // per level: 1 = two-mask kernel, 0 = one-mask, -1 = not decided yet
 };
 
@@ -177,8 +189,10 @@ cudaError_t lane_tables(int k, LaneTables *out)
     return cudaSuccess;
 }
 
-// Staging buffers of the host-pointer entry points come from a pool of the library's own that
-// keeps its memory between calls (the default pool would hand it back at every synchronisation).
+// Staging buffers and small scratch come from a pool of the library's own that keeps up to
+// kPoolKeepBytes between calls (the default pool would hand everything back at every
+// synchronisation); what is free beyond that goes back to the device at the next one.
+constexpr unsigned long long kPoolKeepBytes = 1ull << 30;
 cudaError_t staging_alloc(void **ptr, size_t bytes, cudaStream_t s)
 {
     static std::mutex mu;
@@ -198,7 +212,7 @@ cudaError_t staging_alloc(void **ptr, size_t bytes, cudaStream_t s)
             props.location.id = dev;
             e = cudaMemPoolCreate(&pools[dev], &props);
             if (e != cudaSuccess) return e;
-            unsigned long long keep = ~0ull;
+            unsigned long long keep = kPoolKeepBytes;
             e = cudaMemPoolSetAttribute(pools[dev], cudaMemPoolAttrReleaseThreshold, &keep);
             if (e != cudaSuccess) return e;
         }
@@ -218,6 +232,16 @@ pp_status from_cuda(cudaError_t e)
         cudaError_t e__ = (call);                       \
         if (e__ != cudaSuccess) return from_cuda(e__);  \
     } while (0)
+
+// Multiprocessors of a device, asked for once.
+cudaError_t multiprocessors(int dev, int *sms)
+{
+    static std::atomic<int> known[64];
+    if (dev >= 0 && dev < 64 && (*sms = known[dev].load(std::memory_order_relaxed)) > 0) return cudaSuccess;
+    const cudaError_t e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess && dev >= 0 && dev < 64) known[dev].store(*sms, std::memory_order_relaxed);
+    return e;
+}
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -262,6 +286,208 @@ pp_status validate(int32_t L, const uint64_t *bits, const uint64_t *mem, int32_t
     return PP_OK;
 }
 
+// ---- the bounded search (pp_prune.cu) ----------------------------------------------------------
+
+// Rows of the dense programme: (node set, last node) over all sets of two nodes and more.
+unsigned long long rows_all(int k) { return ((unsigned long long)k << (k - 1)); }
+
+// A synchronous solve gives the bounded search up after this many rows and lets the dense sweep do the
+// rest, which moves more rows per microsecond once the frontier is not sparse.  Up to k = 14 it is never
+// reached.  An asynchronous solve cannot look at the outcome: it has room for every row.
+constexpr unsigned long long kSparseRows = 160000;
+// Without a workspace of the caller the rows live in pooled scratch of at most this size.
+constexpr unsigned long long kSparseScratchBytes = 128ull << 20;
+
+struct SparseLayout {
+    size_t live, rowmap, list, gam, gmin, rows;
+};
+SparseLayout sparse_layout(int k, int Lp)
+{
+    SparseLayout w;
+    size_t o = 0;
+    w.live = o;   o = align_up(o + ((size_t)4 << k), 256);
+    w.rowmap = o; o = align_up(o + ((size_t)k * 8 << k), 256);
+    w.list = o;   o = align_up(o + ((size_t)4 << k), 256);
+    w.gam = o;    o = align_up(o + (size_t)k * k * Lp * 4, 256);
+    w.gmin = o;   o = align_up(o + (size_t)k * k * 4, 256);
+    w.rows = o;
+    return w;
+}
+size_t sparse_bytes(int k, int Lp, unsigned long long limit)
+{
+    const unsigned long long rows = std::min(rows_all(k), limit / ((unsigned long long)Lp * 4));
+    return sparse_layout(k, Lp).rows + (size_t)rows * Lp * 4;
+}
+
+void bind_sparse(PruneDev &q, unsigned char *b, uint64_t bytes)
+{
+    const SparseLayout w = sparse_layout(q.k, q.Lp);
+    q.live = reinterpret_cast<uint32_t *>(b + w.live);
+    q.rowmap = reinterpret_cast<unsigned long long *>(b + w.rowmap);
+    q.list = reinterpret_cast<uint32_t *>(b + w.list);
+    q.gam = reinterpret_cast<uint32_t *>(b + w.gam);
+    q.gmin = reinterpret_cast<uint32_t *>(b + w.gmin);
+    q.rows = reinterpret_cast<uint32_t *>(b + w.rows);
+    q.row_cap = (bytes - w.rows) / ((size_t)q.Lp * 4);
+}
+
+// lo[w][c'] = earliest previous cut c >= 0 such that layers c+1..c' fit on w; c' itself when not even
+// layer c' alone fits.  Non-decreasing in c'.
+void window_table(int L, int k, const uint64_t *M, const uint64_t *cap, int16_t *lo)
+{
+    for (int w = 0; w < k; ++w) {
+        int c = 0;
+        for (int c2 = 0; c2 < L; ++c2) {
+            while (c < c2 && M[c2 + 1] - M[c + 1] > cap[w]) ++c;
+            lo[(size_t)w * L + c2] = (int16_t)c;
+        }
+    }
+}
+
+// Range of the keys: the smallest and the largest positive quotient of Eq. 3 the inputs allow.
+void quotient_range(int L, const uint64_t *num, int n, const uint32_t *den, double *lo, double *hi)
+{
+    uint64_t a = ~0ull, b = 0;
+    uint32_t c = ~0u, e = 0;
+    for (int i = 0; i < L; ++i) {
+        if (num[i]) a = std::min(a, num[i]);
+        b = std::max(b, num[i]);
+    }
+    for (int i = 0; i < n; ++i) {
+        if (den[i]) c = std::min(c, den[i]);
+        e = std::max(e, den[i]);
+    }
+    if (!b || !e) return;  // no positive quotient
+    *lo = std::min(*lo, (double)a / (double)e);
+    *hi = std::max(*hi, (double)b / (double)c);
+}
+
+// Copies the inputs to the device, ordered on the problem's stream.  The staging memory may go as soon
+// as the call returns: copies from pageable memory leave it first.
+pp_status upload_inputs(pp_problem *p, bool wait)
+{
+    if (p->uploaded) return PP_OK;
+    const int L = p->L, k = p->k;
+    std::vector<unsigned char> st;
+    try {
+        st.assign(p->inputs_bytes, 0);
+    } catch (const std::bad_alloc &) {
+        return PP_ERR_NOMEM;
+    }
+    auto put = [&](const void *dst, const void *src, size_t n) {
+        std::memcpy(st.data() + (static_cast<const unsigned char *>(dst) - p->d_inputs), src, n);
+    };
+    put(p->d.bits, p->bits.data(), (size_t)L * 8);
+    put(p->d.M, p->M.data(), (size_t)(L + 1) * 8);
+    put(p->d.cap, p->cap.data(), (size_t)k * 8);
+    put(p->d.bw, p->bw.data(), (size_t)k * k * 4);
+    put(p->d.lo, p->lo.data(), (size_t)k * L * 2);
+    PruneCtl ctl;
+    prune_ctl_init(&ctl);
+    put(p->prune.ctl, &ctl, sizeof ctl);
+    if (wait) PP_CUDA(cudaMemcpy(p->d_inputs, st.data(), st.size(), cudaMemcpyHostToDevice));
+    else PP_CUDA(cudaMemcpyAsync(p->d_inputs, st.data(), st.size(), cudaMemcpyHostToDevice, p->stream));
+    p->uploaded = true;
+    return PP_OK;
+}
+
+// Page-locked result records of the synchronous calls, one per call in flight: the kernel writes its
+// result straight into host memory.  Chunks of 32; all but one chunk are given back when unused.
+struct HostSlot {
+    pp_solution sol;
+    PruneNote note;
+};
+class HostSlots {
+public:
+    HostSlot *take()
+    {
+        std::lock_guard<std::mutex> lock(mu_);
+        for (auto &c : chunks_)
+            if (c.free) return from(c);
+        void *ptr = nullptr;
+        if (cudaHostAlloc(&ptr, 32 * sizeof(HostSlot), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        try {
+            chunks_.push_back({static_cast<HostSlot *>(ptr), 0xFFFFFFFFu});
+        } catch (const std::bad_alloc &) {
+            cudaFreeHost(ptr);
+            return nullptr;
+        }
+        return from(chunks_.back());
+    }
+    void give(HostSlot *s)
+    {
+        std::lock_guard<std::mutex> lock(mu_);
+        for (size_t i = 0; i < chunks_.size(); ++i) {
+            const ptrdiff_t at = s - chunks_[i].base;
+            if (at < 0 || at >= 32) continue;
+            chunks_[i].free |= 1u << at;
+            if (i > 0 && chunks_[i].free == 0xFFFFFFFFu) {
+                cudaFreeHost(chunks_[i].base);
+                chunks_.erase(chunks_.begin() + (long)i);
+            }
+            return;
+        }
+    }
+
+private:
+    struct Chunk {
+        HostSlot *base;
+        uint32_t free;
+    };
+    static HostSlot *from(Chunk &c)
+    {
+        const int at = __builtin_ctz(c.free);
+        c.free &= ~(1u << at);
+        return c.base + at;
+    }
+    std::mutex mu_;
+    std::vector<Chunk> chunks_;
+};
+HostSlots g_slots;
+
+// ---- the dense search (pp_rank.cu, pp_sweep*.cu) ------------------------------------------------
+
+// Sizes of its tables: distinct usable bandwidths, element width, row stride.
+void dense_dims(pp_problem *p)
+{
+    if (p->dense_dims) return;
+    const int k = p->k, L = p->L;
+    std::map<uint32_t, int> seen;
+    p->ubw.clear();
+    p->pair_u.assign((size_t)k * k, -1);
+    for (int v = 0; v < k; ++v)
+        for (int w = 0; w < k; ++w) {
+            uint32_t b = p->bw[(size_t)v * k + w];
+            if (v == w || b == 0) continue;
+            auto it = seen.find(b);
+            if (it == seen.end()) {
+                it = seen.emplace(b, (int)p->ubw.size()).first;
+                p->ubw.push_back(b);
+            }
+            p->pair_u[(size_t)v * k + w] = (int16_t)it->second;
+        }
+    p->U = (int)p->ubw.size();
+    if (p->ubw.empty()) p->ubw.push_back(0);  // keep the upload non-empty; U stays 0
+    // 16-bit ranks when 0, 1..L*U and the +inf code all fit
+    p->elem = ((uint64_t)L * (uint64_t)std::max(p->U, 1) + 1 <= 65534) ? 2 : 4;
+    const int per32 = 32 / p->elem;
+    p->Lpad = (L + per32 - 1) / per32 * per32;
+    Dev &d = p->d;
+    d.Lpad = p->Lpad; d.U = p->U; d.elem = p->elem;
+    p->dense_dims = true;
+}
+
+// Bytes of a workspace that either search can run in.
+uint64_t workspace_bytes(pp_problem *p)
+{
+    dense_dims(p);
+    return std::max<uint64_t>(work_layout(p->L, p->k, p->Lpad, p->U, p->elem).total,
+                              sparse_bytes(p->k, p->prune.Lp, ~0ull));
+}
+
 void bind_work(pp_problem *p)
 {
     WorkLayout w = work_layout(p->L, p->k, p->Lpad, p->U, p->elem);
@@ -281,52 +507,152 @@ void bind_work(pp_problem *p)
 pp_status ensure_work(pp_problem *p)
 {
     if (p->d_work) return PP_OK;
-    WorkLayout w = work_layout(p->L, p->k, p->Lpad, p->U, p->elem);
     void *ptr = nullptr;
     if (alloc_should_fail()) return PP_ERR_NOMEM;
-    PP_CUDA(cudaMalloc(&ptr, w.total));
+    const uint64_t bytes = workspace_bytes(p);
+    PP_CUDA(cudaMalloc(&ptr, bytes));
     p->d_work = static_cast<unsigned char *>(ptr);
-    p->work_bytes = w.total;
+    p->work_bytes = bytes;
     p->own_work = true;
     bind_work(p);
+    bind_sparse(p->prune, p->d_work, bytes);
     return PP_OK;
 }
 
-pp_status queue_solve(pp_problem *p, pp_solution *sol_dev)
+// Window constants of the register-tiled kernels, the list of node sets and the bandwidth classes on
+// the device, and which kernel takes which level.
+pp_status dense_prepare(pp_problem *p)
+{
+    if (p->dense_ready) return PP_OK;
+    const int L = p->L, k = p->k;
+    Dev &d = p->d;
+    try {
+        dense_dims(p);
+        const MaskList &ml = mask_list(k);
+        // constants of the register-tiled sweep, when the instance is inside its envelope
+        std::vector<unsigned char> fmeta(fast_meta_bytes()), pmeta;
+        std::vector<uint32_t> gmeta;
+        const bool tiled = p->elem == 2 && p->Lpad <= 240 && k >= 2;
+        const bool has_fast = tiled && fast_meta_build(L, k, p->lo.data(), fmeta.data());
+        if (has_fast && ml.swaps) {
+            pmeta.resize(pair_meta_bytes());
+            if (!pair_meta_build(L, k, p->lo.data(), pmeta.data())) pmeta.clear();
+        }
+        if (!has_fast && tiled) {
+            gmeta.resize((size_t)k * p->Lpad);
+            d.gen_levels = gen_meta_build(L, k, p->Lpad, p->lo.data(), gmeta.data());
+        }
+        struct Part { const void *src; size_t bytes; size_t off; };
+        Part parts[5] = {{p->pair_u.data(), p->pair_u.size() * 2, 0}, {p->ubw.data(), p->ubw.size() * 4, 0},
+                         {fmeta.data(), fmeta.size(), 0}, {gmeta.data(), gmeta.size() * 4, 0}, {pmeta.data(), pmeta.size(), 0}};
+        size_t total = 0;
+        for (auto &q : parts) { q.off = total; total = align_up(total + q.bytes, 256); }
+        // one staging buffer, one copy: the parts are small and a copy per part costs more than the bytes
+        std::vector<unsigned char> staging(total, 0);
+        for (auto &q : parts)
+            if (q.bytes) std::memcpy(staging.data() + q.off, q.src, q.bytes);
+        DeviceMasks dmasks;
+        PP_CUDA(device_masks(k, ml, &dmasks));
+        if (!p->d_dense) PP_CUDA(staging_alloc(reinterpret_cast<void **>(&p->d_dense), total, nullptr));
+        PP_CUDA(cudaMemcpy(p->d_dense, staging.data(), total, cudaMemcpyHostToDevice));
+        for (auto &e : p->ev)
+            if (!e) PP_CUDA(cudaEventCreate(&e));
+        unsigned char *b = p->d_dense;
+        d.pair_u = reinterpret_cast<int16_t *>(b + parts[0].off);
+        d.ubw = reinterpret_cast<uint32_t *>(b + parts[1].off);
+        d.fast_meta = has_fast ? b + parts[2].off : nullptr;
+        d.gen_meta = gmeta.empty() ? nullptr : reinterpret_cast<uint32_t *>(b + parts[3].off);
+        d.pair_meta = pmeta.empty() ? nullptr : b + parts[4].off;
+        d.masks = dmasks.masks;  // shared by every problem of this k on this device
+        d.level_off = dmasks.level_off;
+        p->pair_lvl.assign(k + 2, -1);
+    } catch (const std::bad_alloc &) {
+        return PP_ERR_NOMEM;
+    }
+    p->dense_ready = true;
+    return PP_OK;
+}
+
+// The kernels the dense search of this problem consists of (also what pp_last_solve_profile reports).
+void dense_plan(pp_problem *p, bool *fast)
+{
+    const Dev &d = p->d;
+    *fast = p->force_generic != 1 && fast_sweep_supported(d);
+    p->pair_levels = 0;
+    const int top = std::min(p->k, p->L);
+    for (int level = 2; level <= top; ++level) {
+        if (!*fast || p->force_generic == 2) continue;
+        if (p->pair_lvl[level] < 0) p->pair_lvl[level] = pair_sweep_takes(d, level, p->force_generic == 3) ? 1 : 0;
+        p->pair_levels += p->pair_lvl[level];
+    }
+    p->fast_used = *fast ? (d.fast_meta ? 1 : 2) : 0;
+}
+
+pp_status queue_dense(pp_problem *p, pp_solution *sol_dev)
 {
     pp_status st = ensure_work(p);
+    if (st == PP_OK) st = upload_inputs(p, false);
+    if (st == PP_OK) st = dense_prepare(p);
     if (st != PP_OK) return st;
     cudaStream_t s = p->stream;
-    bool fast = fast_sweep_supported(p->d);
-    if (p->force_generic == 1) fast = false;
+    bool fast = false;
+    dense_plan(p, &fast);
     const Dev &d = p->d;
     int launches = 0;
     PP_CUDA(cudaEventRecord(p->ev[0], s));
     PP_CUDA(launch_rank_base(d, s, &launches));
     // an event between two kernels ends the programmatic overlap of their launches: only on request
     if (p->profiling) PP_CUDA(cudaEventRecord(p->ev[1], s));
-    int sweep = 0, pairs = 0;
+    int sweep = 0;
     const int top = std::min(p->k, p->L);
     for (int level = 2; level <= top; ++level) {
         const bool first = level == 2;
-        if (fast && p->force_generic != 2) {
-            if (p->pair_lvl[level] < 0) p->pair_lvl[level] = pair_sweep_takes(d, level, p->force_generic == 3) ? 1 : 0;
-            PP_CUDA(p->pair_lvl[level] ? launch_sweep_pair(d, level, s, first) : launch_sweep_fast(d, level, s, first));
-            pairs += p->pair_lvl[level];
-        } else {
-            PP_CUDA(fast ? launch_sweep_fast(d, level, s, first) : launch_sweep_generic(d, level, s));
-        }
+        if (!fast) PP_CUDA(launch_sweep_generic(d, level, s));
+        else if (p->force_generic != 2 && p->pair_lvl[level]) PP_CUDA(launch_sweep_pair(d, level, s, first));
+        else PP_CUDA(launch_sweep_fast(d, level, s, first));
         ++sweep;
     }
     if (p->profiling) PP_CUDA(cudaEventRecord(p->ev[2], s));
     PP_CUDA(launch_finalize(d, sol_dev, s, true));
     PP_CUDA(cudaEventRecord(p->ev[3], s));
     p->sweep_launches = sweep;
-    p->pair_levels = pairs;
-    p->total_launches = launches + sweep + 1;
-    p->fast_used = fast ? (p->d.fast_meta ? 1 : 2) : 0;
+    p->total_launches += launches + sweep + 1;
     p->solved = true;
     p->profiled = p->profiling;
+    p->table_whole = true;
+    return PP_OK;
+}
+
+// The bounded search is the way an ordinary solve takes; a caller that pins a sweep kernel or asks for
+// the times of the dense search's phases gets the dense search.
+bool takes_sparse(const pp_problem *p) { return p->force_generic == -1 && !p->profiling; }
+
+// Scratch of the bounded search: the workspace, else a pooled buffer of its own.
+pp_status ensure_sparse(pp_problem *p)
+{
+    if (p->d_work || p->d_sparse) return PP_OK;
+    const size_t bytes = sparse_bytes(p->k, p->prune.Lp, kSparseScratchBytes);
+    PP_CUDA(staging_alloc(reinterpret_cast<void **>(&p->d_sparse), bytes, p->stream));
+    bind_sparse(p->prune, p->d_sparse, bytes);
+    return PP_OK;
+}
+
+// row_limit: rows after which the search gives up (note->dense).
+pp_status queue_sparse(pp_problem *p, pp_solution *sol, PruneNote *note, unsigned long long row_limit)
+{
+    pp_status st = upload_inputs(p, false);
+    if (st != PP_OK) return st;
+    PruneDev q = p->prune;
+    q.out = sol;
+    q.note = note;
+    q.row_cap = std::min(q.row_cap, row_limit);
+    PP_CUDA(launch_prune(q, p->sms, p->stream));
+    p->total_launches = 1;
+    p->sweep_launches = 1;
+    p->solved = true;
+    p->profiled = false;
+    p->sparse_ran = true;
+    p->table_whole = false;
     return PP_OK;
 }
 
@@ -368,106 +694,23 @@ pp_status pp_problem_create(int32_t L, const uint64_t *layer_out_bits,
         // memory prefix sums: segment first..last needs M[last+1] - M[first] bytes
         p->M.assign(L + 1, 0);
         for (int i = 0; i < L; ++i) p->M[i + 1] = p->M[i] + p->mem[i];
-        // window table: lo[w][c'] = earliest previous cut c >= 0 such that layers c+1..c' fit on
-        // w; c' itself when not even layer c' alone fits.  Non-decreasing in c'.
         p->lo.assign((size_t)k * L, 0);
-        for (int w = 0; w < k; ++w) {
-            int c = 0;
-            for (int c2 = 0; c2 < L; ++c2) {
-                while (c < c2 && p->M[c2 + 1] - p->M[c + 1] > p->cap[w]) ++c;
-                p->lo[(size_t)w * L + c2] = (int16_t)c;
-            }
-        }
-        // distinct usable bandwidths
-        std::map<uint32_t, int> seen;
-        p->pair_u.assign((size_t)k * k, -1);
-        for (int v = 0; v < k; ++v)
-            for (int w = 0; w < k; ++w) {
-                uint32_t b = p->bw[(size_t)v * k + w];
-                if (v == w || b == 0) continue;
-                auto it = seen.find(b);
-                if (it == seen.end()) {
-                    it = seen.emplace(b, (int)p->ubw.size()).first;
-                    p->ubw.push_back(b);
-                }
-                p->pair_u[(size_t)v * k + w] = (int16_t)it->second;
-            }
-        p->U = (int)p->ubw.size();
-        if (p->ubw.empty()) p->ubw.push_back(0);  // keep the upload non-empty; U stays 0
-        // 16-bit ranks when 0, 1..L*U and the +inf code all fit
-        p->elem = ((uint64_t)L * (uint64_t)std::max(p->U, 1) + 1 <= 65534) ? 2 : 4;
-        const int per32 = 32 / p->elem;
-        p->Lpad = (L + per32 - 1) / per32 * per32;
-        // masks by (popcount, value)
-        const MaskList &ml = mask_list(k);
-        p->mask_swaps = ml.swaps;
-        p->pair_lvl.assign(k + 2, -1);
+        window_table(L, k, p->M.data(), p->cap.data(), p->lo.data());
     } catch (const std::bad_alloc &) {
         delete p;
         return PP_ERR_NOMEM;
     }
-
-    // constants of the register-tiled sweep, when the instance is inside its envelope
-    std::vector<unsigned char> fmeta;
-    bool has_fast = false;
-    try {
-        fmeta.resize(fast_meta_bytes());
-        has_fast = p->elem == 2 && p->Lpad <= 240 && k >= 2 &&
-                   fast_meta_build(L, k, p->lo.data(), fmeta.data());
-    } catch (const std::bad_alloc &) {
-        delete p;
-        return PP_ERR_NOMEM;
-    }
-    std::vector<unsigned char> pmeta;
-    try {
-        if (has_fast && p->mask_swaps) {
-            pmeta.resize(pair_meta_bytes());
-            if (!pair_meta_build(L, k, p->lo.data(), pmeta.data())) pmeta.clear();
-        }
-    } catch (const std::bad_alloc &) {
-        delete p;
-        return PP_ERR_NOMEM;
-    }
-    std::vector<uint32_t> gmeta;
-    try {
-        if (!has_fast && p->elem == 2 && p->Lpad <= 240 && k >= 2) {
-            gmeta.resize((size_t)k * p->Lpad);
-            p->d.gen_levels = gen_meta_build(L, k, p->Lpad, p->lo.data(), gmeta.data());
-        }
-    } catch (const std::bad_alloc &) {
-        delete p;
-        return PP_ERR_NOMEM;
-    }
-    // upload the small arrays in one allocation
-    struct Part { const void *src; size_t bytes; size_t off; };
-    std::vector<Part> parts = {
-        {p->bits.data(), p->bits.size() * 8, 0},       {p->M.data(), p->M.size() * 8, 0},
-        {p->cap.data(), p->cap.size() * 8, 0},         {p->bw.data(), p->bw.size() * 4, 0},
-        {p->lo.data(), p->lo.size() * 2, 0},           {p->pair_u.data(), p->pair_u.size() * 2, 0},
-        {p->ubw.data(), p->ubw.size() * 4, 0},
-        {nullptr, 0, 0} /* masks: shared */,           {nullptr, 0, 0} /* level_off: shared */,
-        {nullptr, 8, 0} /* best */,                    {nullptr, 4, 0} /* err */,
-        {nullptr, sizeof(pp_solution), 0} /* solution */,
-        {fmeta.data(), fmeta.size(), 0},
-        {gmeta.data(), gmeta.size() * 4, 0},
-        {pmeta.data(), pmeta.size(), 0}};
-    size_t total = 0;
-    for (auto &q : parts) { q.off = total; total = align_up(total + q.bytes, 256); }
-    // one staging buffer, one copy: the parts are small and a copy per part costs more than the bytes
-    std::vector<unsigned char> staging;
-    try {
-        staging.assign(total, 0);
-    } catch (const std::bad_alloc &) {
-        delete p;
-        return PP_ERR_NOMEM;
-    }
-    for (auto &q : parts)
-        if (q.src && q.bytes) std::memcpy(staging.data() + q.off, q.src, q.bytes);
-    DeviceMasks dmasks;
-    cudaError_t e = device_masks(k, mask_list(k), &dmasks);
+    // one device buffer for the inputs, the counters of the searches and a result record; the copy is
+    // queued by the first call that needs it, on the stream the problem has by then
+    const size_t bytes[9] = {(size_t)L * 8, (size_t)(L + 1) * 8, (size_t)k * 8, (size_t)k * k * 4, (size_t)k * L * 2,
+                             sizeof(PruneCtl), 8 /* best */, 4 /* err */, sizeof(pp_solution) + sizeof(PruneNote)};
+    size_t off[9], total = 0;
+    for (int i = 0; i < 9; ++i) { off[i] = total; total = align_up(total + bytes[i], i < 4 ? 16 : 128); }
+    p->inputs_bytes = total;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = multiprocessors(dev, &p->sms);
     if (e == cudaSuccess) e = staging_alloc(reinterpret_cast<void **>(&p->d_inputs), total, nullptr);
-    if (e == cudaSuccess) e = cudaMemcpy(p->d_inputs, staging.data(), total, cudaMemcpyHostToDevice);
-    for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = cudaEventCreate(&p->ev[i]);
     if (e != cudaSuccess) {
         pp_status rc = from_cuda(e);
         pp_problem_destroy(p);
@@ -475,22 +718,24 @@ pp_status pp_problem_create(int32_t L, const uint64_t *layer_out_bits,
     }
     unsigned char *b = p->d_inputs;
     Dev &d = p->d;
-    d.L = L; d.k = k; d.Lpad = p->Lpad; d.U = p->U; d.elem = p->elem;
-    d.bits = reinterpret_cast<uint64_t *>(b + parts[0].off);
-    d.M = reinterpret_cast<uint64_t *>(b + parts[1].off);
-    d.cap = reinterpret_cast<uint64_t *>(b + parts[2].off);
-    d.bw = reinterpret_cast<uint32_t *>(b + parts[3].off);
-    d.lo = reinterpret_cast<int16_t *>(b + parts[4].off);
-    d.pair_u = reinterpret_cast<int16_t *>(b + parts[5].off);
-    d.ubw = reinterpret_cast<uint32_t *>(b + parts[6].off);
-    d.masks = dmasks.masks;  // shared by every problem of this k on this device
-    d.level_off = dmasks.level_off;
-    d.best = reinterpret_cast<unsigned long long *>(b + parts[9].off);
-    d.err = reinterpret_cast<int32_t *>(b + parts[10].off);
-    p->d_sol = reinterpret_cast<pp_solution *>(b + parts[11].off);
-    d.fast_meta = has_fast ? b + parts[12].off : nullptr;
-    d.gen_meta = gmeta.empty() ? nullptr : reinterpret_cast<uint32_t *>(b + parts[13].off);
-    d.pair_meta = pmeta.empty() ? nullptr : b + parts[14].off;
+    d.L = L; d.k = k;
+    d.bits = reinterpret_cast<uint64_t *>(b + off[0]);
+    d.M = reinterpret_cast<uint64_t *>(b + off[1]);
+    d.cap = reinterpret_cast<uint64_t *>(b + off[2]);
+    d.bw = reinterpret_cast<uint32_t *>(b + off[3]);
+    d.lo = reinterpret_cast<int16_t *>(b + off[4]);
+    d.best = reinterpret_cast<unsigned long long *>(b + off[6]);
+    d.err = reinterpret_cast<int32_t *>(b + off[7]);
+    p->d_sol = reinterpret_cast<pp_solution *>(b + off[8]);
+    p->d_note = reinterpret_cast<PruneNote *>(b + off[8] + sizeof(pp_solution));
+    PruneDev &q = p->prune;
+    q.L = L; q.k = k; q.Lp = prune_row_pad(L);
+    q.bits = d.bits; q.M = d.M; q.cap = d.cap; q.bw = d.bw; q.lo = d.lo;
+    q.ctl = reinterpret_cast<PruneCtl *>(b + off[5]);
+    double lo = std::numeric_limits<double>::max(), hi = 0.0;
+    quotient_range(L, p->bits.data(), k * k, p->bw.data(), &lo, &hi);
+    prune_key_range(hi > 0.0 ? lo : 1.0, hi > 0.0 ? hi : 1.0, &q);
+    prune_node_bounds(p->cap.data(), p->M[L], &q);
     *out = p;
     return PP_OK;
 }
@@ -499,7 +744,8 @@ void pp_problem_destroy(pp_problem *p)
 {
     if (!p) return;
     if (p->own_work && p->d_work) cudaFree(p->d_work);
-    if (p->d_inputs) cudaFreeAsync(p->d_inputs, p->stream);  // ordered after the problem's queued work
+    for (unsigned char *q : {p->d_inputs, p->d_sparse, p->d_dense})
+        if (q) cudaFreeAsync(q, p->stream);  // ordered after the problem's queued work
     for (auto &e : p->ev)
         if (e) cudaEventDestroy(e);
     delete p;
@@ -508,14 +754,21 @@ void pp_problem_destroy(pp_problem *p)
 pp_status pp_problem_set_stream(pp_problem *p, void *cuda_stream)
 {
     if (!p) return PP_ERR_ARG;
-    p->stream = static_cast<cudaStream_t>(cuda_stream);
-    return PP_OK;
+    cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+    if (s == p->stream) return PP_OK;
+    if (p->uploaded || p->d_sparse) PP_CUDA(cudaStreamSynchronize(p->stream));  // copies and scratch are ordered there
+    p->stream = s;
+    return upload_inputs(p, true);
 }
 
 pp_status pp_problem_workspace_bytes(const pp_problem *p, uint64_t *bytes)
 {
     if (!p || !bytes) return PP_ERR_ARG;
-    *bytes = work_layout(p->L, p->k, p->Lpad, p->U, p->elem).total;
+    try {
+        *bytes = workspace_bytes(const_cast<pp_problem *>(p));
+    } catch (const std::bad_alloc &) {
+        return PP_ERR_NOMEM;
+    }
     return PP_OK;
 }
 
@@ -523,7 +776,10 @@ pp_status pp_problem_set_workspace(pp_problem *p, void *device_buffer, uint64_t 
 {
     if (!p || !device_buffer) return PP_ERR_ARG;
     if (reinterpret_cast<uintptr_t>(device_buffer) % 256) return PP_ERR_ARG;
-    if (bytes < work_layout(p->L, p->k, p->Lpad, p->U, p->elem).total) return PP_ERR_NOMEM;
+    uint64_t need = 0;
+    pp_status st = pp_problem_workspace_bytes(p, &need);
+    if (st != PP_OK) return st;
+    if (bytes < need) return PP_ERR_NOMEM;
     if (p->own_work && p->d_work) {
         cudaStreamSynchronize(p->stream);
         cudaFree(p->d_work);
@@ -533,6 +789,7 @@ pp_status pp_problem_set_workspace(pp_problem *p, void *device_buffer, uint64_t 
     p->own_work = false;
     p->solved = false;
     bind_work(p);
+    bind_sparse(p->prune, p->d_work, bytes);
     return PP_OK;
 }
 
@@ -540,7 +797,7 @@ pp_status pp_problem_force_generic(pp_problem *p, int32_t mode)
 {
     if (!p || mode < -1 || mode > 3) return PP_ERR_ARG;
     p->force_generic = mode;
-    p->pair_lvl.assign(p->k + 2, -1);
+    if (p->dense_ready) p->pair_lvl.assign(p->k + 2, -1);
     return PP_OK;
 }
 
@@ -554,38 +811,107 @@ pp_status pp_problem_set_profiling(pp_problem *p, int32_t on)
 pp_status pp_solve_exact_dev(pp_problem *p, pp_solution *solution_dev)
 {
     if (!p || !solution_dev) return PP_ERR_ARG;
-    return queue_solve(p, solution_dev);
+    try {
+        p->total_launches = 0;
+        p->sparse_ran = false;
+        if (!takes_sparse(p)) return queue_dense(p, solution_dev);
+        // room for every row: pooled scratch where that is small, else a workspace
+        pp_status st = sparse_bytes(p->k, p->prune.Lp, ~0ull) <= kSparseScratchBytes ? ensure_sparse(p) : ensure_work(p);
+        if (st == PP_OK) st = queue_sparse(p, solution_dev, p->d_note, ~0ull);
+        p->note_on_device = true;
+        return st;
+    } catch (const std::bad_alloc &) {
+        return PP_ERR_NOMEM;
+    }
+}
+
+// The bounded search with its result in page-locked memory.  PP_ERR_LIMIT: the frontier outgrew its
+// rows, the dense search has to run.
+static pp_status solve_sparse(pp_problem *p, pp_solution *sol)
+{
+    pp_status st = ensure_sparse(p);
+    if (st != PP_OK) return st;
+    HostSlot *slot = g_slots.take();
+    if (!slot) return PP_ERR_NOMEM;
+    slot->note.dense = -1;
+    st = queue_sparse(p, &slot->sol, &slot->note, kSparseRows);
+    const cudaError_t e = cudaStreamSynchronize(p->stream);
+    if (st == PP_OK) st = from_cuda(e);
+    if (st == PP_OK) {
+        p->note = slot->note;
+        p->note_on_device = false;
+        *sol = slot->sol;
+        if (p->note.dense < 0) {  // a barrier of the kernel gave up: put its counters back
+            PruneCtl ctl;
+            prune_ctl_init(&ctl);
+            cudaMemcpy(p->prune.ctl, &ctl, sizeof ctl, cudaMemcpyHostToDevice);
+            st = PP_ERR_CUDA;
+        } else if (p->note.dense) {
+            st = PP_ERR_LIMIT;
+        } else if (sol->status != PP_OK && sol->status != PP_INFEASIBLE) {
+            st = PP_ERR_CUDA;
+        }
+    }
+    g_slots.give(slot);
+    return st;
 }
 
 pp_status pp_solve_exact(pp_problem *p, double *beta_ms, int32_t *m, int32_t *cuts,
                          int32_t *placement)
 {
     if (!p || !beta_ms || !m || !placement || (!cuts && p->k > 1)) return PP_ERR_ARG;
-    PP_CUDA(cudaMemsetAsync(p->d.err, 0, sizeof(int32_t), p->stream));
-    pp_status st = queue_solve(p, p->d_sol);
-    if (st != PP_OK) return st;
-    PP_CUDA(cudaMemcpyAsync(p->h_sol, p->d_sol, sizeof(pp_solution), cudaMemcpyDeviceToHost, p->stream));
-    PP_CUDA(cudaMemcpyAsync(p->h_err, p->d.err, sizeof(int32_t), cudaMemcpyDeviceToHost, p->stream));
-    PP_CUDA(cudaStreamSynchronize(p->stream));
-    if (*p->h_err) return PP_ERR_CUDA;
-    *beta_ms = p->h_sol->beta_ms;
-    *m = p->h_sol->m;
-    for (int j = 0; j < p->k - 1; ++j) cuts[j] = p->h_sol->cuts[j];
-    for (int j = 0; j < p->k; ++j) placement[j] = p->h_sol->placement[j];
-    return static_cast<pp_status>(p->h_sol->status);
+    pp_solution sol{};
+    try {
+        p->total_launches = 0;
+        p->sparse_ran = false;
+        pp_status st = takes_sparse(p) ? solve_sparse(p, &sol) : PP_ERR_LIMIT;
+        if (st == PP_ERR_LIMIT) {
+            int32_t err = 0;
+            st = upload_inputs(p, false);
+            if (st != PP_OK) return st;
+            PP_CUDA(cudaMemsetAsync(p->d.err, 0, sizeof(int32_t), p->stream));
+            st = queue_dense(p, p->d_sol);
+            if (st != PP_OK) return st;
+            PP_CUDA(cudaMemcpyAsync(&sol, p->d_sol, sizeof sol, cudaMemcpyDeviceToHost, p->stream));
+            PP_CUDA(cudaMemcpyAsync(&err, p->d.err, sizeof err, cudaMemcpyDeviceToHost, p->stream));
+            PP_CUDA(cudaStreamSynchronize(p->stream));
+            if (err) return PP_ERR_CUDA;
+        } else if (st != PP_OK) {
+            return st;
+        }
+    } catch (const std::bad_alloc &) {
+        return PP_ERR_NOMEM;
+    }
+    *beta_ms = sol.beta_ms;
+    *m = sol.m;
+    for (int j = 0; j < p->k - 1; ++j) cuts[j] = sol.cuts[j];
+    for (int j = 0; j < p->k; ++j) placement[j] = sol.placement[j];
+    return static_cast<pp_status>(sol.status);
 }
 
 pp_status pp_last_solve_profile(pp_problem *p, pp_profile *out)
 {
     if (!p || !out || !p->solved) return PP_ERR_ARG;
     PP_CUDA(cudaStreamSynchronize(p->stream));
-    out->ms_rank = out->ms_sweep = out->ms_finalize = 0.0f;
+    pp_status st = dense_prepare(p);
+    if (st != PP_OK) return st;
+    bool fast = false;
+    dense_plan(p, &fast);
+    out->ms_rank = out->ms_sweep = out->ms_finalize = out->ms_total = 0.0f;
+    if (p->sparse_ran) {
+        if (p->note_on_device) PP_CUDA(cudaMemcpy(&p->note, p->d_note, sizeof p->note, cudaMemcpyDeviceToHost));
+        out->ms_total = (float)((double)p->note.ns * 1e-6);
+    }
+    if (p->table_whole) {
+        float ms = 0.0f;
+        PP_CUDA(cudaEventElapsedTime(&ms, p->ev[0], p->ev[3]));
+        out->ms_total += ms;
+    }
     if (p->profiled) {
         PP_CUDA(cudaEventElapsedTime(&out->ms_rank, p->ev[0], p->ev[1]));
         PP_CUDA(cudaEventElapsedTime(&out->ms_sweep, p->ev[1], p->ev[2]));
         PP_CUDA(cudaEventElapsedTime(&out->ms_finalize, p->ev[2], p->ev[3]));
     }
-    PP_CUDA(cudaEventElapsedTime(&out->ms_total, p->ev[0], p->ev[3]));
     out->sweep_launches = p->sweep_launches;
     out->total_launches = p->total_launches;
     out->state_bytes = p->elem;
@@ -600,6 +926,8 @@ pp_status pp_eval_plans_dev(pp_problem *p, int64_t B, const uint8_t *nseg, const
     if (!p || B < 0) return PP_ERR_ARG;
     if (B == 0) return PP_OK;
     if (!nseg || !ends || !nodes || !beta_ms || !plan_status) return PP_ERR_ARG;
+    pp_status st = upload_inputs(p, false);
+    if (st != PP_OK) return st;
     PP_CUDA(launch_eval(p->d, B, nseg, ends, nodes, beta_ms, plan_status, p->stream));
     return PP_OK;
 }
@@ -615,6 +943,8 @@ pp_status pp_eval_plans(pp_problem *p, int64_t B, const uint8_t *nseg, const int
     size_t o_ends = align_up(b_nseg, 256), o_nodes = align_up(o_ends + b_rows, 256);
     size_t o_beta = align_up(o_nodes + b_rows, 256), o_st = align_up(o_beta + b_beta, 256);
     size_t total = o_st + (size_t)B;
+    pp_status st = upload_inputs(p, false);
+    if (st != PP_OK) return st;
     unsigned char *buf = nullptr;
     cudaStream_t s = p->stream;
     PP_CUDA(staging_alloc(reinterpret_cast<void **>(&buf), total, s));
@@ -640,6 +970,8 @@ pp_status pp_eval_plans_packed_dev(pp_problem *p, int64_t B, int64_t total, cons
     if (!p || B < 0 || total < 0) return PP_ERR_ARG;
     if (B == 0) return PP_OK;
     if (!nseg || !plan_off || !beta_ms || !plan_status || ((!ends || !nodes) && total > 0)) return PP_ERR_ARG;
+    pp_status st = upload_inputs(p, false);
+    if (st != PP_OK) return st;
     PP_CUDA(launch_eval_packed(p->d, B, total, nseg, plan_off, ends, nodes, beta_ms, plan_status, p->stream));
     return PP_OK;
 }
@@ -655,6 +987,8 @@ pp_status pp_eval_plans_packed(pp_problem *p, int64_t B, int64_t total, const ui
     const size_t o_off = align_up(nB, 256), o_ends = align_up(o_off + (nB + 1) * 4, 256);
     const size_t o_nodes = align_up(o_ends + nT * 2, 256), o_beta = align_up(o_nodes + nT, 256);
     const size_t o_st = align_up(o_beta + nB * 8, 256), bytes = o_st + nB;
+    pp_status st = upload_inputs(p, false);
+    if (st != PP_OK) return st;
     unsigned char *buf = nullptr;
     cudaStream_t s = p->stream;
     PP_CUDA(staging_alloc(reinterpret_cast<void **>(&buf), bytes, s));
@@ -680,6 +1014,8 @@ pp_status pp_random_plans_dev(pp_problem *p, int64_t P, const uint32_t *draws, u
     if (!p || P < 0) return PP_ERR_ARG;
     if (P == 0) return PP_OK;
     if (!draws || !nseg || !ends || !nodes) return PP_ERR_ARG;
+    pp_status st = upload_inputs(p, false);
+    if (st != PP_OK) return st;
     PP_CUDA(launch_random_plans(p->d, P, draws, nseg, ends, nodes, p->stream));
     return PP_OK;
 }
@@ -694,6 +1030,8 @@ pp_status pp_random_plans(pp_problem *p, int64_t P, const uint32_t *draws, uint8
     const size_t b_draws = (size_t)P * 2 * k * 4, b_rows = (size_t)P * k * 4;
     const size_t o_ends = align_up(b_draws, 256), o_nodes = align_up(o_ends + b_rows, 256);
     const size_t o_nseg = align_up(o_nodes + b_rows, 256), total = o_nseg + (size_t)P;
+    pp_status st = upload_inputs(p, false);
+    if (st != PP_OK) return st;
     unsigned char *buf = nullptr;
     cudaStream_t s = p->stream;
     PP_CUDA(staging_alloc(reinterpret_cast<void **>(&buf), total, s));
@@ -1104,62 +1442,81 @@ pp_status pp_solve_exact_compute(int32_t L, const uint64_t *layer_out_bits, cons
     if (L > PP_COMPUTE_MAX_L || k > PP_COMPUTE_MAX_K) return PP_ERR_LIMIT;
     for (int i = 0; i < L; ++i)
         if (layer_work[i] >= PP_MAX_BITS) return PP_ERR_LIMIT;
+    PruneDev q{};
+    q.L = L; q.k = k; q.Lp = prune_row_pad(L);
+    // one staging buffer, one copy: the inputs, their prefix sums, the windows, the counters
+    const size_t bytes[8] = {(size_t)L * 8, (size_t)(L + 1) * 8, (size_t)(L + 1) * 8, (size_t)k * 8,
+                             (size_t)k * k * 4, (size_t)k * 4, (size_t)k * L * 2, sizeof(PruneCtl)};
+    size_t off[8], total = 0;
+    for (int i = 0; i < 8; ++i) { off[i] = total; total = align_up(total + bytes[i], i < 6 ? 16 : 128); }
+    std::vector<unsigned char> st8;
     try {
-        std::vector<uint64_t> M(L + 1, 0), Wp(L + 1, 0);
-        for (int i = 0; i < L; ++i) {
-            M[i + 1] = M[i] + layer_mem_bytes[i];
-            Wp[i + 1] = Wp[i] + layer_work[i];
-        }
-        DeviceMasks dmasks;
-        PP_CUDA(device_masks(k, mask_list(k), &dmasks));
-        struct Part { const void *src; size_t bytes; size_t off; };
-        std::vector<Part> parts = {
-            {layer_out_bits, (size_t)L * 8, 0}, {M.data(), (size_t)(L + 1) * 8, 0}, {Wp.data(), (size_t)(L + 1) * 8, 0},
-            {node_mem_bytes, (size_t)k * 8, 0}, {bw_kbps, (size_t)k * k * 4, 0}, {node_speed, (size_t)k * 4, 0},
-            {nullptr, 16, 0} /* best value, best key */, {nullptr, sizeof(pp_solution), 0},
-            {nullptr, (size_t)k * k * L * 8, 0} /* gamma */, {nullptr, (size_t)k * L * L * 8, 0} /* compute times */,
-            {nullptr, ((size_t)k << k) * L * 8, 0} /* state table */};
-        size_t total = 0;
-        for (auto &q : parts) { q.off = total; total = align_up(total + q.bytes, 256); }
-        unsigned char *buf = nullptr;
-        if (alloc_should_fail()) return PP_ERR_NOMEM;
-        PP_CUDA(cudaMalloc(reinterpret_cast<void **>(&buf), total));
-        struct Release {
-            unsigned char *b;
-            ~Release() { cudaFree(b); }
-        } release{buf};
-        cudaStream_t s = nullptr;
-        for (int i = 0; i < 6; ++i)
-            PP_CUDA(cudaMemcpyAsync(buf + parts[i].off, parts[i].src, parts[i].bytes, cudaMemcpyHostToDevice, s));
-        CtDev d{};
-        d.L = L; d.k = k;
-        d.bits = reinterpret_cast<uint64_t *>(buf + parts[0].off);
-        d.M = reinterpret_cast<uint64_t *>(buf + parts[1].off);
-        d.Wp = reinterpret_cast<uint64_t *>(buf + parts[2].off);
-        d.cap = reinterpret_cast<uint64_t *>(buf + parts[3].off);
-        d.bw = reinterpret_cast<uint32_t *>(buf + parts[4].off);
-        d.speed = reinterpret_cast<uint32_t *>(buf + parts[5].off);
-        d.masks = dmasks.masks;
-        d.level_off = dmasks.level_off;
-        d.best_val = reinterpret_cast<unsigned long long *>(buf + parts[6].off);
-        d.best_key = d.best_val + 1;
-        pp_solution *d_sol = reinterpret_cast<pp_solution *>(buf + parts[7].off);
-        d.gam = reinterpret_cast<double *>(buf + parts[8].off);
-        d.seg = reinterpret_cast<double *>(buf + parts[9].off);
-        d.table = reinterpret_cast<double *>(buf + parts[10].off);
-        PP_CUDA(launch_compute_search(d, d_sol, s));
-        pp_solution h{};
-        PP_CUDA(cudaMemcpyAsync(&h, d_sol, sizeof h, cudaMemcpyDeviceToHost, s));
-        PP_CUDA(cudaStreamSynchronize(s));
-        if (h.status != PP_OK && h.status != PP_INFEASIBLE) return PP_ERR_CUDA;
-        *beta_ms = h.beta_ms;
-        *m = h.m;
-        for (int j = 0; j < k - 1; ++j) cuts[j] = h.cuts[j];
-        for (int j = 0; j < k; ++j) placement[j] = h.placement[j];
-        return static_cast<pp_status>(h.status);
+        st8.assign(total, 0);
     } catch (const std::bad_alloc &) {
         return PP_ERR_NOMEM;
     }
+    unsigned char *h = st8.data();
+    uint64_t *M = reinterpret_cast<uint64_t *>(h + off[1]), *Wp = reinterpret_cast<uint64_t *>(h + off[2]);
+    std::memcpy(h + off[0], layer_out_bits, bytes[0]);
+    for (int i = 0; i < L; ++i) {
+        M[i + 1] = M[i] + layer_mem_bytes[i];
+        Wp[i + 1] = Wp[i] + layer_work[i];
+    }
+    std::memcpy(h + off[3], node_mem_bytes, bytes[3]);
+    std::memcpy(h + off[4], bw_kbps, bytes[4]);
+    std::memcpy(h + off[5], node_speed, bytes[5]);
+    window_table(L, k, M, node_mem_bytes, reinterpret_cast<int16_t *>(h + off[6]));
+    prune_ctl_init(reinterpret_cast<PruneCtl *>(h + off[7]));
+    double lo = std::numeric_limits<double>::max(), hi = 0.0;
+    quotient_range(L, layer_out_bits, k * k, bw_kbps, &lo, &hi);
+    quotient_range(L, layer_work, k, node_speed, &lo, &hi);   // shortest run of layers: one
+    quotient_range(1, Wp + L, k, node_speed, &lo, &hi);       // longest: all of them
+    prune_key_range(hi > 0.0 ? lo : 1.0, hi > 0.0 ? hi : 1.0, &q);
+    prune_node_bounds(node_mem_bytes, M[L], &q);
+    int dev = 0, sms = 0;
+    PP_CUDA(cudaGetDevice(&dev));
+    PP_CUDA(multiprocessors(dev, &sms));
+    cudaStream_t s = nullptr;
+    HostSlot *slot = g_slots.take();
+    if (!slot) return PP_ERR_NOMEM;
+    const size_t seg_bytes = align_up((size_t)k * L * q.Lp * 4, 256), head = align_up(total, 256) + seg_bytes;
+    cudaError_t e = cudaSuccess;
+    // pooled scratch for a frontier that stays small, room for every state if it does not
+    const unsigned long long limits[2] = {kSparseScratchBytes, ~0ull};
+    for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
+        unsigned char *buf = nullptr;
+        const size_t table = sparse_bytes(k, q.Lp, limits[pass]);
+        e = staging_alloc(reinterpret_cast<void **>(&buf), head + table, s);
+        if (e != cudaSuccess) break;
+        q.bits = reinterpret_cast<uint64_t *>(buf + off[0]);
+        q.M = reinterpret_cast<uint64_t *>(buf + off[1]);
+        q.Wp = reinterpret_cast<uint64_t *>(buf + off[2]);
+        q.cap = reinterpret_cast<uint64_t *>(buf + off[3]);
+        q.bw = reinterpret_cast<uint32_t *>(buf + off[4]);
+        q.speed = reinterpret_cast<uint32_t *>(buf + off[5]);
+        q.lo = reinterpret_cast<int16_t *>(buf + off[6]);
+        q.ctl = reinterpret_cast<PruneCtl *>(buf + off[7]);
+        q.seg = reinterpret_cast<uint32_t *>(buf + align_up(total, 256));
+        bind_sparse(q, buf + head, table);
+        q.out = &slot->sol;
+        q.note = &slot->note;
+        slot->note.dense = -1;
+        e = cudaMemcpyAsync(buf, h, total, cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess) e = launch_prune(q, sms, s);
+        cudaFreeAsync(buf, s);
+        const cudaError_t e2 = cudaStreamSynchronize(s);
+        if (e == cudaSuccess) e = e2;
+        if (e == cudaSuccess && slot->note.dense <= 0) break;
+    }
+    const HostSlot got = *slot;
+    g_slots.give(slot);
+    if (e != cudaSuccess) return from_cuda(e);
+    if (got.note.dense != 0 || (got.sol.status != PP_OK && got.sol.status != PP_INFEASIBLE)) return PP_ERR_CUDA;
+    *beta_ms = got.sol.beta_ms;
+    *m = got.sol.m;
+    for (int j = 0; j < k - 1; ++j) cuts[j] = got.sol.cuts[j];
+    for (int j = 0; j < k; ++j) placement[j] = got.sol.placement[j];
+    return static_cast<pp_status>(got.sol.status);
 }
 
 pp_status pp_debug_minmax_rate(int32_t op, int32_t iters, double *warp_instr_per_clk_per_sm)
@@ -1216,6 +1573,10 @@ pp_status pp_debug_read_state_row(pp_problem *p, uint32_t mask, int32_t v, doubl
 {
     if (!p || !row_out || !p->solved) return PP_ERR_ARG;
     if (v < 0 || v >= p->k || mask >= (1u << p->k) || !((mask >> v) & 1u)) return PP_ERR_ARG;
+    if (!p->table_whole) {  // the bounded search keeps no whole table: let the dense one write it
+        pp_status st = queue_dense(p, p->d_sol);
+        if (st != PP_OK) return st;
+    }
     PP_CUDA(cudaStreamSynchronize(p->stream));
     const int L = p->L, U = p->U;
     std::vector<uint32_t> rk((size_t)std::max(U, 1) * L);

@@ -116,6 +116,47 @@ cudaError_t launch_batch_prep(int64_t B, int L, int k, const uint64_t *bits, con
 cudaError_t launch_batch_lanes(int64_t B, int L, int k, const uint64_t *bits, const uint32_t *bw,
                                const BatchLanes &t, double *beta, int32_t *m, int32_t *cuts,
                                int32_t *placement, int8_t *status, cudaStream_t s);
+// The search as a bounded sparse frontier (pp_prune.cu), one launch per solve.
+struct PruneCtl {              // device; the kernel leaves it as it found it
+    unsigned long long best;   // best final state of the levels done: pack_best of its key
+    uint32_t count[64];        // node sets appended to the frontier by the level of that many nodes (a second
+                               // search over the class of the optimum counts from 32)
+    uint32_t arrived, left;    // barrier arrivals; blocks that have left
+    uint32_t failed;           // a barrier ran out of polls
+    uint32_t dense;            // 1 = the frontier outgrew its rows
+};
+struct PruneNote {             // what the host learns about a launch
+    long long ns;              // duration on the device
+    int32_t dense;             // as PruneCtl::dense
+};
+struct PruneDev {
+    int L, k, Lp;              // Lp: row stride in keys
+    int key_shift;             // keys: 1 + (bits of the double - key_base) >> key_shift
+    unsigned long long key_base;
+    uint32_t whole;            // nodes that hold the whole chain
+    uint32_t tight_levels;     // bit j: some rest of the chain may not fit the nodes that j used ones leave
+    const uint64_t *bits, *M, *cap;  // as in Dev
+    const uint32_t *bw;
+    const int16_t *lo;
+    uint32_t *live;            // [2^k] nodes v whose row (S, v) is kept
+    unsigned long long *rowmap;  // [2^k * k] (S, v): smallest key << 32 | row
+    uint32_t *list;            // [2^k] node sets of the frontier, level after level
+    uint32_t *gam;             // [k*k*Lp] key of gamma[c][v][w] at (w*k + v)*Lp + c
+    uint32_t *gmin;            // [k*k] its minimum over the cut positions
+    uint32_t *rows;            // [row_cap * Lp]
+    unsigned long long row_cap;
+    const uint64_t *Wp;        // Eq. 1 only: [L+1] prefix sums of the layers' work,
+    const uint32_t *speed;     //   [k] speeds,
+    uint32_t *seg;             //   [k*L*Lp] keys of the compute times of every run of layers; null for Eq. 2
+    PruneCtl *ctl;
+    pp_solution *out;          // device or mapped host memory
+    PruneNote *note;           // device or mapped host memory
+};
+void prune_key_range(double lo, double hi, PruneDev *d);
+void prune_node_bounds(const uint64_t *cap, uint64_t total, PruneDev *d);
+int prune_row_pad(int L);
+void prune_ctl_init(PruneCtl *c);
+cudaError_t launch_prune(const PruneDev &d, int sms, cudaStream_t s);
 // Random comparison baseline (Section 4): P plans of problem d from 2 k draws each.
 cudaError_t launch_random_plans(const Dev &d, int64_t P, const uint32_t *draws, uint8_t *nseg, int32_t *ends,
                                 int32_t *nodes, cudaStream_t s);
@@ -134,16 +175,6 @@ size_t kpath_smem_bytes(int kk);
 cudaError_t launch_kpath(int n, int kk, int64_t Q, const uint32_t *bw, const uint32_t *threshold, const int32_t *start,
                          const int32_t *end, const unsigned long long *alive, const uint8_t *colours, uint8_t *found,
                          int32_t *path, cudaStream_t s);
-// Exact search under Eq. 1 (compute times in the bottleneck), pp_compute.cu.
-struct CtDev {
-    int L, k;
-    const uint64_t *bits, *M, *Wp, *cap;   // [L], [L+1] memory prefix sums, [L+1] work prefix sums, [k]
-    const uint32_t *bw, *speed;            // [k*k], [k]
-    const uint32_t *masks, *level_off;     // node sets by popcount (any order within a level)
-    double *gam, *seg, *table;             // [k*k*L], [k*L*L], [2^k * k * L]
-    unsigned long long *best_val, *best_key;  // adjacent 64-bit words
-};
-cudaError_t launch_compute_search(const CtDev &d, pp_solution *out, cudaStream_t s);
 // Issue-rate probe (pp_probe.cu): `blocks` blocks of 1024 threads, cycles[b] = SM clocks block b took.
 cudaError_t launch_probe(int op, int iters, int blocks, long long *cycles, uint32_t *sink, cudaStream_t s);
 double probe_instr_per_block(int iters);

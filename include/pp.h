@@ -324,9 +324,9 @@ pp_status pp_kpath_colour_batch_dev(int32_t n, const uint32_t *bw_kbps, int64_t 
  * among the distinct sizes; classes are served from the highest down, within a class the maximal
  * runs of consecutive cuts longest first (equal lengths by first cut); a run of l cuts gets a path
  * of l + 1 unused nodes between its already placed neighbours, at the largest link-bandwidth
- * threshold (Eq. 8) for which the colour-coding search of pp_kpath_colour_batch finds one: the
- * bisection of Algorithm 2 over the sorted bandwidths, each probe a batch of `trials` colourings,
- * the first colouring that finds a path decides.
+ * threshold (Eq. 8) for which the colour-coding search of pp_kpath_colour_batch finds one over
+ * `trials` colourings, which is where the bisection of Algorithm 2 over the sorted bandwidths ends;
+ * the first colouring that finds a path there decides.
  *   n, bw_kbps [n*n]   host: the communication graph (row = sender), n <= 64
  *   n_cuts, sizes [n_cuts]   host: transfer sizes S of the cuts, in chain order
  *   n_classes          number of transfer-size (= bandwidth) classes, >= 1

@@ -391,12 +391,15 @@ pp_status upload_inputs(pp_problem *p, bool wait)
     return PP_OK;
 }
 
-// Page-locked result records of the synchronous calls, one per call in flight: the kernel writes its
-// result straight into host memory.  Chunks of 32; all but one chunk are given back when unused.
+// Page-locked memory of the synchronous calls, one slot per call in flight: the kernel writes its result
+// straight into host memory.  Chunks of kSlots; all but one chunk are given back when unused.
 struct HostSlot {
     pp_solution sol;
     PruneNote note;
+    MatchOut match;
+    alignas(256) unsigned char small[15 * 1024];  // inputs and results of a small call as a whole
 };
+constexpr int kSlots = 8;
 class HostSlots {
 public:
     HostSlot *take()
@@ -405,12 +408,12 @@ public:
         for (auto &c : chunks_)
             if (c.free) return from(c);
         void *ptr = nullptr;
-        if (cudaHostAlloc(&ptr, 32 * sizeof(HostSlot), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+        if (cudaHostAlloc(&ptr, kSlots * sizeof(HostSlot), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
             cudaGetLastError();
             return nullptr;
         }
         try {
-            chunks_.push_back({static_cast<HostSlot *>(ptr), 0xFFFFFFFFu});
+            chunks_.push_back({static_cast<HostSlot *>(ptr), (1u << kSlots) - 1u});
         } catch (const std::bad_alloc &) {
             cudaFreeHost(ptr);
             return nullptr;
@@ -422,9 +425,9 @@ public:
         std::lock_guard<std::mutex> lock(mu_);
         for (size_t i = 0; i < chunks_.size(); ++i) {
             const ptrdiff_t at = s - chunks_[i].base;
-            if (at < 0 || at >= 32) continue;
+            if (at < 0 || at >= kSlots) continue;
             chunks_[i].free |= 1u << at;
-            if (i > 0 && chunks_[i].free == 0xFFFFFFFFu) {
+            if (i > 0 && chunks_[i].free == (1u << kSlots) - 1u) {
                 cudaFreeHost(chunks_[i].base);
                 chunks_.erase(chunks_.begin() + (long)i);
             }
@@ -447,6 +450,10 @@ private:
     std::vector<Chunk> chunks_;
 };
 HostSlots g_slots;
+struct SlotLease {  // a slot for the duration of a call
+    HostSlot *slot = g_slots.take();
+    ~SlotLease() { if (slot) g_slots.give(slot); }
+};
 
 // ---- the dense search (pp_rank.cu, pp_sweep*.cu) ------------------------------------------------
 
@@ -1230,6 +1237,27 @@ pp_status pp_partition_minsum_batch(int64_t B, int32_t L, const uint64_t *cut_we
     const size_t sz[8] = {nB * L * 8, nB * L * 8, nB * 8, nB * 8, nB * 4, rows * 4, rows * 8, nB};
     size_t off[9];
     off[0] = 0;
+    for (int i = 0; i < 8; ++i) off[i + 1] = align_up(off[i] + sz[i], 16);
+    if (off[8] <= sizeof(HostSlot::small)) {
+        // a few chains: the kernel reads and writes page-locked memory, nothing is copied or allocated on
+        // the device (every word crosses the bus once)
+        SlotLease lease;
+        if (!lease.slot) return PP_ERR_NOMEM;
+        unsigned char *h = lease.slot->small;
+        const void *in[3] = {cut_weight, mem, kappa};
+        for (int i = 0; i < 3; ++i) std::memcpy(h + off[i], in[i], sz[i]);
+        PP_CUDA(launch_partition_minsum(B, L, cap_seg, reinterpret_cast<uint64_t *>(h + off[0]),
+                                        reinterpret_cast<uint64_t *>(h + off[1]), reinterpret_cast<uint64_t *>(h + off[2]),
+                                        reinterpret_cast<uint64_t *>(h + off[3]), reinterpret_cast<int32_t *>(h + off[4]),
+                                        reinterpret_cast<int32_t *>(h + off[5]), reinterpret_cast<uint64_t *>(h + off[6]),
+                                        reinterpret_cast<int8_t *>(h + off[7]), nullptr));
+        PP_CUDA(cudaStreamSynchronize(nullptr));
+        void *out[5] = {cost, m, cuts, sizes, status};
+        const size_t n[5] = {sz[3], sz[4], nB * (size_t)cap_seg * 4, nB * (size_t)cap_seg * 8, sz[7]};
+        for (int i = 0; i < 5; ++i)
+            if (out[i] && n[i]) std::memcpy(out[i], h + off[3 + i], n[i]);
+        return PP_OK;
+    }
     for (int i = 0; i < 8; ++i) off[i + 1] = align_up(off[i] + sz[i], 256);
     unsigned char *buf = nullptr;
     cudaStream_t s = nullptr;
@@ -1303,10 +1331,52 @@ pp_status pp_kpath_colour_batch(int32_t n, const uint32_t *bw_kbps, int64_t Q, i
     return from_cuda(e2);
 }
 
-// Placement stage of the paper's heuristic (Section 3.2.2, Algorithms 2 and 3), orchestrated on the
-// host: classes of the cut sizes, runs of cuts per class, and for every run a bisection over the
-// sorted link bandwidths whose probes are batches of colour-coding k-path queries on the device (one
-// query per trial colouring).
+// The whole stage as one launch (pp_match.cu): one copy up, the result in page-locked memory.
+constexpr size_t kMatchSharedBytes = 220 * 1024;
+static pp_status match_one_launch(int32_t n, const uint32_t *bw, int32_t n_cuts, int32_t trials, const uint32_t *draws,
+                                  const std::vector<MatchRun> &order, int kk, int32_t *nodes, uint32_t *cut_threshold,
+                                  cudaStream_t s)
+{
+    int dev = 0, sms = 0;
+    PP_CUDA(cudaGetDevice(&dev));
+    PP_CUDA(multiprocessors(dev, &sms));
+    SlotLease lease;
+    if (!lease.slot) return PP_ERR_NOMEM;
+    const size_t sz[4] = {(size_t)n * n * 4, (size_t)trials * n * 4, order.size() * sizeof(MatchRun), sizeof(MatchCtl)};
+    size_t off[5];
+    off[0] = 0;
+    for (int i = 0; i < 4; ++i) off[i + 1] = align_up(off[i] + sz[i], 128);
+    std::vector<unsigned char> st(off[4], 0);
+    const void *src[3] = {bw, draws, order.data()};
+    for (int i = 0; i < 3; ++i) std::memcpy(st.data() + off[i], src[i], sz[i]);
+    unsigned char *buf = nullptr;
+    PP_CUDA(staging_alloc(reinterpret_cast<void **>(&buf), off[4] + (size_t)2 * sms * PP_KPATH_MAX_K * 4, s));
+    MatchDev d;
+    d.n = n; d.n_cuts = n_cuts; d.n_runs = (int)order.size(); d.trials = trials;
+    d.bw = reinterpret_cast<uint32_t *>(buf + off[0]);
+    d.draws = reinterpret_cast<uint32_t *>(buf + off[1]);
+    d.runs = reinterpret_cast<MatchRun *>(buf + off[2]);
+    d.ctl = reinterpret_cast<MatchCtl *>(buf + off[3]);
+    d.paths = reinterpret_cast<int32_t *>(buf + off[4]);
+    d.out = &lease.slot->match;
+    lease.slot->match.status = (int)PP_ERR_CUDA;
+    cudaError_t e = cudaMemcpyAsync(buf, st.data(), off[4], cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = launch_match(d, kk, sms, s);
+    cudaFreeAsync(buf, s);
+    const cudaError_t e2 = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return from_cuda(e);
+    if (e2 != cudaSuccess) return from_cuda(e2);
+    const MatchOut &got = lease.slot->match;
+    if (got.status != PP_OK && got.status != PP_INFEASIBLE) return PP_ERR_CUDA;
+    std::copy(got.nodes, got.nodes + n_cuts + 1, nodes);
+    if (cut_threshold) std::copy(got.threshold, got.threshold + n_cuts, cut_threshold);
+    return static_cast<pp_status>(got.status);
+}
+
+// Placement stage of the paper's heuristic (Section 3.2.2, Algorithms 2 and 3): classes of the cut sizes
+// and the order of their runs on the host, the paths on the device.  Without the one-launch kernel every
+// run is a bisection over the sorted link bandwidths whose probes are batches of colour-coding k-path
+// queries (one query per trial colouring).
 pp_status pp_kpath_matching(int32_t n, const uint32_t *bw_kbps, int32_t n_cuts, const uint64_t *sizes,
                             int32_t n_classes, int32_t trials, const uint32_t *draws, int32_t *nodes,
                             uint32_t *cut_threshold, void *cuda_stream)
@@ -1333,6 +1403,28 @@ pp_status pp_kpath_matching(int32_t n, const uint32_t *bw_kbps, int32_t n_cuts, 
             const size_t rank = std::lower_bound(distinct.begin(), distinct.end(), sizes[j]) - distinct.begin();
             cls[j] = (int)(rank * (size_t)n_classes / distinct.size());
         }
+        // serving order: classes from the highest down, within a class maximal runs of cuts, longest first,
+        // equal lengths by first cut
+        std::vector<MatchRun> order;
+        int longest = 0;
+        for (int X = n_classes - 1; X >= 0; --X) {
+            const size_t from = order.size();
+            for (int i = 0; i < n_cuts;) {
+                if (cls[i] != X) { ++i; continue; }
+                int j = i;
+                while (j < n_cuts && cls[j] == X) ++j;
+                order.push_back({i, j - i});
+                longest = std::max(longest, j - i);
+                i = j;
+            }
+            std::stable_sort(order.begin() + (long)from, order.end(),
+                             [](const MatchRun &a, const MatchRun &b) { return a.cuts > b.cuts; });
+        }
+        // tables of bottlenecks that fit a block's shared memory: one launch for the whole stage.  Longer
+        // runs (paths of ten vertices and more on large graphs) and plans with more cuts than the kernel's
+        // records hold are bisected with a launch per probe.
+        if (n_cuts < 64 && longest < PP_KPATH_MAX_K && match_smem_bytes(n, longest + 1) <= kMatchSharedBytes)
+            return match_one_launch(n, bw_kbps, n_cuts, trials, draws, order, longest + 1, nodes, cut_threshold, s);
         // link bandwidths in descending order: the thresholds Algorithm 2 bisects over
         std::vector<uint32_t> edge_list;
         for (int v = 0; v < n; ++v)
@@ -1357,20 +1449,9 @@ pp_status pp_kpath_matching(int32_t n, const uint32_t *bw_kbps, int32_t n_cuts, 
         std::vector<uint64_t> h_alive(T);
         std::vector<uint8_t> h_col(T * n), h_found(T);
         uint64_t used = 0;
-        for (int X = n_classes - 1; X >= 0; --X) {
-            // maximal runs of cuts of class X, longest first, equal lengths by first cut
-            std::vector<std::pair<int, int>> runs;  // (first cut, cuts)
-            for (int i = 0; i < n_cuts;) {
-                if (cls[i] != X) { ++i; continue; }
-                int j = i;
-                while (j < n_cuts && cls[j] == X) ++j;
-                runs.emplace_back(i, j - i);
-                i = j;
-            }
-            std::stable_sort(runs.begin(), runs.end(),
-                             [](const std::pair<int, int> &a, const std::pair<int, int> &b) { return a.second > b.second; });
-            for (const auto &run : runs) {
-                const int first = run.first, cuts = run.second, kk = cuts + 1;
+        {
+            for (const MatchRun &run : order) {
+                const int first = run.first, cuts = run.cuts, kk = cuts + 1;
                 if (kk > PP_KPATH_MAX_K) return PP_ERR_LIMIT;
                 const int sv = nodes[first], uv = nodes[first + cuts];
                 uint64_t alive = ~used;

@@ -175,6 +175,28 @@ size_t kpath_smem_bytes(int kk);
 cudaError_t launch_kpath(int n, int kk, int64_t Q, const uint32_t *bw, const uint32_t *threshold, const int32_t *start,
                          const int32_t *end, const unsigned long long *alive, const uint8_t *colours, uint8_t *found,
                          int32_t *path, cudaStream_t s);
+// Placement stage in one launch (pp_match.cu).
+struct MatchRun {
+    int32_t first, cuts;       // a run of cuts of one class, in serving order
+};
+struct MatchCtl {
+    unsigned long long best[64];  // per run: bottleneck << 32 | ~colouring; zero before the launch
+    uint32_t arrived;
+};
+struct MatchOut {
+    int32_t status, nodes[64];
+    uint32_t threshold[64];
+};
+struct MatchDev {
+    int n, n_cuts, n_runs, trials;
+    const uint32_t *bw, *draws;
+    const MatchRun *runs;
+    int32_t *paths;            // [2][blocks][PP_KPATH_MAX_K]
+    MatchCtl *ctl;
+    MatchOut *out;             // mapped host memory
+};
+size_t match_smem_bytes(int n, int kk);
+cudaError_t launch_match(const MatchDev &d, int kk_max, int sms, cudaStream_t s);
 // Issue-rate probe (pp_probe.cu): `blocks` blocks of 1024 threads, cycles[b] = SM clocks block b took.
 cudaError_t launch_probe(int op, int iters, int blocks, long long *cycles, uint32_t *sink, cudaStream_t s);
 double probe_instr_per_block(int iters);

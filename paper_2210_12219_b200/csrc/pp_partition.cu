@@ -11,9 +11,12 @@
 // tie rule "smaller cost, then fewer partitions"; walking forward from point 0 and always taking
 // the earliest e that attains F[i] gives the lexicographically smallest cut list among those.
 //
-// Two kernels.  One warp per chain (any length, small batches): the recurrence is L dependent steps,
-// each a minimum over a window that the lanes scan together; prefix sums of the memory and the G
-// values live in the warp's slice of shared memory, the weights pass through registers 32 at a time.
+// Two kernels.  One warp per chain (any length, small batches): everything about a point that does not
+// depend on the recurrence (prefix sums, weights, the last point hi of its window) is worked out by the
+// lanes in parallel and kept in the warp's slice of shared memory; the recurrence itself is L dependent
+// steps of one lane, a sliding minimum over a queue of candidates with ascending values (a step pushes
+// one and drops the beaten and the expired ones: about 60 cycles, where scanning the window with all lanes
+// and reducing it by shuffles took about 450).
 // One lane per chain (chains of up to 64 points, 8192 chains or more): see k_partition_lanes.
 #include "pp_internal.cuh"
 
@@ -25,14 +28,7 @@ constexpr int kPartWarps = 4;
 constexpr unsigned long long kInfCost = ~0ull;
 constexpr int kPartsBits = 11;  // partitions <= PP_MAX_L = 1024 < 2^11
 
-__device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long x)
-{
-    for (int o = 16; o; o >>= 1) {
-        const unsigned long long y = __shfl_xor_sync(0xFFFFFFFFu, x, o);
-        x = y < x ? y : x;
-    }
-    return x;
-}
+__host__ __device__ inline size_t part_words(int L) { return 3 * (size_t)L + 1 + ((size_t)L + 1) / 2; }
 
 __global__ void __launch_bounds__(kPartWarps * 32)
 k_partition_minsum(int64_t B, int L, int cap_seg, const uint64_t *__restrict__ weight,
@@ -42,8 +38,11 @@ k_partition_minsum(int64_t B, int L, int cap_seg, const uint64_t *__restrict__ w
 {
     extern __shared__ unsigned long long smem_u64[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    unsigned long long *M = smem_u64 + (size_t)wid * (2 * L + 1);  // [L + 1] prefix sums of the memory
-    unsigned long long *G = M + (L + 1);                           // [L]
+    unsigned long long *M = smem_u64 + (size_t)wid * part_words(L);  // [L + 1] prefix sums of the memory
+    unsigned long long *G = M + (L + 1);                             // [L]
+    unsigned long long *Wt = G + L;                                  // [L] weights
+    uint16_t *H = reinterpret_cast<uint16_t *>(Wt + L);              // [L] points after i's window start: hi(i) + 1
+    uint16_t *D = H + L;                                             // [L] queue of candidates
     for (int64_t b = (int64_t)blockIdx.x * kPartWarps + wid; b < B; b += (int64_t)gridDim.x * kPartWarps) {
         const uint64_t *w = weight + b * L, *mm = mem + b * L;
         const unsigned long long cap = kappa[b];
@@ -55,7 +54,9 @@ k_partition_minsum(int64_t B, int L, int cap_seg, const uint64_t *__restrict__ w
         for (int base = 0; base < L; base += 32) {
             const int i = base + lane;
             unsigned long long x = i < L ? mm[i] : 0ull;
-            if (i < L && w[i] >= PP_MAX_BITS) bad = true;
+            const unsigned long long wi = i < L ? w[i] : 0ull;
+            if (wi >= PP_MAX_BITS) bad = true;
+            if (i < L) Wt[i] = wi;
             for (int o = 1; o < 32; o <<= 1) {
                 const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, x, o);
                 if (lane >= o) {
@@ -84,34 +85,43 @@ k_partition_minsum(int64_t B, int L, int cap_seg, const uint64_t *__restrict__ w
             continue;
         }
         __syncwarp();
+        for (int i = lane; i < L; i += 32) {  // points i .. e fit: the prefix sums ascend
+            const unsigned long long base = M[i];
+            int lo = i, hi = L;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (M[mid + 1] - base <= cap) lo = mid + 1; else hi = mid;
+            }
+            H[i] = (uint16_t)lo;
+        }
+        __syncwarp();
         // backward recurrence
-        unsigned long long F = kInfCost, wchunk = 0;
-        int hi = L - 1;
-        for (int i = L - 1; i >= 0; --i) {
-            if (i == L - 1 || (i & 31) == 31) {  // weights of points i-31 .. i (i - 1 is the one needed next)
-                const int e = (i & ~31) + lane;
-                wchunk = e < L ? w[e] : 0ull;
-            }
-            if (i == L - 1) {
-                if (lane == 0) G[L - 1] = 1ull;  // cost 0, one partition
-                __syncwarp();
-            }
-            while (hi >= i && M[hi + 1] - M[i] > cap) --hi;
-            unsigned long long best = kInfCost;
-            for (int e = i + lane; e <= hi; e += 32) {
-                const unsigned long long g = G[e];
-                best = g < best ? g : best;
-            }
-            F = warp_min_u64(best);
-            if (i > 0) {
-                const unsigned long long wi = __shfl_sync(0xFFFFFFFFu, wchunk, (i - 1) & 31);
-                // the chunk that holds point i - 1 is the current one unless i is a multiple of 32
-                unsigned long long wprev = wi;
-                if ((i & 31) == 0) wprev = w[i - 1];
-                if (lane == 0) G[i - 1] = F == kInfCost ? kInfCost : F + (wprev << kPartsBits) + 1ull;
-                __syncwarp();
+        unsigned long long F = kInfCost;
+        if (lane == 0) {
+            unsigned long long g = 1ull;  // G of the point about to be pushed: cost 0, one partition
+            unsigned long long back = 0ull, front = 0ull;
+            int head = 0, tail = -1, oldest = 0;  // D[head .. tail]: points in descending order, values ascending
+            for (int i = L - 1; i >= 0; --i) {
+                const int end = H[i];
+                const unsigned long long wprev = i > 0 ? Wt[i - 1] : 0ull;
+                G[i] = g;
+                while (tail >= head && back >= g) {
+                    --tail;
+                    if (tail >= head) back = G[D[tail]];
+                }
+                D[++tail] = (uint16_t)i;
+                back = g;
+                if (tail == head) { front = g; oldest = i; }
+                while (head <= tail && oldest >= end) {
+                    ++head;
+                    if (head <= tail) { oldest = D[head]; front = G[oldest]; }
+                }
+                F = head <= tail ? front : kInfCost;
+                g = F == kInfCost ? kInfCost : F + (wprev << kPartsBits) + 1ull;
             }
         }
+        __syncwarp();
+        F = __shfl_sync(0xFFFFFFFFu, F, 0);
         if (F == kInfCost) {
             if (lane == 0) {
                 o_cost[b] = 0;
@@ -130,10 +140,8 @@ k_partition_minsum(int64_t B, int L, int cap_seg, const uint64_t *__restrict__ w
         // forward walk: the earliest point that attains the optimum of the suffix
         unsigned long long target = F;
         int i = 0, nc = 0;
-        hi = -1;
         for (;;) {
-            if (hi < i) hi = i;
-            while (hi + 1 < L && M[hi + 2] - M[i] <= cap) ++hi;
+            const int hi = (int)H[i] - 1;
             int found = -1;
             for (int base = i; base <= hi && found < 0; base += 32) {
                 const int e = base + lane;
@@ -141,7 +149,7 @@ k_partition_minsum(int64_t B, int L, int cap_seg, const uint64_t *__restrict__ w
                 if (hits) found = base + __ffs(hits) - 1;
             }
             if (found < 0 || found == L - 1) break;  // found < 0 cannot happen on a consistent table
-            const unsigned long long wf = w[found];
+            const unsigned long long wf = Wt[found];
             if (lane == 0) {
                 if (cuts) cuts[nc] = found;
                 if (sizes) sizes[nc] = wf;
@@ -249,7 +257,7 @@ k_partition_lanes(int64_t B, int L, int cap_seg, const uint64_t *__restrict__ we
 
 }  // namespace
 
-size_t partition_smem_bytes(int L) { return (size_t)kPartWarps * (2 * (size_t)L + 1) * sizeof(unsigned long long); }
+size_t partition_smem_bytes(int L) { return (size_t)kPartWarps * part_words(L) * sizeof(unsigned long long); }
 
 cudaError_t launch_partition_minsum(int64_t B, int L, int cap_seg, const uint64_t *weight, const uint64_t *mem,
                                     const uint64_t *kappa, uint64_t *cost, int32_t *m, int32_t *cuts,

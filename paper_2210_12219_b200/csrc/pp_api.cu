@@ -48,6 +48,7 @@ struct pp_problem {
     std::vector<uint32_t> ubw;
     std::vector<int16_t> pair_u;
     unsigned char *d_dense = nullptr;
+    unsigned char *d_tables = nullptr;  // PlanTables, made by the first call that scores or draws plans
     Dev d{};
     int sweep_launches = 0, total_launches = 0, fast_used = 0, pair_levels = 0;
     std::vector<signed char> pair_lvl;  // per level: 1 = two-mask kernel, 0 = one-mask, -1 = not decided yet
@@ -388,6 +389,17 @@ pp_status upload_inputs(pp_problem *p, bool wait)
     if (wait) PP_CUDA(cudaMemcpy(p->d_inputs, st.data(), st.size(), cudaMemcpyHostToDevice));
     else PP_CUDA(cudaMemcpyAsync(p->d_inputs, st.data(), st.size(), cudaMemcpyHostToDevice, p->stream));
     p->uploaded = true;
+    return PP_OK;
+}
+
+pp_status ensure_tables(pp_problem *p)
+{
+    const pp_status st = upload_inputs(p, false);
+    if (st != PP_OK || p->d_tables) return st;
+    unsigned char *t = nullptr;
+    PP_CUDA(staging_alloc(reinterpret_cast<void **>(&t), plan_tables(p->L, p->k).total, p->stream));
+    p->d_tables = t;
+    PP_CUDA(launch_plan_tables(p->d, t, p->stream));
     return PP_OK;
 }
 
@@ -751,7 +763,7 @@ void pp_problem_destroy(pp_problem *p)
 {
     if (!p) return;
     if (p->own_work && p->d_work) cudaFree(p->d_work);
-    for (unsigned char *q : {p->d_inputs, p->d_sparse, p->d_dense})
+    for (unsigned char *q : {p->d_inputs, p->d_sparse, p->d_dense, p->d_tables})
         if (q) cudaFreeAsync(q, p->stream);  // ordered after the problem's queued work
     for (auto &e : p->ev)
         if (e) cudaEventDestroy(e);
@@ -763,7 +775,7 @@ pp_status pp_problem_set_stream(pp_problem *p, void *cuda_stream)
     if (!p) return PP_ERR_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     if (s == p->stream) return PP_OK;
-    if (p->uploaded || p->d_sparse) PP_CUDA(cudaStreamSynchronize(p->stream));  // copies and scratch are ordered there
+    if (p->uploaded || p->d_sparse || p->d_tables) PP_CUDA(cudaStreamSynchronize(p->stream));  // copies and scratch are ordered there
     p->stream = s;
     return upload_inputs(p, true);
 }
@@ -933,9 +945,9 @@ pp_status pp_eval_plans_dev(pp_problem *p, int64_t B, const uint8_t *nseg, const
     if (!p || B < 0) return PP_ERR_ARG;
     if (B == 0) return PP_OK;
     if (!nseg || !ends || !nodes || !beta_ms || !plan_status) return PP_ERR_ARG;
-    pp_status st = upload_inputs(p, false);
+    pp_status st = ensure_tables(p);
     if (st != PP_OK) return st;
-    PP_CUDA(launch_eval(p->d, B, nseg, ends, nodes, beta_ms, plan_status, p->stream));
+    PP_CUDA(launch_eval(p->d, p->d_tables, B, nseg, ends, nodes, beta_ms, plan_status, p->stream));
     return PP_OK;
 }
 
@@ -950,7 +962,7 @@ pp_status pp_eval_plans(pp_problem *p, int64_t B, const uint8_t *nseg, const int
     size_t o_ends = align_up(b_nseg, 256), o_nodes = align_up(o_ends + b_rows, 256);
     size_t o_beta = align_up(o_nodes + b_rows, 256), o_st = align_up(o_beta + b_beta, 256);
     size_t total = o_st + (size_t)B;
-    pp_status st = upload_inputs(p, false);
+    pp_status st = ensure_tables(p);
     if (st != PP_OK) return st;
     unsigned char *buf = nullptr;
     cudaStream_t s = p->stream;
@@ -959,7 +971,7 @@ pp_status pp_eval_plans(pp_problem *p, int64_t B, const uint8_t *nseg, const int
     if (e == cudaSuccess) e = cudaMemcpyAsync(buf + o_ends, ends, b_rows, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(buf + o_nodes, nodes, b_rows, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
-        e = launch_eval(p->d, B, buf, reinterpret_cast<int32_t *>(buf + o_ends),
+        e = launch_eval(p->d, p->d_tables, B, buf, reinterpret_cast<int32_t *>(buf + o_ends),
                         reinterpret_cast<int32_t *>(buf + o_nodes),
                         reinterpret_cast<double *>(buf + o_beta), buf + o_st, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(beta_ms, buf + o_beta, b_beta, cudaMemcpyDeviceToHost, s);
@@ -977,9 +989,9 @@ pp_status pp_eval_plans_packed_dev(pp_problem *p, int64_t B, int64_t total, cons
     if (!p || B < 0 || total < 0) return PP_ERR_ARG;
     if (B == 0) return PP_OK;
     if (!nseg || !plan_off || !beta_ms || !plan_status || ((!ends || !nodes) && total > 0)) return PP_ERR_ARG;
-    pp_status st = upload_inputs(p, false);
+    pp_status st = ensure_tables(p);
     if (st != PP_OK) return st;
-    PP_CUDA(launch_eval_packed(p->d, B, total, nseg, plan_off, ends, nodes, beta_ms, plan_status, p->stream));
+    PP_CUDA(launch_eval_packed(p->d, p->d_tables, B, total, nseg, plan_off, ends, nodes, beta_ms, plan_status, p->stream));
     return PP_OK;
 }
 
@@ -994,7 +1006,7 @@ pp_status pp_eval_plans_packed(pp_problem *p, int64_t B, int64_t total, const ui
     const size_t o_off = align_up(nB, 256), o_ends = align_up(o_off + (nB + 1) * 4, 256);
     const size_t o_nodes = align_up(o_ends + nT * 2, 256), o_beta = align_up(o_nodes + nT, 256);
     const size_t o_st = align_up(o_beta + nB * 8, 256), bytes = o_st + nB;
-    pp_status st = upload_inputs(p, false);
+    pp_status st = ensure_tables(p);
     if (st != PP_OK) return st;
     unsigned char *buf = nullptr;
     cudaStream_t s = p->stream;
@@ -1004,7 +1016,7 @@ pp_status pp_eval_plans_packed(pp_problem *p, int64_t B, int64_t total, const ui
     if (e == cudaSuccess && nT) e = cudaMemcpyAsync(buf + o_ends, ends, nT * 2, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess && nT) e = cudaMemcpyAsync(buf + o_nodes, nodes, nT, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
-        e = launch_eval_packed(p->d, B, total, buf, reinterpret_cast<uint32_t *>(buf + o_off),
+        e = launch_eval_packed(p->d, p->d_tables, B, total, buf, reinterpret_cast<uint32_t *>(buf + o_off),
                                reinterpret_cast<uint16_t *>(buf + o_ends), buf + o_nodes,
                                reinterpret_cast<double *>(buf + o_beta), buf + o_st, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(beta_ms, buf + o_beta, nB * 8, cudaMemcpyDeviceToHost, s);
@@ -1021,9 +1033,9 @@ pp_status pp_random_plans_dev(pp_problem *p, int64_t P, const uint32_t *draws, u
     if (!p || P < 0) return PP_ERR_ARG;
     if (P == 0) return PP_OK;
     if (!draws || !nseg || !ends || !nodes) return PP_ERR_ARG;
-    pp_status st = upload_inputs(p, false);
+    pp_status st = ensure_tables(p);
     if (st != PP_OK) return st;
-    PP_CUDA(launch_random_plans(p->d, P, draws, nseg, ends, nodes, p->stream));
+    PP_CUDA(launch_random_plans(p->d, p->d_tables, P, draws, nseg, ends, nodes, p->stream));
     return PP_OK;
 }
 
@@ -1037,14 +1049,14 @@ pp_status pp_random_plans(pp_problem *p, int64_t P, const uint32_t *draws, uint8
     const size_t b_draws = (size_t)P * 2 * k * 4, b_rows = (size_t)P * k * 4;
     const size_t o_ends = align_up(b_draws, 256), o_nodes = align_up(o_ends + b_rows, 256);
     const size_t o_nseg = align_up(o_nodes + b_rows, 256), total = o_nseg + (size_t)P;
-    pp_status st = upload_inputs(p, false);
+    pp_status st = ensure_tables(p);
     if (st != PP_OK) return st;
     unsigned char *buf = nullptr;
     cudaStream_t s = p->stream;
     PP_CUDA(staging_alloc(reinterpret_cast<void **>(&buf), total, s));
     cudaError_t e = cudaMemcpyAsync(buf, draws, b_draws, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
-        e = launch_random_plans(p->d, P, reinterpret_cast<uint32_t *>(buf), buf + o_nseg,
+        e = launch_random_plans(p->d, p->d_tables, P, reinterpret_cast<uint32_t *>(buf), buf + o_nseg,
                                 reinterpret_cast<int32_t *>(buf + o_ends),
                                 reinterpret_cast<int32_t *>(buf + o_nodes), s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(nseg, buf + o_nseg, (size_t)P, cudaMemcpyDeviceToHost, s);

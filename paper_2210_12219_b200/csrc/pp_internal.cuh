@@ -79,9 +79,26 @@ bool pair_meta_build(int L, int k, const int16_t *lo, void *out);
 bool pair_sweep_takes(const Dev &d, int level, bool whenever_possible);
 cudaError_t launch_sweep_pair(const Dev &d, int level, cudaStream_t s, bool first_level);
 cudaError_t launch_finalize(const Dev &d, pp_solution *out, cudaStream_t s, bool dependent);
-cudaError_t launch_eval(const Dev &d, int64_t B, const uint8_t *nseg, const int32_t *ends,
+// What the evaluator and the random plans look up, laid out once per problem on the device as their
+// kernels stage it in shared memory: output bits of the layers, bandwidths with a row and a column of
+// zeros for "no such node", forward windows fwd[w * L + first] = layers from `first` on that fit node w
+// (a row of zeros for no such node, one entry more for a segment that would start behind the chain).
+struct PlanTables {
+    size_t bits, bw, fwd, total;
+};
+__host__ __device__ inline PlanTables plan_tables(int L, int k)
+{
+    PlanTables t;
+    t.bits = 0;
+    t.bw = ((size_t)L * 8 + 15) & ~(size_t)15;
+    t.fwd = t.bw + (((size_t)(k + 1) * (k + 1) * 4 + 15) & ~(size_t)15);
+    t.total = t.fwd + ((((size_t)(k + 1) * L + 1) * 2 + 15) & ~(size_t)15);
+    return t;
+}
+cudaError_t launch_plan_tables(const Dev &d, unsigned char *out, cudaStream_t s);
+cudaError_t launch_eval(const Dev &d, const unsigned char *tables, int64_t B, const uint8_t *nseg, const int32_t *ends,
                         const int32_t *nodes, double *beta, uint8_t *status, cudaStream_t s);
-cudaError_t launch_eval_packed(const Dev &d, int64_t B, int64_t total, const uint8_t *nseg, const uint32_t *off,
+cudaError_t launch_eval_packed(const Dev &d, const unsigned char *tables, int64_t B, int64_t total, const uint8_t *nseg, const uint32_t *off,
                                const uint16_t *ends, const uint8_t *nodes, double *beta, uint8_t *status,
                                cudaStream_t s);
 size_t batch_smem_bytes(int L, int k);
@@ -158,8 +175,8 @@ int prune_row_pad(int L);
 void prune_ctl_init(PruneCtl *c);
 cudaError_t launch_prune(const PruneDev &d, int sms, cudaStream_t s);
 // Random comparison baseline (Section 4): P plans of problem d from 2 k draws each.
-cudaError_t launch_random_plans(const Dev &d, int64_t P, const uint32_t *draws, uint8_t *nseg, int32_t *ends,
-                                int32_t *nodes, cudaStream_t s);
+cudaError_t launch_random_plans(const Dev &d, const unsigned char *tables, int64_t P, const uint32_t *draws, uint8_t *nseg,
+                                int32_t *ends, int32_t *nodes, cudaStream_t s);
 // Greedy comparison baseline (Section 4), one warp per instance.
 cudaError_t launch_greedy(int64_t B, int L, int k, const uint64_t *bits, const uint64_t *mem,
                           const uint64_t *cap, const uint32_t *bw, double *beta, int32_t *m, int32_t *cuts,

@@ -7,105 +7,124 @@
 // (nseg = 0, rows of -1) when the chosen node holds not even the next layer, or when all k
 // nodes are used and layers are left over.
 //
-// A plan is 2 k dependent steps of a few dozen scalar instructions; the kernel reads 8 k bytes
-// of draws and writes 1 + 8 k bytes per plan, so with enough plans it is bound by HBM bandwidth.
+// A plan is a chain of dependent steps, so with the tens of thousands of plans of a call the kernel is
+// bound by the latency of a step and by getting the rows in and out.  How many layers from a given one
+// on fit a node is looked up (a table of k * L counts, made once per problem) instead of
+// bisected over the prefix sums, and the r-th free node is found by counting bits in halves: a step is
+// some forty instructions for every lane alike (a bisection and a walk over the free nodes before:
+// 100 003 plans of k = 14, L = 50 in 14.4 us).
 #include "pp_internal.cuh"
 
 namespace pp {
 
 constexpr int kRandomThreads = 128;
 
-// Rows travel through shared memory so that global memory sees whole contiguous blocks: the draws
-// of the block's plans on the way in, their two output rows on the way out.  A thread's outputs
-// overwrite its own draws: step s has read words 2s and 2s+1 before segment n <= s + 1 goes to
-// words 2(n-1) (cut) and 2(n-1)+1 (node).  The row stride is odd, which keeps the threads of a
-// warp, each on its own row, on different banks.  The prefix sums and capacities are staged too:
-// the bisection reads them at dependent addresses.
-__global__ void __launch_bounds__(kRandomThreads)
-k_random_plans(Dev d, int64_t P, const uint32_t *__restrict__ draws, uint8_t *nseg, int32_t *ends, int32_t *nodes)
+// r-th (from 0) set bit of x; r below the number of set bits
+__device__ __forceinline__ int select_bit(uint32_t x, int r)
 {
-    extern __shared__ uint32_t smem_words[];
-    const int k = d.k, L = d.L, W = 2 * k, stride = W + 1, tid = threadIdx.x;
-    uint32_t *sd = smem_words;  // [threads][stride]: draws in, (cut, node) pairs out
-    uint64_t *sM = reinterpret_cast<uint64_t *>(smem_words + ((kRandomThreads * stride + 1) & ~1));  // [L+1]
-    uint64_t *scap = sM + L + 1;                                                                     // [k]
-    for (int i = tid; i <= L; i += kRandomThreads) sM[i] = d.M[i];
-    for (int i = tid; i < k; i += kRandomThreads) scap[i] = d.cap[i];
+    int at = 0;
+#pragma unroll
+    for (int half = 16; half; half >>= 1) {
+        const int below = __popc(x & ((1u << half) - 1u));
+        const bool up = r >= below;
+        r -= up ? below : 0;
+        at += up ? half : 0;
+        x = up ? x >> half : x;
+    }
+    return at;
+}
+
+// Rows travel through shared memory so that global memory sees whole contiguous blocks: the draws
+// of the block's plans on the way in, their two output rows on the way out, a pair of words at a time.  A
+// thread's outputs overwrite its own draws: step s has read pair s before segment n <= s + 1 goes to pair
+// n - 1 as (cut, node).  The row stride is an odd number of pairs, which keeps the threads of a warp, each
+// on its own row, on different banks.
+__global__ void __launch_bounds__(kRandomThreads)
+k_random_plans(const int L, const int k, const uint16_t *__restrict__ fwd, const int64_t P, const uint32_t *__restrict__ draws,
+               uint8_t *nseg, int32_t *ends, int32_t *nodes)
+{
+    extern __shared__ uint2 smem_pairs[];
+    const int stride = k | 1, tid = threadIdx.x;
+    uint2 *sd = smem_pairs;  // [threads][stride]: draws in, (cut, node) pairs out
+    uint16_t *s_fwd = reinterpret_cast<uint16_t *>(smem_pairs + kRandomThreads * stride);  // [k][L]
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // whatever wrote fwd, or reads or writes the plans, is complete
+    asm volatile("griddepcontrol.launch_dependents;");
     const int64_t p0 = (int64_t)blockIdx.x * kRandomThreads;
     const int np = P - p0 < kRandomThreads ? (int)(P - p0) : kRandomThreads;
+    const int r0 = tid / k, c0 = tid - r0 * k, dr = kRandomThreads / k, dc = kRandomThreads - dr * k;
+    const uint32_t *src = draws + p0 * 2 * k;
+    const bool pairs = (reinterpret_cast<uintptr_t>(draws) & 7u) == 0;
     {
-        const uint32_t *src = draws + p0 * W;
-        int r = tid / W, c = tid - r * W;
-        const int dr = kRandomThreads / W, dc = kRandomThreads - dr * W;
-        for (int i = tid; i < np * W; i += kRandomThreads) {
-            sd[r * stride + c] = src[i];
-            r += dr;
+        int at = r0 * stride + c0, c = c0;
+        const int step = dr * stride + dc, carry = stride - k;
+#pragma unroll 4
+        for (int i = tid; i < np * k; i += kRandomThreads) {
+            sd[at] = pairs ? reinterpret_cast<const uint2 *>(src)[i] : make_uint2(src[2 * i], src[2 * i + 1]);
+            at += step;
             c += dc;
-            if (c >= W) { c -= W; ++r; }
+            if (c >= k) { c -= k; at += carry; }
         }
     }
+    for (int i = tid; i < k * L; i += kRandomThreads) s_fwd[i] = fwd[i];
     __syncthreads();
     if (tid < np) {
-        const uint32_t *dr = sd + tid * stride;
-        int32_t *out = reinterpret_cast<int32_t *>(sd + tid * stride);
-        uint32_t used = 0;
+        uint2 *row = sd + tid * stride;
+        uint32_t free_nodes = (1u << k) - 1u;
         int first = 0, n = 0;
         bool done = false;
         for (int step = 0; step < k; ++step) {
-            // node: the r-th node not used yet
-            int r = (int)(((unsigned long long)dr[2 * step] * (unsigned)(k - step)) >> 32);
-            uint32_t free_nodes = ~used & ((1u << k) - 1u);
-            for (; r > 0; --r) free_nodes &= free_nodes - 1;
-            const int node = __ffs(free_nodes) - 1;
-            // segments [first, e] that fit: prefix sums ascend, so a bisection finds how many
-            const uint64_t base = sM[first], room = scap[node];
-            int lo = first, hi = L;  // every e < lo fits, no e >= hi does
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (sM[mid + 1] - base <= room) lo = mid + 1; else hi = mid;
-            }
-            const int count = lo - first;
+            const uint2 draw = row[step];
+            const int node = select_bit(free_nodes, (int)__umulhi(draw.x, (unsigned)(k - step)));
+            const uint32_t count = s_fwd[node * L + first];  // segments [first, e] that fit
             if (count == 0) break;
-            const int last = first + (int)(((unsigned long long)dr[2 * step + 1] * (unsigned)count) >> 32);
-            used |= 1u << node;
-            out[2 * n + 1] = node;
+            const int last = first + (int)__umulhi(draw.y, count);
+            free_nodes &= ~(1u << node);
+            done = last == L - 1;
+            row[n] = make_uint2(done ? 0xFFFFFFFFu : (uint32_t)last, (uint32_t)node);  // the last segment has no cut
             ++n;
-            if (last == L - 1) {
-                done = true;
-                break;
-            }
-            out[2 * n - 2] = last;
+            if (done) break;
             first = last + 1;
         }
         if (!done) n = 0;
         nseg[p0 + tid] = (uint8_t)n;
-        for (int i = n; i < k; ++i) out[2 * i + 1] = -1;
-        for (int i = n > 0 ? n - 1 : 0; i < k; ++i) out[2 * i] = -1;
+        for (int i = n; i < k; ++i) row[i] = make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
     }
     __syncthreads();
     {
         int32_t *de = ends + p0 * k, *dn = nodes + p0 * k;
-        int r = tid / k, c = tid - r * k;
-        const int dr = kRandomThreads / k, dc = kRandomThreads - dr * k;
+        int at = r0 * stride + c0, c = c0;
+        const int step = dr * stride + dc, carry = stride - k;
+#pragma unroll 4
         for (int i = tid; i < np * k; i += kRandomThreads) {
-            de[i] = (int32_t)sd[r * stride + 2 * c];
-            dn[i] = (int32_t)sd[r * stride + 2 * c + 1];
-            r += dr;
+            const uint2 x = sd[at];
+            de[i] = (int32_t)x.x;
+            dn[i] = (int32_t)x.y;
+            at += step;
             c += dc;
-            if (c >= k) { c -= k; ++r; }
+            if (c >= k) { c -= k; at += carry; }
         }
     }
 }
 
-cudaError_t launch_random_plans(const Dev &d, int64_t P, const uint32_t *draws, uint8_t *nseg, int32_t *ends,
-                                int32_t *nodes, cudaStream_t s)
+cudaError_t launch_random_plans(const Dev &d, const unsigned char *tables, int64_t P, const uint32_t *draws, uint8_t *nseg,
+                                int32_t *ends, int32_t *nodes, cudaStream_t s)
 {
     const int64_t blocks = (P + kRandomThreads - 1) / kRandomThreads;
     if (blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
-    const size_t smem = (((size_t)kRandomThreads * (2 * d.k + 1) + 1) & ~(size_t)1) * sizeof(uint32_t) +
-                        ((size_t)d.L + 1 + d.k) * sizeof(uint64_t);  // at most 29 KB (k = 20, L = 1024)
-    k_random_plans<<<(unsigned)blocks, kRandomThreads, smem, s>>>(d, P, draws, nseg, ends, nodes);
-    return cudaGetLastError();
+    const size_t smem = (size_t)kRandomThreads * (d.k | 1) * sizeof(uint2) + (size_t)d.k * d.L * sizeof(uint16_t);
+    cudaError_t e = cudaFuncSetAttribute(k_random_plans, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+    if (e != cudaSuccess) return e;  // at most 62 KB (k = 20, L = 1024)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(kRandomThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_random_plans, d.L, d.k, reinterpret_cast<const uint16_t *>(tables + plan_tables(d.L, d.k).fwd), P, draws, nseg, ends, nodes);
 }
 
 }  // namespace pp

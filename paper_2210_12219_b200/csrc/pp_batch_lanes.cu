@@ -8,7 +8,7 @@
 // few thousand instances), instance-minor: the 32 lanes of a warp read 32 neighbouring words.
 //
 // Per chunk of instances:
-//   1. k_lanes_prep, one warp per instance: staging, windows, the ranking of gamma (Eq. 3); writes
+//   1. k_lanes_prep, one block per instance: staging, windows, the ranking of gamma (Eq. 3); writes
 //      the instance's column of the rank table, the window lengths, the base frontier and the best
 //      single-node plan;
 //   2. one launch per popcount level, k_lanes_level<NV, LH>: a warp takes (group of 32 instances,
@@ -29,10 +29,8 @@ namespace {
 
 constexpr int kLevelWarps = 4;
 constexpr int kLevelFourBlocks = 5;  // source masks of up to this many nodes: registers capped for four blocks per SM
-constexpr int kPrepWarps = 4;
+constexpr int kPrepThreads = 128, kPrepBlocks = 12;  // 18 KB of shared memory a block at most
 constexpr int kFlagLimit = 1;     // BatchLanes::flag: an input beyond the limits
-constexpr int kFlagDeferred = 2;  // ... the first preparing pass left the ranking to the second
-constexpr int kWalks = 2;  // staircase walks a lane runs interleaved: the walk is a chain of dependent loads
 constexpr int kBackWarps = 8;
 constexpr int kLanesMinB = 64;  // below this the block-per-instance kernel keeps more of the GPU busy
 constexpr int kLanesMaxK = 8;   // NV <= 7 rows of a source mask in registers
@@ -61,157 +59,140 @@ __device__ __forceinline__ void st_table(const BatchLanes &t, uint32_t *p, const
     if (PP_IN_BOUNDS(t, (size_t)(p - base), words)) *p = v;
 }
 
-// Shared memory of one warp of the preparing kernel (byte offsets; every part 16-byte aligned).
+// Word e of an instance's column (rows of LH words one after another): the 32 instances of a group lie
+// side by side in pieces of kPiece words, so that a lane moves a piece at a time.
+constexpr int kPiece = 2;   // 4096 x (k = 8, L = 24), us a call: 1 word 261, 2 words 235, 4 words 245 (spills in the level kernels)
+struct alignas(4 * kPiece) Piece {
+    uint32_t w[kPiece];
+};
+__host__ __device__ inline size_t word_at(size_t e) { return e / kPiece * (32 * kPiece) + e % kPiece; }
+__device__ __forceinline__ Piece ld_piece(const BatchLanes &t, const uint32_t *p, const uint32_t *base, size_t words)
+{
+    Piece x;
+    if (PP_IN_BOUNDS(t, (size_t)(p - base), words)) {
+        x = *reinterpret_cast<const Piece *>(p);
+    } else {
+        for (int i = 0; i < kPiece; ++i) x.w[i] = 0xFFFFFFFFu;
+    }
+    return x;
+}
+__device__ __forceinline__ void st_piece(const BatchLanes &t, uint32_t *p, const uint32_t *base, size_t words, const Piece &v)
+{
+    if (PP_IN_BOUNDS(t, (size_t)(p - base), words)) *reinterpret_cast<Piece *>(p) = v;
+}
+
+// Shared memory of an instance in the preparing kernel (byte offsets; every part 16-byte aligned).
+constexpr int kBuckets = 1024;  // of the ranking; two 16-bit counters per word
 struct PrepLayout {
-    size_t K, M, bits, sorted, cap, bw, ubw, rk, pair_u, rowu, pos, total;
-    int Ks;  // row stride of the quotient matrix in keys: a sentinel in front of the L quotients
+    size_t val, M, bits, cap, bw, ubw, hist, rk, pair_u, total;
 };
 
-__host__ __device__ inline PrepLayout prep_layout(int L, int ucap)
+__host__ __device__ inline PrepLayout prep_layout(int L, int k)
 {
     PrepLayout p;
-    const size_t U = (size_t)ucap;  // distinct bandwidths the quotient matrix has room for
+    const size_t n = (size_t)k * (k - 1) * L;  // quotients
     size_t o = 0;
     auto take = [&o](size_t bytes) { size_t at = o; o = (o + bytes + 15) & ~(size_t)15; return at; };
-    p.Ks = L + 1;
-    p.K = take((U + 1) * (size_t)p.Ks * 8);
+    p.val = take(n * 4);
     p.M = take(33 * 8);
     p.bits = take(32 * 8);
-    p.sorted = take(32 * 8);
     p.cap = take(8 * 8);
     p.bw = take(64 * 4);
     p.ubw = take(64 * 4);
-    p.rk = take((U * L + 1) * 2);
+    p.hist = take((size_t)kBuckets / 2 * 4);
+    p.rk = take(n * 4);
     p.pair_u = take(64);
-    p.rowu = take(64);
-    p.pos = take(32);
     p.total = o;
     return p;
 }
 
-// One warp per instance, lane <-> layer (L <= 32) or node pair (k * k <= 64, two per lane): staging,
-// the windows, the ranking of gamma (Eq. 3), and the instance's column of the tables of BatchLanes.
-//   * layers ordered by bits (ties by index), distinct usable bandwidths listed in order of first
-//     appearance, as in the block-per-instance kernel;
+// One block of four warps per instance (L <= 32 layers, k * k <= 64 node pairs): staging, the windows, the
+// ranking of gamma (Eq. 3), and the instance's column of the tables of BatchLanes.
+//   * distinct usable bandwidths listed in order of first appearance;
 //   * window start lo_w(c2) by a branch-free binary search over the memory prefix sums;
-//   * rank = 1 + number of quotients strictly below.  The quotients form a matrix whose rows (one
-//     per distinct bandwidth, widest link first) and columns (layers by ascending bits) both ascend,
-//     so the count for one entry is a staircase walk: in every row step left while the element is
-//     not below the entry, add the column reached, go down a row.  Keys are the bit patterns of the
-//     quotients (positive doubles order like them) plus one, so that a zero in front of every row
-//     stops the walk to the left without a test; row U holds the largest key and empties the column
-//     counter; a walk takes exactly U + L steps.  A lane runs several walks interleaved.
-// The matrix is the bulk of a warp's shared memory, and the walks are chains of dependent loads that
-// want many warps in flight, so the kernel runs twice: the first pass has room for k (k - 1) / 2
-// distinct bandwidths (every symmetric network) and marks an instance that has more; the second pass,
-// with room for k (k - 1), takes only the marked ones and returns at once from all others.
-__global__ void __launch_bounds__(kPrepWarps * 32)
+//   * rank = 1 + number of quotients strictly below, by a bucket sort: a quotient's bucket is its place in
+//     the range of the instance's quotients on the scale of the doubles' bits (monotone, about 1 % wide),
+//     counters in shared memory, their prefix sums, the quotients scattered into the order of the
+//     buckets, and each compared with the few that share its bucket.  Some 90 instructions per quotient
+//     where a staircase walk over the sorted quotient matrix took U + L dependent steps, 350.
+// What is left is a chain of short dependent phases, a third as long with four warps to an instance as with
+// one; the SM's other instances hide it.
+__global__ void __launch_bounds__(kPrepThreads, kPrepBlocks)
 k_lanes_prep(const BatchLanes t, const int64_t B, const int L, const int k, const uint64_t *__restrict__ g_bits,
              const uint64_t *__restrict__ g_mem, const uint64_t *__restrict__ g_cap,
-             const uint32_t *__restrict__ g_bw, const int ucap, const int second_pass)
+             const uint32_t *__restrict__ g_bw)
 {
     extern __shared__ __align__(16) unsigned char smem_prep[];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const PrepLayout lay = prep_layout(L, ucap);
-    unsigned char *base = smem_prep + (size_t)wid * lay.total;
-    unsigned long long *K = reinterpret_cast<unsigned long long *>(base + lay.K);
-    unsigned long long *M = reinterpret_cast<unsigned long long *>(base + lay.M);
-    unsigned long long *s_bits = reinterpret_cast<unsigned long long *>(base + lay.bits);
-    unsigned long long *s_sorted = reinterpret_cast<unsigned long long *>(base + lay.sorted);
-    unsigned long long *s_cap = reinterpret_cast<unsigned long long *>(base + lay.cap);
-    uint32_t *s_bw = reinterpret_cast<uint32_t *>(base + lay.bw);
-    uint32_t *ubw = reinterpret_cast<uint32_t *>(base + lay.ubw);
-    uint16_t *rk = reinterpret_cast<uint16_t *>(base + lay.rk);
-    int8_t *pair_u = reinterpret_cast<int8_t *>(base + lay.pair_u);
-    uint8_t *rowu = base + lay.rowu;
-    uint8_t *pos = base + lay.pos;
-    const int Ks = lay.Ks, LH = t.LH, kk = k * k;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const PrepLayout lay = prep_layout(L, k);
+    uint32_t *s_val = reinterpret_cast<uint32_t *>(smem_prep + lay.val);
+    unsigned long long *M = reinterpret_cast<unsigned long long *>(smem_prep + lay.M);
+    unsigned long long *s_bits = reinterpret_cast<unsigned long long *>(smem_prep + lay.bits);
+    unsigned long long *s_cap = reinterpret_cast<unsigned long long *>(smem_prep + lay.cap);
+    uint32_t *s_bw = reinterpret_cast<uint32_t *>(smem_prep + lay.bw);
+    uint32_t *ubw = reinterpret_cast<uint32_t *>(smem_prep + lay.ubw);
+    uint32_t *hist = reinterpret_cast<uint32_t *>(smem_prep + lay.hist);
+    uint32_t *rk = reinterpret_cast<uint32_t *>(smem_prep + lay.rk);
+    int8_t *pair_u = reinterpret_cast<int8_t *>(smem_prep + lay.pair_u);
+    __shared__ uint32_t s_first[2], s_sum[kPrepThreads / 32];
+    const int LH = t.LH, kk = k * k;
     const uint32_t FULL = 0xFFFFFFFFu;
-    // floor(x / k) for x < 64 and floor(x / L) for x < k (k-1) L <= 1792 by a multiplication
+    // floor(x / k) for x < 64, floor(x / L) for x < k (k-1) L <= 1792, floor(x / LH) for x < k k LH <= 1024
     const uint32_t recip_k = (65536u + (uint32_t)k - 1u) / (uint32_t)k;
     const uint32_t recip_L = (65536u + (uint32_t)L - 1u) / (uint32_t)L;
-    for (int64_t inst = (int64_t)blockIdx.x * kPrepWarps + wid; inst < B; inst += (int64_t)gridDim.x * kPrepWarps) {
-        if (second_pass && !(t.flag[inst] & kFlagDeferred)) continue;  // ranked by the first pass
-        __syncwarp();
+    const uint32_t recip_LH = (65536u + (uint32_t)LH - 1u) / (uint32_t)LH;
+    for (int64_t inst = blockIdx.x; inst < B; inst += gridDim.x) {
+        __syncthreads();
         // ---- staging, prefix sums of the memory ----
-        const unsigned long long b = lane < L ? g_bits[inst * L + lane] : 0ull;
-        const unsigned long long mm = lane < L ? g_mem[inst * L + lane] : 0ull;
-        const uint32_t bw0 = lane < kk ? g_bw[inst * kk + lane] : 0u;
-        const uint32_t bw1 = lane + 32 < kk ? g_bw[inst * kk + lane + 32] : 0u;
-        bool bad = b >= PP_MAX_BITS || bw0 >= PP_MAX_KBPS || bw1 >= PP_MAX_KBPS;
-        unsigned long long x = mm;
+        bool bad = false;
+        if (wid == 0) {
+            const unsigned long long b = lane < L ? g_bits[inst * L + lane] : 0ull;
+            unsigned long long x = lane < L ? g_mem[inst * L + lane] : 0ull;
+            bad = b >= PP_MAX_BITS;
+            s_bits[lane] = b;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long y = __shfl_up_sync(FULL, x, o);
-            if (lane >= o) {
-                if (y > ~0ull - x) bad = true;  // the 64-bit sum would wrap: PP_ERR_LIMIT
-                x += y;
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long y = __shfl_up_sync(FULL, x, o);
+                if (lane >= o) {
+                    if (y > ~0ull - x) bad = true;  // the 64-bit sum would wrap: PP_ERR_LIMIT
+                    x += y;
+                }
             }
+            if (lane == 0) M[0] = 0ull;
+            M[lane + 1] = x;  // beyond L: the total, never read
+        } else if (wid < 3) {
+            const int p = tid - 32, v = (int)(((uint32_t)p * recip_k) >> 16);
+            const uint32_t x = p < kk ? g_bw[inst * kk + p] : 0u;
+            bad = x >= PP_MAX_KBPS;
+            s_bw[p] = p < kk && v != p - v * k ? x : 0u;  // 0: no usable link
+        } else if (lane < k) {
+            s_cap[lane] = g_cap[inst * k + lane];
         }
-        if (lane == 0) M[0] = 0ull;
-        M[lane + 1] = x;  // beyond L: the total, never read
-        s_bits[lane] = b;
-        s_bw[lane] = bw0;
-        s_bw[lane + 32] = bw1;
-        if (lane < k) s_cap[lane] = g_cap[inst * k + lane];
-        bad = __any_sync(FULL, bad);
-        __syncwarp();
-        // ---- layers in ascending order of bits (ties by index) ----
-        {
-            int p = 0;
-            for (int o = 0; o < L; ++o) {
-                const unsigned long long xo = s_bits[o];
-                p += (xo < b) || (xo == b && o < lane);
-            }
-            if (lane < L) {
-                s_sorted[p] = b;
-                pos[lane] = (uint8_t)p;
-            }
-        }
+        reinterpret_cast<uint4 *>(hist)[tid] = make_uint4(0u, 0u, 0u, 0u);
+        bad = __syncthreads_or(bad);
         // ---- distinct usable bandwidths in order of first appearance ----
-        int U;
-        {
-            const int p0 = lane, p1 = lane + 32;
-            const int v0 = (int)(((uint32_t)p0 * recip_k) >> 16), v1 = (int)(((uint32_t)p1 * recip_k) >> 16);
-            const bool us0 = p0 < kk && v0 != p0 - v0 * k && bw0 != 0u;
-            const bool us1 = p1 < kk && v1 != p1 - v1 * k && bw1 != 0u;
-            int f0 = us0 ? p0 : -1, f1 = us1 ? p1 : -1;
-            int v2 = 0, w2 = 0;
-            for (int p2 = 0; p2 < kk; ++p2) {  // ascending: the first match stays
-                const uint32_t b2 = s_bw[p2];
-                const bool us2 = v2 != w2 && b2 != 0u;
-                if (us2 && us0 && b2 == bw0 && p2 < f0) f0 = p2;
-                if (us2 && us1 && b2 == bw1 && p2 < f1) f1 = p2;
-                if (++w2 == k) { w2 = 0; ++v2; }
+        uint32_t x = 0;
+        int f = 0;
+        if (wid < 2) {
+            x = s_bw[tid];
+#pragma unroll 4
+            for (int p4 = 60; p4 >= 0; p4 -= 4) {  // descending: the first appearance stays
+                const uint4 q = *reinterpret_cast<const uint4 *>(s_bw + p4);
+                f = q.w == x ? p4 + 3 : f;
+                f = q.z == x ? p4 + 2 : f;
+                f = q.y == x ? p4 + 1 : f;
+                f = q.x == x ? p4 : f;
             }
-            const bool first0 = us0 && f0 == p0, first1 = us1 && f1 == p1;
-            const uint32_t m0 = __ballot_sync(FULL, first0), m1 = __ballot_sync(FULL, first1);
-            const int n0 = __popc(m0);
-            U = n0 + __popc(m1);
-            auto index_of = [&](int f) {
-                return f < 32 ? __popc(m0 & ((1u << f) - 1u)) : n0 + __popc(m1 & ((1u << (f - 32)) - 1u));
-            };
-            const int u0 = f0 >= 0 ? index_of(f0) : -1, u1 = f1 >= 0 ? index_of(f1) : -1;
-            pair_u[p0] = (int8_t)u0;
-            pair_u[p1] = (int8_t)u1;
-            if (first0) ubw[u0] = bw0;
-            if (first1) ubw[u1] = bw1;
-        }
-        __syncwarp();
-        // rows of the quotient matrix: widest link first (the values of a column then ascend)
-        for (int u = lane; u < U; u += 32) {
-            const uint32_t mine = ubw[u];
-            int r = 0;
-            for (int u2 = 0; u2 < U; ++u2) r += ubw[u2] > mine;
-            rowu[r] = (uint8_t)u;
+            const uint32_t firsts = __ballot_sync(FULL, x != 0u && f == tid);
+            if (lane == 0) s_first[wid] = firsts;
         }
         // ---- windows, base frontier ----
         {
-            uint32_t *lT = t.len + (size_t)(inst >> 5) * (size_t)(k * LH) * 32 + (inst & 31);
-            uint32_t *tT = t.table + (size_t)(inst >> 5) * (size_t)t.rows * LH * 32 + (inst & 31);
-            uint32_t *wT = t.win + (size_t)(inst >> 5) * (size_t)(k * 2 * LH) * 32 + (inst & 31);
+            uint32_t *lT = t.len + (size_t)(inst >> 5) * (size_t)(k * LH) * 32 + (inst & 31) * kPiece;
+            uint32_t *tT = t.table + (size_t)(inst >> 5) * (size_t)t.rows * LH * 32 + (inst & 31) * kPiece;
+            uint32_t *wT = t.win + (size_t)(inst >> 5) * (size_t)(k * 2 * LH) * 32 + (inst & 31) * kPiece;
             const unsigned long long Mc = M[lane + 1];  // memory of layers 0..lane
-            for (int w = 0; w < k; ++w) {
+            for (int w = 3 - wid; w < k; w += kPrepThreads / 32) {
                 const unsigned long long capw = s_cap[w];
                 // c* = number of prefix sums M[0..lane+1] below M[lane+1] - cap: the first start layer
                 // from which the segment ending at this layer fits; window start = max(c* - 1, 0)
@@ -225,97 +206,120 @@ k_lanes_prep(const BatchLanes t, const int64_t B, const int L, const int k, cons
                 const uint32_t inf = (lane < L && Mc <= capw) ? 0u : 0xFFFFu;
                 const uint32_t len0 = __shfl_sync(FULL, len, 2 * lane), len1 = __shfl_sync(FULL, len, 2 * lane + 1);
                 const uint32_t inf0 = __shfl_sync(FULL, inf, 2 * lane), inf1 = __shfl_sync(FULL, inf, 2 * lane + 1);
-                {
-                    // window [lo, lane - 1] of length len >= 1 = union of the two runs of 2^s positions
-                    // that end at lane - 1 and that start at lo, s = floor(log2 len): their sparse-table
-                    // cells; an empty window reads the cell that holds +inf
-                    uint32_t code = win_cell(kWinLevels, 0, LH) * 0x00010001u;
-                    if (len != 0u) {
-                        const int sl = 31 - __clz((int)len);
-                        code = win_cell(sl, lane - 1, LH) | (win_cell(sl, lo + (1 << sl) - 1, LH) << 16);
-                    }
-                    // position 0 has no window: its entry carries the highest level this node's windows read
-                    const uint32_t longest = __reduce_max_sync(FULL, len);
-                    if (lane == 0) code = longest > 1u ? (uint32_t)(31 - __clz((int)longest)) : 0u;
-                    if (lane < 2 * LH) st_table(t, wT + (size_t)(w * 2 * LH + lane) * 32, t.win, t.win_words, code);
+                // window [lo, lane - 1] of length len >= 1 = union of the two runs of 2^s positions
+                // that end at lane - 1 and that start at lo, s = floor(log2 len): their sparse-table
+                // cells; an empty window reads the cell that holds +inf
+                uint32_t code = win_cell(kWinLevels, 0, LH) * 0x00010001u;
+                if (len != 0u) {
+                    const int sl = 31 - __clz((int)len);
+                    code = win_cell(sl, lane - 1, LH) | (win_cell(sl, lo + (1 << sl) - 1, LH) << 16);
                 }
+                // position 0 has no window: its entry carries the highest level this node's windows read
+                const uint32_t longest = __reduce_max_sync(FULL, len);
+                if (lane == 0) code = longest > 1u ? (uint32_t)(31 - __clz((int)longest)) : 0u;
+                if (lane < 2 * LH) st_table(t, wT + word_at(w * 2 * LH + lane), t.win, t.win_words, code);
                 if (lane < LH) {
-                    st_table(t, lT + (size_t)(w * LH + lane) * 32, t.len, t.len_words, lane < 16 ? len0 | (len1 << 16) : 0u);
-                    st_table(t, tT + ((size_t)t.rowoff[1u << w] * LH + lane) * 32, t.table, t.table_words,
+                    st_table(t, lT + word_at(w * LH + lane), t.len, t.len_words, lane < 16 ? len0 | (len1 << 16) : 0u);
+                    st_table(t, tT + word_at((size_t)t.rowoff[1u << w] * LH + lane), t.table, t.table_words,
                              lane < 16 ? inf0 | (inf1 << 16) : 0xFFFFFFFFu);
                 }
             }
-            if (lane == 0) {
-                unsigned long long best = kNoBest;
-                for (int v = k - 1; v >= 0; --v)
-                    if (M[L] <= s_cap[v]) best = pack_best(0u, 1, 1u << v, v);
-                t.key[inst] = best;
-                t.flag[inst] = (int8_t)((bad ? kFlagLimit : 0) | (U > ucap ? kFlagDeferred : 0));
+        }
+        __syncthreads();
+        const uint32_t m0 = s_first[0], m1 = s_first[1];
+        const int n0 = __popc(m0), U = n0 + __popc(m1);
+        if (wid < 2) {
+            const int u = x == 0u ? -1 : f < 32 ? __popc(m0 & ((1u << f) - 1u)) : n0 + __popc(m1 & ((1u << (f - 32)) - 1u));
+            pair_u[tid] = (int8_t)u;
+            if (x != 0u && f == tid) ubw[u] = x;
+        }
+        if (tid == kPrepThreads - 1) {
+            unsigned long long best = kNoBest;
+            for (int v = k - 1; v >= 0; --v)
+                if (M[L] <= s_cap[v]) best = pack_best(0u, 1, 1u << v, v);
+            t.key[inst] = best;
+            t.flag[inst] = (int8_t)(bad ? kFlagLimit : 0);
+        }
+        // ---- ranks of the quotients ----
+        const int n = U * L;
+        // upper words of doubles that no positive quotient lies outside of
+        const unsigned long long b = s_bits[lane];
+        const uint32_t p0 = s_bw[lane], p1 = s_bw[lane + 32];
+        const uint32_t least = __reduce_min_sync(FULL, lane < L && b ? __float_as_uint(__ull2float_rd(b)) : 0x7F800000u);
+        const uint32_t most = __reduce_max_sync(FULL, lane < L ? __float_as_uint(__ull2float_ru(b)) : 0u);
+        const uint32_t fast = __reduce_max_sync(FULL, max(p0, p1));
+        const uint32_t slow = __reduce_min_sync(FULL, min(p0 ? p0 : FULL, p1 ? p1 : FULL));
+        const int hi0 = __double2hiint(__ddiv_rd((double)__uint_as_float(least), (double)fast));
+        const int hi1 = __double2hiint(__ddiv_ru((double)__uint_as_float(most), (double)slow));
+        const int shift = max(0, 32 - __clz(max(hi1 - hi0, 0)) - 10);  // 2^10 = kBuckets
+        const unsigned long long lowest = (unsigned long long)(uint32_t)hi0 << 32;
+        __syncthreads();
+        auto quotient = [&](int e) {
+            const int u = (int)(((uint32_t)e * recip_L) >> 16);
+            return __ddiv_rn((double)s_bits[e - u * L], (double)ubw[u]);
+        };
+        for (int e = tid; e < n; e += kPrepThreads) {
+            // distance of the quotient's bits from the lowest (0.0 counts as the lowest): the upper bits are its
+            // bucket, the next 21 its key within the bucket
+            const unsigned long long q = (unsigned long long)__double_as_longlong(quotient(e));
+            const uint32_t y = (uint32_t)((q > lowest ? q - lowest : 0ull) >> (shift + 11));
+            rk[e] = y;
+            atomicAdd(&hist[y >> 22], 1u << ((y >> 21 & 1u) * 16));
+        }
+        __syncthreads();
+        {  // counters -> first places: a thread takes eight neighbouring buckets
+            const uint4 c = reinterpret_cast<const uint4 *>(hist)[tid];
+            uint32_t sum = c.x + c.y + c.z + c.w;
+            sum = (sum & 0xFFFFu) + (sum >> 16);
+            uint32_t upto = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(FULL, upto, o);
+                if (lane >= o) upto += y;
             }
+            if (lane == 31) s_sum[wid] = upto;
+            __syncthreads();
+            uint32_t place = upto - sum;
+            for (int i = 0; i < wid; ++i) place += s_sum[i];
+            auto next = [&](uint32_t word) {
+                const uint32_t second = place + (word & 0xFFFFu), both = place | (second << 16);
+                place = second + (word >> 16);
+                return both;
+            };
+            uint4 first;
+            first.x = next(c.x); first.y = next(c.y); first.z = next(c.z); first.w = next(c.w);
+            reinterpret_cast<uint4 *>(hist)[tid] = first;
         }
-        if (U > ucap) continue;  // more distinct bandwidths than this pass has room for: left to the second pass
-        __syncwarp();
-        // ---- quotient matrix ----
-        for (int r = 0; r <= U; ++r) {
-            unsigned long long key = ~0ull;
-            if (r < U)
-                key = 1ull + (unsigned long long)__double_as_longlong(
-                                 __ddiv_rn((double)s_sorted[lane < L ? lane : 0], (double)ubw[rowu[r]]));
-            if (lane < L) K[r * Ks + 1 + lane] = key;
-            if (lane == 0) K[r * Ks] = 0ull;
+        __syncthreads();
+        for (int e = tid; e < n; e += kPrepThreads) {
+            const uint32_t y = rk[e], half = (y >> 21 & 1u) * 16;
+            const uint32_t place = (atomicAdd(&hist[y >> 22], 1u << half) >> half) & 0xFFFFu;
+            s_val[place] = (y << 11) | (uint32_t)e;  // key and entry (n < 2^11)
         }
-        __syncwarp();
-        // ---- ranks ----
-        {
-            // The column counter is not kept: a step down from row r at column j leaves from byte
-            // offset 8 (r Ks + j), so the sum of the offsets of the U steps down is
-            // 8 (Ks U (U - 1) / 2 + sum of the columns).
-            const int n = U * L, steps = U + L;
-            const unsigned char *Kb = reinterpret_cast<const unsigned char *>(K);
-            const int down = Ks * 8, start = L * 8;  // the last quotient of row 0
-            const int rows_part = Ks * (U * (U - 1) / 2);
-            for (int e0 = 0; e0 < n; e0 += 32 * kWalks) {
-                unsigned long long x[kWalks];
-                int p[kWalks], sum[kWalks], cell[kWalks];
-#pragma unroll
-                for (int q = 0; q < kWalks; ++q) {
-                    const int e = e0 + 32 * q + lane;
-                    const int r = (int)(((uint32_t)e * recip_L) >> 16), i = e - r * L;
-                    // an idle lane walks with the smallest key: left along row 0, then down the zeros
-                    x[q] = e < n ? K[r * Ks + 1 + i] : 1ull;
-                    cell[q] = e < n ? rowu[r] * L + i : -1;
-                    p[q] = start;
-                    sum[q] = 0;
-                }
-#pragma unroll 2
-                for (int st = 0; st < steps; ++st) {
-#pragma unroll
-                    for (int q = 0; q < kWalks; ++q) {
-                        const bool ge = *reinterpret_cast<const unsigned long long *>(Kb + p[q]) >= x[q];
-                        sum[q] += ge ? 0 : p[q];
-                        p[q] += ge ? -8 : down;
-                    }
-                }
-#pragma unroll
-                for (int q = 0; q < kWalks; ++q)
-                    if (cell[q] >= 0) rk[cell[q]] = (uint16_t)(1 + (sum[q] >> 3) - rows_part);
+        __syncthreads();
+        // a counter now holds the end of its bucket, that is the start of the next one
+        for (int e = tid; e < n; e += kPrepThreads) {
+            const uint32_t y = rk[e], mine = (y << 11) | (uint32_t)e, bk = y >> 21, half = (bk & 1u) * 16;
+            const int start = bk ? (int)((hist[(bk - 1) >> 1] >> (16 - half)) & 0xFFFFu) : 0;
+            const int end = (int)((hist[bk >> 1] >> half) & 0xFFFFu);
+            int below = start;
+            for (int q = start; q < end; ++q) {
+                const uint32_t other = s_val[q];
+                if ((other ^ mine) >= 2048u) below += other < mine;
+                else if (other != mine) below += quotient((int)(other & 2047u)) < quotient(e);  // one key: the doubles decide
             }
+            rk[e] = (uint32_t)(1 + below);
         }
-        __syncwarp();
+        __syncthreads();
         // ---- rank table, two positions per word: rank[v][w][c] = rank of (bandwidth of v -> w, layer c) ----
         {
-            uint32_t *rT = t.rank + (size_t)(inst >> 5) * (size_t)(kk * LH) * 32 + (inst & 31);
-            const int c0 = 2 * lane, c1 = 2 * lane + 1;
-            const int q0 = c0 < L ? pos[c0] : 0, q1 = c1 < L ? pos[c1] : 0;
-            for (int pr = 0; pr < kk; ++pr) {
+            uint32_t *rT = t.rank + (size_t)(inst >> 5) * (size_t)(kk * LH) * 32 + (inst & 31) * kPiece;
+            for (int e = tid; e < kk * LH; e += kPrepThreads) {
+                const int pr = (int)(((uint32_t)e * recip_LH) >> 16), c0 = 2 * (e - pr * LH);
                 const int u = pair_u[pr];
-                uint32_t word = 0xFFFFFFFFu;
-                if (u >= 0) {
-                    const uint32_t a = c0 < L ? rk[u * L + q0] : 0xFFFFu;
-                    const uint32_t c = c1 < L ? rk[u * L + q1] : 0xFFFFu;
-                    word = a | (c << 16);
-                }
-                if (lane < LH) st_table(t, rT + (size_t)(pr * LH + lane) * 32, t.rank, t.rank_words, word);
+                const uint32_t a = u >= 0 && c0 < L ? rk[u * L + c0] : 0xFFFFu;
+                const uint32_t c = u >= 0 && c0 + 1 < L ? rk[u * L + c0 + 1] : 0xFFFFu;
+                st_table(t, rT + word_at(e), t.rank, t.rank_words, a | (c << 16));
             }
         }
     }
@@ -372,10 +376,10 @@ k_lanes_level(const BatchLanes t, const int64_t B, const int k, const int L, con
         const int64_t left = B - g * 32;
         const int valid = left < 32 ? (int)left : 32;
         const int col = lane < valid ? lane : valid - 1;
-        const uint32_t *tab = t.table + (size_t)g * t.rows * (LH * 32) + col;
-        uint32_t *tabw = t.table + (size_t)g * t.rows * (LH * 32) + lane;
-        const uint32_t *rk = t.rank + (size_t)g * (size_t)(k * k) * (LH * 32) + col;
-        const uint32_t *wn = t.win + (size_t)g * (size_t)(k * 2) * (LH * 32) + col;
+        const uint32_t *tab = t.table + (size_t)g * t.rows * (LH * 32) + col * kPiece;
+        uint32_t *tabw = t.table + (size_t)g * t.rows * (LH * 32) + lane * kPiece;
+        const uint32_t *rk = t.rank + (size_t)g * (size_t)(k * k) * (LH * 32) + col * kPiece;
+        const uint32_t *wn = t.win + (size_t)g * (size_t)(k * 2) * (LH * 32) + col * kPiece;
         uint32_t d[NV][LH];
         int vs[NV];
         {
@@ -386,8 +390,11 @@ k_lanes_level(const BatchLanes t, const int64_t B, const int k, const int L, con
                 vs[vi] = __ffs(rem) - 1;
                 rem &= rem - 1;
 #pragma unroll
-                for (int wd = W0; wd < LH; ++wd)
-                    d[vi][wd] = ld_table(t, tab + ((size_t)(row0 + vi) * LH + wd) * 32, t.table, t.table_words);
+                for (int q = W0 / kPiece; q < LH / kPiece; ++q) {
+                    const Piece x = ld_piece(t, tab + word_at((size_t)(row0 + vi) * LH + kPiece * q), t.table, t.table_words);
+#pragma unroll
+                    for (int i = 0; i < kPiece; ++i) d[vi][kPiece * q + i] = x.w[i];
+                }
             }
         }
         unsigned long long key = kNoBest;
@@ -399,29 +406,43 @@ k_lanes_level(const BatchLanes t, const int64_t B, const int k, const int L, con
             // the window cells of this node, asked for before anything else; position 0 has no window
             // and its entry carries the highest level of the sparse table this (instance, node) reads
             uint32_t cw[2 * LH];
-            const uint32_t lvl = ld_table(t, wn + (size_t)(w * 2 * LH) * 32, t.win, t.win_words);
 #pragma unroll
-            for (int c2 = C0; c2 < 2 * LH; ++c2)
-                cw[c2] = ld_table(t, wn + (size_t)(w * 2 * LH + c2) * 32, t.win, t.win_words);
+            for (int q = C0 / kPiece; q < 2 * LH / kPiece; ++q) {
+                const Piece x = ld_piece(t, wn + word_at((size_t)(w * 2 * LH) + kPiece * q), t.win, t.win_words);
+#pragma unroll
+                for (int i = 0; i < kPiece; ++i) cw[kPiece * q + i] = x.w[i];
+            }
+            const uint32_t lvl = C0 < kPiece ? cw[0] : ld_table(t, wn + word_at((size_t)(w * 2 * LH)), t.win, t.win_words);
             uint32_t gg[LH];
-            {
-                const uint32_t *r0 = rk + (size_t)((vs[0] * k + w) * LH) * 32;
+            auto rank_row = [&](int vi, int q) {
+                return ld_piece(t, rk + word_at((size_t)((vs[vi] * k + w) * LH) + kPiece * q), t.rank, t.rank_words);
+            };
 #pragma unroll
-                for (int wd = W0; wd < LH; ++wd) gg[wd] = __vmaxu2(d[0][wd], ld_table(t, r0 + wd * 32, t.rank, t.rank_words));
+            for (int q = W0 / kPiece; q < LH / kPiece; ++q) {
+                const Piece a = rank_row(0, q);
+#pragma unroll
+                for (int i = 0; i < kPiece; ++i) gg[kPiece * q + i] = __vmaxu2(d[0][kPiece * q + i], a.w[i]);
             }
 #pragma unroll
             for (int vi = 1; vi + 1 < NV; vi += 2) {
-                const uint32_t *r1 = rk + (size_t)((vs[vi] * k + w) * LH) * 32;
-                const uint32_t *r2 = rk + (size_t)((vs[vi + 1] * k + w) * LH) * 32;
 #pragma unroll
-                for (int wd = W0; wd < LH; ++wd)
-                    gg[wd] = __vimin3_u16x2(gg[wd], __vmaxu2(d[vi][wd], ld_table(t, r1 + wd * 32, t.rank, t.rank_words)),
-                                            __vmaxu2(d[vi + 1][wd], ld_table(t, r2 + wd * 32, t.rank, t.rank_words)));
+                for (int q = W0 / kPiece; q < LH / kPiece; ++q) {
+                    const Piece a = rank_row(vi, q), b = rank_row(vi + 1, q);
+#pragma unroll
+                    for (int i = 0; i < kPiece; ++i) {
+                        const int wd = kPiece * q + i;
+                        gg[wd] = __vimin3_u16x2(gg[wd], __vmaxu2(d[vi][wd], a.w[i]), __vmaxu2(d[vi + 1][wd], b.w[i]));
+                    }
+                }
             }
             if (!(NV & 1)) {
-                const uint32_t *r1 = rk + (size_t)((vs[NV - 1] * k + w) * LH) * 32;
 #pragma unroll
-                for (int wd = W0; wd < LH; ++wd) gg[wd] = __vminu2(gg[wd], __vmaxu2(d[NV - 1][wd], ld_table(t, r1 + wd * 32, t.rank, t.rank_words)));
+                for (int q = W0 / kPiece; q < LH / kPiece; ++q) {
+                    const Piece a = rank_row(NV - 1, q);
+#pragma unroll
+                    for (int i = 0; i < kPiece; ++i)
+                        gg[kPiece * q + i] = __vminu2(gg[kPiece * q + i], __vmaxu2(d[NV - 1][kPiece * q + i], a.w[i]));
+                }
             }
             // Window minimum over [lo_w(c2), c2 - 1] for every c2: the sparse table of g goes to the
             // lane's column of shared memory, level s from level s - 1 by one packed minimum per word
@@ -466,10 +487,15 @@ k_lanes_level(const BatchLanes t, const int64_t B, const int k, const int L, con
             const uint32_t row = t.rowoff[S2] + (uint32_t)__popc(S2 & ((1u << w) - 1u));
             uint32_t xw = 0xFFFFFFFFu;
 #pragma unroll
-            for (int wd = O0; wd < LH; ++wd) {
-                const uint32_t o = ob[2 * wd] | (ob[2 * wd + 1] << 16);
-                st_table(t, tabw + ((size_t)row * LH + wd) * 32, t.table, t.table_words, o);
-                if (wd == wfin) xw = o;
+            for (int q = O0 / kPiece; q < LH / kPiece; ++q) {
+                Piece o;
+#pragma unroll
+                for (int i = 0; i < kPiece; ++i) {
+                    const int wd = kPiece * q + i;
+                    o.w[i] = wd >= O0 ? ob[2 * wd] | (ob[2 * wd + 1] << 16) : 0xFFFFFFFFu;
+                    if (wd == wfin) xw = o.w[i];
+                }
+                st_piece(t, tabw + word_at((size_t)row * LH + kPiece * q), t.table, t.table_words, o);
             }
             const uint32_t x = (xw >> sfin) & 0xFFFFu;
             if (x != 0xFFFFu) {
@@ -485,7 +511,7 @@ k_lanes_level(const BatchLanes t, const int64_t B, const int k, const int L, con
 __device__ __forceinline__ uint32_t lanes_elem(const BatchLanes &t, const uint32_t *col, const uint32_t *base, size_t words,
                                                size_t row, int LH, int c)
 {
-    return (ld_table(t, col + (row * LH + (size_t)(c >> 1)) * 32, base, words) >> ((c & 1) * 16)) & 0xFFFFu;
+    return (ld_table(t, col + word_at(row * LH + (size_t)(c >> 1)), base, words) >> ((c & 1) * 16)) & 0xFFFFu;
 }
 
 __global__ void __launch_bounds__(kBackWarps * 32)
@@ -503,9 +529,9 @@ k_lanes_back(const BatchLanes t, const int64_t B, const int L, const int k, cons
          inst += (int64_t)gridDim.x * kBackWarps) {
         const size_t g = (size_t)(inst >> 5);
         const int col = (int)(inst & 31);
-        const uint32_t *tab = t.table + g * t.rows * (size_t)(LH * 32) + col;
-        const uint32_t *rk = t.rank + g * (size_t)(k * k) * (size_t)(LH * 32) + col;
-        const uint32_t *ln = t.len + g * (size_t)k * (size_t)(LH * 32) + col;
+        const uint32_t *tab = t.table + g * t.rows * (size_t)(LH * 32) + col * kPiece;
+        const uint32_t *rk = t.rank + g * (size_t)(k * k) * (size_t)(LH * 32) + col * kPiece;
+        const uint32_t *ln = t.len + g * (size_t)k * (size_t)(LH * 32) + col * kPiece;
         const unsigned long long key = t.key[inst];
         const int bad = t.flag[inst] & kFlagLimit;
         int32_t *cuts = o_cuts ? o_cuts + inst * (k - 1) : nullptr;
@@ -513,7 +539,7 @@ k_lanes_back(const BatchLanes t, const int64_t B, const int L, const int k, cons
         if (lane < k) place[lane] = -1;
         if (cuts && lane < k - 1) cuts[lane] = -1;
         __syncwarp();
-        for (int e = lane; e < k * LH; e += 32) mylen[e] = ld_table(t, ln + (size_t)e * 32, t.len, t.len_words);
+        for (int e = lane; e < k * LH; e += 32) mylen[e] = ld_table(t, ln + word_at(e), t.len, t.len_words);
         __syncwarp();
         if (bad || key == kNoBest) {
             if (lane == 0) {
@@ -534,7 +560,7 @@ k_lanes_back(const BatchLanes t, const int64_t B, const int L, const int k, cons
             int found = -1;
 #pragma unroll 8
             for (int e = lane; e < k * k * LH; e += 32) {
-                const uint32_t x = ld_table(t, rk + (size_t)e * 32, t.rank, t.rank_words);
+                const uint32_t x = ld_table(t, rk + word_at(e), t.rank, t.rank_words);
                 if ((x & 0xFFFFu) == rstar) found = 2 * e;
                 if ((x >> 16) == rstar) found = 2 * e + 1;
             }
@@ -647,22 +673,9 @@ cudaError_t launch_batch_prep(int64_t B, int L, int k, const uint64_t *bits, con
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int64_t blocks = (B + kPrepWarps - 1) / kPrepWarps;
-    if (blocks > (int64_t)sms * 16) blocks = (int64_t)sms * 16;
-    const int ufull = k * (k - 1), uhalf = ufull / 2;
-    for (int pass = 0; pass < 2; ++pass) {
-        const int ucap = pass ? ufull : uhalf;
-        const size_t sm = prep_layout(L, ucap).total * kPrepWarps;
-        // the attribute is set to the larger size both times: it belongs to the function, and another
-        // host thread may be between its own two launches
-        cudaError_t e = cudaFuncSetAttribute(k_lanes_prep, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)(prep_layout(L, ufull).total * kPrepWarps));
-        if (e != cudaSuccess) return e;
-        k_lanes_prep<<<(unsigned)blocks, kPrepWarps * 32, sm, s>>>(t, B, L, k, bits, mem, cap, bw, ucap, pass);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    const int64_t blocks = B < (int64_t)sms * 64 ? B : (int64_t)sms * 64;
+    k_lanes_prep<<<(unsigned)blocks, kPrepThreads, prep_layout(L, k).total, s>>>(t, B, L, k, bits, mem, cap, bw);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_batch_lanes(int64_t B, int L, int k, const uint64_t *bits, const uint32_t *bw,

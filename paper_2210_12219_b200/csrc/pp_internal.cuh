@@ -106,13 +106,13 @@ cudaError_t launch_batch(int64_t B, int L, int k, const uint64_t *bits, const ui
                          const uint64_t *cap, const uint32_t *bw, double *beta, int32_t *m,
                          int32_t *cuts, int32_t *placement, int8_t *status, cudaStream_t s);
 // Many-instance search with one instance per lane (pp_batch_lanes.cu): tables of a chunk of
-// instances in global memory, instance-minor, so that the 32 lanes of a warp read 32 neighbouring
-// words.  Group g holds instances 32 g .. 32 g + 31 of the chunk.
+// instances in global memory, instance-minor in pieces of two words, so that the 32 lanes of a warp read
+// 256 neighbouring bytes.  Group g holds instances 32 g .. 32 g + 31 of the chunk.
 struct BatchLanes {
-    uint32_t *table;          // [group][compact row][LH][32]: states, two cut positions per word
-    uint32_t *rank;           // [group][v * k + w][LH][32]: gamma ranks, same packing
-    uint32_t *len;            // [group][w][LH][32]: window lengths c' - lo_w(c'), same packing
-    uint32_t *win;            // [group][w][2 LH][32]: per cut position the two sparse-table cells whose minimum
+    uint32_t *table;          // [group][compact row][LH / 2][32][2]: states, two cut positions per word
+    uint32_t *rank;           // [group][v * k + w][LH / 2][32][2]: gamma ranks, same packing
+    uint32_t *len;            // [group][w][LH / 2][32][2]: window lengths c' - lo_w(c'), same packing
+    uint32_t *win;            // [group][w][LH][32][2]: per cut position the two sparse-table cells whose minimum
                               // is the window minimum, as byte offsets into a warp's table (see pp_batch_lanes.cu)
     unsigned long long *key;  // [group][32]: smallest final state so far (value, popcount, mask, node)
     int8_t *flag;             // [group][32]: 1 = an input beyond the limits
@@ -126,7 +126,7 @@ struct BatchLanes {
 };
 bool batch_lanes_takes(int64_t B, int L, int k);
 int batch_lanes_words(int L);
-// prep: one warp per instance ranks gamma and writes the instance's column of the tables
+// prep: one block per instance ranks gamma and writes the instance's column of the tables
 cudaError_t launch_batch_prep(int64_t B, int L, int k, const uint64_t *bits, const uint64_t *mem,
                               const uint64_t *cap, const uint32_t *bw, const BatchLanes &t, cudaStream_t s);
 // the levels and the backtrack over a prepared chunk; *launches counts the kernels queued

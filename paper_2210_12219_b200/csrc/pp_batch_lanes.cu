@@ -18,10 +18,10 @@
 //      minimum over [lo_w(c'), c'-1] from a sparse table of g in the lane's own column of shared
 //      memory (the one place where a lane needs an index of its own), stores the row of (P + w, w), and keeps the smallest final state
 //      (value, popcount, mask, node), merged into the instance's key with one atomic per lane;
-//   3. k_lanes_back, one warp per instance: the value of the winning rank and the backtrack by the
+//   3. k_lanes_back, one warp per instance: the backtrack by the
 //      threshold rule, lanes over the candidates.
 // Same recurrence, final choice and backtrack rule as the single-instance path (pp_sweep.cu).
-#include "pp_internal.cuh"
+#include "pp_blocks.cuh"
 
 namespace pp {
 
@@ -82,9 +82,8 @@ __device__ __forceinline__ void st_piece(const BatchLanes &t, uint32_t *p, const
 }
 
 // Shared memory of an instance in the preparing kernel (byte offsets; every part 16-byte aligned).
-constexpr int kBuckets = 1024;  // of the ranking; two 16-bit counters per word
 struct PrepLayout {
-    size_t val, M, bits, cap, bw, ubw, hist, rk, pair_u, total;
+    size_t val, key, rk, M, bits, dbits, cap, bw, ubw, hist, pair_u, cls, total;
 };
 
 __host__ __device__ inline PrepLayout prep_layout(int L, int k)
@@ -94,27 +93,26 @@ __host__ __device__ inline PrepLayout prep_layout(int L, int k)
     size_t o = 0;
     auto take = [&o](size_t bytes) { size_t at = o; o = (o + bytes + 15) & ~(size_t)15; return at; };
     p.val = take(n * 4);
+    p.key = take(n * 4);
+    p.rk = take(n * 2);
     p.M = take(33 * 8);
     p.bits = take(32 * 8);
+    p.dbits = take(32 * 8);
     p.cap = take(8 * 8);
     p.bw = take(64 * 4);
     p.ubw = take(64 * 4);
-    p.hist = take((size_t)kBuckets / 2 * 4);
-    p.rk = take(n * 4);
+    p.hist = take((size_t)kRankBuckets * 4);
     p.pair_u = take(64);
+    p.cls = take(32);
     p.total = o;
     return p;
 }
 
 // One block of four warps per instance (L <= 32 layers, k * k <= 64 node pairs): staging, the windows, the
 // ranking of gamma (Eq. 3), and the instance's column of the tables of BatchLanes.
-//   * distinct usable bandwidths listed in order of first appearance;
+//   * distinct usable bandwidths and distinct transfer sizes listed in order of first appearance;
 //   * window start lo_w(c2) by a branch-free binary search over the memory prefix sums;
-//   * rank = 1 + number of quotients strictly below, by a bucket sort: a quotient's bucket is its place in
-//     the range of the instance's quotients on the scale of the doubles' bits (monotone, about 1 % wide),
-//     counters in shared memory, their prefix sums, the quotients scattered into the order of the
-//     buckets, and each compared with the few that share its bucket.  Some 90 instructions per quotient
-//     where a staircase walk over the sorted quotient matrix took U + L dependent steps, 350.
+//   * ranks by rank_quotients.
 // What is left is a chain of short dependent phases, a third as long with four warps to an instance as with
 // one; the SM's other instances hide it.
 __global__ void __launch_bounds__(kPrepThreads, kPrepBlocks)
@@ -132,14 +130,16 @@ k_lanes_prep(const BatchLanes t, const int64_t B, const int L, const int k, cons
     uint32_t *s_bw = reinterpret_cast<uint32_t *>(smem_prep + lay.bw);
     uint32_t *ubw = reinterpret_cast<uint32_t *>(smem_prep + lay.ubw);
     uint32_t *hist = reinterpret_cast<uint32_t *>(smem_prep + lay.hist);
-    uint32_t *rk = reinterpret_cast<uint32_t *>(smem_prep + lay.rk);
+    uint32_t *s_key = reinterpret_cast<uint32_t *>(smem_prep + lay.key);
+    uint16_t *rk = reinterpret_cast<uint16_t *>(smem_prep + lay.rk);
+    unsigned long long *dbits = reinterpret_cast<unsigned long long *>(smem_prep + lay.dbits);
     int8_t *pair_u = reinterpret_cast<int8_t *>(smem_prep + lay.pair_u);
-    __shared__ uint32_t s_first[2], s_sum[kPrepThreads / 32];
+    uint8_t *cls = smem_prep + lay.cls;
+    __shared__ uint32_t s_first[3], s_sum[kPrepThreads / 32];
     const int LH = t.LH, kk = k * k;
     const uint32_t FULL = 0xFFFFFFFFu;
-    // floor(x / k) for x < 64, floor(x / L) for x < k (k-1) L <= 1792, floor(x / LH) for x < k k LH <= 1024
+    // floor(x / k) for x < 64, floor(x / LH) for x < k k LH <= 1024
     const uint32_t recip_k = (65536u + (uint32_t)k - 1u) / (uint32_t)k;
-    const uint32_t recip_L = (65536u + (uint32_t)L - 1u) / (uint32_t)L;
     const uint32_t recip_LH = (65536u + (uint32_t)LH - 1u) / (uint32_t)LH;
     for (int64_t inst = blockIdx.x; inst < B; inst += gridDim.x) {
         __syncthreads();
@@ -168,9 +168,8 @@ k_lanes_prep(const BatchLanes t, const int64_t B, const int L, const int k, cons
         } else if (lane < k) {
             s_cap[lane] = g_cap[inst * k + lane];
         }
-        reinterpret_cast<uint4 *>(hist)[tid] = make_uint4(0u, 0u, 0u, 0u);
         bad = __syncthreads_or(bad);
-        // ---- distinct usable bandwidths in order of first appearance ----
+        // ---- distinct usable bandwidths, distinct sizes, in order of first appearance ----
         uint32_t x = 0;
         int f = 0;
         if (wid < 2) {
@@ -185,6 +184,19 @@ k_lanes_prep(const BatchLanes t, const int64_t B, const int L, const int k, cons
             }
             const uint32_t firsts = __ballot_sync(FULL, x != 0u && f == tid);
             if (lane == 0) s_first[wid] = firsts;
+        } else if (wid == 3) {
+            const unsigned long long mine = s_bits[lane];
+#pragma unroll 4
+            for (int i = 30; i >= 0; i -= 2) {
+                const ulonglong2 q = *reinterpret_cast<const ulonglong2 *>(s_bits + i);
+                f = q.y == mine ? i + 1 : f;
+                f = q.x == mine ? i : f;
+            }
+            const uint32_t firsts = __ballot_sync(FULL, lane < L && f == lane);
+            const int c = __popc(firsts & ((1u << f) - 1u));
+            cls[lane] = (uint8_t)c;
+            if (lane < L && f == lane) dbits[c] = mine;
+            if (lane == 0) s_first[2] = firsts;
         }
         // ---- windows, base frontier ----
         {
@@ -241,84 +253,27 @@ k_lanes_prep(const BatchLanes t, const int64_t B, const int L, const int k, cons
             t.flag[inst] = (int8_t)(bad ? kFlagLimit : 0);
         }
         // ---- ranks of the quotients ----
-        const int n = U * L;
-        // upper words of doubles that no positive quotient lies outside of
-        const unsigned long long b = s_bits[lane];
-        const uint32_t p0 = s_bw[lane], p1 = s_bw[lane + 32];
-        const uint32_t least = __reduce_min_sync(FULL, lane < L && b ? __float_as_uint(__ull2float_rd(b)) : 0x7F800000u);
-        const uint32_t most = __reduce_max_sync(FULL, lane < L ? __float_as_uint(__ull2float_ru(b)) : 0u);
-        const uint32_t fast = __reduce_max_sync(FULL, max(p0, p1));
-        const uint32_t slow = __reduce_min_sync(FULL, min(p0 ? p0 : FULL, p1 ? p1 : FULL));
-        const int hi0 = __double2hiint(__ddiv_rd((double)__uint_as_float(least), (double)fast));
-        const int hi1 = __double2hiint(__ddiv_ru((double)__uint_as_float(most), (double)slow));
-        const int shift = max(0, 32 - __clz(max(hi1 - hi0, 0)) - 10);  // 2^10 = kBuckets
-        const unsigned long long lowest = (unsigned long long)(uint32_t)hi0 << 32;
-        __syncthreads();
-        auto quotient = [&](int e) {
-            const int u = (int)(((uint32_t)e * recip_L) >> 16);
-            return __ddiv_rn((double)s_bits[e - u * L], (double)ubw[u]);
-        };
-        for (int e = tid; e < n; e += kPrepThreads) {
-            // distance of the quotient's bits from the lowest (0.0 counts as the lowest): the upper bits are its
-            // bucket, the next 21 its key within the bucket
-            const unsigned long long q = (unsigned long long)__double_as_longlong(quotient(e));
-            const uint32_t y = (uint32_t)((q > lowest ? q - lowest : 0ull) >> (shift + 11));
-            rk[e] = y;
-            atomicAdd(&hist[y >> 22], 1u << ((y >> 21 & 1u) * 16));
+        {
+            const unsigned long long b = s_bits[lane];
+            const uint32_t p0 = s_bw[lane], p1 = s_bw[lane + 32];
+            const uint32_t least = __reduce_min_sync(FULL, lane < L && b ? __float_as_uint(__ull2float_rd(b)) : 0x7F800000u);
+            const uint32_t most = __reduce_max_sync(FULL, lane < L ? __float_as_uint(__ull2float_ru(b)) : 0u);
+            const uint32_t fast = __reduce_max_sync(FULL, max(p0, p1));
+            const uint32_t slow = __reduce_min_sync(FULL, min(p0 ? p0 : FULL, p1 ? p1 : FULL));
+            rank_quotients<kPrepThreads, uint32_t, 11>(dbits, ubw, U, __popc(s_first[2]),
+                                                       __ddiv_rd((double)__uint_as_float(least), (double)fast),
+                                                       __ddiv_ru((double)__uint_as_float(most), (double)slow), s_key, s_val,
+                                                       hist, rk, s_sum);
         }
-        __syncthreads();
-        {  // counters -> first places: a thread takes eight neighbouring buckets
-            const uint4 c = reinterpret_cast<const uint4 *>(hist)[tid];
-            uint32_t sum = c.x + c.y + c.z + c.w;
-            sum = (sum & 0xFFFFu) + (sum >> 16);
-            uint32_t upto = sum;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(FULL, upto, o);
-                if (lane >= o) upto += y;
-            }
-            if (lane == 31) s_sum[wid] = upto;
-            __syncthreads();
-            uint32_t place = upto - sum;
-            for (int i = 0; i < wid; ++i) place += s_sum[i];
-            auto next = [&](uint32_t word) {
-                const uint32_t second = place + (word & 0xFFFFu), both = place | (second << 16);
-                place = second + (word >> 16);
-                return both;
-            };
-            uint4 first;
-            first.x = next(c.x); first.y = next(c.y); first.z = next(c.z); first.w = next(c.w);
-            reinterpret_cast<uint4 *>(hist)[tid] = first;
-        }
-        __syncthreads();
-        for (int e = tid; e < n; e += kPrepThreads) {
-            const uint32_t y = rk[e], half = (y >> 21 & 1u) * 16;
-            const uint32_t place = (atomicAdd(&hist[y >> 22], 1u << half) >> half) & 0xFFFFu;
-            s_val[place] = (y << 11) | (uint32_t)e;  // key and entry (n < 2^11)
-        }
-        __syncthreads();
-        // a counter now holds the end of its bucket, that is the start of the next one
-        for (int e = tid; e < n; e += kPrepThreads) {
-            const uint32_t y = rk[e], mine = (y << 11) | (uint32_t)e, bk = y >> 21, half = (bk & 1u) * 16;
-            const int start = bk ? (int)((hist[(bk - 1) >> 1] >> (16 - half)) & 0xFFFFu) : 0;
-            const int end = (int)((hist[bk >> 1] >> half) & 0xFFFFu);
-            int below = start;
-            for (int q = start; q < end; ++q) {
-                const uint32_t other = s_val[q];
-                if ((other ^ mine) >= 2048u) below += other < mine;
-                else if (other != mine) below += quotient((int)(other & 2047u)) < quotient(e);  // one key: the doubles decide
-            }
-            rk[e] = (uint32_t)(1 + below);
-        }
-        __syncthreads();
         // ---- rank table, two positions per word: rank[v][w][c] = rank of (bandwidth of v -> w, layer c) ----
         {
+            const int D = __popc(s_first[2]);
             uint32_t *rT = t.rank + (size_t)(inst >> 5) * (size_t)(kk * LH) * 32 + (inst & 31) * kPiece;
             for (int e = tid; e < kk * LH; e += kPrepThreads) {
                 const int pr = (int)(((uint32_t)e * recip_LH) >> 16), c0 = 2 * (e - pr * LH);
                 const int u = pair_u[pr];
-                const uint32_t a = u >= 0 && c0 < L ? rk[u * L + c0] : 0xFFFFu;
-                const uint32_t c = u >= 0 && c0 + 1 < L ? rk[u * L + c0 + 1] : 0xFFFFu;
+                const uint32_t a = u >= 0 && c0 < L ? rk[u * D + cls[c0]] : 0xFFFFu;
+                const uint32_t c = u >= 0 && c0 + 1 < L ? rk[u * D + cls[c0 + 1]] : 0xFFFFu;
                 st_table(t, rT + word_at(e), t.rank, t.rank_words, a | (c << 16));
             }
         }
@@ -553,26 +508,8 @@ k_lanes_back(const BatchLanes t, const int64_t B, const int L, const int k, cons
         const int m = (int)((key >> 25) & 31);
         uint32_t S = (uint32_t)((key >> 5) & 0xFFFFF);
         int w = (int)(key & 31), c2 = L - 1;
-        double bstar = 0.0;
-        if (rstar != 0) {
-            // an entry of the rank table that carries the winning rank names a (node pair, layer) whose
-            // quotient is beta* (equal ranks hold equal doubles)
-            int found = -1;
-#pragma unroll 8
-            for (int e = lane; e < k * k * LH; e += 32) {
-                const uint32_t x = ld_table(t, rk + word_at(e), t.rank, t.rank_words);
-                if ((x & 0xFFFFu) == rstar) found = 2 * e;
-                if ((x >> 16) == rstar) found = 2 * e + 1;
-            }
-            for (int o = 16; o; o >>= 1) {
-                const int other = __shfl_xor_sync(0xFFFFFFFFu, found, o);
-                found = other > found ? other : found;
-            }
-            const int r = (found >> 1) / LH, c = 2 * ((found >> 1) - r * LH) + (found & 1);
-            bstar = __ddiv_rn((double)g_bits[inst * L + c], (double)g_bw[inst * k * k + r]);
-        }
+        int my_cut = 0, my_node = 0;  // lane j: cut and node of segment j
         if (lane == 0) {
-            o_beta[inst] = bstar;
             o_m[inst] = m;
             o_status[inst] = (int8_t)PP_OK;
 #ifdef PP_DEBUG_BOUNDS
@@ -580,7 +517,9 @@ k_lanes_back(const BatchLanes t, const int64_t B, const int L, const int k, cons
 #endif
         }
         for (int j = m - 1; j >= 0; --j) {
-            if (lane == 0) {
+            if (lane == j) {
+                my_node = w;
+                my_cut = c2;
                 place[j] = w;
                 if (j < m - 1) cuts[j] = c2;
             }
@@ -591,22 +530,21 @@ k_lanes_back(const BatchLanes t, const int64_t B, const int L, const int k, cons
             const int np = __popc(P), total = (c2 - l0) * np;
             // candidates (position, node of P), lanes over all of them at once: the loads of a step are
             // independent, the smallest (position, node) that meets the threshold wins
+            const uint32_t recip = (65536u + (uint32_t)np - 1u) / (uint32_t)np;  // floor(x / np) for x <= 31 * 7
+            uint32_t nodes = 0;  // the nodes of P, four bits each
+            int n = 0;
+            for (uint32_t rem = P; rem; rem &= rem - 1, n += 4) nodes |= (uint32_t)(__ffs(rem) - 1) << n;
             unsigned int pick = 0xFFFFFFFFu;
-#pragma unroll 2
+#pragma unroll 1
             for (int it = lane; it < total; it += 32) {
-                const int ci = it / np, vi = it - ci * np;
-                const int c = l0 + ci, v = (int)__fns(P, 0, vi + 1);
+                const int ci = (int)(((uint32_t)it * recip) >> 16), vi = it - ci * np;
+                const int c = l0 + ci, v = (int)((nodes >> (4 * vi)) & 15u);
                 // a state of np segments ends at layer np - 1 at the earliest; earlier positions were never written
                 const uint32_t a = c >= np - 1 ? lanes_elem(t, tab, t.table, t.table_words, (size_t)prow + vi, LH, c) : 0xFFFFu;
                 const uint32_t b = lanes_elem(t, rk, t.rank, t.rank_words, (size_t)(v * k + w), LH, c);
-                const uint32_t mx = a > b ? a : b;
-                const unsigned int kk = ((unsigned)c << 5) | (unsigned)v;
-                if (mx <= rstar && kk < pick) pick = kk;
+                if (max(a, b) <= rstar) pick = min(pick, ((unsigned)c << 5) | (unsigned)v);
             }
-            for (int o = 16; o; o >>= 1) {
-                const unsigned int other = __shfl_xor_sync(0xFFFFFFFFu, pick, o);
-                pick = other < pick ? other : pick;
-            }
+            pick = __reduce_min_sync(0xFFFFFFFFu, pick);
             if (pick == 0xFFFFFFFFu) {  // inconsistent table: flag the instance, keep going
                 if (lane == 0) o_status[inst] = (int8_t)PP_ERR_CUDA;
                 break;
@@ -615,6 +553,18 @@ k_lanes_back(const BatchLanes t, const int64_t B, const int L, const int k, cons
             w = (int)(pick & 31u);
             c2 = (int)(pick >> 5);
         }
+        // beta* is the bottleneck of the plan: no link of it ranks above the optimum, and no plan is better
+        const int next_node = __shfl_down_sync(0xFFFFFFFFu, my_node, 1);
+        unsigned long long worst = 0ull;  // non-negative doubles order like their bits
+        if (lane < m - 1)
+            worst = (unsigned long long)__double_as_longlong(
+                __ddiv_rn((double)g_bits[inst * L + my_cut], (double)g_bw[inst * k * k + my_node * k + next_node]));
+#pragma unroll
+        for (int o = 4; o; o >>= 1) {
+            const unsigned long long other = __shfl_xor_sync(0xFFFFFFFFu, worst, o);
+            worst = other > worst ? other : worst;
+        }
+        if (lane == 0) o_beta[inst] = __longlong_as_double((long long)worst);
     }
 }
 

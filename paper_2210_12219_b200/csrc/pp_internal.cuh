@@ -102,7 +102,13 @@ cudaError_t launch_eval_packed(const Dev &d, const unsigned char *tables, int64_
                                const uint16_t *ends, const uint8_t *nodes, double *beta, uint8_t *status,
                                cudaStream_t s);
 size_t batch_smem_bytes(int L, int k);
-cudaError_t launch_batch(int64_t B, int L, int k, const uint64_t *bits, const uint64_t *mem,
+// Row numbering of the batched search, per (device, k): rows ordered by (popcount, mask, node), the masks
+// listed by (popcount, value) with the first of each popcount, source mask | target node << 16 of every row
+// with the first row of each popcount.
+struct LaneTables {
+    const uint32_t *rowoff = nullptr, *mlist = nullptr, *moff = nullptr, *rows = nullptr, *first = nullptr;
+};
+cudaError_t launch_batch(int64_t B, int L, int k, const LaneTables &lt, int sms, const uint64_t *bits, const uint64_t *mem,
                          const uint64_t *cap, const uint32_t *bw, double *beta, int32_t *m,
                          int32_t *cuts, int32_t *placement, int8_t *status, cudaStream_t s);
 // Many-instance search with one instance per lane (pp_batch_lanes.cu): tables of a chunk of

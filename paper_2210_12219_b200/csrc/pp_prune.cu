@@ -31,13 +31,11 @@
 //             of S that can still matter, and writes the row of (S + w, w) if any of its states does
 //   end       once a level has little work block 0 goes on alone (its barrier costs nothing); it walks
 //             back by the threshold rule, checks the class of beta*, and writes the result record
-// A group of G lanes holds a row, P consecutive cut positions per lane.  The window minimum is the
-// tail of the block (= lane) that holds lo (suffix minima, through shared memory), whole blocks in
-// between (a sparse table over the G block minima), and the own prefix.
+// A group of G lanes holds a row, P consecutive cut positions per lane.
 #include <algorithm>
 #include <cstring>
 
-#include "pp_internal.cuh"
+#include "pp_blocks.cuh"
 
 namespace pp {
 
@@ -47,7 +45,6 @@ constexpr uint32_t kFull = 0xFFFFFFFFu;
 constexpr uint32_t kInfKey = 0xFFFFFFFFu;
 constexpr int kSpinLimit = 1 << 22;  // polls of a barrier before the kernel gives up
 constexpr int kAloneRounds = 2;      // a level of at most this many rounds of one block is done by block 0 alone
-constexpr int log2i(int x) { return x <= 1 ? 0 : 1 + log2i(x / 2); }
 __host__ __device__ constexpr int prune_threads(int P) { return P <= 16 ? 512 : 256; }
 
 // Which class of doubles a key stands for.
@@ -88,9 +85,9 @@ __device__ __forceinline__ uint32_t group_min(uint32_t u)
 
 // Shared memory: the part common to the block, then one strip per group of lanes.
 struct PruneLayout {
-    size_t bits, M, cap, bw, gmin, lo, strips, total;
+    size_t bits, M, cap, bw, gmin, lo, code, strips, total;
 };
-__host__ __device__ inline PruneLayout prune_layout(int L, int k, int Lp, int groups, size_t strip)
+__host__ __device__ inline PruneLayout prune_layout(int L, int k, int Lp, int groups, size_t strip, bool codes)
 {
     PruneLayout p;
     size_t o = 0;
@@ -101,64 +98,18 @@ __host__ __device__ inline PruneLayout prune_layout(int L, int k, int Lp, int gr
     p.bw = take((size_t)k * k * 4);
     p.gmin = take((size_t)k * k * 4);
     p.lo = take((size_t)k * Lp * 2);
+    p.code = take(codes ? (size_t)k * Lp * sizeof(WindowCode) : 0);
     p.strips = o;
     p.total = o + (size_t)groups * strip;
     return p;
 }
-template <int G, int P>
-struct Strip {
-    static constexpr int kLevels = log2i(G) + 1;
-    static constexpr int kSuffix = G * (P + 1);  // lanes write at an odd stride of words: no bank conflicts
-    static constexpr int kTable = kLevels * G;
-    static constexpr int kIds = 20;              // row ids of the source rows
-    static constexpr size_t kBytes = ((size_t)(kSuffix + kTable + kIds) * 4 + 15) & ~(size_t)15;
-};
+// Window codes where a warp works off several rows of every node: short chains, few blocks.
+template <int G, bool CT>
+constexpr bool kCodes = G <= 16 && !CT;
 
-// out[i] = min of g over [lo[i], pos0 + i - 1] for this lane's P positions
+// strip of a group: its window minima, then the ids of the source rows
 template <int G, int P>
-__device__ __forceinline__ void window_min(const uint32_t (&g)[P], const int16_t *lo, uint32_t *suffix, uint32_t *table,
-                                           int sl, uint32_t (&out)[P])
-{
-    uint32_t s = g[P - 1], pre[P];
-    pre[0] = g[0];
-#pragma unroll
-    for (int i = 1; i < P; ++i) pre[i] = min(pre[i - 1], g[i]);
-    uint32_t D = pre[P - 1];
-    table[sl] = D;
-    uint32_t *mine = suffix + sl * (P + 1);
-    mine[P - 1] = s;
-#pragma unroll
-    for (int i = P - 2; i >= 0; --i) {
-        s = min(s, g[i]);
-        mine[i] = s;
-    }
-#pragma unroll
-    for (int t = 1; t < Strip<G, P>::kLevels; ++t) {  // D = minimum of the last 2^t blocks
-        D = min(D, __shfl_up_sync(kFull, D, 1 << (t - 1), G));  // a lane without a source lane gets its own back
-        table[t * G + sl] = D;
-    }
-    __syncwarp();
-    const int pos0 = sl * P;
-#pragma unroll
-    for (int i = 0; i < P; ++i) {
-        const int l = lo[i];
-        const int bl = l / P, n = sl - 1 - bl;  // whole blocks between lo's and this one
-        uint32_t v = i > 0 ? pre[i > 0 ? i - 1 : 0] : kInfKey;
-        if (n >= 0) {
-            v = min(v, suffix[bl * (P + 1) + (l & (P - 1))]);
-            if (n > 0) {
-                const int t = 31 - __clz(n);
-                v = min(v, min(table[t * G + sl - 1], table[t * G + bl + (1 << t)]));
-            }
-        } else if (l > pos0) {  // the window starts inside this lane's own block
-            v = kInfKey;
-#pragma unroll
-            for (int q = 1; q < i; ++q)
-                if (q >= l - pos0) v = min(v, g[q]);
-        }
-        out[i] = v;
-    }
-}
+constexpr size_t kStripBytes = ((size_t)(Strip<G, P>::kSize + PP_MAX_K) * 4 + 15) & ~(size_t)15;
 
 template <int P>
 __device__ __forceinline__ void load_row(const uint32_t *p, uint32_t (&x)[P])
@@ -215,23 +166,22 @@ template <int G, int P, bool CT>
 __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d)
 {
     constexpr int kThreads = prune_threads(P), kWarps = kThreads / 32, kGroups = kThreads / G, kPerWarp = 32 / G;
-    using St = Strip<G, P>;
     extern __shared__ __align__(16) unsigned char smem_prune[];
     const int k = d.k, L = d.L, Lp = d.Lp, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int sl = lane & (G - 1), gb = lane & ~(G - 1);  // position in the group, first lane of the group
     const int at = sl * P;                                // this lane's first cut position
     const bool in_row = at < Lp;
     const int at0 = in_row ? at : 0;
-    const PruneLayout lay = prune_layout(L, k, Lp, kGroups, St::kBytes);
+    const PruneLayout lay = prune_layout(L, k, Lp, kGroups, kStripBytes<G, P>, kCodes<G, CT>);
     double *s_bits = reinterpret_cast<double *>(smem_prune + lay.bits);
     unsigned long long *s_M = reinterpret_cast<unsigned long long *>(smem_prune + lay.M);
     unsigned long long *s_cap = reinterpret_cast<unsigned long long *>(smem_prune + lay.cap);
     uint32_t *s_bw = reinterpret_cast<uint32_t *>(smem_prune + lay.bw);
     uint32_t *s_gmin = reinterpret_cast<uint32_t *>(smem_prune + lay.gmin);
     int16_t *s_lo = reinterpret_cast<int16_t *>(smem_prune + lay.lo);
-    uint32_t *s_suffix = reinterpret_cast<uint32_t *>(smem_prune + lay.strips + (size_t)(tid / G) * St::kBytes);
-    uint32_t *s_table = s_suffix + St::kSuffix;
-    uint32_t *s_ids = s_table + St::kTable;
+    WindowCode *s_code = reinterpret_cast<WindowCode *>(smem_prune + lay.code);
+    uint32_t *s_strip = reinterpret_cast<uint32_t *>(smem_prune + lay.strips + (size_t)(tid / G) * kStripBytes<G, P>);
+    uint32_t *s_ids = s_strip + Strip<G, P>::kSize;
     __shared__ unsigned long long s_best;  // best final state the block knows of
     __shared__ unsigned int s_pick[kWarps];
     __shared__ int s_cut[PP_MAX_K], s_node[PP_MAX_K];
@@ -251,8 +201,13 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d)
     for (int c = tid; c <= L; c += kThreads) s_M[c] = d.M[c];
     if (tid < k) s_cap[tid] = d.cap[tid];
     for (int e = tid; e < k * k; e += kThreads) s_bw[e] = d.bw[e];
+    if (sl == 0) s_strip[Strip<G, P>::kNone] = kInfKey;
     for (int w = wid; w < k; w += kWarps)
-        for (int c = lane; c < Lp; c += 32) s_lo[w * Lp + c] = c < L ? d.lo[w * L + c] : (int16_t)c;
+        for (int c = lane; c < Lp; c += 32) {
+            const int l = c < L ? d.lo[w * L + c] : c;
+            s_lo[w * Lp + c] = (int16_t)l;
+            if constexpr (kCodes<G, CT>) s_code[w * Lp + c] = window_code<G, P, uint32_t>(c, l);
+        }
     for (int e = tid; e < k * k; e += kThreads) s_gmin[e] = kInfKey;
     if (tid == 0) s_best = kNoBest;
     __syncthreads();
@@ -277,15 +232,16 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d)
     auto make_row = [&](const uint32_t (&g)[P], uint32_t (&out)[P], uint32_t S2, int w, int level, uint32_t lim, bool on,
                         uint32_t &rmin) -> bool {
         if constexpr (!CT) {
-            window_min<G, P>(g, s_lo + (size_t)w * Lp + at0, s_suffix, s_table, sl, out);
+            if constexpr (kCodes<G, CT>) window_min<G, P>(g, s_code + (size_t)w * Lp + at0, s_strip, sl, kInfKey, out);
+            else window_min_direct<G, P>(g, s_lo + (size_t)w * Lp + at0, s_strip, sl, kInfKey, out);
         } else {
             // the compute time of the last partition depends on both its ends: every output scans its
             // window, nearest start first, until the compute time alone is too much
 #pragma unroll
-            for (int i = 0; i < P; ++i) s_suffix[at + i] = g[i];
+            for (int i = 0; i < P; ++i) s_strip[at + i] = g[i];
             __syncwarp();
             uint32_t cur[P];
-            cur[0] = at > 0 ? s_suffix[at - 1] : kInfKey;
+            cur[0] = at > 0 ? s_strip[at - 1] : kInfKey;
 #pragma unroll
             for (int i = 1; i < P; ++i) cur[i] = g[i - 1];
 #pragma unroll
@@ -303,7 +259,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d)
                 if (!more || at + P - 2 - dd < 0) break;
 #pragma unroll
                 for (int i = P - 1; i > 0; --i) cur[i] = cur[i - 1];
-                cur[0] = at - 2 - dd >= 0 ? s_suffix[at - 2 - dd] : kInfKey;
+                cur[0] = at - 2 - dd >= 0 ? s_strip[at - 2 - dd] : kInfKey;
             }
         }
         const bool tight = (tight_levels >> level) & 1u;
@@ -680,7 +636,7 @@ cudaError_t launch_shape(const PruneDev &d, int sms, cudaStream_t s)
         constexpr int G = decltype(g)::value, P = decltype(p)::value;
         if (sh.G == G && sh.P == P) {
             kernel = k_prune<G, P, CT>;
-            strip = Strip<G, P>::kBytes;
+            strip = kStripBytes<G, P>;
         }
     };
     using std::integral_constant;
@@ -704,7 +660,7 @@ cudaError_t launch_shape(const PruneDev &d, int sms, cudaStream_t s)
     }
     int blocks = (int)std::min<unsigned long long>((widest + groups - 1) / groups, (unsigned long long)sms);
     if (blocks <= 2) blocks = 1;
-    const size_t sm = prune_layout(d.L, d.k, d.Lp, groups, strip).total;
+    const size_t sm = prune_layout(d.L, d.k, d.Lp, groups, strip, sh.G <= 16 && !CT).total;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};

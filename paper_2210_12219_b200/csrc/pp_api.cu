@@ -369,12 +369,21 @@ void quotient_range(int L, const uint64_t *num, int n, const uint32_t *den, doub
 
 // Copies the inputs to the device, ordered on the problem's stream.  The staging memory may go as soon
 // as the call returns: copies from pageable memory leave it first.
+void ensure_windows(pp_problem *p)
+{
+    if (!p->lo.empty()) return;
+    std::vector<int16_t> lo((size_t)p->k * p->L);
+    window_table(p->L, p->k, p->M.data(), p->cap.data(), lo.data());
+    p->lo.swap(lo);
+}
+
 pp_status upload_inputs(pp_problem *p, bool wait)
 {
     if (p->uploaded) return PP_OK;
     const int L = p->L, k = p->k;
     std::vector<unsigned char> st;
     try {
+        ensure_windows(p);
         st.assign(p->inputs_bytes, 0);
     } catch (const std::bad_alloc &) {
         return PP_ERR_NOMEM;
@@ -413,6 +422,7 @@ struct HostSlot {
     pp_solution sol;
     PruneNote note;
     MatchOut match;
+    PruneCtl *ctl;             // counters of a search, on the chunk's device
     alignas(256) unsigned char small[15 * 1024];  // inputs and results of a small call as a whole
 };
 constexpr int kSlots = 8;
@@ -420,31 +430,46 @@ class HostSlots {
 public:
     HostSlot *take()
     {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
         std::lock_guard<std::mutex> lock(mu_);
         for (auto &c : chunks_)
-            if (c.free) return from(c);
-        void *ptr = nullptr;
-        if (cudaHostAlloc(&ptr, kSlots * sizeof(HostSlot), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+            if (c.free && c.dev == dev) return from(c);
+        Chunk c{nullptr, nullptr, (1u << kSlots) - 1u, dev};
+        try {
+            chunks_.reserve(chunks_.size() + 1);
+        } catch (const std::bad_alloc &) {
+            return nullptr;
+        }
+        PruneCtl init[kSlots];
+        for (auto &x : init) prune_ctl_init(&x);
+        cudaError_t e = cudaHostAlloc(reinterpret_cast<void **>(&c.base), kSlots * sizeof(HostSlot),
+                                      cudaHostAllocPortable | cudaHostAllocMapped);
+        if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&c.ctl), sizeof init);
+        if (e == cudaSuccess) e = cudaMemcpy(c.ctl, init, sizeof init, cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) {
+            cudaFreeHost(c.base);
+            cudaFree(c.ctl);
             cudaGetLastError();
             return nullptr;
         }
-        try {
-            chunks_.push_back({static_cast<HostSlot *>(ptr), (1u << kSlots) - 1u});
-        } catch (const std::bad_alloc &) {
-            cudaFreeHost(ptr);
-            return nullptr;
-        }
+        for (int i = 0; i < kSlots; ++i) c.base[i].ctl = c.ctl + i;
+        chunks_.push_back(c);
         return from(chunks_.back());
     }
     void give(HostSlot *s)
     {
         std::lock_guard<std::mutex> lock(mu_);
         for (size_t i = 0; i < chunks_.size(); ++i) {
-            const ptrdiff_t at = s - chunks_[i].base;
+            Chunk &c = chunks_[i];
+            const ptrdiff_t at = s - c.base;
             if (at < 0 || at >= kSlots) continue;
-            chunks_[i].free |= 1u << at;
-            if (i > 0 && chunks_[i].free == (1u << kSlots) - 1u) {
-                cudaFreeHost(chunks_[i].base);
+            c.free |= 1u << at;
+            bool another = false;  // the first chunk of a device stays
+            for (size_t j = 0; j < i; ++j) another |= chunks_[j].dev == c.dev;
+            if (another && c.free == (1u << kSlots) - 1u) {
+                cudaFreeHost(c.base);
+                cudaFree(c.ctl);
                 chunks_.erase(chunks_.begin() + (long)i);
             }
             return;
@@ -454,7 +479,9 @@ public:
 private:
     struct Chunk {
         HostSlot *base;
+        PruneCtl *ctl;
         uint32_t free;
+        int dev;
     };
     static HostSlot *from(Chunk &c)
     {
@@ -503,6 +530,13 @@ private:
 };
 PinnedBuffers g_pinned;
 
+// After a search that did not come to its end: its kernel has not cleared the counters.
+void reset_counters(HostSlot *slot)
+{
+    PruneCtl ctl;
+    prune_ctl_init(&ctl);
+    cudaMemcpy(slot->ctl, &ctl, sizeof ctl, cudaMemcpyHostToDevice);
+}
 struct SlotLease {  // a slot for the duration of a call
     HostSlot *slot = g_slots.take();
     ~SlotLease() { if (slot) g_slots.give(slot); }
@@ -588,6 +622,7 @@ pp_status dense_prepare(pp_problem *p)
     Dev &d = p->d;
     try {
         dense_dims(p);
+        ensure_windows(p);
         const MaskList &ml = mask_list(k);
         // constants of the register-tiled sweep, when the instance is inside its envelope
         std::vector<unsigned char> fmeta(fast_meta_bytes()), pmeta;
@@ -698,15 +733,16 @@ pp_status ensure_sparse(pp_problem *p)
 }
 
 // row_limit: rows after which the search gives up (note->dense).
-pp_status queue_sparse(pp_problem *p, pp_solution *sol, PruneNote *note, unsigned long long row_limit)
+pp_status queue_sparse(pp_problem *p, PruneCtl *ctl, pp_solution *sol, PruneNote *note, unsigned long long row_limit)
 {
-    pp_status st = upload_inputs(p, false);
-    if (st != PP_OK) return st;
     PruneDev q = p->prune;
+    q.ctl = ctl;
+    q.lo = p->uploaded ? p->d.lo : nullptr;
     q.out = sol;
     q.note = note;
     q.row_cap = std::min(q.row_cap, row_limit);
-    PP_CUDA(launch_prune(q, p->sms, p->stream));
+    const PruneHost h{p->bits.data(), p->M.data(), p->cap.data(), p->bw.data(), nullptr, nullptr};
+    PP_CUDA(launch_prune(q, h, p->sms, p->stream));
     p->total_launches = 1;
     p->sweep_launches = 1;
     p->solved = true;
@@ -754,8 +790,6 @@ pp_status pp_problem_create(int32_t L, const uint64_t *layer_out_bits,
         // memory prefix sums: segment first..last needs M[last+1] - M[first] bytes
         p->M.assign(L + 1, 0);
         for (int i = 0; i < L; ++i) p->M[i + 1] = p->M[i] + p->mem[i];
-        p->lo.assign((size_t)k * L, 0);
-        window_table(L, k, p->M.data(), p->cap.data(), p->lo.data());
     } catch (const std::bad_alloc &) {
         delete p;
         return PP_ERR_NOMEM;
@@ -790,7 +824,6 @@ pp_status pp_problem_create(int32_t L, const uint64_t *layer_out_bits,
     p->d_note = reinterpret_cast<PruneNote *>(b + off[8] + sizeof(pp_solution));
     PruneDev &q = p->prune;
     q.L = L; q.k = k; q.Lp = prune_row_pad(L);
-    q.bits = d.bits; q.M = d.M; q.cap = d.cap; q.bw = d.bw; q.lo = d.lo;
     q.ctl = reinterpret_cast<PruneCtl *>(b + off[5]);
     double lo = std::numeric_limits<double>::max(), hi = 0.0;
     quotient_range(L, p->bits.data(), k * k, p->bw.data(), &lo, &hi);
@@ -877,7 +910,8 @@ pp_status pp_solve_exact_dev(pp_problem *p, pp_solution *solution_dev)
         if (!takes_sparse(p)) return queue_dense(p, solution_dev);
         // room for every row: pooled scratch where that is small, else a workspace
         pp_status st = sparse_bytes(p->k, p->prune.Lp, ~0ull) <= kSparseScratchBytes ? ensure_sparse(p) : ensure_work(p);
-        if (st == PP_OK) st = queue_sparse(p, solution_dev, p->d_note, ~0ull);
+        if (st == PP_OK) st = upload_inputs(p, false);  // the counters
+        if (st == PP_OK) st = queue_sparse(p, p->prune.ctl, solution_dev, p->d_note, ~0ull);
         p->note_on_device = true;
         return st;
     } catch (const std::bad_alloc &) {
@@ -894,7 +928,7 @@ static pp_status solve_sparse(pp_problem *p, pp_solution *sol)
     HostSlot *slot = g_slots.take();
     if (!slot) return PP_ERR_NOMEM;
     slot->note.dense = -1;
-    st = queue_sparse(p, &slot->sol, &slot->note, kSparseRows);
+    st = queue_sparse(p, slot->ctl, &slot->sol, &slot->note, kSparseRows);
     const cudaError_t e = cudaStreamSynchronize(p->stream);
     if (st == PP_OK) st = from_cuda(e);
     if (st == PP_OK) {
@@ -902,9 +936,7 @@ static pp_status solve_sparse(pp_problem *p, pp_solution *sol)
         p->note_on_device = false;
         *sol = slot->sol;
         if (p->note.dense < 0) {  // a barrier of the kernel gave up: put its counters back
-            PruneCtl ctl;
-            prune_ctl_init(&ctl);
-            cudaMemcpy(p->prune.ctl, &ctl, sizeof ctl, cudaMemcpyHostToDevice);
+            reset_counters(slot);
             st = PP_ERR_CUDA;
         } else if (p->note.dense) {
             st = PP_ERR_LIMIT;
@@ -1605,29 +1637,13 @@ pp_status pp_solve_exact_compute(int32_t L, const uint64_t *layer_out_bits, cons
         if (layer_work[i] >= PP_MAX_BITS) return PP_ERR_LIMIT;
     PruneDev q{};
     q.L = L; q.k = k; q.Lp = prune_row_pad(L);
-    // one staging buffer, one copy: the inputs, their prefix sums, the windows, the counters
-    const size_t bytes[8] = {(size_t)L * 8, (size_t)(L + 1) * 8, (size_t)(L + 1) * 8, (size_t)k * 8,
-                             (size_t)k * k * 4, (size_t)k * 4, (size_t)k * L * 2, sizeof(PruneCtl)};
-    size_t off[8], total = 0;
-    for (int i = 0; i < 8; ++i) { off[i] = total; total = align_up(total + bytes[i], i < 6 ? 16 : 128); }
-    std::vector<unsigned char> st8;
-    try {
-        st8.assign(total, 0);
-    } catch (const std::bad_alloc &) {
-        return PP_ERR_NOMEM;
-    }
-    unsigned char *h = st8.data();
-    uint64_t *M = reinterpret_cast<uint64_t *>(h + off[1]), *Wp = reinterpret_cast<uint64_t *>(h + off[2]);
-    std::memcpy(h + off[0], layer_out_bits, bytes[0]);
+    uint64_t M[PP_COMPUTE_MAX_L + 1], Wp[PP_COMPUTE_MAX_L + 1];
+    M[0] = Wp[0] = 0;
     for (int i = 0; i < L; ++i) {
         M[i + 1] = M[i] + layer_mem_bytes[i];
         Wp[i + 1] = Wp[i] + layer_work[i];
     }
-    std::memcpy(h + off[3], node_mem_bytes, bytes[3]);
-    std::memcpy(h + off[4], bw_kbps, bytes[4]);
-    std::memcpy(h + off[5], node_speed, bytes[5]);
-    window_table(L, k, M, node_mem_bytes, reinterpret_cast<int16_t *>(h + off[6]));
-    prune_ctl_init(reinterpret_cast<PruneCtl *>(h + off[7]));
+    const PruneHost h{layer_out_bits, M, node_mem_bytes, bw_kbps, Wp, node_speed};
     double lo = std::numeric_limits<double>::max(), hi = 0.0;
     quotient_range(L, layer_out_bits, k * k, bw_kbps, &lo, &hi);
     quotient_range(L, layer_work, k, node_speed, &lo, &hi);   // shortest run of layers: one
@@ -1640,7 +1656,7 @@ pp_status pp_solve_exact_compute(int32_t L, const uint64_t *layer_out_bits, cons
     cudaStream_t s = nullptr;
     HostSlot *slot = g_slots.take();
     if (!slot) return PP_ERR_NOMEM;
-    const size_t seg_bytes = align_up((size_t)k * L * q.Lp * 4, 256), head = align_up(total, 256) + seg_bytes;
+    const size_t head = align_up((size_t)k * L * q.Lp * 4, 256);
     cudaError_t e = cudaSuccess;
     // pooled scratch for a frontier that stays small, room for every state if it does not
     const unsigned long long limits[2] = {kSparseScratchBytes, ~0ull};
@@ -1649,35 +1665,29 @@ pp_status pp_solve_exact_compute(int32_t L, const uint64_t *layer_out_bits, cons
         const size_t table = sparse_bytes(k, q.Lp, limits[pass]);
         e = staging_alloc(reinterpret_cast<void **>(&buf), head + table, s);
         if (e != cudaSuccess) break;
-        q.bits = reinterpret_cast<uint64_t *>(buf + off[0]);
-        q.M = reinterpret_cast<uint64_t *>(buf + off[1]);
-        q.Wp = reinterpret_cast<uint64_t *>(buf + off[2]);
-        q.cap = reinterpret_cast<uint64_t *>(buf + off[3]);
-        q.bw = reinterpret_cast<uint32_t *>(buf + off[4]);
-        q.speed = reinterpret_cast<uint32_t *>(buf + off[5]);
-        q.lo = reinterpret_cast<int16_t *>(buf + off[6]);
-        q.ctl = reinterpret_cast<PruneCtl *>(buf + off[7]);
-        q.seg = reinterpret_cast<uint32_t *>(buf + align_up(total, 256));
+        q.ctl = slot->ctl;
+        q.seg = reinterpret_cast<uint32_t *>(buf);
         bind_sparse(q, buf + head, table);
         q.out = &slot->sol;
         q.note = &slot->note;
         slot->note.dense = -1;
-        e = cudaMemcpyAsync(buf, h, total, cudaMemcpyHostToDevice, s);
-        if (e == cudaSuccess) e = launch_prune(q, sms, s);
+        e = launch_prune(q, h, sms, s);
         cudaFreeAsync(buf, s);
         const cudaError_t e2 = cudaStreamSynchronize(s);
         if (e == cudaSuccess) e = e2;
         if (e == cudaSuccess && slot->note.dense <= 0) break;
     }
-    const HostSlot got = *slot;
+    const pp_solution sol = slot->sol;
+    const int32_t dense = slot->note.dense;
+    if (e == cudaSuccess && dense < 0) reset_counters(slot);
     g_slots.give(slot);
     if (e != cudaSuccess) return from_cuda(e);
-    if (got.note.dense != 0 || (got.sol.status != PP_OK && got.sol.status != PP_INFEASIBLE)) return PP_ERR_CUDA;
-    *beta_ms = got.sol.beta_ms;
-    *m = got.sol.m;
-    for (int j = 0; j < k - 1; ++j) cuts[j] = got.sol.cuts[j];
-    for (int j = 0; j < k; ++j) placement[j] = got.sol.placement[j];
-    return static_cast<pp_status>(got.sol.status);
+    if (dense != 0 || (sol.status != PP_OK && sol.status != PP_INFEASIBLE)) return PP_ERR_CUDA;
+    *beta_ms = sol.beta_ms;
+    *m = sol.m;
+    for (int j = 0; j < k - 1; ++j) cuts[j] = sol.cuts[j];
+    for (int j = 0; j < k; ++j) placement[j] = sol.placement[j];
+    return static_cast<pp_status>(sol.status);
 }
 
 pp_status pp_debug_minmax_rate(int32_t op, int32_t iters, double *warp_instr_per_clk_per_sm)

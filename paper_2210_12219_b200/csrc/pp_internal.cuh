@@ -158,9 +158,7 @@ struct PruneDev {
     unsigned long long key_base;
     uint32_t whole;            // nodes that hold the whole chain
     uint32_t tight_levels;     // bit j: some rest of the chain may not fit the nodes that j used ones leave
-    const uint64_t *bits, *M, *cap;  // as in Dev
-    const uint32_t *bw;
-    const int16_t *lo;
+    const int16_t *lo;         // [k*L] window starts (see Dev), or null: the kernel works them out
     uint32_t *live;            // [2^k] nodes v whose row (S, v) is kept
     unsigned long long *rowmap;  // [2^k * k] (S, v): smallest key << 32 | row
     uint32_t *list;            // [2^k] node sets of the frontier, level after level
@@ -168,9 +166,7 @@ struct PruneDev {
     uint32_t *gmin;            // [k*k] its minimum over the cut positions
     uint32_t *rows;            // [row_cap * Lp]
     unsigned long long row_cap;
-    const uint64_t *Wp;        // Eq. 1 only: [L+1] prefix sums of the layers' work,
-    const uint32_t *speed;     //   [k] speeds,
-    uint32_t *seg;             //   [k*L*Lp] keys of the compute times of every run of layers; null for Eq. 2
+    uint32_t *seg;             // Eq. 1: [k*L*Lp] keys of the compute times of every run of layers; null for Eq. 2
     PruneCtl *ctl;
     pp_solution *out;          // device or mapped host memory
     PruneNote *note;           // device or mapped host memory
@@ -179,7 +175,13 @@ void prune_key_range(double lo, double hi, PruneDev *d);
 void prune_node_bounds(const uint64_t *cap, uint64_t total, PruneDev *d);
 int prune_row_pad(int L);
 void prune_ctl_init(PruneCtl *c);
-cudaError_t launch_prune(const PruneDev &d, int sms, cudaStream_t s);
+struct PruneHost {             // host arrays, read before launch_prune returns
+    const uint64_t *bits, *M, *cap;  // [L], [L+1] memory prefix sums, [k]
+    const uint32_t *bw;        // [k*k]
+    const uint64_t *Wp;        // Eq. 1 only: [L+1] prefix sums of the layers' work, [k] speeds
+    const uint32_t *speed;
+};
+cudaError_t launch_prune(const PruneDev &d, const PruneHost &h, int sms, cudaStream_t s);
 // Random comparison baseline (Section 4): P plans of problem d from 2 k draws each.
 cudaError_t launch_random_plans(const Dev &d, const unsigned char *tables, int64_t P, const uint32_t *draws, uint8_t *nseg,
                                 int32_t *ends, int32_t *nodes, cudaStream_t s);

@@ -85,9 +85,9 @@ __device__ __forceinline__ uint32_t group_min(uint32_t u)
 
 // Shared memory: the part common to the block, then one strip per group of lanes.
 struct PruneLayout {
-    size_t bits, M, cap, bw, gmin, lo, code, strips, total;
+    size_t bits, M, cap, bw, gmin, lo, code, Wp, speed, strips, total;
 };
-__host__ __device__ inline PruneLayout prune_layout(int L, int k, int Lp, int groups, size_t strip, bool codes)
+__host__ __device__ inline PruneLayout prune_layout(int L, int k, int Lp, int groups, size_t strip, bool codes, bool compute)
 {
     PruneLayout p;
     size_t o = 0;
@@ -99,6 +99,8 @@ __host__ __device__ inline PruneLayout prune_layout(int L, int k, int Lp, int gr
     p.gmin = take((size_t)k * k * 4);
     p.lo = take((size_t)k * Lp * 2);
     p.code = take(codes ? (size_t)k * Lp * sizeof(WindowCode) : 0);
+    p.Wp = take(compute ? (size_t)(L + 1) * 8 : 0);
+    p.speed = take(compute ? (size_t)k * 4 : 0);
     p.strips = o;
     p.total = o + (size_t)groups * strip;
     return p;
@@ -155,6 +157,20 @@ __device__ __forceinline__ bool grid_barrier(PruneCtl *ctl, uint32_t target)
     return s_ok != 0;
 }
 
+// The inputs travel as a kernel parameter (4 KB for chains of up to 128 layers, 18 KB for the longest): no
+// copy to queue in front of the search and to wait for.
+template <int N, bool CT>
+struct PruneIn {
+    unsigned long long bits[N], M[N + 1], cap[PP_MAX_K];
+    uint32_t bw[PP_MAX_K * PP_MAX_K];
+};
+template <int N>
+struct PruneIn<N, true> {
+    unsigned long long bits[N], M[N + 1], cap[PP_MAX_K];
+    uint32_t bw[PP_MAX_K * PP_MAX_K], speed[PP_MAX_K];
+    unsigned long long Wp[N + 1];
+};
+
 // n-th (from 0) set bit of x
 __device__ __forceinline__ int nth_bit(uint32_t x, int n)
 {
@@ -163,7 +179,7 @@ __device__ __forceinline__ int nth_bit(uint32_t x, int n)
 }
 
 template <int G, int P, bool CT>
-__global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d)
+__global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d, const __grid_constant__ PruneIn<G * P, CT> params)
 {
     constexpr int kThreads = prune_threads(P), kWarps = kThreads / 32, kGroups = kThreads / G, kPerWarp = 32 / G;
     extern __shared__ __align__(16) unsigned char smem_prune[];
@@ -172,14 +188,16 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d)
     const int at = sl * P;                                // this lane's first cut position
     const bool in_row = at < Lp;
     const int at0 = in_row ? at : 0;
-    const PruneLayout lay = prune_layout(L, k, Lp, kGroups, kStripBytes<G, P>, kCodes<G, CT>);
+    const PruneLayout lay = prune_layout(L, k, Lp, kGroups, kStripBytes<G, P>, kCodes<G, CT>, CT);
     double *s_bits = reinterpret_cast<double *>(smem_prune + lay.bits);
     unsigned long long *s_M = reinterpret_cast<unsigned long long *>(smem_prune + lay.M);
     unsigned long long *s_cap = reinterpret_cast<unsigned long long *>(smem_prune + lay.cap);
     uint32_t *s_bw = reinterpret_cast<uint32_t *>(smem_prune + lay.bw);
     uint32_t *s_gmin = reinterpret_cast<uint32_t *>(smem_prune + lay.gmin);
     int16_t *s_lo = reinterpret_cast<int16_t *>(smem_prune + lay.lo);
-    WindowCode *s_code = reinterpret_cast<WindowCode *>(smem_prune + lay.code);
+    [[maybe_unused]] unsigned long long *s_Wp = reinterpret_cast<unsigned long long *>(smem_prune + lay.Wp);
+    [[maybe_unused]] uint32_t *s_speed = reinterpret_cast<uint32_t *>(smem_prune + lay.speed);
+    [[maybe_unused]] WindowCode *s_code = reinterpret_cast<WindowCode *>(smem_prune + lay.code);
     uint32_t *s_strip = reinterpret_cast<uint32_t *>(smem_prune + lay.strips + (size_t)(tid / G) * kStripBytes<G, P>);
     uint32_t *s_ids = s_strip + Strip<G, P>::kSize;
     __shared__ unsigned long long s_best;  // best final state the block knows of
@@ -197,19 +215,57 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d)
     unsigned long long t_start = 0;
     if (blockIdx.x == 0 && tid == 0) asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t_start));
     // ---- inputs ----
-    for (int c = tid; c < Lp; c += kThreads) s_bits[c] = c < L ? (double)d.bits[c] : 0.0;
-    for (int c = tid; c <= L; c += kThreads) s_M[c] = d.M[c];
-    if (tid < k) s_cap[tid] = d.cap[tid];
-    for (int e = tid; e < k * k; e += kThreads) s_bw[e] = d.bw[e];
-    if (sl == 0) s_strip[Strip<G, P>::kNone] = kInfKey;
-    for (int w = wid; w < k; w += kWarps)
-        for (int c = lane; c < Lp; c += 32) {
-            const int l = c < L ? d.lo[w * L + c] : c;
-            s_lo[w * Lp + c] = (int16_t)l;
-            if constexpr (kCodes<G, CT>) s_code[w * Lp + c] = window_code<G, P, uint32_t>(c, l);
-        }
-    for (int e = tid; e < k * k; e += kThreads) s_gmin[e] = kInfKey;
+    // read through an address of their own: neighbouring threads read neighbouring words, which the constant
+    // bank would serve one after another
+    const PruneIn<G * P, CT> *in = &params;
+    asm volatile("" : "+l"(in));
+    for (int c = tid; c < Lp; c += kThreads) s_bits[c] = c < L ? (double)in->bits[c] : 0.0;
+    for (int c = tid; c <= L; c += kThreads) s_M[c] = in->M[c];
+    for (int e = tid; e < k * k; e += kThreads) {
+        s_bw[e] = in->bw[e];
+        s_gmin[e] = kInfKey;
+    }
+    if (tid < k) s_cap[tid] = in->cap[tid];
     if (tid == 0) s_best = kNoBest;
+    if constexpr (CT) {
+        for (int c = tid; c <= L; c += kThreads) s_Wp[c] = in->Wp[c];
+        if (tid < k) s_speed[tid] = in->speed[tid];
+    }
+    if (sl == 0) s_strip[Strip<G, P>::kNone] = kInfKey;
+    __syncthreads();
+    auto set_window = [&](int w, int c, int l) {
+        s_lo[w * Lp + c] = (int16_t)l;
+        if constexpr (kCodes<G, CT>) s_code[w * Lp + c] = window_code<G, P, uint32_t>(c, l);
+    };
+    // window starts: lo[w][c'] = earliest previous cut c >= 0 such that layers c+1..c' fit on w, c' itself when
+    // not even layer c' alone does; a lane takes a run of neighbouring positions, found by bisection for the
+    // first and by stepping on for the others
+    if (d.lo)  // a problem that is solved again and again has them on the device
+        for (int w = wid; w < k; w += kWarps)
+            for (int c = lane; c < Lp; c += 32) set_window(w, c, c < L ? (int)d.lo[w * L + c] : c);
+    else
+    for (int w = wid; w < k; w += kWarps) {
+        const int run = (Lp + 31) / 32, c0 = lane * run, c1 = min(c0 + run, Lp);
+        const unsigned long long capw = s_cap[w];
+        int l = 0;
+        for (int c = c0; c < c1; ++c) {
+            if (c < L) {
+                const unsigned long long need = s_M[c + 1], thr = need > capw ? need - capw : 0ull;
+                if (c == c0) {
+                    int hi = c;  // M[c + 1] >= thr
+                    while (l < hi) {
+                        const int mid = (l + hi) >> 1;
+                        if (s_M[mid + 1] < thr) l = mid + 1; else hi = mid;
+                    }
+                } else {
+                    while (s_M[l + 1] < thr) ++l;
+                }
+            } else {
+                l = c;
+            }
+            set_window(w, c, l);
+        }
+    }
     __syncthreads();
     const unsigned long long total = s_M[L];
     const uint32_t tight_levels = d.tight_levels, whole = d.whole;
@@ -224,7 +280,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d)
     // base state of one node: layers 0..c on v
     auto base_key = [&](int v, int c) -> uint32_t {
         if (s_M[c + 1] > s_cap[v]) return kInfKey;
-        if constexpr (CT) return d.speed[v] ? key_of(__ddiv_rn((double)d.Wp[c + 1], (double)d.speed[v])) : kInfKey;
+        if constexpr (CT) return s_speed[v] ? key_of(__ddiv_rn((double)s_Wp[c + 1], (double)s_speed[v])) : kInfKey;
         return 0u;
     };
     // row of (S2, w) from g: window minimum, then drop what cannot matter, note a final state; returns
@@ -324,9 +380,9 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d)
             for (int e = (nblk == 1 ? 0 : (int)blockIdx.x) * kThreads + tid; e < n; e += nblk * kThreads) {
                 const int r = e / Lp, c2 = e - r * Lp, w = r / L, first = c2 - (r - w * L);
                 uint32_t key = kInfKey;
-                const uint32_t sp = d.speed[w];
+                const uint32_t sp = s_speed[w];
                 if (c2 < L && first >= 0 && sp != 0 && s_M[c2 + 1] - s_M[first] <= s_cap[w])
-                    key = key_of(__ddiv_rn((double)(d.Wp[c2 + 1] - d.Wp[first]), (double)sp));
+                    key = key_of(__ddiv_rn((double)(s_Wp[c2 + 1] - s_Wp[first]), (double)sp));
                 d.seg[e] = key;
             }
             if (tid == 0)
@@ -530,7 +586,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d)
             if (tid < m - 1) x = __ddiv_rn(s_bits[s_cut[tid]], (double)s_bw[s_node[tid] * k + s_node[tid + 1]]);
             if constexpr (CT) {
                 const int first = tid ? s_cut[tid - 1] + 1 : 0, last = tid < m - 1 ? s_cut[tid] : L - 1;
-                const double y = __ddiv_rn((double)(d.Wp[last + 1] - d.Wp[first]), (double)d.speed[s_node[tid]]);
+                const double y = __ddiv_rn((double)(s_Wp[last + 1] - s_Wp[first]), (double)s_speed[s_node[tid]]);
                 x = y > x ? y : x;
             }
             atomicMax(&s_worst, (unsigned long long)__double_as_longlong(x));
@@ -565,7 +621,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d)
             for (int e = tid; e < k * L * Lp; e += kThreads)
                 if (__ldcg(d.seg + e) == vstar) {
                     const int r = e / Lp, last = e - r * Lp, w2 = r / L, first = last - (r - w2 * L);
-                    if ((unsigned long long)__double_as_longlong(__ddiv_rn((double)(d.Wp[last + 1] - d.Wp[first]), (double)d.speed[w2])) < worst)
+                    if ((unsigned long long)__double_as_longlong(__ddiv_rn((double)(s_Wp[last + 1] - s_Wp[first]), (double)s_speed[w2])) < worst)
                         s_zoom = 1;
                 }
         }
@@ -626,31 +682,19 @@ PruneShape prune_shape(int L)
     return s;
 }
 
-template <bool CT>
-cudaError_t launch_shape(const PruneDev &d, int sms, cudaStream_t s)
+template <int G, int P, bool CT>
+cudaError_t launch_shape(const PruneDev &d, const PruneHost &h, int sms, cudaStream_t s)
 {
-    const PruneShape sh = prune_shape(d.L);
-    void (*kernel)(PruneDev) = nullptr;
-    size_t strip = 0;
-    auto pick = [&](auto g, auto p) {
-        constexpr int G = decltype(g)::value, P = decltype(p)::value;
-        if (sh.G == G && sh.P == P) {
-            kernel = k_prune<G, P, CT>;
-            strip = kStripBytes<G, P>;
-        }
-    };
-    using std::integral_constant;
-    pick(integral_constant<int, 4>{}, integral_constant<int, 4>{});
-    pick(integral_constant<int, 8>{}, integral_constant<int, 4>{});
-    pick(integral_constant<int, 16>{}, integral_constant<int, 4>{});
-    pick(integral_constant<int, 32>{}, integral_constant<int, 4>{});
-    pick(integral_constant<int, 32>{}, integral_constant<int, 8>{});
-    if constexpr (!CT) {
-        pick(integral_constant<int, 32>{}, integral_constant<int, 16>{});
-        pick(integral_constant<int, 32>{}, integral_constant<int, 32>{});
+    PruneIn<G * P, CT> in;
+    std::memcpy(in.bits, h.bits, (size_t)d.L * 8);
+    std::memcpy(in.M, h.M, (size_t)(d.L + 1) * 8);
+    std::memcpy(in.cap, h.cap, (size_t)d.k * 8);
+    std::memcpy(in.bw, h.bw, (size_t)d.k * d.k * 4);
+    if constexpr (CT) {
+        std::memcpy(in.Wp, h.Wp, (size_t)(d.L + 1) * 8);
+        std::memcpy(in.speed, h.speed, (size_t)d.k * 4);
     }
-    if (!kernel) return cudaErrorInvalidValue;
-    const int threads = prune_threads(sh.P), groups = threads / sh.G;
+    constexpr int threads = prune_threads(P), groups = threads / G;
     // blocks: one round over the targets of the widest level if it is kept whole; a single block where
     // two rounds of it do, its barrier costs next to nothing
     unsigned long long widest = 1, binom = 1;
@@ -660,8 +704,8 @@ cudaError_t launch_shape(const PruneDev &d, int sms, cudaStream_t s)
     }
     int blocks = (int)std::min<unsigned long long>((widest + groups - 1) / groups, (unsigned long long)sms);
     if (blocks <= 2) blocks = 1;
-    const size_t sm = prune_layout(d.L, d.k, d.Lp, groups, strip, sh.G <= 16 && !CT).total;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const size_t sm = prune_layout(d.L, d.k, d.Lp, groups, kStripBytes<G, P>, kCodes<G, CT>, CT).total;
+    cudaError_t e = cudaFuncSetAttribute(k_prune<G, P, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)blocks);
@@ -673,7 +717,7 @@ cudaError_t launch_shape(const PruneDev &d, int sms, cudaStream_t s)
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = blocks > 1 ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, d);
+    return cudaLaunchKernelEx(&cfg, k_prune<G, P, CT>, d, in);
 }
 
 }  // namespace
@@ -721,9 +765,18 @@ void prune_node_bounds(const uint64_t *cap, uint64_t total, PruneDev *d)
     }
 }
 
-cudaError_t launch_prune(const PruneDev &d, int sms, cudaStream_t s)
+cudaError_t launch_prune(const PruneDev &d, const PruneHost &h, int sms, cudaStream_t s)
 {
-    return d.seg ? launch_shape<true>(d, sms, s) : launch_shape<false>(d, sms, s);
+    const PruneShape sh = prune_shape(d.L);
+    switch (sh.G * 100 + sh.P) {
+#define PP_CASE(g, p) \
+    case g * 100 + p: return d.seg ? launch_shape<g, p, true>(d, h, sms, s) : launch_shape<g, p, false>(d, h, sms, s);
+        PP_CASE(4, 4) PP_CASE(8, 4) PP_CASE(16, 4) PP_CASE(32, 4) PP_CASE(32, 8)
+#undef PP_CASE
+        case 3216: return launch_shape<32, 16, false>(d, h, sms, s);  // Eq. 1 stops at 256 layers
+        case 3232: return launch_shape<32, 32, false>(d, h, sms, s);
+    }
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace pp

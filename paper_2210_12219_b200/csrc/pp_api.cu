@@ -303,21 +303,6 @@ constexpr unsigned long long kSparseRows = 160000;
 // Without a workspace of the caller the rows live in pooled scratch of at most this size.
 constexpr unsigned long long kSparseScratchBytes = 128ull << 20;
 
-struct SparseLayout {
-    size_t live, rowmap, list, gam, gmin, rows;
-};
-SparseLayout sparse_layout(int k, int Lp)
-{
-    SparseLayout w;
-    size_t o = 0;
-    w.live = o;   o = align_up(o + ((size_t)4 << k), 256);
-    w.rowmap = o; o = align_up(o + ((size_t)k * 8 << k), 256);
-    w.list = o;   o = align_up(o + ((size_t)4 << k), 256);
-    w.gam = o;    o = align_up(o + (size_t)k * k * Lp * 4, 256);
-    w.gmin = o;   o = align_up(o + (size_t)k * k * 4, 256);
-    w.rows = o;
-    return w;
-}
 size_t sparse_bytes(int k, int Lp, unsigned long long limit)
 {
     const unsigned long long rows = std::min(rows_all(k), limit / ((unsigned long long)Lp * 4));
@@ -823,7 +808,7 @@ pp_status pp_problem_create(int32_t L, const uint64_t *layer_out_bits,
     p->d_sol = reinterpret_cast<pp_solution *>(b + off[8]);
     p->d_note = reinterpret_cast<PruneNote *>(b + off[8] + sizeof(pp_solution));
     PruneDev &q = p->prune;
-    q.L = L; q.k = k; q.Lp = prune_row_pad(L);
+    q.L = L; q.k = k; q.Lp = prune_row_pad(L, k);
     q.ctl = reinterpret_cast<PruneCtl *>(b + off[5]);
     double lo = std::numeric_limits<double>::max(), hi = 0.0;
     quotient_range(L, p->bits.data(), k * k, p->bw.data(), &lo, &hi);
@@ -909,7 +894,9 @@ pp_status pp_solve_exact_dev(pp_problem *p, pp_solution *solution_dev)
         p->sparse_ran = false;
         if (!takes_sparse(p)) return queue_dense(p, solution_dev);
         // room for every row: pooled scratch where that is small, else a workspace
-        pp_status st = sparse_bytes(p->k, p->prune.Lp, ~0ull) <= kSparseScratchBytes ? ensure_sparse(p) : ensure_work(p);
+        pp_status st = PP_OK;
+        if (!prune_in_shared(p->L, p->k, false))
+            st = sparse_bytes(p->k, p->prune.Lp, ~0ull) <= kSparseScratchBytes ? ensure_sparse(p) : ensure_work(p);
         if (st == PP_OK) st = upload_inputs(p, false);  // the counters
         if (st == PP_OK) st = queue_sparse(p, p->prune.ctl, solution_dev, p->d_note, ~0ull);
         p->note_on_device = true;
@@ -923,7 +910,7 @@ pp_status pp_solve_exact_dev(pp_problem *p, pp_solution *solution_dev)
 // rows, the dense search has to run.
 static pp_status solve_sparse(pp_problem *p, pp_solution *sol)
 {
-    pp_status st = ensure_sparse(p);
+    pp_status st = prune_in_shared(p->L, p->k, false) ? PP_OK : ensure_sparse(p);
     if (st != PP_OK) return st;
     HostSlot *slot = g_slots.take();
     if (!slot) return PP_ERR_NOMEM;
@@ -1636,7 +1623,7 @@ pp_status pp_solve_exact_compute(int32_t L, const uint64_t *layer_out_bits, cons
     for (int i = 0; i < L; ++i)
         if (layer_work[i] >= PP_MAX_BITS) return PP_ERR_LIMIT;
     PruneDev q{};
-    q.L = L; q.k = k; q.Lp = prune_row_pad(L);
+    q.L = L; q.k = k; q.Lp = prune_row_pad(L, k);
     uint64_t M[PP_COMPUTE_MAX_L + 1], Wp[PP_COMPUTE_MAX_L + 1];
     M[0] = Wp[0] = 0;
     for (int i = 0; i < L; ++i) {
@@ -1662,17 +1649,19 @@ pp_status pp_solve_exact_compute(int32_t L, const uint64_t *layer_out_bits, cons
     const unsigned long long limits[2] = {kSparseScratchBytes, ~0ull};
     for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
         unsigned char *buf = nullptr;
-        const size_t table = sparse_bytes(k, q.Lp, limits[pass]);
-        e = staging_alloc(reinterpret_cast<void **>(&buf), head + table, s);
-        if (e != cudaSuccess) break;
+        if (!prune_in_shared(L, k, true)) {
+            const size_t table = sparse_bytes(k, q.Lp, limits[pass]);
+            e = staging_alloc(reinterpret_cast<void **>(&buf), head + table, s);
+            if (e != cudaSuccess) break;
+            q.seg = reinterpret_cast<uint32_t *>(buf);
+            bind_sparse(q, buf + head, table);
+        }
         q.ctl = slot->ctl;
-        q.seg = reinterpret_cast<uint32_t *>(buf);
-        bind_sparse(q, buf + head, table);
         q.out = &slot->sol;
         q.note = &slot->note;
         slot->note.dense = -1;
         e = launch_prune(q, h, sms, s);
-        cudaFreeAsync(buf, s);
+        if (buf) cudaFreeAsync(buf, s);
         const cudaError_t e2 = cudaStreamSynchronize(s);
         if (e == cudaSuccess) e = e2;
         if (e == cudaSuccess && slot->note.dense <= 0) break;

@@ -1,5 +1,5 @@
 // Building blocks shared by the kernels that work on one instance in shared memory: the window minimum
-// over a row held by a group of lanes, and the ranking of an instance's quotients by one block.
+// over a row held by a group of lanes, the ranking of an instance's quotients by one block, bit selection.
 #pragma once
 #include "pp_internal.cuh"
 
@@ -132,6 +132,21 @@ __device__ __forceinline__ void window_min(const uint32_t (&g)[P], const WindowC
             out[i + h] = min(min(own, tail), min(left, right));
         }
     }
+}
+
+// r-th (from 0) set bit of x; r below the number of set bits
+__device__ __forceinline__ int select_bit(uint32_t x, int r)
+{
+    int at = 0;
+#pragma unroll
+    for (int half = 16; half; half >>= 1) {
+        const int below = __popc(x & ((1u << half) - 1u));
+        const bool up = r >= below;
+        r -= up ? below : 0;
+        at += up ? half : 0;
+        x = up ? x >> half : x;
+    }
+    return at;
 }
 
 constexpr int kRankBuckets = 1024;

@@ -154,6 +154,7 @@ struct PruneNote {             // what the host learns about a launch
 };
 struct PruneDev {
     int L, k, Lp;              // Lp: row stride in keys
+    int clustered;             // the blocks are one cluster (set by the launch)
     int key_shift;             // keys: 1 + (bits of the double - key_base) >> key_shift
     unsigned long long key_base;
     uint32_t whole;            // nodes that hold the whole chain
@@ -173,8 +174,27 @@ struct PruneDev {
 };
 void prune_key_range(double lo, double hi, PruneDev *d);
 void prune_node_bounds(const uint64_t *cap, uint64_t total, PruneDev *d);
-int prune_row_pad(int L);
+int prune_row_pad(int L, int k);
 void prune_ctl_init(PruneCtl *c);
+// Tables of the bounded search, in scratch memory or in a block's shared memory; the rows come last.
+struct SparseLayout {
+    size_t live, rowmap, list, gam, gmin, rows;
+};
+__host__ __device__ inline SparseLayout sparse_layout(int k, int Lp)
+{
+    SparseLayout w;
+    size_t o = 0;
+    auto take = [&o](size_t bytes) { size_t at = o; o = (o + bytes + 255) & ~(size_t)255; return at; };
+    w.live = take((size_t)4 << k);
+    w.rowmap = take((size_t)k * 8 << k);
+    w.list = take((size_t)4 << k);
+    w.gam = take((size_t)k * k * Lp * 4);
+    w.gmin = take((size_t)k * k * 4);
+    w.rows = o;
+    return w;
+}
+// whether the search of such a problem needs no scratch in global memory; compute: the one of Eq. 1
+bool prune_in_shared(int L, int k, bool compute);
 struct PruneHost {             // host arrays, read before launch_prune returns
     const uint64_t *bits, *M, *cap;  // [L], [L+1] memory prefix sums, [k]
     const uint32_t *bw;        // [k*k]

@@ -43,9 +43,15 @@ namespace {
 
 constexpr uint32_t kFull = 0xFFFFFFFFu;
 constexpr uint32_t kInfKey = 0xFFFFFFFFu;
+constexpr int kClusterBlocks = 8, kClusterRounds = 2;
+constexpr int kWideK = 10;  // nodes up to which short rows take two positions a lane (k = 14, L = 60: 192 us, with four 144)
+constexpr int kSharedRounds = 3;  // k = 6, L = 12: 17 -> 12 us a solve; k = 7 (5 rounds) no gain, k = 8 a loss
+constexpr size_t kSharedBytes = 220 * 1024;
+constexpr int kAhead = 8;             // steps of a window scan whose compute times are asked for at a time
 constexpr int kSpinLimit = 1 << 22;  // polls of a barrier before the kernel gives up
 constexpr int kAloneRounds = 2;      // a level of at most this many rounds of one block is done by block 0 alone
-__host__ __device__ constexpr int prune_threads(int P) { return P <= 16 ? 512 : 256; }
+// P = 8 (up to 256 layers): 20 warps, so that the 2448 targets of the node sets of two of 18 nodes are one round
+__host__ __device__ constexpr int prune_threads(int P) { return P == 8 ? 640 : P <= 16 ? 512 : 256; }
 
 // Which class of doubles a key stands for.
 struct KeyMap {
@@ -106,36 +112,45 @@ __host__ __device__ inline PruneLayout prune_layout(int L, int k, int Lp, int gr
     return p;
 }
 // Window codes where a warp works off several rows of every node: short chains, few blocks.
-template <int G, bool CT>
-constexpr bool kCodes = G <= 16 && !CT;
+template <int G, int P, bool CT>
+constexpr bool kCodes = G * P <= 64 && !CT;
 
 // strip of a group: its window minima, then the ids of the source rows
 template <int G, int P>
 constexpr size_t kStripBytes = ((size_t)(Strip<G, P>::kSize + PP_MAX_K) * 4 + 15) & ~(size_t)15;
 
-template <int P>
+// What another block may have written: past L1.  SM: the tables are in shared memory.
+template <bool SM, typename T>
+__device__ __forceinline__ T ld_now(const T *p)
+{
+    if constexpr (SM) return *p;
+    else return __ldcg(p);
+}
+
+// P keys of a row; CA: as they are, through L1 or in shared memory
+template <int P, bool CA>
 __device__ __forceinline__ void load_row(const uint32_t *p, uint32_t (&x)[P])
 {
+    if constexpr (P == 2) {
+        const uint2 t = CA ? *reinterpret_cast<const uint2 *>(p) : __ldcg(reinterpret_cast<const uint2 *>(p));
+        x[0] = t.x; x[1] = t.y;
+    } else {
 #pragma unroll
-    for (int i = 0; i < P; i += 4) {
-        const uint4 t = __ldcg(reinterpret_cast<const uint4 *>(p + i));
-        x[i] = t.x; x[i + 1] = t.y; x[i + 2] = t.z; x[i + 3] = t.w;
-    }
-}
-template <int P>
-__device__ __forceinline__ void load_row_ca(const uint32_t *p, uint32_t (&x)[P])  // through L1: written before the last barrier
-{
-#pragma unroll
-    for (int i = 0; i < P; i += 4) {
-        const uint4 t = *reinterpret_cast<const uint4 *>(p + i);
-        x[i] = t.x; x[i + 1] = t.y; x[i + 2] = t.z; x[i + 3] = t.w;
+        for (int i = 0; i < P; i += 4) {
+            const uint4 t = CA ? *reinterpret_cast<const uint4 *>(p + i) : __ldcg(reinterpret_cast<const uint4 *>(p + i));
+            x[i] = t.x; x[i + 1] = t.y; x[i + 2] = t.z; x[i + 3] = t.w;
+        }
     }
 }
 template <int P>
 __device__ __forceinline__ void store_row(uint32_t *p, const uint32_t (&x)[P])
 {
+    if constexpr (P == 2) {
+        *reinterpret_cast<uint2 *>(p) = make_uint2(x[0], x[1]);
+    } else {
 #pragma unroll
-    for (int i = 0; i < P; i += 4) *reinterpret_cast<uint4 *>(p + i) = make_uint4(x[i], x[i + 1], x[i + 2], x[i + 3]);
+        for (int i = 0; i < P; i += 4) *reinterpret_cast<uint4 *>(p + i) = make_uint4(x[i], x[i + 1], x[i + 2], x[i + 3]);
+    }
 }
 
 // All blocks of the grid; false when the wait ran out (the caller returns).
@@ -171,14 +186,8 @@ struct PruneIn<N, true> {
     unsigned long long Wp[N + 1];
 };
 
-// n-th (from 0) set bit of x
-__device__ __forceinline__ int nth_bit(uint32_t x, int n)
-{
-    for (; n > 0; --n) x &= x - 1;
-    return __ffs(x) - 1;
-}
-
-template <int G, int P, bool CT>
+// SM: the tables of the search in shared memory, one block (launch_prune)
+template <int G, int P, bool CT, bool SM>
 __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d, const __grid_constant__ PruneIn<G * P, CT> params)
 {
     constexpr int kThreads = prune_threads(P), kWarps = kThreads / 32, kGroups = kThreads / G, kPerWarp = 32 / G;
@@ -188,7 +197,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
     const int at = sl * P;                                // this lane's first cut position
     const bool in_row = at < Lp;
     const int at0 = in_row ? at : 0;
-    const PruneLayout lay = prune_layout(L, k, Lp, kGroups, kStripBytes<G, P>, kCodes<G, CT>, CT);
+    const PruneLayout lay = prune_layout(L, k, Lp, kGroups, kStripBytes<G, P>, kCodes<G, P, CT>, CT);
     double *s_bits = reinterpret_cast<double *>(smem_prune + lay.bits);
     unsigned long long *s_M = reinterpret_cast<unsigned long long *>(smem_prune + lay.M);
     unsigned long long *s_cap = reinterpret_cast<unsigned long long *>(smem_prune + lay.cap);
@@ -204,9 +213,20 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
     __shared__ unsigned int s_pick[kWarps];
     __shared__ int s_cut[PP_MAX_K], s_node[PP_MAX_K];
     __shared__ unsigned long long s_worst;  // bits of the plan's bottleneck
-    __shared__ int s_zoom, s_nlinks;
-    __shared__ uint16_t s_links[PP_MAX_K * PP_MAX_K];  // links with a quotient no larger than the optimum
+    __shared__ unsigned long long s_low;    // bits of the smallest quotient in the optimum's class
+    __shared__ uint32_t s_cnt;
+    __shared__ int s_fail;
     PruneCtl *ctl = d.ctl;
+    __shared__ uint32_t s_count[SM ? 64 : 1];
+    unsigned char *tables = smem_prune + lay.total;  // SM: in the layout they have in global memory
+    const SparseLayout tl = sparse_layout(k, Lp);
+    uint32_t *t_live = SM ? reinterpret_cast<uint32_t *>(tables + tl.live) : d.live;
+    unsigned long long *t_rowmap = SM ? reinterpret_cast<unsigned long long *>(tables + tl.rowmap) : d.rowmap;
+    uint32_t *t_list = SM ? reinterpret_cast<uint32_t *>(tables + tl.list) : d.list;
+    uint32_t *t_gam = SM ? reinterpret_cast<uint32_t *>(tables + tl.gam) : d.gam;
+    uint32_t *t_gmin = SM ? reinterpret_cast<uint32_t *>(tables + tl.gmin) : d.gmin;
+    uint32_t *t_rows = SM ? reinterpret_cast<uint32_t *>(tables + tl.rows) : d.rows;
+    [[maybe_unused]] uint32_t *t_seg = SM ? t_rows + (((size_t)k << (k - 1)) * Lp) : d.seg;
     const double kInf = __longlong_as_double(0x7FF0000000000000ll);
     const int top = k < L ? k : L;
     const uint32_t full = (1u << k) - 1u;
@@ -226,6 +246,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
         s_gmin[e] = kInfKey;
     }
     if (tid < k) s_cap[tid] = in->cap[tid];
+    if (SM && tid < 64) s_count[tid] = 0u;
     if (tid == 0) s_best = kNoBest;
     if constexpr (CT) {
         for (int c = tid; c <= L; c += kThreads) s_Wp[c] = in->Wp[c];
@@ -235,7 +256,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
     __syncthreads();
     auto set_window = [&](int w, int c, int l) {
         s_lo[w * Lp + c] = (int16_t)l;
-        if constexpr (kCodes<G, CT>) s_code[w * Lp + c] = window_code<G, P, uint32_t>(c, l);
+        if constexpr (kCodes<G, P, CT>) s_code[w * Lp + c] = window_code<G, P, uint32_t>(c, l);
     };
     // window starts: lo[w][c'] = earliest previous cut c >= 0 such that layers c+1..c' fit on w, c' itself when
     // not even layer c' alone does; a lane takes a run of neighbouring positions, found by bisection for the
@@ -269,11 +290,22 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
     __syncthreads();
     const unsigned long long total = s_M[L];
     const uint32_t tight_levels = d.tight_levels, whole = d.whole;
+    __shared__ double s_room[384];  // memory of a set of nodes, seven of them at a time
+    if (tight_levels)
+        for (int e = tid; e < 384; e += kThreads) {
+            double sum = 0.0;
+            for (int b = 0; b < 7; ++b) {
+                const int v = (e >> 7) * 7 + b;
+                if (((e >> b) & 1) && v < k) sum += (double)s_cap[v];
+            }
+            s_room[e] = sum;
+        }
+    __syncthreads();
 
     KeyMap key_of{d.key_base, d.key_shift, 0u};
     bool dense = false;
     uint32_t barriers = 0;
-    int nblk = gridDim.x;  // blocks that work on the search: 1 once block 0 goes on alone
+    int nblk = SM ? 1 : (int)gridDim.x;  // blocks that work on the search: 1 once block 0 goes on alone
     int m = 0, w_end = 0, status = (int)PP_INFEASIBLE;
     double beta = kInf;
 
@@ -288,7 +320,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
     auto make_row = [&](const uint32_t (&g)[P], uint32_t (&out)[P], uint32_t S2, int w, int level, uint32_t lim, bool on,
                         uint32_t &rmin) -> bool {
         if constexpr (!CT) {
-            if constexpr (kCodes<G, CT>) window_min<G, P>(g, s_code + (size_t)w * Lp + at0, s_strip, sl, kInfKey, out);
+            if constexpr (kCodes<G, P, CT>) window_min<G, P>(g, s_code + (size_t)w * Lp + at0, s_strip, sl, kInfKey, out);
             else window_min_direct<G, P>(g, s_lo + (size_t)w * Lp + at0, s_strip, sl, kInfKey, out);
         } else {
             // the compute time of the last partition depends on both its ends: every output scans its
@@ -302,34 +334,40 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
             for (int i = 1; i < P; ++i) cur[i] = g[i - 1];
 #pragma unroll
             for (int i = 0; i < P; ++i) out[i] = kInfKey;
-            const uint32_t *seg = d.seg + (size_t)w * L * Lp + at0;
-            for (int dd = 0; dd < L; ++dd) {
-                uint32_t x[P];
+            const uint32_t *seg = t_seg + (size_t)w * L * Lp + at0;
+            for (int d0 = 0; d0 < L; d0 += kAhead) {  // the loads of kAhead steps are in flight together
+                uint32_t x[kAhead][P];
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) load_row<P, true>(seg + (size_t)min(d0 + u, L - 1) * Lp, x[u]);
                 bool more = false;
-                load_row_ca<P>(seg + (size_t)dd * Lp, x);
 #pragma unroll
-                for (int i = 0; i < P; ++i) {
-                    out[i] = min(out[i], max(cur[i], x[i]));
-                    more |= x[i] < lim;
+                for (int u = 0; u < kAhead; ++u) {
+                    const int dd = d0 + u;
+#pragma unroll
+                    for (int i = 0; i < P; ++i) {
+                        out[i] = min(out[i], max(cur[i], x[u][i]));
+                        more |= x[u][i] < lim;
+                    }
+#pragma unroll
+                    for (int i = P - 1; i > 0; --i) cur[i] = cur[i - 1];
+                    cur[0] = at - 2 - dd >= 0 ? s_strip[at - 2 - dd] : kInfKey;
                 }
-                if (!more || at + P - 2 - dd < 0) break;
-#pragma unroll
-                for (int i = P - 1; i > 0; --i) cur[i] = cur[i - 1];
-                cur[0] = at - 2 - dd >= 0 ? s_strip[at - 2 - dd] : kInfKey;
+                if (!more || at + P - 1 - kAhead - d0 < 0) break;
             }
         }
         const bool tight = (tight_levels >> level) & 1u;
-        double room = kInf;
+        unsigned long long must = 0ull;  // layers 0..c have to hold this much for the unused nodes to hold the rest
         if (tight) {
-            room = 0.0;
-            for (uint32_t rest = full & ~S2; rest; rest &= rest - 1) room += (double)s_cap[__ffs(rest) - 1];
+            const uint32_t rest = full & ~S2;
+            double room = s_room[rest & 127u] + s_room[128 + (rest >> 7 & 127u)] + s_room[256 + (rest >> 14)];
             room *= 1.0 + 1e-9;  // rounding of the sums must not drop a state
+            must = room < (double)total ? total - (unsigned long long)room : 0ull;
         }
         uint32_t least = kInfKey, x = kInfKey;
 #pragma unroll
         for (int i = 0; i < P; ++i) {
             const int c = at + i;
-            if (!on || out[i] >= lim || c >= L || (tight && (double)(total - s_M[c + 1]) > room)) out[i] = kInfKey;
+            if (!on || out[i] >= lim || c >= L || (tight && s_M[c + 1] < must)) out[i] = kInfKey;
             least = min(least, out[i]);
             if (c == L - 1) x = out[i];
         }
@@ -341,18 +379,27 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
         return rmin != kInfKey;
     };
     // end of a level: the block's best final state goes to the others; false = a barrier gave up
-    auto level_end = [&](unsigned long long best_before) -> bool {
+    // and s_cnt has the node sets it added to the frontier
+    auto level_end = [&](unsigned long long best_before, const uint32_t *added) -> bool {
+        __syncthreads();
         if (nblk == 1) {
+            if (tid == 0 && added) s_cnt = ld_now<SM>(added);
             __syncthreads();
             return true;
         }
-        __syncthreads();
         if (tid == 0 && s_best < best_before)
             asm volatile("red.relaxed.gpu.global.min.u64 [%0], %1;" ::"l"(&ctl->best), "l"(s_best) : "memory");
-        barriers += gridDim.x;
-        if (!grid_barrier(ctl, barriers)) return false;
-        const unsigned long long seen = __ldcg(&ctl->best);
-        if (tid == 0 && seen < s_best) s_best = seen;
+        if (d.clustered) {
+            asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        } else {
+            barriers += gridDim.x;
+            if (!grid_barrier(ctl, barriers)) return false;
+        }
+        if (tid == 0) {
+            const unsigned long long seen = __ldcg(&ctl->best);
+            if (added) s_cnt = __ldcg(added);
+            if (seen < s_best) s_best = seen;
+        }
         __syncthreads();
         return true;
     };
@@ -372,8 +419,8 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
         const int slots = nblk * kWarps, my_slot = wid * nblk + (nblk == 1 ? 0 : (int)blockIdx.x);
         // node sets of three nodes and more start without rows (those of two nodes are all written below)
         for (uint32_t S = (nblk == 1 ? 0 : blockIdx.x) * kThreads + tid; S < (1u << k); S += nblk * kThreads)
-            if (__popc(S) > 2) d.live[S] = 0u;
-        uint32_t *const count = ctl->count + (key_of.zoom ? 32 : 0);
+            if (__popc(S) > 2) t_live[S] = 0u;
+        uint32_t *const count = (SM ? s_count : ctl->count) + (key_of.zoom ? 32 : 0);
         if constexpr (CT) {
             // compute times of every run of layers: seg[(w * L + d) * Lp + c'] = layers c'-d .. c' on w
             const int n = k * L * Lp;
@@ -383,14 +430,14 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                 const uint32_t sp = s_speed[w];
                 if (c2 < L && first >= 0 && sp != 0 && s_M[c2 + 1] - s_M[first] <= s_cap[w])
                     key = key_of(__ddiv_rn((double)(s_Wp[c2 + 1] - s_Wp[first]), (double)sp));
-                d.seg[e] = key;
+                t_seg[e] = key;
             }
             if (tid == 0)
                 for (int v = 0; v < k; ++v) {
                     const uint32_t x = base_key(v, L - 1);
                     if (x != kInfKey) s_best = min(s_best, pack_best(x, 1, 1u << v, v));
                 }
-            if (!level_end(kNoBest)) return;
+            if (!level_end(kNoBest, nullptr)) return;
         }
         // ---- two nodes: the keys of every link, the rows of every pair ----
         if (top >= 2) {
@@ -409,9 +456,9 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                     g[i] = (link != 0 && c < L) ? key_of(__ddiv_rn(s_bits[c], div)) : kInfKey;
                     if (c < L - 1) gm = min(gm, g[i]);
                 }
-                if (on && in_row) store_row<P>(d.gam + (size_t)(w * k + v) * Lp + at, g);
+                if (on && in_row) store_row<P>(t_gam + (size_t)(w * k + v) * Lp + at, g);
                 gm = group_min<G>(gm);
-                if (on && sl == 0) d.gmin[w * k + v] = gm;
+                if (on && sl == 0) t_gmin[w * k + v] = gm;
 #pragma unroll
                 for (int i = 0; i < P; ++i) {
                     const int c = at + i;
@@ -423,18 +470,18 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                 const int a = v < w ? v : w, b = v < w ? w : v;
                 const int pr = a * (2 * k - a - 1) / 2 + (b - a - 1);
                 const uint32_t id = 2u * (uint32_t)pr + (w == b ? 1u : 0u);
-                if (keep && in_row) store_row<P>(d.rows + (size_t)id * Lp + at, out);
+                if (keep && in_row) store_row<P>(t_rows + (size_t)id * Lp + at, out);
                 if (on && sl == 0) {
-                    d.rowmap[(size_t)S2 * k + w] = ((unsigned long long)rmin << 32) | id;
+                    t_rowmap[(size_t)S2 * k + w] = ((unsigned long long)rmin << 32) | id;
                     if (w == b) {
-                        d.list[pr] = S2;
-                        d.live[S2] = S2;
+                        t_list[pr] = S2;
+                        t_live[S2] = S2;
                     }
                 }
                 __syncwarp();
             }
-            if (!level_end(before)) return;
-            for (int e = tid; e < k * k; e += kThreads) s_gmin[e] = (e / k != e % k) ? __ldcg(d.gmin + e) : kInfKey;
+            if (!level_end(before, nullptr)) return;
+            for (int e = tid; e < k * k; e += kThreads) s_gmin[e] = (e / k != e % k) ? ld_now<SM>(t_gmin + e) : kInfKey;
             __syncthreads();
         }
 
@@ -444,6 +491,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
         bool alone = nblk == 1;
         for (int level = 3; level <= top && cnt; ++level) {
             const int nw = k - (level - 1);
+            const uint32_t recip_nw = 0xFFFFFFFFu / (uint32_t)nw + 1u;  // floor(it / nw) by a multiplication: it < 2^27
             const unsigned long long items = (unsigned long long)cnt * nw;
             if (used + items > d.row_cap) {
                 dense = true;
@@ -459,10 +507,10 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
             for (unsigned long long base = (unsigned long long)my * kPerWarp; base < items; base += (unsigned long long)all * kPerWarp) {
                 const unsigned long long it = base + lane / G;
                 const bool on = it < items;
-                const uint32_t li = on ? (uint32_t)it / (uint32_t)nw : 0u;
-                const uint32_t S = __ldcg(d.list + beg + li);
-                const int w = nth_bit(full & ~S, on ? (int)((uint32_t)it - li * (uint32_t)nw) : 0);
-                const uint32_t rows_of_S = __ldcg(d.live + S);
+                const uint32_t li = on ? (nw > 1 ? __umulhi((uint32_t)it, recip_nw) : (uint32_t)it) : 0u;
+                const uint32_t S = ld_now<SM>(t_list + beg + li);
+                const int w = select_bit(full & ~S, on ? (int)((uint32_t)it - li * (uint32_t)nw) : 0);
+                const uint32_t rows_of_S = ld_now<SM>(t_live + S);
                 const uint32_t lim = limit_of(*reinterpret_cast<volatile unsigned long long *>(&s_best), level);
                 // source rows that can still matter: their smallest value and the link's smallest key
                 uint32_t src = 0;
@@ -472,7 +520,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                     const int v = v0 + sl;
                     bool ok = false;
                     if (v < k && ((S >> v) & 1u)) {
-                        const unsigned long long e = __ldcg(d.rowmap + (size_t)S * k + v);
+                        const unsigned long long e = ld_now<SM>(t_rowmap + (size_t)S * k + v);
                         s_ids[v] = (uint32_t)e;
                         ok = on && ((rows_of_S >> v) & 1u) && max((uint32_t)(e >> 32), s_gmin[w * k + v]) < lim;
                     }
@@ -491,10 +539,10 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                     src &= src - 1;
                     if (in_row) {
                         uint32_t a[P], b[P], a2[P], b2[P];
-                        load_row<P>(d.rows + (size_t)s_ids[v] * Lp + at, a);
-                        load_row<P>(d.gam + (size_t)(w * k + v) * Lp + at, b);
-                        load_row<P>(d.rows + (size_t)s_ids[v2] * Lp + at, a2);
-                        load_row<P>(d.gam + (size_t)(w * k + v2) * Lp + at, b2);
+                        load_row<P, SM>(t_rows + (size_t)s_ids[v] * Lp + at, a);
+                        load_row<P, SM>(t_gam + (size_t)(w * k + v) * Lp + at, b);
+                        load_row<P, SM>(t_rows + (size_t)s_ids[v2] * Lp + at, a2);
+                        load_row<P, SM>(t_gam + (size_t)(w * k + v2) * Lp + at, b2);
 #pragma unroll
                         for (int i = 0; i < P; ++i) g[i] = min(g[i], min(max(a[i], b[i]), max(a2[i], b2[i])));
                     }
@@ -506,19 +554,19 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                 const uint32_t S2 = S | (1u << w);
                 if (make_row(g, out, S2, w, level, lim, on, rmin)) {
                     const uint32_t id = (uint32_t)(used + it);
-                    if (in_row) store_row<P>(d.rows + (size_t)id * Lp + at, out);
+                    if (in_row) store_row<P>(t_rows + (size_t)id * Lp + at, out);
                     if (sl == 0) {
-                        d.rowmap[(size_t)S2 * k + w] = ((unsigned long long)rmin << 32) | id;
-                        if (atomicOr(d.live + S2, 1u << w) == 0u)
-                            d.list[beg + cnt + atomicAdd(&count[level], 1u)] = S2;
+                        t_rowmap[(size_t)S2 * k + w] = ((unsigned long long)rmin << 32) | id;
+                        if (atomicOr(t_live + S2, 1u << w) == 0u)
+                            t_list[beg + cnt + atomicAdd(&count[level], 1u)] = S2;
                     }
                 }
                 __syncwarp();
             }
             used += items;
-            if (!level_end(before)) return;
+            if (!level_end(before, &count[level])) return;
             beg += cnt;
-            cnt = __ldcg(&count[level]);
+            cnt = s_cnt;
         }
         if (blockIdx.x != 0 || dense) break;  // block 0 finishes
         __syncthreads();
@@ -532,54 +580,107 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
         uint32_t S = (uint32_t)(best >> 5) & 0xFFFFFu;
         int w = (int)best & 31, c2 = L - 1;
         if (tid < PP_MAX_K) s_cut[tid] = s_node[tid] = -1;
-        if (tid == 0) s_worst = 0ull;
+        if (tid == 0) {
+            s_worst = 0ull;
+            s_low = ~0ull;
+            s_fail = 0;
+        }
         __syncthreads();
-        for (int j = m - 1; j >= 0; --j) {
-            if (tid == 0) {
-                s_node[j] = w;
-                if (j < m - 1) s_cut[j] = c2;
-            }
-            if (j == 0) break;
-            const uint32_t from = S & ~(1u << w);
-            const int lo = s_lo[(size_t)w * Lp + c2], np = __popc(from);
-            const uint32_t rows_of = np > 1 ? __ldcg(d.live + from) : from;
-            unsigned int bestk = 0xFFFFFFFFu;
-            for (int vi = wid; vi < np; vi += kWarps) {
-                const int v = nth_bit(from, vi);
-                const unsigned long long e = np > 1 ? __ldcg(d.rowmap + (size_t)from * k + v) : 0ull;
-                if (!((rows_of >> v) & 1u) || (uint32_t)(e >> 32) > vstar) continue;
-                const uint32_t *row = d.rows + (size_t)(uint32_t)e * Lp, *gm = d.gam + (size_t)(w * k + v) * Lp;
-                for (int c0 = lo; c0 < c2; c0 += 32) {
-                    const int c = c0 + lane;
-                    bool hit = false;
-                    if (c < c2) {
-                        uint32_t x = max(np > 1 ? __ldcg(row + c) : base_key(v, c), __ldcg(gm + c));
-                        if constexpr (CT) x = max(x, __ldcg(d.seg + (size_t)(w * L + c2 - c - 1) * Lp + c2));
-                        hit = x <= vstar;
+        // half of the warps walk back, the others look for the smallest quotient in the optimum's class
+        constexpr int kBack = kWarps / 2;
+        if (wid < kBack) {
+            for (int j = m - 1; j >= 0; --j) {
+                if (tid == 0) {
+                    s_node[j] = w;
+                    if (j < m - 1) s_cut[j] = c2;
+                }
+                if (j == 0) break;
+                const uint32_t from = S & ~(1u << w);
+                const int lo = s_lo[(size_t)w * Lp + c2], np = __popc(from);
+                const uint32_t rows_of = np > 1 ? ld_now<SM>(t_live + from) : from;
+                unsigned int pick = 0xFFFFFFFFu;
+                for (int vi = wid; vi < np; vi += kBack) {
+                    const int v = select_bit(from, vi);
+                    const unsigned long long e = np > 1 ? ld_now<SM>(t_rowmap + (size_t)from * k + v) : 0ull;
+                    if (!((rows_of >> v) & 1u) || (uint32_t)(e >> 32) > vstar) continue;
+                    const uint32_t *row = t_rows + (size_t)(uint32_t)e * Lp, *gm = t_gam + (size_t)(w * k + v) * Lp;
+                    constexpr int kChunks = 4;  // of 32 positions, their loads in flight together
+                    bool hit_one = false;
+                    for (int c0 = lo; c0 < c2 && !hit_one; c0 += 32 * kChunks) {
+                        uint32_t x[kChunks];
+#pragma unroll
+                        for (int u = 0; u < kChunks; ++u) {
+                            const int c = c0 + 32 * u + lane;
+                            x[u] = kInfKey;
+                            if (c < c2) {
+                                x[u] = max(np > 1 ? ld_now<SM>(row + c) : base_key(v, c), ld_now<SM>(gm + c));
+                                if constexpr (CT) x[u] = max(x[u], ld_now<SM>(t_seg + (size_t)(w * L + c2 - c - 1) * Lp + c2));
+                            }
+                        }
+#pragma unroll
+                        for (int u = 0; u < kChunks; ++u) {
+                            const unsigned int hits = __ballot_sync(kFull, x[u] <= vstar);
+                            if (hits && !hit_one) {
+                                pick = min(pick, ((unsigned)(c0 + 32 * u + __ffs(hits) - 1) << 5) | (unsigned)v);
+                                hit_one = true;
+                            }
+                        }
                     }
-                    const unsigned int hits = __ballot_sync(kFull, hit);
-                    if (hits) {
-                        const unsigned int kk = ((unsigned)(c0 + __ffs(hits) - 1) << 5) | (unsigned)v;
-                        bestk = kk < bestk ? kk : bestk;
-                        break;
+                }
+                if (lane == 0) s_pick[wid] = pick;
+                asm volatile("bar.sync 1, %0;" ::"n"(kBack * 32) : "memory");
+                pick = __reduce_min_sync(kFull, s_pick[lane < kBack ? lane : 0]);
+                asm volatile("bar.sync 1, %0;" ::"n"(kBack * 32) : "memory");
+                if (pick == 0xFFFFFFFFu) {  // cannot happen on a consistent frontier; report, do not trap
+                    s_fail = 1;
+                    break;
+                }
+                S = from;
+                w = (int)(pick & 31u);
+                c2 = (int)(pick >> 5);
+            }
+        } else if (!key_of.zoom && key_of.shift != 0 && vstar != 0u) {
+            // They lie within 2^-24 of the lower end of the class (a class spans at most 2^27 of the 2^52
+            // mantissas), so that a multiplication per link and two per layer find the few candidates; few
+            // links have a quotient below the optimum at all.
+            constexpr double kNear = 1.0 / (1 << 23);
+            constexpr int kOthers = kWarps - kBack;
+            const double edge = __longlong_as_double((long long)(key_of.base + ((unsigned long long)(vstar - 1u) << key_of.shift)));
+            auto candidate = [&](double q) {
+                if (key_of(q) == vstar) atomicMin(&s_low, (unsigned long long)__double_as_longlong(q));
+            };
+            for (int p0 = 0; p0 < k * k; p0 += 32 * kOthers) {
+                const int p = p0 + lane * kOthers + wid - kBack, w2 = p / k, v2 = p - w2 * k;
+                const bool has = p < k * k && s_gmin[p] <= vstar;
+                const double link = has ? (double)s_bw[v2 * k + w2] : 0.0;
+                for (uint32_t hits = __ballot_sync(kFull, has); hits; hits &= hits - 1) {
+                    const double div = __shfl_sync(kFull, link, __ffs(hits) - 1), near = edge * div;
+                    for (int c = lane; c < L - 1; c += 32) {
+                        const double b = s_bits[c];
+                        if (fabs(b - near) <= near * kNear) candidate(__ddiv_rn(b, div));
                     }
                 }
             }
-            if (lane == 0) s_pick[wid] = bestk;
-            __syncthreads();
-            unsigned int pick = s_pick[lane < kWarps ? lane : 0];
-            pick = __reduce_min_sync(kFull, pick);
-            __syncthreads();
-            if (pick == 0xFFFFFFFFu) {  // cannot happen on a consistent frontier; report, do not trap
-                status = (int)PP_ERR_CUDA;
-                break;
+            if constexpr (CT) {  // compute times: for every end of a run the starts that come near, by bisection
+                for (int e = tid - kBack * 32; e < k * L; e += kOthers * 32) {
+                    const int w2 = e / L, last = e - w2 * L;
+                    const double div = (double)s_speed[w2], near = edge * div, work = (double)s_Wp[last + 1];
+                    if (div == 0.0) continue;
+                    int a = 0, b = last + 1;
+                    while (a < b) {
+                        const int mid = (a + b) >> 1;
+                        if ((double)s_Wp[mid] < work - near - near * kNear) a = mid + 1; else b = mid;
+                    }
+                    for (; a <= last && (double)s_Wp[a] <= work - near + near * kNear; ++a)
+                        candidate(__ddiv_rn((double)(s_Wp[last + 1] - s_Wp[a]), div));
+                }
             }
-            S = from;
-            w = (int)(pick & 31u);
-            c2 = (int)(pick >> 5);
         }
         __syncthreads();
-        if (status != (int)PP_OK) break;
+        if (s_fail) {
+            status = (int)PP_ERR_CUDA;
+            break;
+        }
         // the plan's own bottleneck
         if (tid < m) {
             double x = 0.0;
@@ -591,42 +692,11 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
             }
             atomicMax(&s_worst, (unsigned long long)__double_as_longlong(x));
         }
-        if (tid == 0) s_zoom = 0;
         __syncthreads();
         const unsigned long long worst = s_worst;
         beta = __longlong_as_double((long long)worst);
-        if (key_of.zoom || key_of.shift == 0 || worst == 0ull) break;  // every key is one double
-        // a smaller quotient in the same class?  Few links have one at all below the optimum.
-        if (tid < 32) {
-            int n = 0;
-            for (int p0 = 0; p0 < k * k; p0 += 32) {
-                const int p = p0 + lane;
-                const bool has = p < k * k && s_gmin[p] <= vstar;
-                const uint32_t hit = __ballot_sync(kFull, has);
-                if (has) s_links[n + __popc(hit & ((1u << lane) - 1u))] = (uint16_t)p;
-                n += __popc(hit);
-            }
-            if (lane == 0) s_nlinks = n;
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int e = tid; e < s_nlinks * L; e += kThreads) {
-            const int p = s_links[e / L], c = e % L;
-            if (c < L - 1 && d.gam[(size_t)p * Lp + c] == vstar) {
-                const int w2 = p / k, v2 = p - w2 * k;
-                if ((unsigned long long)__double_as_longlong(__ddiv_rn(s_bits[c], (double)s_bw[v2 * k + w2])) < worst) s_zoom = 1;
-            }
-        }
-        if constexpr (CT) {
-            for (int e = tid; e < k * L * Lp; e += kThreads)
-                if (__ldcg(d.seg + e) == vstar) {
-                    const int r = e / Lp, last = e - r * Lp, w2 = r / L, first = last - (r - w2 * L);
-                    if ((unsigned long long)__double_as_longlong(__ddiv_rn((double)(s_Wp[last + 1] - s_Wp[first]), (double)s_speed[w2])) < worst)
-                        s_zoom = 1;
-                }
-        }
-        __syncthreads();
-        if (!s_zoom) break;
+        // exact unless the class of the optimum holds a quotient smaller than the plan's own bottleneck
+        if (key_of.zoom || s_low >= worst) break;
         key_of.zoom = vstar;  // once more, this class resolved
         nblk = 1;
         if (tid == 0) s_best = kNoBest;
@@ -653,6 +723,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
             ctl->dense = dense ? 1 : 0;
         }
     }
+    if constexpr (SM) return;  // the counters in global memory are as they were
     // the last block to leave clears the counters for the next launch
     __shared__ uint32_t s_left;
     __syncthreads();
@@ -674,12 +745,38 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
 struct PruneShape {
     int G, P;
 };
-PruneShape prune_shape(int L)
+// Lanes and positions a lane of a row.  Short rows of few nodes take two positions a lane: there are warps
+// to spare, and the time of a level is that of a lane's own chain of instructions.
+PruneShape prune_shape(int L, int k)
 {
-    PruneShape s{4, 4};
+    PruneShape s = L <= 64 && k <= kWideK ? PruneShape{8, 2} : PruneShape{4, 4};
     while (s.G * s.P < L && s.G < 32) s.G *= 2;
     while (s.G * s.P < L) s.P *= 2;
     return s;
+}
+
+// targets of the widest level if it is kept whole
+unsigned long long widest_level(int k)
+{
+    unsigned long long widest = 1, binom = 1;
+    for (int j = 1; j <= k; ++j) {
+        binom = binom * (unsigned)(k - j + 1) / (unsigned)j;  // C(k, j)
+        widest = std::max(widest, binom * (unsigned)(k - j));
+    }
+    return widest;
+}
+
+// Shared memory of a block that holds the whole search; 0 when it does not fit or the widest level takes
+// more than kSharedRounds rounds of a block's groups.  With the tables in shared memory a round takes 1.4 us
+// against 3.3 in global memory, and there is no barrier of blocks (2 us a level and more).
+template <int G, int P, bool CT>
+size_t shared_bytes(int L, int k, int Lp)
+{
+    constexpr int groups = prune_threads(P) / G;
+    if (k > 10 || widest_level(k) > (unsigned long long)kSharedRounds * groups) return 0;
+    const size_t rows = ((size_t)k << (k - 1)) * Lp * 4, seg = CT ? (size_t)k * L * Lp * 4 : 0;
+    const size_t all = prune_layout(L, k, Lp, groups, kStripBytes<G, P>, kCodes<G, P, CT>, CT).total + sparse_layout(k, Lp).rows + rows + seg;
+    return all <= kSharedBytes ? all : 0;
 }
 
 template <int G, int P, bool CT>
@@ -695,36 +792,53 @@ cudaError_t launch_shape(const PruneDev &d, const PruneHost &h, int sms, cudaStr
         std::memcpy(in.speed, h.speed, (size_t)d.k * 4);
     }
     constexpr int threads = prune_threads(P), groups = threads / G;
+    PruneDev q = d;
+    q.clustered = 0;
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = s;
+    cfg.attrs = attr;
+    if (const size_t all = shared_bytes<G, P, CT>(d.L, d.k, d.Lp)) {
+        cudaError_t e = cudaFuncSetAttribute(k_prune<G, P, CT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)all);
+        if (e != cudaSuccess) return e;
+        q.row_cap = (unsigned long long)d.k << (d.k - 1);
+        cfg.dynamicSmemBytes = all;
+        return cudaLaunchKernelEx(&cfg, k_prune<G, P, CT, true>, q, in);
+    }
     // blocks: one round over the targets of the widest level if it is kept whole; a single block where
     // two rounds of it do, its barrier costs next to nothing
-    unsigned long long widest = 1, binom = 1;
-    for (int j = 1; j <= d.k; ++j) {
-        binom = binom * (unsigned)(d.k - j + 1) / (unsigned)j;  // C(k, j)
-        widest = std::max(widest, binom * (unsigned)(d.k - j));
-    }
+    const unsigned long long widest = widest_level(d.k);
     int blocks = (int)std::min<unsigned long long>((widest + groups - 1) / groups, (unsigned long long)sms);
     if (blocks <= 2) blocks = 1;
-    const size_t sm = prune_layout(d.L, d.k, d.Lp, groups, kStripBytes<G, P>, kCodes<G, CT>, CT).total;
-    cudaError_t e = cudaFuncSetAttribute(k_prune<G, P, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    // up to kClusterRounds rounds of 8 blocks: one cluster, whose barrier is the hardware's (0.3 us; one in
+    // global memory 1.5 to 2)
+    const bool cluster = blocks > 1 && widest <= (unsigned long long)kClusterRounds * kClusterBlocks * groups;
+    if (cluster) blocks = kClusterBlocks;
+    const size_t sm = prune_layout(d.L, d.k, d.Lp, groups, kStripBytes<G, P>, kCodes<G, P, CT>, CT).total;
+    cudaError_t e = cudaFuncSetAttribute(k_prune<G, P, CT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)blocks);
-    cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = sm;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
+    if (cluster) {
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)blocks;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    } else {
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+    }
     cfg.numAttrs = blocks > 1 ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k_prune<G, P, CT>, d, in);
+    q.clustered = cluster ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k_prune<G, P, CT, false>, q, in);
 }
 
 }  // namespace
 
-int prune_row_pad(int L)
+int prune_row_pad(int L, int k)
 {
-    const int P = prune_shape(L).P;
+    const int P = prune_shape(L, k).P;
     return (L + P - 1) / P * P;
 }
 
@@ -765,15 +879,33 @@ void prune_node_bounds(const uint64_t *cap, uint64_t total, PruneDev *d)
     }
 }
 
-cudaError_t launch_prune(const PruneDev &d, const PruneHost &h, int sms, cudaStream_t s)
+// F<G, P, CT> of the shape of a row of L layers among k nodes; Eq. 1 stops at 256 layers
+#define PP_SHAPES(CASE) CASE(8, 2) CASE(16, 2) CASE(32, 2) CASE(4, 4) CASE(8, 4) CASE(16, 4) CASE(32, 4) CASE(32, 8)
+
+bool prune_in_shared(int L, int k, bool compute)
 {
-    const PruneShape sh = prune_shape(d.L);
+    const PruneShape sh = prune_shape(L, k);
+    const int Lp = prune_row_pad(L, k);
     switch (sh.G * 100 + sh.P) {
 #define PP_CASE(g, p) \
-    case g * 100 + p: return d.seg ? launch_shape<g, p, true>(d, h, sms, s) : launch_shape<g, p, false>(d, h, sms, s);
-        PP_CASE(4, 4) PP_CASE(8, 4) PP_CASE(16, 4) PP_CASE(32, 4) PP_CASE(32, 8)
+    case g * 100 + p: return (compute ? shared_bytes<g, p, true>(L, k, Lp) : shared_bytes<g, p, false>(L, k, Lp)) != 0;
+        PP_SHAPES(PP_CASE)
 #undef PP_CASE
-        case 3216: return launch_shape<32, 16, false>(d, h, sms, s);  // Eq. 1 stops at 256 layers
+        case 3216: return !compute && shared_bytes<32, 16, false>(L, k, Lp) != 0;
+        case 3232: return !compute && shared_bytes<32, 32, false>(L, k, Lp) != 0;
+    }
+    return false;
+}
+
+cudaError_t launch_prune(const PruneDev &d, const PruneHost &h, int sms, cudaStream_t s)
+{
+    const PruneShape sh = prune_shape(d.L, d.k);
+    switch (sh.G * 100 + sh.P) {
+#define PP_CASE(g, p) \
+    case g * 100 + p: return h.Wp ? launch_shape<g, p, true>(d, h, sms, s) : launch_shape<g, p, false>(d, h, sms, s);
+        PP_SHAPES(PP_CASE)
+#undef PP_CASE
+        case 3216: return launch_shape<32, 16, false>(d, h, sms, s);
         case 3232: return launch_shape<32, 32, false>(d, h, sms, s);
     }
     return cudaErrorInvalidValue;

@@ -13,26 +13,11 @@
 // bisected over the prefix sums, and the r-th free node is found by counting bits in halves: a step is
 // some forty instructions for every lane alike (a bisection and a walk over the free nodes before:
 // 100 003 plans of k = 14, L = 50 in 14.4 us).
-#include "pp_internal.cuh"
+#include "pp_blocks.cuh"
 
 namespace pp {
 
 constexpr int kRandomThreads = 128;
-
-// r-th (from 0) set bit of x; r below the number of set bits
-__device__ __forceinline__ int select_bit(uint32_t x, int r)
-{
-    int at = 0;
-#pragma unroll
-    for (int half = 16; half; half >>= 1) {
-        const int below = __popc(x & ((1u << half) - 1u));
-        const bool up = r >= below;
-        r -= up ? below : 0;
-        at += up ? half : 0;
-        x = up ? x >> half : x;
-    }
-    return at;
-}
 
 // Rows travel through shared memory so that global memory sees whole contiguous blocks: the draws
 // of the block's plans on the way in, their two output rows on the way out, a pair of words at a time.  A

@@ -1431,7 +1431,7 @@ pp_status pp_kpath_colour_batch(int32_t n, const uint32_t *bw_kbps, int64_t Q, i
 }
 
 // The whole stage as one launch (pp_match.cu): one copy up, the result in page-locked memory.
-constexpr size_t kMatchSharedBytes = 220 * 1024;
+constexpr size_t kMatchSharedBytes = 224 * 1024;
 static pp_status match_one_launch(int32_t n, const uint32_t *bw, int32_t n_cuts, int32_t trials, const uint32_t *draws,
                                   const std::vector<MatchRun> &order, int kk, int32_t *nodes, uint32_t *cut_threshold,
                                   cudaStream_t s)
@@ -1441,7 +1441,8 @@ static pp_status match_one_launch(int32_t n, const uint32_t *bw, int32_t n_cuts,
     PP_CUDA(multiprocessors(dev, &sms));
     SlotLease lease;
     if (!lease.slot) return PP_ERR_NOMEM;
-    const size_t sz[4] = {(size_t)n * n * 4, (size_t)trials * n * 4, order.size() * sizeof(MatchRun), sizeof(MatchCtl)};
+    const size_t sz[4] = {(size_t)n * n * 4, (size_t)trials * n * 4, order.size() * sizeof(MatchRun),
+                          (size_t)2 * std::min(trials, sms) * 32};
     size_t off[5];
     off[0] = 0;
     for (int i = 0; i < 4; ++i) off[i + 1] = align_up(off[i] + sz[i], 128);
@@ -1449,18 +1450,17 @@ static pp_status match_one_launch(int32_t n, const uint32_t *bw, int32_t n_cuts,
     const void *src[3] = {bw, draws, order.data()};
     for (int i = 0; i < 3; ++i) std::memcpy(st.data() + off[i], src[i], sz[i]);
     unsigned char *buf = nullptr;
-    PP_CUDA(staging_alloc(reinterpret_cast<void **>(&buf), off[4] + (size_t)2 * sms * PP_KPATH_MAX_K * 4, s));
+    PP_CUDA(staging_alloc(reinterpret_cast<void **>(&buf), off[4], s));
     MatchDev d;
-    d.n = n; d.n_cuts = n_cuts; d.n_runs = (int)order.size(); d.trials = trials;
+    d.n = n; d.n_cuts = n_cuts; d.n_runs = (int)order.size(); d.trials = trials; d.kk = kk;
     d.bw = reinterpret_cast<uint32_t *>(buf + off[0]);
     d.draws = reinterpret_cast<uint32_t *>(buf + off[1]);
     d.runs = reinterpret_cast<MatchRun *>(buf + off[2]);
-    d.ctl = reinterpret_cast<MatchCtl *>(buf + off[3]);
-    d.paths = reinterpret_cast<int32_t *>(buf + off[4]);
+    d.records = reinterpret_cast<unsigned long long *>(buf + off[3]);
     d.out = &lease.slot->match;
     lease.slot->match.status = (int)PP_ERR_CUDA;
     cudaError_t e = cudaMemcpyAsync(buf, st.data(), off[4], cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = launch_match(d, kk, sms, s);
+    if (e == cudaSuccess) e = launch_match(d, sms, s);
     cudaFreeAsync(buf, s);
     const cudaError_t e2 = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return from_cuda(e);

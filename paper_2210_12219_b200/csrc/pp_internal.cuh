@@ -224,24 +224,19 @@ cudaError_t launch_kpath(int n, int kk, int64_t Q, const uint32_t *bw, const uin
 struct MatchRun {
     int32_t first, cuts;       // a run of cuts of one class, in serving order
 };
-struct MatchCtl {
-    unsigned long long best[64];  // per run: bottleneck << 32 | ~colouring; zero before the launch
-    uint32_t arrived;
-};
 struct MatchOut {
     int32_t status, nodes[64];
     uint32_t threshold[64];
 };
 struct MatchDev {
-    int n, n_cuts, n_runs, trials;
+    int n, n_cuts, n_runs, trials, kk;  // kk: vertices of the longest path
     const uint32_t *bw, *draws;
     const MatchRun *runs;
-    int32_t *paths;            // [2][blocks][PP_KPATH_MAX_K]
-    MatchCtl *ctl;
+    unsigned long long *records;  // [2][blocks][4]; no tag of a run in it before the launch
     MatchOut *out;             // mapped host memory
 };
 size_t match_smem_bytes(int n, int kk);
-cudaError_t launch_match(const MatchDev &d, int kk_max, int sms, cudaStream_t s);
+cudaError_t launch_match(const MatchDev &d, int sms, cudaStream_t s);
 // Issue-rate probe (pp_probe.cu): `blocks` blocks of 1024 threads, cycles[b] = SM clocks block b took.
 cudaError_t launch_probe(int op, int iters, int blocks, long long *cycles, uint32_t *sink, cudaStream_t s);
 double probe_instr_per_block(int iters);

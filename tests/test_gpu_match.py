@@ -21,7 +21,7 @@ def _built():
 
 
 @pytest.mark.parametrize("n,cuts,classes,trials", [(12, 5, 2, 200), (13, 8, 1, 60), (14, 9, 1, 40), (64, 4, 2, 10), (2, 1, 1, 3),
-                                                   (13, 11, 1, 30)])
+                                                   (13, 11, 1, 30), (32, 5, 2, 9), (33, 5, 2, 9), (3, 2, 1, 149)])
 def test_matching_shapes(n, cuts, classes, trials):
     rng = np.random.default_rng(n * 100 + cuts)
     for sym in (True, False):

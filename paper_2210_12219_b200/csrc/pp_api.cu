@@ -1343,13 +1343,18 @@ pp_status pp_partition_minsum_batch(int64_t B, int32_t L, const uint64_t *cut_we
         SlotLease lease;
         if (!lease.slot) return PP_ERR_NOMEM;
         unsigned char *h = lease.slot->small;
-        const void *in[3] = {cut_weight, mem, kappa};
-        for (int i = 0; i < 3; ++i) std::memcpy(h + off[i], in[i], sz[i]);
-        PP_CUDA(launch_partition_minsum(B, L, cap_seg, reinterpret_cast<uint64_t *>(h + off[0]),
-                                        reinterpret_cast<uint64_t *>(h + off[1]), reinterpret_cast<uint64_t *>(h + off[2]),
-                                        reinterpret_cast<uint64_t *>(h + off[3]), reinterpret_cast<int32_t *>(h + off[4]),
-                                        reinterpret_cast<int32_t *>(h + off[5]), reinterpret_cast<uint64_t *>(h + off[6]),
-                                        reinterpret_cast<int8_t *>(h + off[7]), nullptr));
+        uint64_t *o_cost = reinterpret_cast<uint64_t *>(h + off[3]), *o_sizes = reinterpret_cast<uint64_t *>(h + off[6]);
+        int32_t *o_m = reinterpret_cast<int32_t *>(h + off[4]), *o_cuts = reinterpret_cast<int32_t *>(h + off[5]);
+        int8_t *o_status = reinterpret_cast<int8_t *>(h + off[7]);
+        if (partition_as_params(B, L)) {
+            PP_CUDA(launch_partition_params(B, L, cap_seg, cut_weight, mem, kappa, o_cost, o_m, o_cuts, o_sizes, o_status, nullptr));
+        } else {
+            const void *in[3] = {cut_weight, mem, kappa};
+            for (int i = 0; i < 3; ++i) std::memcpy(h + off[i], in[i], sz[i]);
+            PP_CUDA(launch_partition_minsum(B, L, cap_seg, reinterpret_cast<uint64_t *>(h + off[0]),
+                                            reinterpret_cast<uint64_t *>(h + off[1]), reinterpret_cast<uint64_t *>(h + off[2]),
+                                            o_cost, o_m, o_cuts, o_sizes, o_status, nullptr));
+        }
         PP_CUDA(cudaStreamSynchronize(nullptr));
         void *out[5] = {cost, m, cuts, sizes, status};
         const size_t n[5] = {sz[3], sz[4], nB * (size_t)cap_seg * 4, nB * (size_t)cap_seg * 8, sz[7]};

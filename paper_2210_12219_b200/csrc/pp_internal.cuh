@@ -215,6 +215,12 @@ size_t partition_smem_bytes(int L);
 cudaError_t launch_partition_minsum(int64_t B, int L, int cap_seg, const uint64_t *weight, const uint64_t *mem,
                                     const uint64_t *kappa, uint64_t *cost, int32_t *m, int32_t *cuts,
                                     uint64_t *sizes, int8_t *status, cudaStream_t s);
+// The same for a few chains in host arrays that travel as kernel parameters (partition_as_params says which);
+// the outputs are device or page-locked memory.
+bool partition_as_params(int64_t B, int L);
+cudaError_t launch_partition_params(int64_t B, int L, int cap_seg, const uint64_t *weight, const uint64_t *mem,
+                                    const uint64_t *kappa, uint64_t *cost, int32_t *m, int32_t *cuts, uint64_t *sizes,
+                                    int8_t *status, cudaStream_t s);
 // Colour-coding k-path search of the placement stage (Algorithm 2's K-PATH), one block per query.
 size_t kpath_smem_bytes(int kk);
 cudaError_t launch_kpath(int n, int kk, int64_t Q, const uint32_t *bw, const uint32_t *threshold, const int32_t *start,

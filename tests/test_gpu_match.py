@@ -40,7 +40,7 @@ def test_matching_shapes(n, cuts, classes, trials):
             assert (thr[first:first + run] == t).all()
 
 
-@pytest.mark.parametrize("L", [1, 2, 31, 33, 100, 1024])
+@pytest.mark.parametrize("L", [1, 2, 31, 32, 33, 64, 65, 100, 128, 129, 1024])
 def test_partition_windows(L):
     # windows from a single point to the whole chain, equal and rising and falling weights
     rng = np.random.default_rng(L)
@@ -49,7 +49,7 @@ def test_partition_windows(L):
     for w in weights:
         for m in mem:
             for kappa in (int(m.max()), int(m.max()) + 1, int(m.sum()) // 3 + 9, int(m.sum())):
-                want = OP.minsum_partition([int(x) for x in w], [int(x) for x in m], kappa) if L <= 100 else None
+                want = OP.minsum_partition([int(x) for x in w], [int(x) for x in m], kappa) if L <= 129 else None
                 got = pp.partition_minsum_batch(w[None].astype(np.uint64), m[None].astype(np.uint64),
                                                 np.array([kappa], np.uint64), L)
                 many = pp.partition_minsum_batch(np.repeat(w[None], 40, 0).astype(np.uint64),

@@ -8,6 +8,7 @@
 #include <functional>
 #include <limits>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -408,6 +409,8 @@ struct HostSlot {
     PruneNote note;
     MatchOut match;
     PruneCtl *ctl;             // counters of a search, on the chunk's device
+    unsigned long long *records;  // of the placement stage, on the chunk's device: MatchDev::records
+    int half;
     alignas(256) unsigned char small[15 * 1024];  // inputs and results of a small call as a whole
 };
 constexpr int kSlots = 8;
@@ -420,7 +423,10 @@ public:
         std::lock_guard<std::mutex> lock(mu_);
         for (auto &c : chunks_)
             if (c.free && c.dev == dev) return from(c);
-        Chunk c{nullptr, nullptr, (1u << kSlots) - 1u, dev};
+        int sms = 0;
+        if (multiprocessors(dev, &sms) != cudaSuccess) return nullptr;
+        Chunk c{nullptr, nullptr, nullptr, (1u << kSlots) - 1u, dev};
+        const size_t records = match_record_bytes(sms);
         try {
             chunks_.reserve(chunks_.size() + 1);
         } catch (const std::bad_alloc &) {
@@ -431,14 +437,21 @@ public:
         cudaError_t e = cudaHostAlloc(reinterpret_cast<void **>(&c.base), kSlots * sizeof(HostSlot),
                                       cudaHostAllocPortable | cudaHostAllocMapped);
         if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&c.ctl), sizeof init);
+        if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&c.records), kSlots * records);
+        if (e == cudaSuccess) e = cudaMemset(c.records, 0, kSlots * records);
         if (e == cudaSuccess) e = cudaMemcpy(c.ctl, init, sizeof init, cudaMemcpyHostToDevice);
         if (e != cudaSuccess) {
             cudaFreeHost(c.base);
             cudaFree(c.ctl);
+            cudaFree(c.records);
             cudaGetLastError();
             return nullptr;
         }
-        for (int i = 0; i < kSlots; ++i) c.base[i].ctl = c.ctl + i;
+        for (int i = 0; i < kSlots; ++i) {
+            c.base[i].ctl = c.ctl + i;
+            c.base[i].records = reinterpret_cast<unsigned long long *>(c.records + i * records);
+            c.base[i].half = 0;
+        }
         chunks_.push_back(c);
         return from(chunks_.back());
     }
@@ -455,6 +468,7 @@ public:
             if (another && c.free == (1u << kSlots) - 1u) {
                 cudaFreeHost(c.base);
                 cudaFree(c.ctl);
+                cudaFree(c.records);
                 chunks_.erase(chunks_.begin() + (long)i);
             }
             return;
@@ -465,6 +479,7 @@ private:
     struct Chunk {
         HostSlot *base;
         PruneCtl *ctl;
+        unsigned char *records;
         uint32_t free;
         int dev;
     };
@@ -1446,32 +1461,40 @@ static pp_status match_one_launch(int32_t n, const uint32_t *bw, int32_t n_cuts,
     PP_CUDA(multiprocessors(dev, &sms));
     SlotLease lease;
     if (!lease.slot) return PP_ERR_NOMEM;
-    const size_t sz[4] = {(size_t)n * n * 4, (size_t)trials * n * 4, order.size() * sizeof(MatchRun),
-                          (size_t)2 * std::min(trials, sms) * 32};
-    size_t off[5];
-    off[0] = 0;
-    for (int i = 0; i < 4; ++i) off[i + 1] = align_up(off[i] + sz[i], 128);
-    std::vector<unsigned char> st(off[4], 0);
-    const void *src[3] = {bw, draws, order.data()};
-    for (int i = 0; i < 3; ++i) std::memcpy(st.data() + off[i], src[i], sz[i]);
-    unsigned char *buf = nullptr;
-    PP_CUDA(staging_alloc(reinterpret_cast<void **>(&buf), off[4], s));
+    HostSlot &slot = *lease.slot;
     MatchDev d;
     d.n = n; d.n_cuts = n_cuts; d.n_runs = (int)order.size(); d.trials = trials; d.kk = kk;
-    d.bw = reinterpret_cast<uint32_t *>(buf + off[0]);
-    d.draws = reinterpret_cast<uint32_t *>(buf + off[1]);
-    d.runs = reinterpret_cast<MatchRun *>(buf + off[2]);
-    d.records = reinterpret_cast<unsigned long long *>(buf + off[3]);
-    d.out = &lease.slot->match;
-    lease.slot->match.status = (int)PP_ERR_CUDA;
-    cudaError_t e = cudaMemcpyAsync(buf, st.data(), off[4], cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = launch_match(d, sms, s);
-    cudaFreeAsync(buf, s);
+    d.bw = d.draws = nullptr;
+    d.runs = nullptr;
+    d.records = slot.records;
+    d.half = slot.half;
+    d.stride = sms;
+    d.out = &slot.match;
+    slot.match.status = (int)PP_ERR_CUDA;
+    const size_t nn = (size_t)n * n, at = match_runs_at(n, trials), words = at + order.size() * (sizeof(MatchRun) / 4);
+    std::unique_ptr<uint32_t[]> in(new uint32_t[words]);
+    std::memcpy(in.get(), bw, nn * 4);
+    std::memcpy(in.get() + nn, draws, (size_t)trials * n * 4);
+    std::memcpy(in.get() + at, order.data(), order.size() * sizeof(MatchRun));
+    uint32_t *buf = nullptr;
+    cudaError_t e = cudaSuccess;
+    if (!match_as_params(words)) {
+        PP_CUDA(staging_alloc(reinterpret_cast<void **>(&buf), words * 4, s));
+        d.bw = buf;
+        d.draws = buf + nn;
+        d.runs = reinterpret_cast<MatchRun *>(buf + at);
+        e = cudaMemcpyAsync(buf, in.get(), words * 4, cudaMemcpyHostToDevice, s);
+    }
+    if (e == cudaSuccess) e = launch_match(d, in.get(), words, s);
+    if (buf) cudaFreeAsync(buf, s);
     const cudaError_t e2 = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return from_cuda(e);
-    if (e2 != cudaSuccess) return from_cuda(e2);
-    const MatchOut &got = lease.slot->match;
-    if (got.status != PP_OK && got.status != PP_INFEASIBLE) return PP_ERR_CUDA;
+    slot.half ^= 1;
+    if (e != cudaSuccess || e2 != cudaSuccess || slot.match.status == (int)PP_ERR_CUDA) {
+        cudaMemset(slot.records, 0, match_record_bytes(sms));  // not cleared for the next call
+        cudaStreamSynchronize(nullptr);
+        return e != cudaSuccess ? from_cuda(e) : e2 != cudaSuccess ? from_cuda(e2) : PP_ERR_CUDA;
+    }
+    const MatchOut &got = slot.match;
     std::copy(got.nodes, got.nodes + n_cuts + 1, nodes);
     if (cut_threshold) std::copy(got.threshold, got.threshold + n_cuts, cut_threshold);
     return static_cast<pp_status>(got.status);

@@ -238,11 +238,17 @@ struct MatchDev {
     int n, n_cuts, n_runs, trials, kk;  // kk: vertices of the longest path
     const uint32_t *bw, *draws;
     const MatchRun *runs;
-    unsigned long long *records;  // [2][blocks][4]; no tag of a run in it before the launch
+    unsigned long long *records;  // [2][2][stride][4]: by `half`, by the parity of the run, by block; this half is
+    int half, stride;             // zero before the launch and the launch zeroes the other; stride: blocks at most
     MatchOut *out;             // mapped host memory
 };
 size_t match_smem_bytes(int n, int kk);
-cudaError_t launch_match(const MatchDev &d, int sms, cudaStream_t s);
+// The inputs one after another: bandwidths, draws, at an even word the runs.
+__host__ __device__ inline size_t match_runs_at(int n, int trials) { return ((size_t)n * n + (size_t)trials * n + 1) & ~(size_t)1; }
+bool match_as_params(size_t words);
+size_t match_record_bytes(int sms);
+// d.bw null: the inputs go with the launch, from host memory.
+cudaError_t launch_match(const MatchDev &d, const uint32_t *in, size_t words, cudaStream_t s);
 // Issue-rate probe (pp_probe.cu): `blocks` blocks of 1024 threads, cycles[b] = SM clocks block b took.
 cudaError_t launch_probe(int op, int iters, int blocks, long long *cycles, uint32_t *sink, cudaStream_t s);
 double probe_instr_per_block(int iters);

@@ -25,15 +25,17 @@
 // probes of a launch, two copies and a synchronisation (45 us) for each run.
 #include "pp_internal.cuh"
 
+#include <cstring>
+
 namespace pp {
 
 namespace {
 
-constexpr int kMatchThreads = 512;
-constexpr int kMatchWarps = kMatchThreads / 32;
+constexpr int kShortPath = 4;
 constexpr uint32_t kFull = 0xFFFFFFFFu;
 constexpr int kSpinLimit = 1 << 22;
 constexpr int kMaxRuns = 64;
+constexpr int kRecordWords = 8;  // of a block: two records of four words, by the parity of the run
 constexpr int kAhead = 4;      // predecessors at a time
 constexpr int kPadWords = 64;  // a lane without a second vertex reads this far beyond a row, and drops what it read
 constexpr int kWordNodes = 9;  // nodes of a path in the third word of a record, the others in the fourth; 6 bits each
@@ -63,8 +65,22 @@ __device__ __forceinline__ void st_relaxed(unsigned long long *p, unsigned long 
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-__global__ void __launch_bounds__(kMatchThreads, 1) k_match(const MatchDev d)
+// WORDS > 0: bandwidths, draws and runs travel as parameters of the launch.  Up to 8 KB that costs a call 2 us
+// less than a copy in front of it; of 16 KB the parameters take longer than the copy (a launch carries all of
+// its struct, 0.3 us for each KB beyond four).
+template <int WORDS>
+struct MatchIn {
+    uint32_t v[WORDS];
+};
+template <>
+struct MatchIn<0> {};
+
+// Paths of up to kShortPath vertices have no work for more than eight warps, and every barrier costs by the warp
+// (three runs of four vertices and less: 21.7 us a call with 512 threads, 20.9 with 256; ten vertices 118 and 140).
+template <int kMatchThreads, int WORDS>
+__global__ void __launch_bounds__(kMatchThreads, 1) k_match(const __grid_constant__ MatchDev d, const __grid_constant__ MatchIn<WORDS> in)
 {
+    constexpr int kMatchWarps = kMatchThreads / 32;
     extern __shared__ __align__(16) uint32_t smem_match[];
     const int n = d.n, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     uint32_t *s_bw = smem_match;       // [n][n]
@@ -75,14 +91,27 @@ __global__ void __launch_bounds__(kMatchThreads, 1) k_match(const MatchDev d)
     __shared__ uint32_t s_thr[64];
     __shared__ MatchRun s_runs[kMaxRuns];
     __shared__ unsigned long long s_top[kMatchWarps], s_path[2];
-    const uint32_t draw = tid < n ? d.draws[(size_t)blockIdx.x * n + tid] : 0u;  // of the block's first colouring
+    const uint32_t *g_bw = d.bw, *g_draws = d.draws;
+    const MatchRun *g_runs = d.runs;
+    if constexpr (WORDS > 0) {
+        g_bw = in.v;
+        // an address of their own: neighbouring threads read neighbouring words, which the constant bank would
+        // serve one after another
+        asm volatile("" : "+l"(g_bw));
+        g_draws = g_bw + n * n;
+        g_runs = reinterpret_cast<const MatchRun *>(g_bw + match_runs_at(n, d.trials));
+    }
+    // the records of the launch before this one lie in the other half: no tag in it for the launch after
+    if (blockIdx.x == 0)
+        for (int i = tid; i < kRecordWords * d.stride; i += kMatchThreads) d.records[(size_t)(d.half ^ 1) * kRecordWords * d.stride + i] = 0ull;
+    const uint32_t draw = tid < n ? g_draws[(size_t)blockIdx.x * n + tid] : 0u;  // of the block's first colouring
     uint32_t part[PP_KPATH_MAX_N * PP_KPATH_MAX_N / kMatchThreads];  // of the bandwidths, on their way while the sets are listed
 #pragma unroll
     for (int i = 0; i < PP_KPATH_MAX_N * PP_KPATH_MAX_N / kMatchThreads; ++i) {
         const int e = tid + i * kMatchThreads;
-        part[i] = e < n * n ? d.bw[e] : 0u;
+        part[i] = e < n * n ? g_bw[e] : 0u;
     }
-    if (tid < d.n_runs) s_runs[tid] = d.runs[tid];
+    if (tid < d.n_runs) s_runs[tid] = g_runs[tid];
     if (tid < 64) {
         s_nodes[tid] = -1;
         s_thr[tid] = 0u;
@@ -127,7 +156,7 @@ __global__ void __launch_bounds__(kMatchThreads, 1) k_match(const MatchDev d)
         for (int t = blockIdx.x; t < d.trials; t += gridDim.x) {
             if (t != (int)blockIdx.x) {
                 __syncthreads();  // the path has been read from the table
-                prepare(tid < n ? d.draws[(size_t)t * n + tid] : 0u, kk);
+                prepare(tid < n ? g_draws[(size_t)t * n + tid] : 0u, kk);
             }
             __syncthreads();
             if (tid < n && tid != uv && ((alive >> tid) & 1ull) && (sv < 0 || sv == tid)) W[(1u << s_col[tid]) * n + tid] = kFull;
@@ -201,7 +230,7 @@ __global__ void __launch_bounds__(kMatchThreads, 1) k_match(const MatchDev d)
             }
         }
         // records of this parity were read by every block before it posted the run in between
-        unsigned long long *rec = d.records + (size_t)(run & 1) * gridDim.x * 4;
+        unsigned long long *rec = d.records + ((size_t)d.half * 2 + (run & 1)) * d.stride * 4;
         const unsigned long long tag = (unsigned long long)(run + 1);
         if (wid == 0) {
             const uint32_t id = lane < kk && best != 0ull ? (uint32_t)node : 0u;
@@ -273,14 +302,19 @@ __global__ void __launch_bounds__(kMatchThreads, 1) k_match(const MatchDev d)
 
 size_t match_smem_bytes(int n, int kk) { return ((size_t)n * n + kPadWords + ((size_t)n << kk)) * 4 + ((size_t)2 << kk); }
 
-cudaError_t launch_match(const MatchDev &d, int sms, cudaStream_t s)
+size_t match_record_bytes(int sms) { return (size_t)2 * kRecordWords * 8 * sms; }
+
+namespace {
+
+template <int THREADS, int WORDS>
+cudaError_t launch_match_of(const MatchDev &d, const MatchIn<WORDS> &in, cudaStream_t s)
 {
     const size_t sm = match_smem_bytes(d.n, d.kk);
-    cudaError_t e = cudaFuncSetAttribute(k_match, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = cudaFuncSetAttribute(k_match<THREADS, WORDS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(d.trials < sms ? d.trials : sms));
-    cfg.blockDim = dim3(kMatchThreads);
+    cfg.gridDim = dim3((unsigned)(d.trials < d.stride ? d.trials : d.stride));
+    cfg.blockDim = dim3(THREADS);
     cfg.dynamicSmemBytes = sm;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -288,7 +322,27 @@ cudaError_t launch_match(const MatchDev &d, int sms, cudaStream_t s)
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_match, d);
+    return cudaLaunchKernelEx(&cfg, k_match<THREADS, WORDS>, d, in);
 }
+
+template <int WORDS>
+cudaError_t launch_match_in(const MatchDev &d, const MatchIn<WORDS> &in, cudaStream_t s)
+{
+    return d.kk <= kShortPath ? launch_match_of<256>(d, in, s) : launch_match_of<512>(d, in, s);
+}
+
+constexpr int kParamWords = 2000;
+
+}  // namespace
+
+cudaError_t launch_match(const MatchDev &d, const uint32_t *in, size_t words, cudaStream_t s)
+{
+    if (d.bw) return launch_match_in<0>(d, MatchIn<0>{}, s);
+    MatchIn<kParamWords> params;
+    std::memcpy(params.v, in, words * 4);
+    return launch_match_in<kParamWords>(d, params, s);
+}
+
+bool match_as_params(size_t words) { return words <= (size_t)kParamWords; }
 
 }  // namespace pp

@@ -195,9 +195,13 @@ k_partition_warp(const __grid_constant__ std::conditional_t<PARAMS, PartIn, Part
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     unsigned long long *M = s_M[wid];
     if constexpr (PARAMS) {
-        weight = params.v;
-        mem = params.v + B * L;
-        kappa = params.v + 2 * B * L;
+        const uint64_t *in = params.v;
+        // an address of its own: neighbouring lanes read neighbouring words, which the constant bank would serve
+        // one after another
+        asm volatile("" : "+l"(in));
+        weight = in;
+        mem = in + B * L;
+        kappa = in + 2 * B * L;
     }
     for (int64_t b = (int64_t)blockIdx.x * kPartWarps + wid; b < B; b += (int64_t)gridDim.x * kPartWarps) {
         unsigned long long wt[NQ], x[NQ];

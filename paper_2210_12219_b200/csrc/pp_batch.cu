@@ -42,6 +42,7 @@ __host__ __device__ inline BatchShape batch_shape(int L)
 struct BatchLayout {
     size_t dp, key, val, rk, hist, rank, M, cap, bits, dbits, bw, ubw, rowoff, pair_u, cls, lo, code, strips, total;
     int Ls;  // row stride: whole pieces of four positions
+    int Lc;  // row stride of the window codes: a lane reads those of all its P positions
 };
 
 __host__ __device__ inline BatchLayout batch_layout(int L, int k)
@@ -52,6 +53,7 @@ __host__ __device__ inline BatchLayout batch_layout(int L, int k)
     const size_t Ls = ((size_t)L + 3) & ~(size_t)3;
     const BatchShape sh = batch_shape(L);
     b.Ls = (int)Ls;
+    b.Lc = (L + sh.P - 1) / sh.P * sh.P;
     size_t o = 0;
     auto up16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
     auto take = [&](size_t bytes) { size_t at = o; o = up16(o + bytes); return at; };
@@ -66,7 +68,7 @@ __host__ __device__ inline BatchLayout batch_layout(int L, int k)
     b.rank = take((size_t)k * k * Ls * sizeof(uint16_t));
     b.pair_u = take((size_t)k * k * sizeof(int16_t));
     b.cls = take((size_t)L * sizeof(uint16_t));
-    b.code = take((size_t)k * Ls * sizeof(WindowCode));
+    b.code = take((size_t)k * b.Lc * sizeof(WindowCode));
     // The scratch of the ranking is dead before the first state is written: it shares the bytes of the state
     // table and the strips.
     const size_t table = up16(rows * Ls * sizeof(uint16_t));
@@ -127,10 +129,10 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
 
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int sl = lane & (G - 1), at = sl * P;
-    const int Ls = lay.Ls;
+    const int Ls = lay.Ls, Lc = lay.Lc;
     const bool in_row = at < Ls;
     const int at0 = in_row ? at : 0;
-    WindowCode *code = reinterpret_cast<WindowCode *>(smem + lay.code);  // [w][Ls]
+    WindowCode *code = reinterpret_cast<WindowCode *>(smem + lay.code);  // [w][Lc]
     uint16_t *strip = reinterpret_cast<uint16_t *>(smem + lay.strips) + (size_t)(tid / G) * Strip<G, P>::kSize;
     const double kInf = __longlong_as_double(0x7FF0000000000000ll);
     const uint32_t FULL = 0xFFFFFFFFu;
@@ -218,7 +220,7 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
         // windows: lo = max(c* - 1, 0), c* = first start layer from which the segment ending at layer c2 fits
         for (int w = wid; w < k; w += kBatchWarps) {
             const unsigned long long capw = cap[w];
-            for (int c2 = lane; c2 < Ls; c2 += 32) {
+            for (int c2 = lane; c2 < Lc; c2 += 32) {
                 int a = 0, b = c2;
                 if (c2 < L) {
                     const unsigned long long need = M[c2 + 1];
@@ -232,8 +234,8 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
                 } else {
                     a = c2;  // the pad: an empty window
                 }
-                lo[w * Ls + c2] = (int16_t)a;
-                code[w * Ls + c2] = window_code<G, P, uint16_t>(c2, a);
+                if (c2 < Ls) lo[w * Ls + c2] = (int16_t)a;
+                code[w * Lc + c2] = window_code<G, P, uint16_t>(c2, a);
             }
         }
         __syncthreads();
@@ -294,7 +296,7 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
 #pragma unroll
                 for (int i = 0; i < P; ++i) g[i] = (i & 1) ? g2[i / 2] >> 16 : g2[i / 2] & 0xFFFFu;
                 __syncwarp();  // the previous row's readers are done
-                window_min<G, P>(g, code + w * Ls + at0, strip, sl, kInf16, out);
+                window_min<G, P>(g, code + w * Lc + at0, strip, sl, kInf16, out);
                 const uint32_t S2 = S | (1u << w);
                 uint16_t *dst = dp + (size_t)row * Ls + at;
 #pragma unroll

@@ -46,3 +46,23 @@ def test_extreme_and_close_quotients(L, k):
         want = oracle.dp_naive(inst)
         assert got.status[b] == want.status and got.plan(b) == want.plan(), (L, k, b)
         assert got.beta_ms[b] == want.beta_ms or np.isinf(want.beta_ms), (L, k, b)
+
+
+@pytest.mark.parametrize("L,k", [(3, 2), (16, 5), (17, 4), (31, 6), (33, 6), (45, 7), (66, 5), (127, 4), (129, 4), (132, 3), (258, 3),
+                                 (516, 2)])
+def test_block_per_instance_shapes(L, k):
+    """Rows of every number of positions a lane, whole and ragged ones, in the block-per-instance kernel."""
+    build.build()
+    n = 8 if L <= 66 else 3
+    insts = []
+    for i in range(n):
+        base = W.random_small(97000 + 100 * L + i, L, k)
+        scale = (1.2 + 0.3 * i) * float(base.layer_mem_bytes.sum()) / float(base.node_mem_bytes.sum())
+        insts.append(W.Instance(L, k, base.layer_out_bits, base.layer_mem_bytes,
+                                np.ceil(base.node_mem_bytes * scale).astype(np.uint64), base.bw_kbps, f"shape[{i}]"))
+    got = pp.solve_exact_batch(L, k, *(np.stack([getattr(i, f) for i in insts]) for f in (
+        "layer_out_bits", "layer_mem_bytes", "node_mem_bytes", "bw_kbps")))
+    for b, inst in enumerate(insts):
+        want = oracle.dp_naive(inst)
+        assert got.status[b] == want.status and got.plan(b) == want.plan(), (L, k, b)
+        assert got.beta_ms[b] == want.beta_ms or np.isinf(want.beta_ms), (L, k, b)

@@ -9,11 +9,15 @@
 //   3. sweeps the popcount levels: a group of G lanes takes a target row (P + w, w), P positions a lane,
 //      forms g[c] = min_v max(dp[P][v][c], rank[v][w][c]) on packed pairs of positions and takes the
 //      window minimum over [lo_w(c'), c'-1] (window_min); one block barrier a level;
-//   4. walks back from the smallest final state (value, popcount, mask, node) by the threshold rule, a warp
-//      per source node, and takes beta from the plan's own quotients.
+//   4. walks back from the smallest final state (value, popcount, mask, node) by the threshold rule, one warp,
+//      lanes over the positions, and takes beta from the plan's own quotients.
 // An instance is a chain of some twenty short phases; what bounds a batch of a few hundred is the length of
-// that chain.  300 x (k = 7, L = 45), us in the kernel: 66 with a walk of U + L steps per rank, windows
-// scanned position by position and one warp walking back; see launch_batch for what it is now.
+// that chain.  300 x (k = 7, L = 45), us in the kernel: 66 with a walk of U + L steps per rank and windows
+// scanned position by position, about 40 with the phases above.  Of 93 000 cycles 26 000 then went to the
+// inputs (three dependent trips over the bus, contended 64-bit maxima in shared memory): 9 000 with all loads
+// of a thread in flight and warp reductions, 74 000 in all.  A call from host arrays 88.2 -> 85.8 us, 155 x (k = 8,
+// L = 47) 138.7 -> 133.4, 1616 x (k = 5, L = 53) on the device 72.0 -> 68.3.  Levels take half of it, bound by
+// instruction issue: 8 positions a lane where 4 fit 92.8 us, blocks of 512 threads 91.9, of 256 87.0.
 #include <algorithm>
 
 #include "pp_blocks.cuh"
@@ -121,11 +125,10 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
     int16_t *pair_u = reinterpret_cast<int16_t *>(smem + lay.pair_u);
     uint16_t *cls = reinterpret_cast<uint16_t *>(smem + lay.cls);
     int16_t *lo = reinterpret_cast<int16_t *>(smem + lay.lo);        // [w][Ls]
-    __shared__ unsigned long long s_best, s_least, s_most, s_worst;
+    __shared__ unsigned long long s_best;
+    __shared__ uint32_t s_least, s_most;  // sizes as floats, rounded down and up
     __shared__ uint32_t s_slow, s_fast, s_U, s_D;
     __shared__ uint32_t s_sum[kBatchWarps];
-    __shared__ unsigned int s_pick[kBatchWarps];
-    __shared__ int s_cut[16], s_node[16];
 
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int sl = lane & (G - 1), at = sl * P;
@@ -142,23 +145,69 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
     for (int64_t inst = blockIdx.x; inst < B; inst += gridDim.x) {
         const uint64_t *bits = g_bits + inst * L, *mem = g_mem + inst * L;
         const uint32_t *bw = g_bw + inst * kk;
-        __syncthreads();
-        // ---- 1. stage inputs, prefix sums of the memory (warp 0), bounds of the values ----
+        // ---- 1. stage inputs, bounds of the values ----
+        // The arrays may lie across the bus: every thread asks for its words of all of them before it uses one.
+        unsigned long long x_bits = 0ull, x_mem = 0ull, x_cap = 0ull;
+        uint32_t x_bw = 0u;
+        if (tid < L) {
+            x_bits = bits[tid];
+            x_mem = mem[tid];
+        }
+        if (tid < kk) x_bw = bw[tid];
+        if (tid < k) x_cap = g_cap[inst * k + tid];
+        __syncthreads();  // the instance before this one is done
         if (tid == 0) {
-            s_least = ~0ull;
-            s_most = 0ull;
+            s_least = 0x7F800000u;
+            s_most = 0u;
             s_slow = FULL;
             s_fast = s_U = s_D = 0u;
             s_best = kNoBest;
-            s_worst = 0ull;
+            M[0] = 0ull;
         }
         __syncthreads();
         bool bad = false;
+        {
+            uint32_t least = 0x7F800000u, most = 0u;
+            for (int i = tid; i < L; i += kBatchThreads) {
+                if (i >= kBatchThreads) {
+                    x_bits = bits[i];
+                    x_mem = mem[i];
+                }
+                s_bits[i] = x_bits;
+                M[i + 1] = x_mem;
+                bad |= x_bits >= PP_MAX_BITS;
+                if (x_bits) least = min(least, __float_as_uint(__ull2float_rd(x_bits)));
+                most = max(most, __float_as_uint(__ull2float_ru(x_bits)));
+            }
+            uint32_t usable = 0u;
+            if (tid < kk) {  // k <= 12
+                bad |= x_bw >= PP_MAX_KBPS;
+                usable = tid / k != tid - tid / k * k ? x_bw : 0u;
+                s_bw[tid] = usable;
+            }
+            if (tid < k) cap[tid] = x_cap;
+            if (wid * 32 < L) {
+                least = __reduce_min_sync(FULL, least);
+                most = __reduce_max_sync(FULL, most);
+                if (lane == 0) {
+                    atomicMin(&s_least, least);
+                    atomicMax(&s_most, most);
+                }
+            }
+            if (wid * 32 < kk) {
+                const uint32_t slow = __reduce_min_sync(FULL, usable ? usable : FULL), fast = __reduce_max_sync(FULL, usable);
+                if (lane == 0) {
+                    atomicMin(&s_slow, slow);
+                    atomicMax(&s_fast, fast);
+                }
+            }
+        }
+        __syncthreads();
+        // ---- prefix sums of the memory: the first warp, while the others look for equal values ----
         if (wid == 0) {
             unsigned long long carry = 0;
-            if (lane == 0) M[0] = 0ull;
             for (int base = 0; base < L; base += 32) {
-                unsigned long long x = base + lane < L ? mem[base + lane] : 0ull;
+                unsigned long long x = base + lane < L ? M[base + lane + 1] : 0ull;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
                     const unsigned long long y = __shfl_up_sync(FULL, x, o);
@@ -172,30 +221,10 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
                 if (base + lane < L) M[base + lane + 1] = x;
                 carry = __shfl_sync(FULL, x, 31);
             }
-        } else {
-            for (int i = tid - 32; i < L; i += kBatchThreads - 32) {
-                const unsigned long long x = bits[i];
-                s_bits[i] = x;
-                bad |= x >= PP_MAX_BITS;
-                if (x) atomicMin(&s_least, x);
-                atomicMax(&s_most, x);
-            }
-            for (int p = tid - 32; p < kk; p += kBatchThreads - 32) {
-                const uint32_t x = bw[p];
-                bad |= x >= PP_MAX_KBPS;
-                const uint32_t usable = p / k != p - p / k * k ? x : 0u;
-                s_bw[p] = usable;
-                if (usable) {
-                    atomicMin(&s_slow, usable);
-                    atomicMax(&s_fast, usable);
-                }
-            }
-            if (tid - 32 < k) cap[tid - 32] = g_cap[inst * k + tid - 32];
         }
-        bad = __syncthreads_or(bad);
         // ---- distinct bandwidths and sizes: a value's class is that of its first appearance, and the first
         // appearances are numbered as they come ----
-        for (int p = tid; p < kk; p += kBatchThreads) {
+        for (int p = tid - 32; p >= 0 && p < kk; p += kBatchThreads) {
             const uint32_t x = s_bw[p];
             int f = p;
             for (int q = p - 1; q >= 0; --q) f = s_bw[q] == x ? q : f;
@@ -206,7 +235,7 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
             }
             pair_u[p] = (int16_t)(x == 0u ? -1 : f == p ? u : -2 - f);  // -2 - f: as pair f
         }
-        for (int c = kBatchThreads - 1 - tid; c < L; c += kBatchThreads) {
+        for (int c = kBatchThreads - 1 - tid; wid > 0 && c < L; c += kBatchThreads - 32) {
             const unsigned long long x = s_bits[c];
             int f = c;
             for (int q = c - 1; q >= 0; --q) f = s_bits[q] == x ? q : f;
@@ -217,6 +246,7 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
             }
             cls[c] = (uint16_t)d;
         }
+        bad = __syncthreads_or(bad);
         // windows: lo = max(c* - 1, 0), c* = first start layer from which the segment ending at layer c2 fits
         for (int w = wid; w < k; w += kBatchWarps) {
             const unsigned long long capw = cap[w];
@@ -242,7 +272,8 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
         const int U = (int)s_U, D = (int)s_D;
         // ---- 2. ranks of the quotients, spread out as rank[v][w][c] ----
         rank_quotients<kBatchThreads, unsigned long long, 16>(
-            dbits, ubw, U, D, __ddiv_rd((double)s_least, (double)s_fast), __ddiv_ru((double)s_most, (double)s_slow),
+            dbits, ubw, U, D, __ddiv_rd((double)__uint_as_float(s_least), (double)s_fast),
+            __ddiv_ru((double)__uint_as_float(s_most), (double)s_slow),
             reinterpret_cast<uint32_t *>(smem + lay.key), reinterpret_cast<unsigned long long *>(smem + lay.val),
             reinterpret_cast<uint32_t *>(smem + lay.hist), rk, s_sum);
         for (int pr = wid; pr < kk; pr += kBatchWarps) {
@@ -331,35 +362,28 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
         const int m = (int)((key >> 25) & 31);
         uint32_t S = (uint32_t)((key >> 5) & 0xFFFFF);
         int w = (int)(key & 31), c2 = L - 1, status = (int)PP_OK;
-        if (tid < 16) s_cut[tid] = s_node[tid] = -1;
-        __syncthreads();
+        if (wid > 0) continue;
+        // One warp: a step is a handful of candidates, and a barrier costs more than they do.  Lanes over the
+        // positions, every lane walks the nodes in ascending order: the smallest (position, node) within the
+        // threshold wins.
+        int my_cut = -1, my_node = -1;  // lane j: cut and node of segment j
         for (int j = m - 1; j >= 0; --j) {
-            if (tid == 0) {
-                s_node[j] = w;
-                if (j < m - 1) s_cut[j] = c2;
+            if (lane == j) {
+                my_node = w;
+                if (j < m - 1) my_cut = c2;
             }
             if (j == 0) break;
             const uint32_t from = S & ~(1u << w);
-            const int l0 = lo[w * Ls + c2], np = __popc(from);
             unsigned int pick = FULL;
-            if (wid < np) {
-                uint32_t rem = from;
-                for (int i = wid; i > 0; --i) rem &= rem - 1;
-                const int v = __ffs(rem) - 1;
-                const uint16_t *row = dp + (size_t)(rowoff[from] + wid) * Ls, *rw = rank + (size_t)(v * k + w) * Ls;
-                for (int c0 = l0; c0 < c2; c0 += 32) {
-                    const int c = c0 + lane;
-                    const uint32_t hits = __ballot_sync(FULL, c < c2 && max((uint32_t)row[c], (uint32_t)rw[c]) <= rstar);
-                    if (hits) {
-                        pick = ((unsigned)(c0 + __ffs(hits) - 1) << 5) | (unsigned)v;
-                        break;
-                    }
+            for (int c0 = lo[w * Ls + c2]; c0 < c2 && pick == FULL; c0 += 32) {
+                const int c = min(c0 + lane, c2 - 1);
+                const uint16_t *row = dp + (size_t)rowoff[from] * Ls + c, *rw = rank + (size_t)w * Ls + c;
+                for (uint32_t rem = from; rem; rem &= rem - 1, row += Ls) {
+                    const int v = __ffs(rem) - 1;
+                    if (max((uint32_t)*row, (uint32_t)rw[v * k * Ls]) <= rstar) pick = min(pick, ((unsigned)c << 5) | (unsigned)v);
                 }
+                pick = __reduce_min_sync(FULL, pick);
             }
-            if (lane == 0) s_pick[wid] = pick;
-            __syncthreads();
-            pick = __reduce_min_sync(FULL, s_pick[lane < kBatchWarps ? lane : 0]);
-            __syncthreads();
             if (pick == FULL) {  // inconsistent table: flag the instance, keep going
                 status = (int)PP_ERR_CUDA;
                 break;
@@ -368,25 +392,22 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
             w = (int)(pick & 31u);
             c2 = (int)(pick >> 5);
         }
-        __syncthreads();
         // beta* is the bottleneck of the plan: no link of it ranks above the optimum, and no plan is better
-        if (tid < 32) {
-            double x = 0.0;
-            if (status == (int)PP_OK && lane < m - 1)
-                x = __ddiv_rn((double)s_bits[s_cut[lane]], (double)s_bw[s_node[lane] * k + s_node[lane + 1]]);
-            unsigned long long worst = (unsigned long long)__double_as_longlong(x);  // order like the values
+        const int next = __shfl_down_sync(FULL, my_node, 1);
+        double x = 0.0;
+        if (status == (int)PP_OK && lane < m - 1) x = __ddiv_rn((double)s_bits[my_cut], (double)s_bw[my_node * k + next]);
+        unsigned long long worst = (unsigned long long)__double_as_longlong(x);  // order like the values
 #pragma unroll
-            for (int o = 8; o; o >>= 1) {
-                const unsigned long long other = __shfl_xor_sync(FULL, worst, o);
-                worst = other > worst ? other : worst;
-            }
-            if (lane < k) place[lane] = s_node[lane];
-            if (cuts && lane < k - 1) cuts[lane] = s_cut[lane];
-            if (lane == 0) {
-                o_beta[inst] = __longlong_as_double((long long)worst);
-                o_m[inst] = m;
-                o_status[inst] = (int8_t)status;
-            }
+        for (int o = 8; o; o >>= 1) {
+            const unsigned long long other = __shfl_xor_sync(FULL, worst, o);
+            worst = other > worst ? other : worst;
+        }
+        if (lane < k) place[lane] = my_node;
+        if (cuts && lane < k - 1) cuts[lane] = my_cut;
+        if (lane == 0) {
+            o_beta[inst] = __longlong_as_double((long long)worst);
+            o_m[inst] = m;
+            o_status[inst] = (int8_t)status;
         }
     }
 }

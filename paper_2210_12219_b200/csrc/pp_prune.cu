@@ -119,6 +119,25 @@ constexpr bool kCodes = G * P <= 64 && !CT;
 template <int G, int P>
 constexpr size_t kStripBytes = ((size_t)(Strip<G, P>::kSize + PP_MAX_K) * 4 + 15) & ~(size_t)15;
 
+// Long rows of the first level: a team of four warps to a row, so that no lane has a chain of P divisions and P
+// window minima while most warps of the GPU have no row at all (level of 156 rows of 337 positions, P = 16:
+// 14 300 cycles by one warp a row, 6500 so; 306 rows of 200, P = 8: 6400 and 4200).  Up to two rounds of them; with more rows
+// than that a warp a row keeps the SMs as busy.
+constexpr int kTeam = 128;
+template <int G, int P, bool CT>
+constexpr bool kByTeams = !CT && G == 32 && P >= 8;
+
+// Barrier of a team, and whether any of its threads says so.
+__device__ __forceinline__ bool team_any(int team, bool mine)
+{
+    uint32_t any;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, %2, %3, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                 : "=r"(any)
+                 : "r"((uint32_t)mine), "r"(2 + team), "n"(kTeam)
+                 : "memory");
+    return any != 0u;
+}
+
 // What another block may have written: past L1.  SM: the tables are in shared memory.
 template <bool SM, typename T>
 __device__ __forceinline__ T ld_now(const T *p)
@@ -216,6 +235,11 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
     __shared__ unsigned long long s_low;    // bits of the smallest quotient in the optimum's class
     __shared__ uint32_t s_cnt;
     __shared__ int s_fail;
+    [[maybe_unused]] constexpr int kTeams = kThreads / kTeam, kOwn = (G * P + kTeam - 1) / kTeam;
+    [[maybe_unused]] const int team = tid / kTeam, in_team = tid % kTeam;
+    [[maybe_unused]] uint32_t *team_row =  // two rows, in the strips of the team's warps
+        reinterpret_cast<uint32_t *>(smem_prune + lay.strips + (size_t)team * (kTeam / G) * kStripBytes<G, P>);
+    __shared__ uint32_t s_team[kWarps][2];
     PruneCtl *ctl = d.ctl;
     __shared__ uint32_t s_count[SM ? 64 : 1];
     unsigned char *tables = smem_prune + lay.total;  // SM: in the layout they have in global memory
@@ -259,32 +283,35 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
         if constexpr (kCodes<G, P, CT>) s_code[w * Lp + c] = window_code<G, P, uint32_t>(c, l);
     };
     // window starts: lo[w][c'] = earliest previous cut c >= 0 such that layers c+1..c' fit on w, c' itself when
-    // not even layer c' alone does; a lane takes a run of neighbouring positions, found by bisection for the
-    // first and by stepping on for the others
+    // not even layer c' alone does; by bisection, a lane has four positions of a node in flight (runs of
+    // neighbouring positions, found by stepping on from one to the next: 9300 cycles at k = 13, L = 337)
     if (d.lo)  // a problem that is solved again and again has them on the device
         for (int w = wid; w < k; w += kWarps)
             for (int c = lane; c < Lp; c += 32) set_window(w, c, c < L ? (int)d.lo[w * L + c] : c);
     else
     for (int w = wid; w < k; w += kWarps) {
-        const int run = (Lp + 31) / 32, c0 = lane * run, c1 = min(c0 + run, Lp);
+        constexpr int kU = G * P >= 128 ? 4 : G * P >= 64 ? 2 : 1;
         const unsigned long long capw = s_cap[w];
-        int l = 0;
-        for (int c = c0; c < c1; ++c) {
-            if (c < L) {
-                const unsigned long long need = s_M[c + 1], thr = need > capw ? need - capw : 0ull;
-                if (c == c0) {
-                    int hi = c;  // M[c + 1] >= thr
-                    while (l < hi) {
-                        const int mid = (l + hi) >> 1;
-                        if (s_M[mid + 1] < thr) l = mid + 1; else hi = mid;
-                    }
-                } else {
-                    while (s_M[l + 1] < thr) ++l;
-                }
-            } else {
-                l = c;
+        for (int c0 = lane; c0 < Lp; c0 += 32 * kU) {
+            unsigned long long thr[kU];
+            int l[kU], last[kU];  // l: largest index <= last with M[l] < thr, 0 when there is none
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                last[u] = min(c0 + 32 * u, L - 1);
+                const unsigned long long need = s_M[last[u] + 1];
+                thr[u] = need > capw ? need - capw : 0ull;
+                l[u] = 0;
             }
-            set_window(w, c, l);
+#pragma unroll
+            for (int step = G * P / 2; step; step >>= 1)
+#pragma unroll
+                for (int u = 0; u < kU; ++u)
+                    if (l[u] + step <= last[u] && s_M[l[u] + step] < thr[u]) l[u] += step;
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const int c = c0 + 32 * u;
+                if (c < Lp) set_window(w, c, c < L ? l[u] : c);
+            }
         }
     }
     __syncthreads();
@@ -314,6 +341,17 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
         if (s_M[c + 1] > s_cap[v]) return kInfKey;
         if constexpr (CT) return s_speed[v] ? key_of(__ddiv_rn((double)s_Wp[c + 1], (double)s_speed[v])) : kInfKey;
         return 0u;
+    };
+    // layers 0..c have to hold this much for the nodes outside S2 to hold the rest
+    auto must_hold = [&](uint32_t S2) -> unsigned long long {
+        const uint32_t rest = full & ~S2;
+        double room = s_room[rest & 127u] + s_room[128 + (rest >> 7 & 127u)] + s_room[256 + (rest >> 14)];
+        room *= 1.0 + 1e-9;  // rounding of the sums must not drop a state
+        return room < (double)total ? total - (unsigned long long)room : 0ull;
+    };
+    auto note_final = [&](uint32_t x, int level, uint32_t S2, int w) {
+        const unsigned long long cand = pack_best(x, level, S2, w);
+        if (cand < *reinterpret_cast<volatile unsigned long long *>(&s_best)) atomicMin(&s_best, cand);
     };
     // row of (S2, w) from g: window minimum, then drop what cannot matter, note a final state; returns
     // whether the group keeps the row, and its smallest value
@@ -356,13 +394,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
             }
         }
         const bool tight = (tight_levels >> level) & 1u;
-        unsigned long long must = 0ull;  // layers 0..c have to hold this much for the unused nodes to hold the rest
-        if (tight) {
-            const uint32_t rest = full & ~S2;
-            double room = s_room[rest & 127u] + s_room[128 + (rest >> 7 & 127u)] + s_room[256 + (rest >> 14)];
-            room *= 1.0 + 1e-9;  // rounding of the sums must not drop a state
-            must = room < (double)total ? total - (unsigned long long)room : 0ull;
-        }
+        const unsigned long long must = tight ? must_hold(S2) : 0ull;
         uint32_t least = kInfKey, x = kInfKey;
 #pragma unroll
         for (int i = 0; i < P; ++i) {
@@ -371,10 +403,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
             least = min(least, out[i]);
             if (c == L - 1) x = out[i];
         }
-        if (x != kInfKey) {
-            const unsigned long long cand = pack_best(x, level, S2, w);
-            if (cand < *reinterpret_cast<volatile unsigned long long *>(&s_best)) atomicMin(&s_best, cand);
-        }
+        if (x != kInfKey) note_final(x, level, S2, w);
         rmin = group_min<G>(least);
         return rmin != kInfKey;
     };
@@ -443,7 +472,101 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
         if (top >= 2) {
             const unsigned long long before = s_best;
             const int items = k * (k - 1);
-            for (int base = my_slot * kPerWarp; base < items; base += slots * kPerWarp) {
+            bool by_teams = false;
+            if constexpr (kByTeams<G, P, CT>) {
+                by_teams = items <= 2 * nblk * kTeams;
+                if (by_teams) {
+                    for (int it = team * nblk + (nblk == 1 ? 0 : (int)blockIdx.x); it < items; it += nblk * kTeams) {
+                        const int v = it / (k - 1), o = it - v * (k - 1), w = o + (o >= v ? 1 : 0);
+                        const uint32_t link = s_bw[v * k + w], S2 = (1u << v) | (1u << w);
+                        const double div = (double)link;
+                        uint32_t x[kOwn], out[kOwn], gm = kInfKey, least = kInfKey;
+                        int lo[kOwn], t[kOwn];  // t: log2 of the window's length, -1: no window
+#pragma unroll
+                        for (int q = 0; q < kOwn; ++q) {
+                            const int c = in_team + q * kTeam;
+                            uint32_t key = kInfKey;
+                            x[q] = out[q] = kInfKey;
+                            lo[q] = 0;
+                            t[q] = -1;
+                            if (c < L) {
+                                if (link != 0) key = key_of(__ddiv_rn(s_bits[c], div));
+                                if (c < L - 1) gm = min(gm, key);
+                                x[q] = max(key, base_key(v, c));
+                                lo[q] = s_lo[w * Lp + c];
+                                if (lo[q] < c) t[q] = 31 - __clz(c - lo[q]);
+                            }
+                            if (c < Lp) {
+                                t_gam[(size_t)(w * k + v) * Lp + c] = key;
+                                team_row[c] = x[q];
+                            }
+                        }
+                        // sparse table of the row, one level at a time: out = min over [lo, c - 1]
+                        uint32_t *cur = team_row, *next = team_row + Lp;
+                        for (int s = 0;; ++s) {
+                            bool more = false;
+#pragma unroll
+                            for (int q = 0; q < kOwn; ++q) more |= t[q] > s;
+                            more = team_any(team, more);
+#pragma unroll
+                            for (int q = 0; q < kOwn; ++q)
+                                if (t[q] == s) out[q] = min(cur[in_team + q * kTeam - 1], cur[lo[q] + (1 << s) - 1]);
+                            if (!more) break;
+#pragma unroll
+                            for (int q = 0; q < kOwn; ++q) {
+                                const int c = in_team + q * kTeam;
+                                if (c < Lp) {
+                                    if (c >= 1 << s) x[q] = min(x[q], cur[c - (1 << s)]);
+                                    next[c] = x[q];
+                                }
+                            }
+                            uint32_t *const swap = cur;
+                            cur = next;
+                            next = swap;
+                        }
+                        const uint32_t lim = limit_of(*reinterpret_cast<volatile unsigned long long *>(&s_best), 2);
+                        const bool tight = (tight_levels >> 2) & 1u;
+                        const unsigned long long must = tight ? must_hold(S2) : 0ull;
+#pragma unroll
+                        for (int q = 0; q < kOwn; ++q) {
+                            const int c = in_team + q * kTeam;
+                            if (out[q] >= lim || c >= L || (tight && s_M[c + 1] < must)) out[q] = kInfKey;
+                            least = min(least, out[q]);
+                            if (c == L - 1 && out[q] != kInfKey) note_final(out[q], 2, S2, w);
+                        }
+                        least = __reduce_min_sync(kFull, least);
+                        gm = __reduce_min_sync(kFull, gm);
+                        if (lane == 0) {
+                            s_team[wid][0] = least;
+                            s_team[wid][1] = gm;
+                        }
+                        team_any(team, false);
+#pragma unroll
+                        for (int i = 0; i < kTeam / 32; ++i) {
+                            least = min(least, s_team[team * (kTeam / 32) + i][0]);
+                            gm = min(gm, s_team[team * (kTeam / 32) + i][1]);
+                        }
+                        const int a = v < w ? v : w, b = v < w ? w : v;
+                        const int pr = a * (2 * k - a - 1) / 2 + (b - a - 1);
+                        const uint32_t id = 2u * (uint32_t)pr + (w == b ? 1u : 0u);
+                        if (least != kInfKey)
+#pragma unroll
+                            for (int q = 0; q < kOwn; ++q) {
+                                const int c = in_team + q * kTeam;
+                                if (c < Lp) t_rows[(size_t)id * Lp + c] = out[q];
+                            }
+                        if (in_team == 0) {
+                            t_gmin[w * k + v] = gm;
+                            t_rowmap[(size_t)S2 * k + w] = ((unsigned long long)least << 32) | id;
+                            if (w == b) {
+                                t_list[pr] = S2;
+                                t_live[S2] = S2;
+                            }
+                        }
+                    }
+                }
+            }
+            for (int base = by_teams ? items : my_slot * kPerWarp; base < items; base += slots * kPerWarp) {
                 const int it = base + lane / G;
                 const bool on = it < items;
                 const int v = on ? it / (k - 1) : 0, x = on ? it - v * (k - 1) : 0, w = x + (x >= v ? 1 : 0);
@@ -581,7 +704,6 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
         int w = (int)best & 31, c2 = L - 1;
         if (tid < PP_MAX_K) s_cut[tid] = s_node[tid] = -1;
         if (tid == 0) {
-            s_worst = 0ull;
             s_low = ~0ull;
             s_fail = 0;
         }
@@ -682,15 +804,23 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
             break;
         }
         // the plan's own bottleneck
-        if (tid < m) {
+        if (wid == 0) {
             double x = 0.0;
             if (tid < m - 1) x = __ddiv_rn(s_bits[s_cut[tid]], (double)s_bw[s_node[tid] * k + s_node[tid + 1]]);
             if constexpr (CT) {
-                const int first = tid ? s_cut[tid - 1] + 1 : 0, last = tid < m - 1 ? s_cut[tid] : L - 1;
-                const double y = __ddiv_rn((double)(s_Wp[last + 1] - s_Wp[first]), (double)s_speed[s_node[tid]]);
-                x = y > x ? y : x;
+                if (tid < m) {
+                    const int first = tid ? s_cut[tid - 1] + 1 : 0, last = tid < m - 1 ? s_cut[tid] : L - 1;
+                    const double y = __ddiv_rn((double)(s_Wp[last + 1] - s_Wp[first]), (double)s_speed[s_node[tid]]);
+                    x = y > x ? y : x;
+                }
             }
-            atomicMax(&s_worst, (unsigned long long)__double_as_longlong(x));
+            unsigned long long bits = (unsigned long long)__double_as_longlong(x);
+#pragma unroll
+            for (int o = 16; o; o >>= 1) {
+                const unsigned long long other = __shfl_xor_sync(kFull, bits, o);
+                bits = other > bits ? other : bits;
+            }
+            if (tid == 0) s_worst = bits;
         }
         __syncthreads();
         const unsigned long long worst = s_worst;

@@ -142,9 +142,10 @@ cudaError_t launch_batch_lanes(int64_t B, int L, int k, const uint64_t *bits, co
 // The search as a bounded sparse frontier (pp_prune.cu), one launch per solve.
 struct PruneCtl {              // device; the kernel leaves it as it found it
     unsigned long long best;   // best final state of the levels done: pack_best of its key
-    uint32_t count[64];        // node sets appended to the frontier by the level of that many nodes (a second
-                               // search over the class of the optimum counts from 32)
-    uint32_t arrived, left;    // barrier arrivals; blocks that have left
+    unsigned long long count[64];  // node sets appended to the frontier by the level of that many nodes (a second
+                               // search over the class of the optimum counts from 32); in the upper half the
+                               // blocks that have arrived at the level's end
+    uint32_t left;             // blocks that have left
     uint32_t failed;           // a barrier ran out of polls
     uint32_t dense;            // 1 = the frontier outgrew its rows
 };

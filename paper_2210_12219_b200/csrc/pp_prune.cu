@@ -172,19 +172,24 @@ __device__ __forceinline__ void store_row(uint32_t *p, const uint32_t (&x)[P])
     }
 }
 
-// All blocks of the grid; false when the wait ran out (the caller returns).
-__device__ __forceinline__ bool grid_barrier(PruneCtl *ctl, uint32_t target)
+// All blocks of the grid; false when the wait ran out (the caller returns).  A level's word holds the blocks
+// that have arrived above the node sets it added (32 bits each), so that the last poll brings both; *best,
+// polled along, may miss what the last blocks found, which only makes it a weaker bound.  (Reading both after
+// the barrier cost another trip to L2, 600 cycles a level: k = 16, L = 136 28.7 -> 26.8 us, k = 10, L = 50 48.8 -> 47.9.)
+__device__ __forceinline__ bool grid_barrier(PruneCtl *ctl, unsigned long long *word, unsigned long long *best, uint32_t *added)
 {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        uint32_t seen;
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&ctl->arrived) : "memory");
+        unsigned long long seen;
+        asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(word), "l"(1ull << 32) : "memory");
         int spins = 0;
         do {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&ctl->arrived) : "memory");
-        } while (seen < target && ++spins < kSpinLimit);
-        s_ok = seen >= target;
+            asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(*best) : "l"(&ctl->best) : "memory");
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(seen) : "l"(word) : "memory");
+        } while ((uint32_t)(seen >> 32) < gridDim.x && ++spins < kSpinLimit);
+        *added = (uint32_t)seen;
+        s_ok = (uint32_t)(seen >> 32) >= gridDim.x;
         if (!s_ok) ctl->failed = 1;
     }
     __syncthreads();
@@ -331,7 +336,6 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
 
     KeyMap key_of{d.key_base, d.key_shift, 0u};
     bool dense = false;
-    uint32_t barriers = 0;
     int nblk = SM ? 1 : (int)gridDim.x;  // blocks that work on the search: 1 once block 0 goes on alone
     int m = 0, w_end = 0, status = (int)PP_INFEASIBLE;
     double beta = kInf;
@@ -409,24 +413,28 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
     };
     // end of a level: the block's best final state goes to the others; false = a barrier gave up
     // and s_cnt has the node sets it added to the frontier
-    auto level_end = [&](unsigned long long best_before, const uint32_t *added) -> bool {
+    auto level_end = [&](unsigned long long best_before, int level) -> bool {
         __syncthreads();
         if (nblk == 1) {
-            if (tid == 0 && added) s_cnt = ld_now<SM>(added);
+            if (tid == 0) s_cnt = SM ? s_count[(key_of.zoom ? 32 : 0) + level] : (uint32_t)__ldcg(ctl->count + (key_of.zoom ? 32 : 0) + level);
             __syncthreads();
             return true;
         }
         if (tid == 0 && s_best < best_before)
             asm volatile("red.relaxed.gpu.global.min.u64 [%0], %1;" ::"l"(&ctl->best), "l"(s_best) : "memory");
+        unsigned long long seen = kNoBest;
+        uint32_t added = 0;
         if (d.clustered) {
             asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-        } else {
-            barriers += gridDim.x;
-            if (!grid_barrier(ctl, barriers)) return false;
+            if (tid == 0) {
+                seen = __ldcg(&ctl->best);
+                added = (uint32_t)__ldcg(ctl->count + level);
+            }
+        } else if (!grid_barrier(ctl, ctl->count + level, &seen, &added)) {
+            return false;
         }
         if (tid == 0) {
-            const unsigned long long seen = __ldcg(&ctl->best);
-            if (added) s_cnt = __ldcg(added);
+            s_cnt = added;
             if (seen < s_best) s_best = seen;
         }
         __syncthreads();
@@ -444,12 +452,16 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
             s_node[tid] = tid == 0 ? w_end : -1;
         }
     }
+    auto next_place = [&](int level) -> uint32_t {  // of a level's node sets in the frontier
+        const int at = (key_of.zoom ? 32 : 0) + level;
+        if constexpr (SM) return atomicAdd(&s_count[at], 1u);
+        else return (uint32_t)atomicAdd(ctl->count + at, 1ull);
+    };
     while (!found) {
         const int slots = nblk * kWarps, my_slot = wid * nblk + (nblk == 1 ? 0 : (int)blockIdx.x);
         // node sets of three nodes and more start without rows (those of two nodes are all written below)
         for (uint32_t S = (nblk == 1 ? 0 : blockIdx.x) * kThreads + tid; S < (1u << k); S += nblk * kThreads)
             if (__popc(S) > 2) t_live[S] = 0u;
-        uint32_t *const count = (SM ? s_count : ctl->count) + (key_of.zoom ? 32 : 0);
         if constexpr (CT) {
             // compute times of every run of layers: seg[(w * L + d) * Lp + c'] = layers c'-d .. c' on w
             const int n = k * L * Lp;
@@ -466,7 +478,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                     const uint32_t x = base_key(v, L - 1);
                     if (x != kInfKey) s_best = min(s_best, pack_best(x, 1, 1u << v, v));
                 }
-            if (!level_end(kNoBest, nullptr)) return;
+            if (!level_end(kNoBest, 1)) return;
         }
         // ---- two nodes: the keys of every link, the rows of every pair ----
         if (top >= 2) {
@@ -603,7 +615,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                 }
                 __syncwarp();
             }
-            if (!level_end(before, nullptr)) return;
+            if (!level_end(before, 2)) return;
             for (int e = tid; e < k * k; e += kThreads) s_gmin[e] = (e / k != e % k) ? ld_now<SM>(t_gmin + e) : kInfKey;
             __syncthreads();
         }
@@ -681,17 +693,18 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                     if (sl == 0) {
                         t_rowmap[(size_t)S2 * k + w] = ((unsigned long long)rmin << 32) | id;
                         if (atomicOr(t_live + S2, 1u << w) == 0u)
-                            t_list[beg + cnt + atomicAdd(&count[level], 1u)] = S2;
+                            t_list[beg + cnt + next_place(level)] = S2;
                     }
                 }
                 __syncwarp();
             }
             used += items;
-            if (!level_end(before, &count[level])) return;
+            if (!level_end(before, level)) return;
             beg += cnt;
             cnt = s_cnt;
         }
         if (blockIdx.x != 0 || dense) break;  // block 0 finishes
+        if (!SM && tid == 0 && gridDim.x > 1 && !d.clustered && !key_of.zoom) s_best = min(s_best, __ldcg(&ctl->best));
         __syncthreads();
         const unsigned long long best = s_best;
         if (best == kNoBest) break;  // no plan
@@ -863,10 +876,9 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
     }
     __syncthreads();
     if (s_left == gridDim.x - 1) {
-        if (tid < 64) ctl->count[tid] = 0u;
+        if (tid < 64) ctl->count[tid] = 0ull;
         if (tid == 0) {
             ctl->best = kNoBest;
-            ctl->arrived = 0u;
             ctl->left = 0u;
         }
     }

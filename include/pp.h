@@ -200,7 +200,8 @@ pp_status pp_eval_plans_packed_dev(pp_problem *p, int64_t B, int64_t total, cons
  * Otherwise one thread block solves one instance with its whole state table in shared memory.
  * Returns PP_ERR_LIMIT without touching outputs when the instance shape does not fit one block:
  * k > 12, k*(k-1)*L + 1 > 65534 (ranks are 16-bit), or k * 2^(k-1) * L 16-bit states plus the
- * rank tables beyond the shared memory of a block (k = 8, L = 24 needs 73 KB).  Host variant is
+ * rank tables beyond the shared memory of a block (k = 8, L = 24 needs 62 KB).  The host variant works on a
+ * batch of up to 1 MB where it lies in page-locked memory, larger ones go through device memory; it is
  * synchronous and uses the legacy default stream; the _dev variant takes device pointers and a
  * stream and is asynchronous.  cuts may be NULL when k == 1.
  */

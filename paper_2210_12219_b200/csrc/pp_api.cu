@@ -50,6 +50,7 @@ struct pp_problem {
     std::vector<int16_t> pair_u;
     unsigned char *d_dense = nullptr;
     unsigned char *d_tables = nullptr;  // PlanTables, made by the first call that scores or draws plans
+    bool tables_read = false;           // a launch has been ordered behind the one that makes them
     Dev d{};
     int sweep_launches = 0, total_launches = 0, fast_used = 0, pair_levels = 0;
     std::vector<signed char> pair_lvl;  // per level: 1 = two-mask kernel, 0 = one-mask, -1 = not decided yet
@@ -389,6 +390,15 @@ pp_status upload_inputs(pp_problem *p, bool wait)
     else PP_CUDA(cudaMemcpyAsync(p->d_inputs, st.data(), st.size(), cudaMemcpyHostToDevice, p->stream));
     p->uploaded = true;
     return PP_OK;
+}
+
+// Whether a launch over n plans may start before the one in front of it has ended: the one that makes the
+// tables is not that one.
+bool early(pp_problem *p, int64_t n)
+{
+    const bool was = p->tables_read;
+    p->tables_read = was || n > 0;
+    return was;
 }
 
 pp_status ensure_tables(pp_problem *p)
@@ -1022,7 +1032,7 @@ pp_status pp_eval_plans_dev(pp_problem *p, int64_t B, const uint8_t *nseg, const
     if (!nseg || !ends || !nodes || !beta_ms || !plan_status) return PP_ERR_ARG;
     pp_status st = ensure_tables(p);
     if (st != PP_OK) return st;
-    PP_CUDA(launch_eval(p->d, p->d_tables, B, nseg, ends, nodes, beta_ms, plan_status, p->stream));
+    PP_CUDA(launch_eval(p->d, p->d_tables, B, nseg, ends, nodes, beta_ms, plan_status, early(p, B), p->stream));
     return PP_OK;
 }
 
@@ -1048,7 +1058,7 @@ pp_status pp_eval_plans(pp_problem *p, int64_t B, const uint8_t *nseg, const int
     if (e == cudaSuccess)
         e = launch_eval(p->d, p->d_tables, B, buf, reinterpret_cast<int32_t *>(buf + o_ends),
                         reinterpret_cast<int32_t *>(buf + o_nodes),
-                        reinterpret_cast<double *>(buf + o_beta), buf + o_st, s);
+                        reinterpret_cast<double *>(buf + o_beta), buf + o_st, early(p, B), s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(beta_ms, buf + o_beta, b_beta, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(plan_status, buf + o_st, (size_t)B, cudaMemcpyDeviceToHost, s);
     cudaFreeAsync(buf, s);
@@ -1066,7 +1076,7 @@ pp_status pp_eval_plans_packed_dev(pp_problem *p, int64_t B, int64_t total, cons
     if (!nseg || !plan_off || !beta_ms || !plan_status || ((!ends || !nodes) && total > 0)) return PP_ERR_ARG;
     pp_status st = ensure_tables(p);
     if (st != PP_OK) return st;
-    PP_CUDA(launch_eval_packed(p->d, p->d_tables, B, total, nseg, plan_off, ends, nodes, beta_ms, plan_status, p->stream));
+    PP_CUDA(launch_eval_packed(p->d, p->d_tables, B, total, nseg, plan_off, ends, nodes, beta_ms, plan_status, early(p, B), p->stream));
     return PP_OK;
 }
 
@@ -1093,7 +1103,7 @@ pp_status pp_eval_plans_packed(pp_problem *p, int64_t B, int64_t total, const ui
     if (e == cudaSuccess)
         e = launch_eval_packed(p->d, p->d_tables, B, total, buf, reinterpret_cast<uint32_t *>(buf + o_off),
                                reinterpret_cast<uint16_t *>(buf + o_ends), buf + o_nodes,
-                               reinterpret_cast<double *>(buf + o_beta), buf + o_st, s);
+                               reinterpret_cast<double *>(buf + o_beta), buf + o_st, early(p, B), s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(beta_ms, buf + o_beta, nB * 8, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(plan_status, buf + o_st, nB, cudaMemcpyDeviceToHost, s);
     cudaFreeAsync(buf, s);
@@ -1110,7 +1120,7 @@ pp_status pp_random_plans_dev(pp_problem *p, int64_t P, const uint32_t *draws, u
     if (!draws || !nseg || !ends || !nodes) return PP_ERR_ARG;
     pp_status st = ensure_tables(p);
     if (st != PP_OK) return st;
-    PP_CUDA(launch_random_plans(p->d, p->d_tables, P, draws, nseg, ends, nodes, p->stream));
+    PP_CUDA(launch_random_plans(p->d, p->d_tables, P, draws, nseg, ends, nodes, early(p, P), p->stream));
     return PP_OK;
 }
 
@@ -1133,7 +1143,7 @@ pp_status pp_random_plans(pp_problem *p, int64_t P, const uint32_t *draws, uint8
     if (e == cudaSuccess)
         e = launch_random_plans(p->d, p->d_tables, P, reinterpret_cast<uint32_t *>(buf), buf + o_nseg,
                                 reinterpret_cast<int32_t *>(buf + o_ends),
-                                reinterpret_cast<int32_t *>(buf + o_nodes), s);
+                                reinterpret_cast<int32_t *>(buf + o_nodes), early(p, P), s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(nseg, buf + o_nseg, (size_t)P, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(ends, buf + o_ends, b_rows, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(nodes, buf + o_nodes, b_rows, cudaMemcpyDeviceToHost, s);

@@ -13,7 +13,7 @@
 // is one look into the table of forward windows.  One pass over a row collects all
 // flags; an index that is out of range reads a padding entry and has raised its flag already.
 // 262 144 compressed plans of k = 18, L = 200, a queued call: 21.7 us with a thread to a plan as they come, a division
-// a cut and the row read along the way, 11.9 so.  256 threads, five blocks per SM: 128 or 512 threads, four, six or
+// a cut and the row read along the way, 11.9 so, 11.4 with the tables fetched while the launch in front runs out.  256 threads, five blocks per SM: 128 or 512 threads, four, six or
 // seven blocks 12.0 to 13.8.
 #include "pp_internal.cuh"
 
@@ -63,9 +63,6 @@ k_eval(const int L, const int k, const unsigned char *__restrict__ tables, const
     __shared__ uint32_t s_start[kEvalThreads];  // PACKED: first entry of the row within the staged stretch, or kFar
     __shared__ uint32_t s_first[2][32];
     constexpr uint32_t kFar = 0xFFFFFFFFu;
-    // launched as a dependent of whatever writes the plans (or the tables): only now is it complete
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;");
     const int mmax = k < L ? k : L;
     const double kInf = __longlong_as_double(0x7FF0000000000000ll);
     // what a batch needs to know before its rows can be fetched; asked for one batch ahead
@@ -86,10 +83,14 @@ k_eval(const int L, const int k, const unsigned char *__restrict__ tables, const
             }
         }
     };
-    look_ahead((int64_t)blockIdx.x * kEvalThreads);
     if (tid < 32) s_first[0][tid] = s_first[1][tid] = 0u;
     for (int i = tid; i < (int)(tab.total / 16); i += kEvalThreads)
         reinterpret_cast<uint4 *>(smem_eval)[i] = reinterpret_cast<const uint4 *>(tables)[i];
+    // launched as a dependent of whatever writes the plans: only now is it complete (the tables are
+    // older than that, see launch_eval)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    look_ahead((int64_t)blockIdx.x * kEvalThreads);
     int turn = 0;
     for (int64_t base = (int64_t)blockIdx.x * kEvalThreads; base < B; base += (int64_t)gridDim.x * kEvalThreads, turn ^= 1) {
         const int rows = B - base < kEvalThreads ? (int)(B - base) : kEvalThreads;
@@ -235,7 +236,7 @@ __global__ void k_plan_tables(const Dev d, unsigned char *out)
 
 template <bool PACKED, typename E, typename N>
 cudaError_t launch(const Dev &d, const unsigned char *tables, int64_t B, int64_t total, const uint8_t *nseg, const uint32_t *off, const E *ends,
-                   const N *nodes, double *beta, uint8_t *status, cudaStream_t s)
+                   const N *nodes, double *beta, uint8_t *status, bool early, cudaStream_t s)
 {
     if (B <= 0) return cudaSuccess;
     cudaError_t e = cudaFuncSetAttribute(k_eval<PACKED, E, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
@@ -252,7 +253,7 @@ cudaError_t launch(const Dev &d, const unsigned char *tables, int64_t B, int64_t
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, k_eval<PACKED, E, N>, d.L, d.k, tables, B, total, nseg, off, ends, nodes, beta, status);
 }
 
@@ -266,15 +267,15 @@ cudaError_t launch_plan_tables(const Dev &d, unsigned char *out, cudaStream_t s)
 
 cudaError_t launch_eval_packed(const Dev &d, const unsigned char *tables, int64_t B, int64_t total, const uint8_t *nseg, const uint32_t *off,
                                const uint16_t *ends, const uint8_t *nodes, double *beta, uint8_t *status,
-                               cudaStream_t s)
+                               bool early, cudaStream_t s)
 {
-    return launch<true>(d, tables, B, total, nseg, off, ends, nodes, beta, status, s);
+    return launch<true>(d, tables, B, total, nseg, off, ends, nodes, beta, status, early, s);
 }
 
 cudaError_t launch_eval(const Dev &d, const unsigned char *tables, int64_t B, const uint8_t *nseg, const int32_t *ends,
-                        const int32_t *nodes, double *beta, uint8_t *status, cudaStream_t s)
+                        const int32_t *nodes, double *beta, uint8_t *status, bool early, cudaStream_t s)
 {
-    return launch<false>(d, tables, B, 0, nseg, static_cast<const uint32_t *>(nullptr), ends, nodes, beta, status, s);
+    return launch<false>(d, tables, B, 0, nseg, static_cast<const uint32_t *>(nullptr), ends, nodes, beta, status, early, s);
 }
 
 }  // namespace pp

@@ -96,11 +96,13 @@ __host__ __device__ inline PlanTables plan_tables(int L, int k)
     return t;
 }
 cudaError_t launch_plan_tables(const Dev &d, unsigned char *out, cudaStream_t s);
+// early: the launch may start before the one in front of it on the stream has ended, and reads the tables at once.
+// Not for the first launch after launch_plan_tables.
 cudaError_t launch_eval(const Dev &d, const unsigned char *tables, int64_t B, const uint8_t *nseg, const int32_t *ends,
-                        const int32_t *nodes, double *beta, uint8_t *status, cudaStream_t s);
+                        const int32_t *nodes, double *beta, uint8_t *status, bool early, cudaStream_t s);
 cudaError_t launch_eval_packed(const Dev &d, const unsigned char *tables, int64_t B, int64_t total, const uint8_t *nseg, const uint32_t *off,
                                const uint16_t *ends, const uint8_t *nodes, double *beta, uint8_t *status,
-                               cudaStream_t s);
+                               bool early, cudaStream_t s);
 size_t batch_smem_bytes(int L, int k);
 // Row numbering of the batched search, per (device, k): rows ordered by (popcount, mask, node), the masks
 // listed by (popcount, value) with the first of each popcount, source mask | target node << 16 of every row
@@ -205,7 +207,7 @@ struct PruneHost {             // host arrays, read before launch_prune returns
 cudaError_t launch_prune(const PruneDev &d, const PruneHost &h, int sms, cudaStream_t s);
 // Random comparison baseline (Section 4): P plans of problem d from 2 k draws each.
 cudaError_t launch_random_plans(const Dev &d, const unsigned char *tables, int64_t P, const uint32_t *draws, uint8_t *nseg,
-                                int32_t *ends, int32_t *nodes, cudaStream_t s);
+                                int32_t *ends, int32_t *nodes, bool early, cudaStream_t s);
 // Greedy comparison baseline (Section 4), one warp per instance.
 cudaError_t launch_greedy(int64_t B, int L, int k, const uint64_t *bits, const uint64_t *mem,
                           const uint64_t *cap, const uint32_t *bw, double *beta, int32_t *m, int32_t *cuts,

@@ -32,7 +32,9 @@ k_random_plans(const int L, const int k, const uint16_t *__restrict__ fwd, const
     const int stride = k | 1, tid = threadIdx.x;
     uint2 *sd = smem_pairs;  // [threads][stride]: draws in, (cut, node) pairs out
     uint16_t *s_fwd = reinterpret_cast<uint16_t *>(smem_pairs + kRandomThreads * stride);  // [k][L]
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // whatever wrote fwd, or reads or writes the plans, is complete
+    for (int i = tid; i < k * L; i += kRandomThreads) s_fwd[i] = fwd[i];
+    // whatever wrote the draws, or reads or writes the plans, is complete (fwd is older, see launch_eval)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
     const int64_t p0 = (int64_t)blockIdx.x * kRandomThreads;
     const int np = P - p0 < kRandomThreads ? (int)(P - p0) : kRandomThreads;
@@ -50,7 +52,6 @@ k_random_plans(const int L, const int k, const uint16_t *__restrict__ fwd, const
             if (c >= k) { c -= k; at += carry; }
         }
     }
-    for (int i = tid; i < k * L; i += kRandomThreads) s_fwd[i] = fwd[i];
     __syncthreads();
     if (tid < np) {
         uint2 *row = sd + tid * stride;
@@ -92,7 +93,7 @@ k_random_plans(const int L, const int k, const uint16_t *__restrict__ fwd, const
 }
 
 cudaError_t launch_random_plans(const Dev &d, const unsigned char *tables, int64_t P, const uint32_t *draws, uint8_t *nseg,
-                                int32_t *ends, int32_t *nodes, cudaStream_t s)
+                                int32_t *ends, int32_t *nodes, bool early, cudaStream_t s)
 {
     const int64_t blocks = (P + kRandomThreads - 1) / kRandomThreads;
     if (blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
@@ -108,7 +109,7 @@ cudaError_t launch_random_plans(const Dev &d, const unsigned char *tables, int64
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, k_random_plans, d.L, d.k, reinterpret_cast<const uint16_t *>(tables + plan_tables(d.L, d.k).fwd), P, draws, nseg, ends, nodes);
 }
 

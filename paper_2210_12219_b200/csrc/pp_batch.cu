@@ -109,6 +109,8 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
         const uint64_t *__restrict__ g_cap, const uint32_t *__restrict__ g_bw, double *__restrict__ o_beta,
         int32_t *__restrict__ o_m, int32_t *__restrict__ o_cuts, int32_t *__restrict__ o_place, int8_t *__restrict__ o_status)
 {
+    // The next piece of a batch that is launched in pieces shares nothing with this one and may start beside it.
+    asm volatile("griddepcontrol.launch_dependents;");
     constexpr int kGroups = kBatchThreads / G;
     extern __shared__ __align__(16) unsigned char smem[];
     const BatchLayout lay = batch_layout(L, k);
@@ -410,34 +412,44 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
             o_status[inst] = (int8_t)status;
         }
     }
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // no launch is complete before the one in front of it
 }
 
 template <int G, int P>
 cudaError_t launch_shape(int64_t B, int L, int k, const LaneTables &lt, int sms, const uint64_t *bits, const uint64_t *mem,
                          const uint64_t *cap, const uint32_t *bw, double *beta, int32_t *m, int32_t *cuts,
-                         int32_t *placement, int8_t *status, cudaStream_t s)
+                         int32_t *placement, int8_t *status, bool early, cudaStream_t s)
 {
     const size_t sm = batch_smem_bytes(L, k);
     cudaError_t e = cudaFuncSetAttribute(k_batch<G, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     // a block per instance while they fit a few rounds of the GPU; beyond that blocks take several in turn
     const int64_t grid = std::min<int64_t>(B, (int64_t)sms * 16);
-    k_batch<G, P><<<(unsigned)grid, kBatchThreads, sm, s>>>(B, L, k, lt.rowoff, lt.rows, lt.first, bits, mem, cap, bw, beta, m,
-                                                            cuts, placement, status);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kBatchThreads);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k_batch<G, P>, B, L, k, lt.rowoff, lt.rows, lt.first, bits, mem, cap, bw, beta, m, cuts,
+                              placement, status);
 }
 
 }  // namespace
 
 cudaError_t launch_batch(int64_t B, int L, int k, const LaneTables &lt, int sms, const uint64_t *bits, const uint64_t *mem,
                          const uint64_t *cap, const uint32_t *bw, double *beta, int32_t *m, int32_t *cuts,
-                         int32_t *placement, int8_t *status, cudaStream_t s)
+                         int32_t *placement, int8_t *status, bool early, cudaStream_t s)
 {
     if (B <= 0) return cudaSuccess;
     const BatchShape sh = batch_shape(L);
     switch (sh.G * 100 + sh.P) {
 #define PP_CASE(g, p) \
-    case g * 100 + p: return launch_shape<g, p>(B, L, k, lt, sms, bits, mem, cap, bw, beta, m, cuts, placement, status, s);
+    case g * 100 + p: return launch_shape<g, p>(B, L, k, lt, sms, bits, mem, cap, bw, beta, m, cuts, placement, status, early, s);
         PP_CASE(4, 4) PP_CASE(8, 4) PP_CASE(16, 4) PP_CASE(32, 4) PP_CASE(32, 8) PP_CASE(32, 16) PP_CASE(32, 32)
 #undef PP_CASE
     }

@@ -110,9 +110,10 @@ size_t batch_smem_bytes(int L, int k);
 struct LaneTables {
     const uint32_t *rowoff = nullptr, *mlist = nullptr, *moff = nullptr, *rows = nullptr, *first = nullptr;
 };
+// early: may start beside the launch in front of it on the stream, which is a piece of the same batch.
 cudaError_t launch_batch(int64_t B, int L, int k, const LaneTables &lt, int sms, const uint64_t *bits, const uint64_t *mem,
                          const uint64_t *cap, const uint32_t *bw, double *beta, int32_t *m,
-                         int32_t *cuts, int32_t *placement, int8_t *status, cudaStream_t s);
+                         int32_t *cuts, int32_t *placement, int8_t *status, bool early, cudaStream_t s);
 // Many-instance search with one instance per lane (pp_batch_lanes.cu): tables of a chunk of
 // instances in global memory, instance-minor in pieces of two words, so that the 32 lanes of a warp read
 // 256 neighbouring bytes.  Group g holds instances 32 g .. 32 g + 31 of the chunk.

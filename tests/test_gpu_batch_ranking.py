@@ -66,3 +66,23 @@ def test_block_per_instance_shapes(L, k):
         want = oracle.dp_naive(inst)
         assert got.status[b] == want.status and got.plan(b) == want.plan(), (L, k, b)
         assert got.beta_ms[b] == want.beta_ms or np.isinf(want.beta_ms), (L, k, b)
+
+
+@pytest.mark.parametrize("B", [395, 396, 800])
+def test_host_batch_in_pieces(B):
+    """A host batch that is launched in pieces (two or more from 256 KB of inputs on) gives what small ones give."""
+    build.build()
+    L, k = 40, 4
+    insts = [W.random_small(99000 + i % 97, L, k) for i in range(B)]
+    cap = [np.ceil(i.node_mem_bytes * (1.4 * float(i.layer_mem_bytes.sum()) / float(i.node_mem_bytes.sum()))).astype(np.uint64)
+           for i in insts]
+    arrays = (np.stack([i.layer_out_bits for i in insts]), np.stack([i.layer_mem_bytes for i in insts]), np.stack(cap),
+              np.stack([i.bw_kbps for i in insts]))
+    got = pp.solve_exact_batch(L, k, *arrays)
+    for b in range(0, B, 97):  # the instances repeat after 97
+        n = min(97, B - b)
+        part = pp.solve_exact_batch(L, k, *(a[:n] for a in arrays))
+        for x, y in zip((got.beta_ms, got.m, got.cuts, got.placement, got.status),
+                        (part.beta_ms, part.m, part.cuts, part.placement, part.status)):
+            assert np.array_equal(x[b:b + n], y)
+    assert (got.status == pp.PP_OK).any()

@@ -12,9 +12,9 @@
 // one division at the end gives the largest of the rounded quotients.  Whether a segment fits its node
 // is one look into the table of forward windows.  One pass over a row collects all
 // flags; an index that is out of range reads a padding entry and has raised its flag already.
-// 262 144 compressed plans of k = 18, L = 200, a queued call: 21.7 us with a thread to a plan as they come, a division
-// a cut and the row read along the way, 11.9 so, 11.4 with the tables fetched while the launch in front runs out.  256 threads, five blocks per SM: 128 or 512 threads, four, six or
-// seven blocks 12.0 to 13.8.
+// 262 144 compressed plans of k = 18, L = 200, a queued call: 21.7 us with a thread to a plan as they come, a
+// division a cut and the row read along the way, 11.9 so, 11.4 with the tables fetched while the launch in
+// front runs out.  256 threads, five blocks per SM: 128 or 512 threads, four, six or seven blocks 12.0 to 13.8.
 #include "pp_internal.cuh"
 
 namespace pp {

@@ -69,7 +69,8 @@ typedef enum {
 /* Result record of the exact search as the device writes it. */
 typedef struct {
     double beta_ms;              /* beta*, +inf if infeasible */
-    int32_t status;              /* PP_OK or PP_INFEASIBLE; PP_ERR_CUDA when the backtrack broke off */
+    int32_t status;              /* PP_OK or PP_INFEASIBLE; PP_ERR_CUDA when the backtrack broke off or the
+                                    blocks' wait for one another ran out */
     int32_t m;                   /* number of segments, 0 if infeasible */
     int32_t cuts[PP_MAX_K];      /* e_1 .. e_{m-1}; unused slots are -1 */
     int32_t placement[PP_MAX_K]; /* n_1 .. n_m;     unused slots are -1 */
@@ -400,6 +401,12 @@ pp_status pp_debug_minmax_rate(int32_t op, int32_t iters, double *warp_instr_per
  * PP_ERR_NOMEM come back from pp_problem_create, pp_solve_exact and the host-pointer entry points on
  * a device that has memory to spare. */
 pp_status pp_debug_fail_alloc(int32_t nth);
+
+/* Test hook: the next launch whose blocks wait for one another (a bounded search spread over the GPU, the
+ * placement stage) waits for one block more than it has and gives up after `polls` polls; 0 clears a
+ * pending request.  Lets a test see what a search whose wait runs out reports, and that the one after
+ * it is sound. */
+pp_status pp_debug_starve(int32_t polls);
 
 /* Force (1) or forbid (0) the generic sweep kernel; 2 = automatic choice among the kernels that
  * take one source mask per warp (the two-mask kernel is left out); 3 = the two-mask kernel on every

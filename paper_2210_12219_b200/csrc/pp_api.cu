@@ -110,6 +110,9 @@ bool alloc_should_fail()
     return c == 1;
 }
 
+// Test hook (pp_debug_starve).
+std::atomic<int> g_starved_polls{0};
+
 // Device copy of a mask list, uploaded once per (device, k) and kept for the life of the process:
 // masks [2^k - 1] followed (256-byte aligned) by level_off [k + 2].
 struct DeviceMasks {
@@ -540,13 +543,6 @@ private:
 };
 PinnedBuffers g_pinned;
 
-// After a search that did not come to its end: its kernel has not cleared the counters.
-void reset_counters(HostSlot *slot)
-{
-    PruneCtl ctl;
-    prune_ctl_init(&ctl);
-    cudaMemcpy(slot->ctl, &ctl, sizeof ctl, cudaMemcpyHostToDevice);
-}
 struct SlotLease {  // a slot for the duration of a call
     HostSlot *slot = g_slots.take();
     ~SlotLease() { if (slot) g_slots.give(slot); }
@@ -764,6 +760,8 @@ pp_status queue_sparse(pp_problem *p, PruneCtl *ctl, pp_solution *sol, PruneNote
 
 }  // namespace
 
+int pp::starved_polls() { return g_starved_polls.load(std::memory_order_relaxed) ? g_starved_polls.exchange(0) : 0; }
+
 extern "C" {
 
 const char *pp_status_str(pp_status s)
@@ -939,7 +937,6 @@ static pp_status solve_sparse(pp_problem *p, pp_solution *sol)
     if (st != PP_OK) return st;
     HostSlot *slot = g_slots.take();
     if (!slot) return PP_ERR_NOMEM;
-    slot->note.dense = -1;
     st = queue_sparse(p, slot->ctl, &slot->sol, &slot->note, kSparseRows);
     const cudaError_t e = cudaStreamSynchronize(p->stream);
     if (st == PP_OK) st = from_cuda(e);
@@ -947,14 +944,8 @@ static pp_status solve_sparse(pp_problem *p, pp_solution *sol)
         p->note = slot->note;
         p->note_on_device = false;
         *sol = slot->sol;
-        if (p->note.dense < 0) {  // a barrier of the kernel gave up: put its counters back
-            reset_counters(slot);
-            st = PP_ERR_CUDA;
-        } else if (p->note.dense) {
-            st = PP_ERR_LIMIT;
-        } else if (sol->status != PP_OK && sol->status != PP_INFEASIBLE) {
-            st = PP_ERR_CUDA;
-        }
+        if (p->note.dense) st = PP_ERR_LIMIT;
+        else if (sol->status != PP_OK && sol->status != PP_INFEASIBLE) st = PP_ERR_CUDA;
     }
     g_slots.give(slot);
     return st;
@@ -1721,16 +1712,14 @@ pp_status pp_solve_exact_compute(int32_t L, const uint64_t *layer_out_bits, cons
         q.ctl = slot->ctl;
         q.out = &slot->sol;
         q.note = &slot->note;
-        slot->note.dense = -1;
         e = launch_prune(q, h, sms, s);
         if (buf) cudaFreeAsync(buf, s);
         const cudaError_t e2 = cudaStreamSynchronize(s);
         if (e == cudaSuccess) e = e2;
-        if (e == cudaSuccess && slot->note.dense <= 0) break;
+        if (e == cudaSuccess && !slot->note.dense) break;
     }
     const pp_solution sol = slot->sol;
     const int32_t dense = slot->note.dense;
-    if (e == cudaSuccess && dense < 0) reset_counters(slot);
     g_slots.give(slot);
     if (e != cudaSuccess) return from_cuda(e);
     if (dense != 0 || (sol.status != PP_OK && sol.status != PP_INFEASIBLE)) return PP_ERR_CUDA;
@@ -1774,6 +1763,13 @@ pp_status pp_debug_fail_alloc(int32_t nth)
 {
     if (nth < 0) return PP_ERR_ARG;
     g_fail_alloc_countdown.store(nth);
+    return PP_OK;
+}
+
+pp_status pp_debug_starve(int32_t polls)
+{
+    if (polls < 0) return PP_ERR_ARG;
+    g_starved_polls.store(polls);
     return PP_OK;
 }
 

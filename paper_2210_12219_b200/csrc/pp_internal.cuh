@@ -149,16 +149,17 @@ struct PruneCtl {              // device; the kernel leaves it as it found it
                                // search over the class of the optimum counts from 32); in the upper half the
                                // blocks that have arrived at the level's end
     uint32_t left;             // blocks that have left
-    uint32_t failed;           // a barrier ran out of polls
-    uint32_t dense;            // 1 = the frontier outgrew its rows
+    uint32_t failed;           // a barrier ran out of polls: the other blocks need not wait any longer
 };
 struct PruneNote {             // what the host learns about a launch
     long long ns;              // duration on the device
-    int32_t dense;             // as PruneCtl::dense
+    int32_t dense;             // 1 = the frontier outgrew its rows
 };
 struct PruneDev {
     int L, k, Lp;              // Lp: row stride in keys
     int clustered;             // the blocks are one cluster (set by the launch)
+    uint32_t arrivals;         // blocks a barrier in global memory waits for, and polls before it gives up (set by
+    int polls;                 // the launch)
     int key_shift;             // keys: 1 + (bits of the double - key_base) >> key_shift
     unsigned long long key_base;
     uint32_t whole;            // nodes that hold the whole chain
@@ -176,6 +177,9 @@ struct PruneDev {
     pp_solution *out;          // device or mapped host memory
     PruneNote *note;           // device or mapped host memory
 };
+// Test hook (pp_debug_starve): polls of the next launch whose blocks meet, which then waits for one block
+// more than it has; 0 = an ordinary launch.  Asking for it uses it up.
+int starved_polls();
 void prune_key_range(double lo, double hi, PruneDev *d);
 void prune_node_bounds(const uint64_t *cap, uint64_t total, PruneDev *d);
 int prune_row_pad(int L, int k);
@@ -244,6 +248,7 @@ struct MatchDev {
     const MatchRun *runs;
     unsigned long long *records;  // [2][2][stride][4]: by `half`, by the parity of the run, by block; this half is
     int half, stride;             // zero before the launch and the launch zeroes the other; stride: blocks at most
+    int posts, polls;             // records a run waits for, and polls before it gives up (set by the launch)
     MatchOut *out;             // mapped host memory
 };
 size_t match_smem_bytes(int n, int kk);

@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(kMatchThreads, 1) k_match(const __grid_constan
         }
         unsigned long long key = 0ull, p0 = 0ull, p1 = 0ull;
         bool late = false;
-        if (tid < (int)gridDim.x) {
+        if (tid < d.posts) {
             const unsigned long long *r = rec + (size_t)tid * 4;
             int spins = 0;
             for (;;) {
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kMatchThreads, 1) k_match(const __grid_constan
                     key = a << 32 | (uint32_t)b;
                     break;
                 }
-                if (++spins >= kSpinLimit) {
+                if (++spins >= d.polls) {
                     late = true;
                     break;
                 }
@@ -312,8 +312,15 @@ cudaError_t launch_match_of(const MatchDev &d, const MatchIn<WORDS> &in, cudaStr
     const size_t sm = match_smem_bytes(d.n, d.kk);
     cudaError_t e = cudaFuncSetAttribute(k_match<THREADS, WORDS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
+    MatchDev q = d;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(d.trials < d.stride ? d.trials : d.stride));
+    q.posts = (int)cfg.gridDim.x;
+    q.polls = kSpinLimit;
+    if (const int polls = q.posts < q.stride ? starved_polls() : 0) {  // test hook: a block that never comes
+        ++q.posts;
+        q.polls = polls;
+    }
     cfg.blockDim = dim3(THREADS);
     cfg.dynamicSmemBytes = sm;
     cfg.stream = s;
@@ -322,7 +329,7 @@ cudaError_t launch_match_of(const MatchDev &d, const MatchIn<WORDS> &in, cudaStr
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_match<THREADS, WORDS>, d, in);
+    return cudaLaunchKernelEx(&cfg, k_match<THREADS, WORDS>, q, in);
 }
 
 template <int WORDS>

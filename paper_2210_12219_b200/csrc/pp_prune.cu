@@ -172,25 +172,29 @@ __device__ __forceinline__ void store_row(uint32_t *p, const uint32_t (&x)[P])
     }
 }
 
-// All blocks of the grid; false when the wait ran out (the caller returns).  A level's word holds the blocks
+// All blocks of the grid; false when the wait ran out, here or in another block (the caller reports it and
+// leaves by the end of the kernel, so that the counters are cleared).  A level's word holds the blocks
 // that have arrived above the node sets it added (32 bits each), so that the last poll brings both; *best,
 // polled along, may miss what the last blocks found, which only makes it a weaker bound.  (Reading both after
 // the barrier cost another trip to L2, 600 cycles a level: k = 16, L = 136 28.7 -> 26.8 us, k = 10, L = 50 48.8 -> 47.9.)
-__device__ __forceinline__ bool grid_barrier(PruneCtl *ctl, unsigned long long *word, unsigned long long *best, uint32_t *added)
+__device__ __forceinline__ bool grid_barrier(const PruneDev &d, unsigned long long *word, unsigned long long *best, uint32_t *added)
 {
     __shared__ int s_ok;
+    PruneCtl *ctl = d.ctl;
     __syncthreads();
     if (threadIdx.x == 0) {
         unsigned long long seen;
         asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(word), "l"(1ull << 32) : "memory");
         int spins = 0;
+        uint32_t failed = 0;
         do {
             asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(*best) : "l"(&ctl->best) : "memory");
             asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(seen) : "l"(word) : "memory");
-        } while ((uint32_t)(seen >> 32) < gridDim.x && ++spins < kSpinLimit);
+            if ((++spins & 1023) == 0) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(failed) : "l"(&ctl->failed) : "memory");
+        } while ((uint32_t)(seen >> 32) < d.arrivals && spins < d.polls && !failed);
         *added = (uint32_t)seen;
-        s_ok = (uint32_t)(seen >> 32) >= gridDim.x;
-        if (!s_ok) ctl->failed = 1;
+        s_ok = (uint32_t)(seen >> 32) >= d.arrivals;
+        if (!s_ok) asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(&ctl->failed), "r"(1u) : "memory");
     }
     __syncthreads();
     return s_ok != 0;
@@ -430,7 +434,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                 seen = __ldcg(&ctl->best);
                 added = (uint32_t)__ldcg(ctl->count + level);
             }
-        } else if (!grid_barrier(ctl, ctl->count + level, &seen, &added)) {
+        } else if (!grid_barrier(d, ctl->count + level, &seen, &added)) {
             return false;
         }
         if (tid == 0) {
@@ -478,7 +482,10 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                     const uint32_t x = base_key(v, L - 1);
                     if (x != kInfKey) s_best = min(s_best, pack_best(x, 1, 1u << v, v));
                 }
-            if (!level_end(kNoBest, 1)) return;
+            if (!level_end(kNoBest, 1)) {
+                status = (int)PP_ERR_CUDA;
+                break;
+            }
         }
         // ---- two nodes: the keys of every link, the rows of every pair ----
         if (top >= 2) {
@@ -615,7 +622,10 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                 }
                 __syncwarp();
             }
-            if (!level_end(before, 2)) return;
+            if (!level_end(before, 2)) {
+                status = (int)PP_ERR_CUDA;
+                break;
+            }
             for (int e = tid; e < k * k; e += kThreads) s_gmin[e] = (e / k != e % k) ? ld_now<SM>(t_gmin + e) : kInfKey;
             __syncthreads();
         }
@@ -699,11 +709,14 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                 __syncwarp();
             }
             used += items;
-            if (!level_end(before, level)) return;
+            if (!level_end(before, level)) {
+                status = (int)PP_ERR_CUDA;
+                break;
+            }
             beg += cnt;
             cnt = s_cnt;
         }
-        if (blockIdx.x != 0 || dense) break;  // block 0 finishes
+        if (blockIdx.x != 0 || dense || status == (int)PP_ERR_CUDA) break;  // block 0 finishes
         if (!SM && tid == 0 && gridDim.x > 1 && !d.clustered && !key_of.zoom) s_best = min(s_best, __ldcg(&ctl->best));
         __syncthreads();
         const unsigned long long best = s_best;
@@ -881,11 +894,11 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
             asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t_end));
             d.note->ns = (long long)(t_end - t_start);
             d.note->dense = dense ? 1 : 0;
-            ctl->dense = dense ? 1 : 0;
         }
     }
     if constexpr (SM) return;  // the counters in global memory are as they were
-    // the last block to leave clears the counters for the next launch
+    // The last block to leave clears the counters for the next launch.  Every block comes here, also one whose
+    // wait ran out.
     __shared__ uint32_t s_left;
     __syncthreads();
     if (tid == 0) {
@@ -897,7 +910,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
         if (tid < 64) ctl->count[tid] = 0ull;
         if (tid == 0) {
             ctl->best = kNoBest;
-            ctl->left = 0u;
+            ctl->left = ctl->failed = 0u;
         }
     }
 }
@@ -991,6 +1004,12 @@ cudaError_t launch_shape(const PruneDev &d, const PruneHost &h, int sms, cudaStr
     }
     cfg.numAttrs = blocks > 1 ? 1 : 0;
     q.clustered = cluster ? 1 : 0;
+    q.arrivals = (uint32_t)blocks;
+    q.polls = kSpinLimit;
+    if (const int polls = blocks > 1 && !cluster ? starved_polls() : 0) {  // test hook: a block that never comes
+        ++q.arrivals;
+        q.polls = polls;
+    }
     return cudaLaunchKernelEx(&cfg, k_prune<G, P, CT, false>, q, in);
 }
 

@@ -113,6 +113,15 @@ bool alloc_should_fail()
 // Test hook (pp_debug_starve).
 std::atomic<int> g_starved_polls{0};
 
+// A copy from pageable memory that is complete when the call returns.  cudaMemcpy may return while the last
+// bytes are still under way, which a stream that does not wait for the legacy stream would not notice.
+cudaError_t copy_in(void *dst, const void *src, size_t n)
+{
+    const cudaError_t e = cudaMemcpyAsync(dst, src, n, cudaMemcpyHostToDevice, nullptr);
+    const cudaError_t e2 = cudaStreamSynchronize(nullptr);
+    return e != cudaSuccess ? e : e2;
+}
+
 // Device copy of a mask list, uploaded once per (device, k) and kept for the life of the process:
 // masks [2^k - 1] followed (256-byte aligned) by level_off [k + 2].
 struct DeviceMasks {
@@ -132,8 +141,8 @@ cudaError_t device_masks(int k, const MaskList &ml, DeviceMasks *out)
         unsigned char *buf = nullptr;
         e = alloc_should_fail() ? cudaErrorMemoryAllocation : cudaMalloc(reinterpret_cast<void **>(&buf), mb + lb);
         if (e != cudaSuccess) return e;
-        e = cudaMemcpy(buf, ml.masks.data(), ml.masks.size() * 4, cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(buf + mb, ml.level_off.data(), lb, cudaMemcpyHostToDevice);
+        e = copy_in(buf, ml.masks.data(), ml.masks.size() * 4);
+        if (e == cudaSuccess) e = copy_in(buf + mb, ml.level_off.data(), lb);
         if (e != cudaSuccess) {
             cudaFree(buf);
             return e;
@@ -182,7 +191,7 @@ cudaError_t lane_tables(int k, LaneTables *out)
         e = alloc_should_fail() ? cudaErrorMemoryAllocation
                                 : cudaMalloc(reinterpret_cast<void **>(&buf), host.size() * 4);
         if (e != cudaSuccess) return e;
-        e = cudaMemcpy(buf, host.data(), host.size() * 4, cudaMemcpyHostToDevice);
+        e = copy_in(buf, host.data(), host.size() * 4);
         if (e != cudaSuccess) {
             cudaFree(buf);
             return e;
@@ -389,7 +398,7 @@ pp_status upload_inputs(pp_problem *p, bool wait)
     PruneCtl ctl;
     prune_ctl_init(&ctl);
     put(p->prune.ctl, &ctl, sizeof ctl);
-    if (wait) PP_CUDA(cudaMemcpy(p->d_inputs, st.data(), st.size(), cudaMemcpyHostToDevice));
+    if (wait) PP_CUDA(copy_in(p->d_inputs, st.data(), st.size()));
     else PP_CUDA(cudaMemcpyAsync(p->d_inputs, st.data(), st.size(), cudaMemcpyHostToDevice, p->stream));
     p->uploaded = true;
     return PP_OK;
@@ -451,8 +460,8 @@ public:
                                       cudaHostAllocPortable | cudaHostAllocMapped);
         if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&c.ctl), sizeof init);
         if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&c.records), kSlots * records);
-        if (e == cudaSuccess) e = cudaMemset(c.records, 0, kSlots * records);
-        if (e == cudaSuccess) e = cudaMemcpy(c.ctl, init, sizeof init, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c.records, 0, kSlots * records, nullptr);
+        if (e == cudaSuccess) e = copy_in(c.ctl, init, sizeof init);  // the same stream: both are complete
         if (e != cudaSuccess) {
             cudaFreeHost(c.base);
             cudaFree(c.ctl);
@@ -655,7 +664,7 @@ pp_status dense_prepare(pp_problem *p)
         DeviceMasks dmasks;
         PP_CUDA(device_masks(k, ml, &dmasks));
         if (!p->d_dense) PP_CUDA(staging_alloc(reinterpret_cast<void **>(&p->d_dense), total, nullptr));
-        PP_CUDA(cudaMemcpy(p->d_dense, staging.data(), total, cudaMemcpyHostToDevice));
+        PP_CUDA(copy_in(p->d_dense, staging.data(), total));
         for (auto &e : p->ev)
             if (!e) PP_CUDA(cudaEventCreate(&e));
         unsigned char *b = p->d_dense;

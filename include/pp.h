@@ -100,8 +100,11 @@ typedef struct {
  *   node_mem_bytes  host [k]    capacity of each node in bytes (heterogeneous; the paper's
  *                               homogeneous case is all entries equal)
  *   bw_kbps         host [k*k]  row-major, [v*k + w] = bandwidth of the link v -> w; 0 = no link
- * Validates, builds the uint64 memory prefix sums and the per-node window table (for each
- * node w and segment end c', the earliest segment start that still fits), uploads them.
+ * Validates, copies the inputs, builds the uint64 memory prefix sums and allocates the device
+ * memory of the inputs.  Nothing is sent to the device yet: a synchronous solve takes the inputs
+ * along with its launch; the first pp_problem_set_stream, or else the first call that reads them
+ * there, builds the per-node window tables (for each node w and segment end c' the earliest segment
+ * start that still fits, for each start the number of layers that fit) and copies everything.
  * *out receives the handle; free it with pp_problem_destroy.
  * The list of node sets the dense sweep walks depends on k only: its device copy (4 * 2^k bytes) is
  * made by the first sweep of that k on a device and kept until the process ends.
@@ -116,7 +119,9 @@ pp_status pp_problem_create(int32_t L, const uint64_t *layer_out_bits,
 void pp_problem_destroy(pp_problem *p);
 
 /* Use `cuda_stream` (a cudaStream_t, e.g. torch.cuda.current_stream().cuda_stream) for all
- * later work of this problem.  NULL selects the legacy default stream. */
+ * later work of this problem.  NULL selects the legacy default stream.  Waits for the work queued for
+ * the problem on the stream it used before; the first call copies the inputs to the device, complete
+ * when it returns (on the legacy stream in order). */
 pp_status pp_problem_set_stream(pp_problem *p, void *cuda_stream);
 
 /* Bytes of device scratch the exact search needs (state table, gamma and rank tables).  Without a
@@ -161,6 +166,8 @@ pp_status pp_solve_exact_dev(pp_problem *p, pp_solution *solution_dev);
  *                      DEAD_LINK are only evaluated when ENDS and NODE are clean.
  * pp_eval_plans takes host pointers and is synchronous; pp_eval_plans_dev takes device
  * pointers and is asynchronous on the problem's stream.  B == 0 is a no-op.
+ * The _dev calls over plans (pp_eval_plans_dev, pp_eval_plans_packed_dev, pp_random_plans_dev)
+ * allocate nothing; once pp_problem_set_stream has been called they are plain launches.
  */
 pp_status pp_eval_plans(pp_problem *p, int64_t B, const uint8_t *nseg, const int32_t *ends,
                         const int32_t *nodes, double *beta_ms, uint8_t *plan_status);

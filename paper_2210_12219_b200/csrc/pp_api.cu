@@ -22,9 +22,12 @@ struct pp_problem {
     std::vector<uint64_t> bits, mem, cap, M;
     std::vector<uint32_t> bw;
     std::vector<int16_t> lo;
+    std::vector<uint16_t> fwd;
     unsigned char *d_inputs = nullptr;  // one allocation: the inputs, the counters, a result record
     size_t inputs_bytes = 0;
     bool uploaded = false;              // the inputs have been copied (queued on `stream`)
+    bool tables_ready = false;          // a launch may read them before the work in front of it on `stream` is done:
+                                        // the copy is complete, or another launch is ordered behind it
     unsigned char *d_sparse = nullptr;  // scratch of the bounded search when there is no workspace
     unsigned char *d_work = nullptr;    // workspace (own or caller's): either search runs in it
     uint64_t work_bytes = 0;
@@ -34,6 +37,7 @@ struct pp_problem {
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};  // of the dense search, created by its first run
     pp_solution *d_sol = nullptr;
     PruneNote *d_note = nullptr;
+    unsigned char *d_tables = nullptr;  // PlanTables, in d_inputs
     PruneDev prune{};
     bool solved = false, profiled = false;
     bool sparse_ran = false;            // the last solve ran the bounded search
@@ -49,8 +53,6 @@ struct pp_problem {
     std::vector<uint32_t> ubw;
     std::vector<int16_t> pair_u;
     unsigned char *d_dense = nullptr;
-    unsigned char *d_tables = nullptr;  // PlanTables, made by the first call that scores or draws plans
-    bool tables_read = false;           // a launch has been ordered behind the one that makes them
     Dev d{};
     int sweep_launches = 0, total_launches = 0, fast_used = 0, pair_levels = 0;
     std::vector<signed char> pair_lvl;  // per level: 1 = two-mask kernel, 0 = one-mask, -1 = not decided yet
@@ -336,15 +338,16 @@ void bind_sparse(PruneDev &q, unsigned char *b, uint64_t bytes)
 }
 
 // lo[w][c'] = earliest previous cut c >= 0 such that layers c+1..c' fit on w; c' itself when not even
-// layer c' alone fits.  Non-decreasing in c'.
-void window_table(int L, int k, const uint64_t *M, const uint64_t *cap, int16_t *lo)
+// layer c' alone fits.  fwd[w][c] = layers from c on that fit w.
+void window_table(int L, int k, const uint64_t *M, const uint64_t *cap, int16_t *lo, uint16_t *fwd)
 {
-    for (int w = 0; w < k; ++w) {
-        int c = 0;
+    for (int w = 0; w < k; ++w, lo += L, fwd += L) {
+        int a = 0;  // first layer such that layers a .. c2 fit
         for (int c2 = 0; c2 < L; ++c2) {
-            while (c < c2 && M[c2 + 1] - M[c + 1] > cap[w]) ++c;
-            lo[(size_t)w * L + c2] = (int16_t)c;
+            for (; a <= c2 && M[c2 + 1] - M[a] > cap[w]; ++a) fwd[a] = (uint16_t)(c2 - a);
+            lo[c2] = (int16_t)std::max(a - 1, 0);
         }
+        for (; a < L; ++a) fwd[a] = (uint16_t)(L - a);
     }
 }
 
@@ -366,16 +369,32 @@ void quotient_range(int L, const uint64_t *num, int n, const uint32_t *den, doub
     *hi = std::max(*hi, (double)b / (double)c);
 }
 
-// Copies the inputs to the device, ordered on the problem's stream.  The staging memory may go as soon
-// as the call returns: copies from pageable memory leave it first.
 void ensure_windows(pp_problem *p)
 {
     if (!p->lo.empty()) return;
     std::vector<int16_t> lo((size_t)p->k * p->L);
-    window_table(p->L, p->k, p->M.data(), p->cap.data(), lo.data());
+    std::vector<uint16_t> fwd((size_t)p->k * p->L);
+    window_table(p->L, p->k, p->M.data(), p->cap.data(), lo.data(), fwd.data());
     p->lo.swap(lo);
+    p->fwd.swap(fwd);
 }
 
+// PlanTables of the problem at `out` (zeros so far).  They come out of the pass that makes the window starts and go
+// up with the inputs.  Made by a kernel of the first scoring call they cost that call an allocation, a launch and
+// the overlap with the launch in front (k = 14, L = 50, 100 003 plans: first call 32.3 us so, 21.4 now; with
+// create and set stream 59.5 and 54.7).
+void fill_plan_tables(const pp_problem *p, unsigned char *out)
+{
+    const int L = p->L, k = p->k;
+    const PlanTables t = plan_tables(L, k);
+    std::memcpy(out + t.bits, p->bits.data(), (size_t)L * 8);
+    uint32_t *bw = reinterpret_cast<uint32_t *>(out + t.bw);
+    for (int v = 0; v < k; ++v) std::memcpy(bw + (size_t)v * (k + 1), p->bw.data() + (size_t)v * k, (size_t)k * 4);
+    std::memcpy(out + t.fwd, p->fwd.data(), p->fwd.size() * 2);
+}
+
+// Copies the inputs to the device, ordered on the problem's stream.  The staging memory may go as soon
+// as the call returns: copies from pageable memory leave it first.
 pp_status upload_inputs(pp_problem *p, bool wait)
 {
     if (p->uploaded) return PP_OK;
@@ -398,30 +417,20 @@ pp_status upload_inputs(pp_problem *p, bool wait)
     PruneCtl ctl;
     prune_ctl_init(&ctl);
     put(p->prune.ctl, &ctl, sizeof ctl);
+    fill_plan_tables(p, st.data() + (p->d_tables - p->d_inputs));
     if (wait) PP_CUDA(copy_in(p->d_inputs, st.data(), st.size()));
     else PP_CUDA(cudaMemcpyAsync(p->d_inputs, st.data(), st.size(), cudaMemcpyHostToDevice, p->stream));
     p->uploaded = true;
+    p->tables_ready = wait;
     return PP_OK;
 }
 
-// Whether a launch over n plans may start before the one in front of it has ended: the one that makes the
-// tables is not that one.
-bool early(pp_problem *p, int64_t n)
+// Whether a launch over plans may start before the one in front of it has ended.
+bool early(pp_problem *p)
 {
-    const bool was = p->tables_read;
-    p->tables_read = was || n > 0;
+    const bool was = p->tables_ready;
+    p->tables_ready = true;  // for the launch behind this one
     return was;
-}
-
-pp_status ensure_tables(pp_problem *p)
-{
-    const pp_status st = upload_inputs(p, false);
-    if (st != PP_OK || p->d_tables) return st;
-    unsigned char *t = nullptr;
-    PP_CUDA(staging_alloc(reinterpret_cast<void **>(&t), plan_tables(p->L, p->k).total, p->stream));
-    p->d_tables = t;
-    PP_CUDA(launch_plan_tables(p->d, t, p->stream));
-    return PP_OK;
 }
 
 // Page-locked memory of the synchronous calls, one slot per call in flight: the kernel writes its result
@@ -813,10 +822,11 @@ pp_status pp_problem_create(int32_t L, const uint64_t *layer_out_bits,
     }
     // one device buffer for the inputs, the counters of the searches and a result record; the copy is
     // queued by the first call that needs it, on the stream the problem has by then
-    const size_t bytes[9] = {(size_t)L * 8, (size_t)(L + 1) * 8, (size_t)k * 8, (size_t)k * k * 4, (size_t)k * L * 2,
-                             sizeof(PruneCtl), 8 /* best */, 4 /* err */, sizeof(pp_solution) + sizeof(PruneNote)};
-    size_t off[9], total = 0;
-    for (int i = 0; i < 9; ++i) { off[i] = total; total = align_up(total + bytes[i], i < 4 ? 16 : 128); }
+    const size_t bytes[10] = {(size_t)L * 8, (size_t)(L + 1) * 8, (size_t)k * 8, (size_t)k * k * 4, (size_t)k * L * 2,
+                             sizeof(PruneCtl), 8 /* best */, 4 /* err */, sizeof(pp_solution) + sizeof(PruneNote),
+                              plan_tables(L, k).total};
+    size_t off[10], total = 0;
+    for (int i = 0; i < 10; ++i) { off[i] = total; total = align_up(total + bytes[i], i < 4 ? 16 : 128); }
     p->inputs_bytes = total;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -839,6 +849,7 @@ pp_status pp_problem_create(int32_t L, const uint64_t *layer_out_bits,
     d.err = reinterpret_cast<int32_t *>(b + off[7]);
     p->d_sol = reinterpret_cast<pp_solution *>(b + off[8]);
     p->d_note = reinterpret_cast<PruneNote *>(b + off[8] + sizeof(pp_solution));
+    p->d_tables = b + off[9];
     PruneDev &q = p->prune;
     q.L = L; q.k = k; q.Lp = prune_row_pad(L, k);
     q.ctl = reinterpret_cast<PruneCtl *>(b + off[5]);
@@ -854,7 +865,7 @@ void pp_problem_destroy(pp_problem *p)
 {
     if (!p) return;
     if (p->own_work && p->d_work) cudaFree(p->d_work);
-    for (unsigned char *q : {p->d_inputs, p->d_sparse, p->d_dense, p->d_tables})
+    for (unsigned char *q : {p->d_inputs, p->d_sparse, p->d_dense})
         if (q) cudaFreeAsync(q, p->stream);  // ordered after the problem's queued work
     for (auto &e : p->ev)
         if (e) cudaEventDestroy(e);
@@ -865,10 +876,12 @@ pp_status pp_problem_set_stream(pp_problem *p, void *cuda_stream)
 {
     if (!p) return PP_ERR_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    if (s == p->stream) return PP_OK;
-    if (p->uploaded || p->d_sparse || p->d_tables) PP_CUDA(cudaStreamSynchronize(p->stream));  // copies and scratch are ordered there
+    if (s != p->stream && (p->uploaded || p->d_sparse)) {  // copies and scratch are ordered there
+        PP_CUDA(cudaStreamSynchronize(p->stream));
+        p->tables_ready = p->uploaded;
+    }
     p->stream = s;
-    return upload_inputs(p, true);
+    return upload_inputs(p, s != nullptr);  // the legacy stream, on which the buffer was allocated, has it in order
 }
 
 pp_status pp_problem_workspace_bytes(const pp_problem *p, uint64_t *bytes)
@@ -1030,9 +1043,9 @@ pp_status pp_eval_plans_dev(pp_problem *p, int64_t B, const uint8_t *nseg, const
     if (!p || B < 0) return PP_ERR_ARG;
     if (B == 0) return PP_OK;
     if (!nseg || !ends || !nodes || !beta_ms || !plan_status) return PP_ERR_ARG;
-    pp_status st = ensure_tables(p);
+    pp_status st = upload_inputs(p, false);
     if (st != PP_OK) return st;
-    PP_CUDA(launch_eval(p->d, p->d_tables, B, nseg, ends, nodes, beta_ms, plan_status, early(p, B), p->stream));
+    PP_CUDA(launch_eval(p->d, p->d_tables, B, nseg, ends, nodes, beta_ms, plan_status, early(p), p->stream));
     return PP_OK;
 }
 
@@ -1047,7 +1060,7 @@ pp_status pp_eval_plans(pp_problem *p, int64_t B, const uint8_t *nseg, const int
     size_t o_ends = align_up(b_nseg, 256), o_nodes = align_up(o_ends + b_rows, 256);
     size_t o_beta = align_up(o_nodes + b_rows, 256), o_st = align_up(o_beta + b_beta, 256);
     size_t total = o_st + (size_t)B;
-    pp_status st = ensure_tables(p);
+    pp_status st = upload_inputs(p, false);
     if (st != PP_OK) return st;
     unsigned char *buf = nullptr;
     cudaStream_t s = p->stream;
@@ -1058,7 +1071,7 @@ pp_status pp_eval_plans(pp_problem *p, int64_t B, const uint8_t *nseg, const int
     if (e == cudaSuccess)
         e = launch_eval(p->d, p->d_tables, B, buf, reinterpret_cast<int32_t *>(buf + o_ends),
                         reinterpret_cast<int32_t *>(buf + o_nodes),
-                        reinterpret_cast<double *>(buf + o_beta), buf + o_st, early(p, B), s);
+                        reinterpret_cast<double *>(buf + o_beta), buf + o_st, early(p), s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(beta_ms, buf + o_beta, b_beta, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(plan_status, buf + o_st, (size_t)B, cudaMemcpyDeviceToHost, s);
     cudaFreeAsync(buf, s);
@@ -1074,9 +1087,9 @@ pp_status pp_eval_plans_packed_dev(pp_problem *p, int64_t B, int64_t total, cons
     if (!p || B < 0 || total < 0) return PP_ERR_ARG;
     if (B == 0) return PP_OK;
     if (!nseg || !plan_off || !beta_ms || !plan_status || ((!ends || !nodes) && total > 0)) return PP_ERR_ARG;
-    pp_status st = ensure_tables(p);
+    pp_status st = upload_inputs(p, false);
     if (st != PP_OK) return st;
-    PP_CUDA(launch_eval_packed(p->d, p->d_tables, B, total, nseg, plan_off, ends, nodes, beta_ms, plan_status, early(p, B), p->stream));
+    PP_CUDA(launch_eval_packed(p->d, p->d_tables, B, total, nseg, plan_off, ends, nodes, beta_ms, plan_status, early(p), p->stream));
     return PP_OK;
 }
 
@@ -1091,7 +1104,7 @@ pp_status pp_eval_plans_packed(pp_problem *p, int64_t B, int64_t total, const ui
     const size_t o_off = align_up(nB, 256), o_ends = align_up(o_off + (nB + 1) * 4, 256);
     const size_t o_nodes = align_up(o_ends + nT * 2, 256), o_beta = align_up(o_nodes + nT, 256);
     const size_t o_st = align_up(o_beta + nB * 8, 256), bytes = o_st + nB;
-    pp_status st = ensure_tables(p);
+    pp_status st = upload_inputs(p, false);
     if (st != PP_OK) return st;
     unsigned char *buf = nullptr;
     cudaStream_t s = p->stream;
@@ -1103,7 +1116,7 @@ pp_status pp_eval_plans_packed(pp_problem *p, int64_t B, int64_t total, const ui
     if (e == cudaSuccess)
         e = launch_eval_packed(p->d, p->d_tables, B, total, buf, reinterpret_cast<uint32_t *>(buf + o_off),
                                reinterpret_cast<uint16_t *>(buf + o_ends), buf + o_nodes,
-                               reinterpret_cast<double *>(buf + o_beta), buf + o_st, early(p, B), s);
+                               reinterpret_cast<double *>(buf + o_beta), buf + o_st, early(p), s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(beta_ms, buf + o_beta, nB * 8, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(plan_status, buf + o_st, nB, cudaMemcpyDeviceToHost, s);
     cudaFreeAsync(buf, s);
@@ -1118,9 +1131,9 @@ pp_status pp_random_plans_dev(pp_problem *p, int64_t P, const uint32_t *draws, u
     if (!p || P < 0) return PP_ERR_ARG;
     if (P == 0) return PP_OK;
     if (!draws || !nseg || !ends || !nodes) return PP_ERR_ARG;
-    pp_status st = ensure_tables(p);
+    pp_status st = upload_inputs(p, false);
     if (st != PP_OK) return st;
-    PP_CUDA(launch_random_plans(p->d, p->d_tables, P, draws, nseg, ends, nodes, early(p, P), p->stream));
+    PP_CUDA(launch_random_plans(p->d, p->d_tables, P, draws, nseg, ends, nodes, early(p), p->stream));
     return PP_OK;
 }
 
@@ -1134,7 +1147,7 @@ pp_status pp_random_plans(pp_problem *p, int64_t P, const uint32_t *draws, uint8
     const size_t b_draws = (size_t)P * 2 * k * 4, b_rows = (size_t)P * k * 4;
     const size_t o_ends = align_up(b_draws, 256), o_nodes = align_up(o_ends + b_rows, 256);
     const size_t o_nseg = align_up(o_nodes + b_rows, 256), total = o_nseg + (size_t)P;
-    pp_status st = ensure_tables(p);
+    pp_status st = upload_inputs(p, false);
     if (st != PP_OK) return st;
     unsigned char *buf = nullptr;
     cudaStream_t s = p->stream;
@@ -1143,7 +1156,7 @@ pp_status pp_random_plans(pp_problem *p, int64_t P, const uint32_t *draws, uint8
     if (e == cudaSuccess)
         e = launch_random_plans(p->d, p->d_tables, P, reinterpret_cast<uint32_t *>(buf), buf + o_nseg,
                                 reinterpret_cast<int32_t *>(buf + o_ends),
-                                reinterpret_cast<int32_t *>(buf + o_nodes), early(p, P), s);
+                                reinterpret_cast<int32_t *>(buf + o_nodes), early(p), s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(nseg, buf + o_nseg, (size_t)P, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(ends, buf + o_ends, b_rows, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(nodes, buf + o_nodes, b_rows, cudaMemcpyDeviceToHost, s);

@@ -209,31 +209,6 @@ k_eval(const int L, const int k, const unsigned char *__restrict__ tables, const
     }
 }
 
-// The tables of a problem in the layout the kernels stage: see PlanTables.
-__global__ void k_plan_tables(const Dev d, unsigned char *out)
-{
-    const int L = d.L, k = d.k, k1 = k + 1, gtid = blockIdx.x * blockDim.x + threadIdx.x, gsize = gridDim.x * blockDim.x;
-    const PlanTables tab = plan_tables(L, k);
-    unsigned long long *bits = reinterpret_cast<unsigned long long *>(out + tab.bits);
-    uint32_t *bw = reinterpret_cast<uint32_t *>(out + tab.bw);
-    uint16_t *fwd = reinterpret_cast<uint16_t *>(out + tab.fwd);
-    for (int i = gtid; i < L; i += gsize) bits[i] = d.bits[i];
-    for (int i = gtid; i < k1 * k1; i += gsize) {
-        const int v = i / k1, w = i - v * k1;
-        bw[i] = v < k && w < k ? d.bw[v * k + w] : 0u;
-    }
-    for (int i = gtid; i < k1 * L + 1; i += gsize) {
-        const int w = i / L, first = i - w * L;
-        int lo = first, hi = w < k ? L : first;  // every layer below lo fits, none from hi on does
-        const uint64_t base = d.M[first], room = w < k ? d.cap[w] : 0ull;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (d.M[mid + 1] - base <= room) lo = mid + 1; else hi = mid;
-        }
-        fwd[i] = (uint16_t)(lo - first);
-    }
-}
-
 template <bool PACKED, typename E, typename N>
 cudaError_t launch(const Dev &d, const unsigned char *tables, int64_t B, int64_t total, const uint8_t *nseg, const uint32_t *off, const E *ends,
                    const N *nodes, double *beta, uint8_t *status, bool early, cudaStream_t s)
@@ -258,12 +233,6 @@ cudaError_t launch(const Dev &d, const unsigned char *tables, int64_t B, int64_t
 }
 
 }  // namespace
-
-cudaError_t launch_plan_tables(const Dev &d, unsigned char *out, cudaStream_t s)
-{
-    k_plan_tables<<<((d.k + 1) * d.L + 128) / 128, 128, 0, s>>>(d, out);
-    return cudaGetLastError();
-}
 
 cudaError_t launch_eval_packed(const Dev &d, const unsigned char *tables, int64_t B, int64_t total, const uint8_t *nseg, const uint32_t *off,
                                const uint16_t *ends, const uint8_t *nodes, double *beta, uint8_t *status,

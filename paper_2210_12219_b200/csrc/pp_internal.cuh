@@ -79,7 +79,7 @@ bool pair_meta_build(int L, int k, const int16_t *lo, void *out);
 bool pair_sweep_takes(const Dev &d, int level, bool whenever_possible);
 cudaError_t launch_sweep_pair(const Dev &d, int level, cudaStream_t s, bool first_level);
 cudaError_t launch_finalize(const Dev &d, pp_solution *out, cudaStream_t s, bool dependent);
-// What the evaluator and the random plans look up, laid out once per problem on the device as their
+// What the evaluator and the random plans look up, laid out with the inputs of a problem as their
 // kernels stage it in shared memory: output bits of the layers, bandwidths with a row and a column of
 // zeros for "no such node", forward windows fwd[w * L + first] = layers from `first` on that fit node w
 // (a row of zeros for no such node, one entry more for a segment that would start behind the chain).
@@ -95,9 +95,8 @@ __host__ __device__ inline PlanTables plan_tables(int L, int k)
     t.total = t.fwd + ((((size_t)(k + 1) * L + 1) * 2 + 15) & ~(size_t)15);
     return t;
 }
-cudaError_t launch_plan_tables(const Dev &d, unsigned char *out, cudaStream_t s);
 // early: the launch may start before the one in front of it on the stream has ended, and reads the tables at once.
-// Not for the first launch after launch_plan_tables.
+// Not where the copy of the tables may still be under way.
 cudaError_t launch_eval(const Dev &d, const unsigned char *tables, int64_t B, const uint8_t *nseg, const int32_t *ends,
                         const int32_t *nodes, double *beta, uint8_t *status, bool early, cudaStream_t s);
 cudaError_t launch_eval_packed(const Dev &d, const unsigned char *tables, int64_t B, int64_t total, const uint8_t *nseg, const uint32_t *off,

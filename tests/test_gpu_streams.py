@@ -7,6 +7,7 @@ import pytest
 
 import oracle
 import paper_2210_12219_b200 as pp
+from oracle import random_plans as OR
 from paper_2210_12219_b200 import build
 from paper_2210_12219_b200 import workloads as W
 
@@ -50,3 +51,60 @@ def test_first_calls_of_new_handles(mode):
         assert got.status == want.status and (np.isinf(want.beta_ms) or got.beta_ms == want.beta_ms)
         assert (got.m, tuple(got.cuts[: max(got.m - 1, 0)]), tuple(got.placement[: got.m])) == want.plan()
         assert np.array_equal(beta.cpu().numpy(), scored[0]) and np.array_equal(stat.cpu().numpy(), scored[1])
+
+
+def test_first_calls_over_plans_are_plain_launches():
+    # nothing is allocated, so that a first call can be recorded into a graph, and the tables are there for it
+    import torch
+    inst = W.random_small(96000, 61, 9)
+    inst.node_mem_bytes[:] = np.uint64(int(inst.layer_mem_bytes.sum()) // 3 + 1)
+    B = 700
+    nseg, ends, nodes = W.random_plans(inst, B, seed=4, invalid_fraction=0.2)
+    off, e16, n8 = W.pack_plans(nseg, ends, nodes)
+    want = oracle.eval_plans(inst, nseg, ends, nodes)
+    draws = np.random.default_rng(3).integers(0, 2**32, size=(B, 2 * inst.k), dtype=np.uint64).astype(np.uint32)
+    drawn = OR.random_plans(inst, draws)
+    dev = [torch.from_numpy(a.view("i%d" % a.itemsize) if a.itemsize > 1 else a).cuda()
+           for a in (nseg, ends, nodes, off, e16, n8, draws)]
+    beta = torch.zeros(B, dtype=torch.float64, device="cuda")
+    stat = torch.zeros(B, dtype=torch.uint8, device="cuda")
+    out = (torch.zeros(B, dtype=torch.uint8, device="cuda"), torch.zeros((B, inst.k), dtype=torch.int32, device="cuda"),
+           torch.zeros((B, inst.k), dtype=torch.int32, device="cuda"))
+    ptr = lambda *t: [x.data_ptr() for x in t]
+    calls = {"eval": lambda p: p.eval_plans_dev(B, *ptr(*dev[:3], beta, stat)),
+             "packed": lambda p: p.eval_plans_packed_dev(B, e16.size, *ptr(dev[0], *dev[3:6], beta, stat)),
+             "random": lambda p: p.random_plans_dev(B, *ptr(dev[6], *out))}
+    s = torch.cuda.Stream()
+
+    def check(name):
+        torch.cuda.synchronize()
+        if name == "random":
+            assert [t.cpu().numpy().tolist() for t in out] == list(drawn)
+        else:
+            assert np.array_equal(beta.cpu().numpy(), want[0]) and np.array_equal(stat.cpu().numpy(), want[1])
+        for t in (beta, stat, *out):
+            t.zero_()
+        torch.cuda.synchronize()
+
+    for name, call in calls.items():
+        for stream in (0, s.cuda_stream):
+            with pp.Problem.from_instance(inst) as p:
+                p.set_stream(stream)
+                pp.debug_fail_alloc(1)  # the next allocation would fail
+                try:
+                    call(p)
+                finally:
+                    pp.debug_fail_alloc(0)
+                check(name)
+        with pp.Problem.from_instance(inst) as p:
+            p.set_stream(s.cuda_stream)
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=s):
+                call(p)
+                call(p)
+            for _ in range(2):
+                g.replay()
+                check(name)
+            del g
+            call(p)  # the handle does not live on the graph's memory
+            check(name)

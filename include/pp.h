@@ -121,7 +121,9 @@ void pp_problem_destroy(pp_problem *p);
 /* Use `cuda_stream` (a cudaStream_t, e.g. torch.cuda.current_stream().cuda_stream) for all
  * later work of this problem.  NULL selects the legacy default stream.  Waits for the work queued for
  * the problem on the stream it used before; the first call copies the inputs to the device, complete
- * when it returns (on the legacy stream in order). */
+ * when it returns (on the legacy stream in order).  May be called while `cuda_stream` is recorded
+ * into a graph: nothing the handle keeps becomes part of the graph, and the caller sees to it that the
+ * graph runs after the work the handle has queued elsewhere and before the handle is destroyed. */
 pp_status pp_problem_set_stream(pp_problem *p, void *cuda_stream);
 
 /* Bytes of device scratch the exact search needs (state table, gamma and rank tables).  Without a

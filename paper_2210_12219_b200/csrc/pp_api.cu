@@ -23,7 +23,10 @@ struct pp_problem {
     std::vector<uint32_t> bw;
     std::vector<int16_t> lo;
     std::vector<uint16_t> fwd;
-    unsigned char *d_inputs = nullptr;  // one allocation: the inputs, the counters, a result record
+    unsigned char *d_inputs = nullptr;  // one allocation: see bind_inputs
+    unsigned char *d_spare = nullptr;   // the one of pp_problem_create where the inputs are elsewhere: see upload_inputs
+    unsigned char *mallocs[4] = {};     // of the kept buffers those that are not of the pool
+    int n_mallocs = 0;
     size_t inputs_bytes = 0;
     bool uploaded = false;              // the inputs have been copied (queued on `stream`)
     bool tables_ready = false;          // a launch may read them before the work in front of it on `stream` is done:
@@ -115,12 +118,43 @@ bool alloc_should_fail()
 // Test hook (pp_debug_starve).
 std::atomic<int> g_starved_polls{0};
 
+// Whether the stream is being recorded into a graph (the legacy stream cannot be).
+bool recording(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    return s && cudaStreamIsCapturing(s, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone;
+}
+
+// What a handle or the process keeps must not become part of a graph that happens to be recorded when it is first
+// needed: such memory comes from cudaMalloc and is filled through copy_stream(), which this thread may use meanwhile.
+struct OutsideCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    OutsideCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~OutsideCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+// A stream of the library's own for copies to memory that no stream owns, one per device, kept.
+cudaError_t copy_stream(cudaStream_t *out)
+{
+    static std::mutex mu;
+    static cudaStream_t streams[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    *out = nullptr;
+    if (e != cudaSuccess || dev < 0 || dev >= 64) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    if (!streams[dev]) e = cudaStreamCreateWithFlags(&streams[dev], cudaStreamNonBlocking);
+    *out = streams[dev];
+    return e;
+}
+
 // A copy from pageable memory that is complete when the call returns.  cudaMemcpy may return while the last
 // bytes are still under way, which a stream that does not wait for the legacy stream would not notice.
-cudaError_t copy_in(void *dst, const void *src, size_t n)
+// via: the legacy stream for memory of the pool, copy_stream() for memory of cudaMalloc.
+cudaError_t copy_in(void *dst, const void *src, size_t n, cudaStream_t via)
 {
-    const cudaError_t e = cudaMemcpyAsync(dst, src, n, cudaMemcpyHostToDevice, nullptr);
-    const cudaError_t e2 = cudaStreamSynchronize(nullptr);
+    const cudaError_t e = cudaMemcpyAsync(dst, src, n, cudaMemcpyHostToDevice, via);
+    const cudaError_t e2 = cudaStreamSynchronize(via);
     return e != cudaSuccess ? e : e2;
 }
 
@@ -141,10 +175,14 @@ cudaError_t device_masks(int k, const MaskList &ml, DeviceMasks *out)
     if (it == cache.end()) {
         const size_t mb = (ml.masks.size() * 4 + 255) / 256 * 256, lb = ml.level_off.size() * 4;
         unsigned char *buf = nullptr;
+        OutsideCapture outside;
+        cudaStream_t via = nullptr;
+        e = copy_stream(&via);
+        if (e != cudaSuccess) return e;
         e = alloc_should_fail() ? cudaErrorMemoryAllocation : cudaMalloc(reinterpret_cast<void **>(&buf), mb + lb);
         if (e != cudaSuccess) return e;
-        e = copy_in(buf, ml.masks.data(), ml.masks.size() * 4);
-        if (e == cudaSuccess) e = copy_in(buf + mb, ml.level_off.data(), lb);
+        e = copy_in(buf, ml.masks.data(), ml.masks.size() * 4, via);
+        if (e == cudaSuccess) e = copy_in(buf + mb, ml.level_off.data(), lb, via);
         if (e != cudaSuccess) {
             cudaFree(buf);
             return e;
@@ -190,10 +228,14 @@ cudaError_t lane_tables(int k, LaneTables *out)
         moff[k + 1] = masks;
         first[k + 1] = rows;
         uint32_t *buf = nullptr;
+        OutsideCapture outside;
+        cudaStream_t via = nullptr;
+        e = copy_stream(&via);
+        if (e != cudaSuccess) return e;
         e = alloc_should_fail() ? cudaErrorMemoryAllocation
                                 : cudaMalloc(reinterpret_cast<void **>(&buf), host.size() * 4);
         if (e != cudaSuccess) return e;
-        e = copy_in(buf, host.data(), host.size() * 4);
+        e = copy_in(buf, host.data(), host.size() * 4, via);
         if (e != cudaSuccess) {
             cudaFree(buf);
             return e;
@@ -369,6 +411,44 @@ void quotient_range(int L, const uint64_t *num, int n, const uint32_t *den, doub
     *hi = std::max(*hi, (double)b / (double)c);
 }
 
+// Device memory that the handle keeps: of the pool, ordered on its stream, else of cudaMalloc.
+cudaError_t kept_alloc(pp_problem *p, unsigned char **out, size_t bytes, bool rec)
+{
+    if (!rec) return staging_alloc(reinterpret_cast<void **>(out), bytes, p->stream);
+    if (alloc_should_fail()) return cudaErrorMemoryAllocation;
+    OutsideCapture outside;
+    const cudaError_t e = cudaMalloc(reinterpret_cast<void **>(out), bytes);
+    if (e == cudaSuccess) p->mallocs[p->n_mallocs++] = *out;
+    return e;
+}
+
+// The parts of the buffer of the inputs: the inputs, the counters of the searches, a result record, the tables of the
+// scoring calls.
+size_t bind_inputs(pp_problem *p, unsigned char *b)
+{
+    const int L = p->L, k = p->k;
+    const size_t bytes[10] = {(size_t)L * 8, (size_t)(L + 1) * 8, (size_t)k * 8, (size_t)k * k * 4, (size_t)k * L * 2,
+                              sizeof(PruneCtl), 8 /* best */, 4 /* err */, sizeof(pp_solution) + sizeof(PruneNote),
+                              plan_tables(L, k).total};
+    size_t off[10], total = 0;
+    for (int i = 0; i < 10; ++i) { off[i] = total; total = align_up(total + bytes[i], i < 4 ? 16 : 128); }
+    if (!b) return total;
+    p->d_inputs = b;
+    Dev &d = p->d;
+    d.bits = reinterpret_cast<uint64_t *>(b + off[0]);
+    d.M = reinterpret_cast<uint64_t *>(b + off[1]);
+    d.cap = reinterpret_cast<uint64_t *>(b + off[2]);
+    d.bw = reinterpret_cast<uint32_t *>(b + off[3]);
+    d.lo = reinterpret_cast<int16_t *>(b + off[4]);
+    p->prune.ctl = reinterpret_cast<PruneCtl *>(b + off[5]);
+    d.best = reinterpret_cast<unsigned long long *>(b + off[6]);
+    d.err = reinterpret_cast<int32_t *>(b + off[7]);
+    p->d_sol = reinterpret_cast<pp_solution *>(b + off[8]);
+    p->d_note = reinterpret_cast<PruneNote *>(b + off[8] + sizeof(pp_solution));
+    p->d_tables = b + off[9];
+    return total;
+}
+
 void ensure_windows(pp_problem *p)
 {
     if (!p->lo.empty()) return;
@@ -398,6 +478,13 @@ void fill_plan_tables(const pp_problem *p, unsigned char *out)
 pp_status upload_inputs(pp_problem *p, bool wait)
 {
     if (p->uploaded) return PP_OK;
+    const bool rec = recording(p->stream);
+    if (rec && !p->d_spare) {  // the buffer of pp_problem_create is ordered on the legacy stream, which is out of reach now
+        unsigned char *b = nullptr;
+        PP_CUDA(kept_alloc(p, &b, p->inputs_bytes, true));
+        p->d_spare = p->d_inputs;
+        bind_inputs(p, b);
+    }
     const int L = p->L, k = p->k;
     std::vector<unsigned char> st;
     try {
@@ -418,10 +505,16 @@ pp_status upload_inputs(pp_problem *p, bool wait)
     prune_ctl_init(&ctl);
     put(p->prune.ctl, &ctl, sizeof ctl);
     fill_plan_tables(p, st.data() + (p->d_tables - p->d_inputs));
-    if (wait) PP_CUDA(copy_in(p->d_inputs, st.data(), st.size()));
-    else PP_CUDA(cudaMemcpyAsync(p->d_inputs, st.data(), st.size(), cudaMemcpyHostToDevice, p->stream));
+    if (rec) {
+        OutsideCapture outside;
+        cudaStream_t via = nullptr;
+        PP_CUDA(copy_stream(&via));
+        PP_CUDA(copy_in(p->d_inputs, st.data(), st.size(), via));
+    } else if (wait) {
+        PP_CUDA(copy_in(p->d_inputs, st.data(), st.size(), nullptr));
+    } else PP_CUDA(cudaMemcpyAsync(p->d_inputs, st.data(), st.size(), cudaMemcpyHostToDevice, p->stream));
     p->uploaded = true;
-    p->tables_ready = wait;
+    p->tables_ready = wait || rec;
     return PP_OK;
 }
 
@@ -469,8 +562,10 @@ public:
                                       cudaHostAllocPortable | cudaHostAllocMapped);
         if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&c.ctl), sizeof init);
         if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&c.records), kSlots * records);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c.records, 0, kSlots * records, nullptr);
-        if (e == cudaSuccess) e = copy_in(c.ctl, init, sizeof init);  // the same stream: both are complete
+        cudaStream_t via = nullptr;
+        if (e == cudaSuccess) e = copy_stream(&via);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c.records, 0, kSlots * records, via);
+        if (e == cudaSuccess) e = copy_in(c.ctl, init, sizeof init, via);  // the same stream: both are complete
         if (e != cudaSuccess) {
             cudaFreeHost(c.base);
             cudaFree(c.ctl);
@@ -628,6 +723,7 @@ pp_status ensure_work(pp_problem *p)
     void *ptr = nullptr;
     if (alloc_should_fail()) return PP_ERR_NOMEM;
     const uint64_t bytes = workspace_bytes(p);
+    OutsideCapture outside;
     PP_CUDA(cudaMalloc(&ptr, bytes));
     p->d_work = static_cast<unsigned char *>(ptr);
     p->work_bytes = bytes;
@@ -672,8 +768,17 @@ pp_status dense_prepare(pp_problem *p)
             if (q.bytes) std::memcpy(staging.data() + q.off, q.src, q.bytes);
         DeviceMasks dmasks;
         PP_CUDA(device_masks(k, ml, &dmasks));
-        if (!p->d_dense) PP_CUDA(staging_alloc(reinterpret_cast<void **>(&p->d_dense), total, nullptr));
-        PP_CUDA(copy_in(p->d_dense, staging.data(), total));
+        {
+            const bool rec = recording(p->stream);
+            OutsideCapture outside;
+            cudaStream_t via = nullptr;
+            if (rec) PP_CUDA(copy_stream(&via));
+            if (!p->d_dense) {
+                if (rec) PP_CUDA(kept_alloc(p, &p->d_dense, total, true));
+                else PP_CUDA(staging_alloc(reinterpret_cast<void **>(&p->d_dense), total, nullptr));
+            }
+            PP_CUDA(copy_in(p->d_dense, staging.data(), total, via));
+        }
         for (auto &e : p->ev)
             if (!e) PP_CUDA(cudaEventCreate(&e));
         unsigned char *b = p->d_dense;
@@ -751,7 +856,7 @@ pp_status ensure_sparse(pp_problem *p)
 {
     if (p->d_work || p->d_sparse) return PP_OK;
     const size_t bytes = sparse_bytes(p->k, p->prune.Lp, kSparseScratchBytes);
-    PP_CUDA(staging_alloc(reinterpret_cast<void **>(&p->d_sparse), bytes, p->stream));
+    PP_CUDA(kept_alloc(p, &p->d_sparse, bytes, recording(p->stream)));
     bind_sparse(p->prune, p->d_sparse, bytes);
     return PP_OK;
 }
@@ -820,39 +925,22 @@ pp_status pp_problem_create(int32_t L, const uint64_t *layer_out_bits,
         delete p;
         return PP_ERR_NOMEM;
     }
-    // one device buffer for the inputs, the counters of the searches and a result record; the copy is
-    // queued by the first call that needs it, on the stream the problem has by then
-    const size_t bytes[10] = {(size_t)L * 8, (size_t)(L + 1) * 8, (size_t)k * 8, (size_t)k * k * 4, (size_t)k * L * 2,
-                             sizeof(PruneCtl), 8 /* best */, 4 /* err */, sizeof(pp_solution) + sizeof(PruneNote),
-                              plan_tables(L, k).total};
-    size_t off[10], total = 0;
-    for (int i = 0; i < 10; ++i) { off[i] = total; total = align_up(total + bytes[i], i < 4 ? 16 : 128); }
-    p->inputs_bytes = total;
+    // one device buffer; the copy is queued by pp_problem_set_stream or by the first call that needs it
+    p->inputs_bytes = bind_inputs(p, nullptr);
     int dev = 0;
+    unsigned char *b = nullptr;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = multiprocessors(dev, &p->sms);
-    if (e == cudaSuccess) e = staging_alloc(reinterpret_cast<void **>(&p->d_inputs), total, nullptr);
+    if (e == cudaSuccess) e = staging_alloc(reinterpret_cast<void **>(&b), p->inputs_bytes, nullptr);
     if (e != cudaSuccess) {
         pp_status rc = from_cuda(e);
         pp_problem_destroy(p);
         return rc;
     }
-    unsigned char *b = p->d_inputs;
-    Dev &d = p->d;
-    d.L = L; d.k = k;
-    d.bits = reinterpret_cast<uint64_t *>(b + off[0]);
-    d.M = reinterpret_cast<uint64_t *>(b + off[1]);
-    d.cap = reinterpret_cast<uint64_t *>(b + off[2]);
-    d.bw = reinterpret_cast<uint32_t *>(b + off[3]);
-    d.lo = reinterpret_cast<int16_t *>(b + off[4]);
-    d.best = reinterpret_cast<unsigned long long *>(b + off[6]);
-    d.err = reinterpret_cast<int32_t *>(b + off[7]);
-    p->d_sol = reinterpret_cast<pp_solution *>(b + off[8]);
-    p->d_note = reinterpret_cast<PruneNote *>(b + off[8] + sizeof(pp_solution));
-    p->d_tables = b + off[9];
+    p->d.L = L; p->d.k = k;
+    bind_inputs(p, b);
     PruneDev &q = p->prune;
     q.L = L; q.k = k; q.Lp = prune_row_pad(L, k);
-    q.ctl = reinterpret_cast<PruneCtl *>(b + off[5]);
     double lo = std::numeric_limits<double>::max(), hi = 0.0;
     quotient_range(L, p->bits.data(), k * k, p->bw.data(), &lo, &hi);
     prune_key_range(hi > 0.0 ? lo : 1.0, hi > 0.0 ? hi : 1.0, &q);
@@ -865,8 +953,10 @@ void pp_problem_destroy(pp_problem *p)
 {
     if (!p) return;
     if (p->own_work && p->d_work) cudaFree(p->d_work);
-    for (unsigned char *q : {p->d_inputs, p->d_sparse, p->d_dense})
-        if (q) cudaFreeAsync(q, p->stream);  // ordered after the problem's queued work
+    for (unsigned char *q : {p->d_inputs, p->d_spare, p->d_sparse, p->d_dense})
+        if (q && std::find(p->mallocs, p->mallocs + p->n_mallocs, q) == p->mallocs + p->n_mallocs)
+            cudaFreeAsync(q, p->stream);  // ordered after the problem's queued work
+    for (int i = 0; i < p->n_mallocs; ++i) cudaFree(p->mallocs[i]);
     for (auto &e : p->ev)
         if (e) cudaEventDestroy(e);
     delete p;
@@ -876,7 +966,7 @@ pp_status pp_problem_set_stream(pp_problem *p, void *cuda_stream)
 {
     if (!p) return PP_ERR_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    if (s != p->stream && (p->uploaded || p->d_sparse)) {  // copies and scratch are ordered there
+    if (s != p->stream && (p->uploaded || p->d_sparse) && !recording(s)) {  // copies and scratch are ordered there
         PP_CUDA(cudaStreamSynchronize(p->stream));
         p->tables_ready = p->uploaded;
     }

@@ -108,3 +108,56 @@ def test_first_calls_over_plans_are_plain_launches():
             del g
             call(p)  # the handle does not live on the graph's memory
             check(name)
+
+
+@pytest.mark.parametrize("L,k,mode,workspace", [(12, 6, -1, False), (50, 10, -1, False), (90, 12, -1, False), (337, 9, -1, False),
+                                                (50, 10, 0, False), (60, 9, 0, True), (100, 14, -1, True)])
+def test_handle_that_meets_its_stream_in_a_recording(L, k, mode, workspace):
+    # created before, used for the first time while a graph is recorded: nothing of the handle belongs to the graph
+    import torch
+    inst = W.random_small(97000 + L, L, k)
+    inst.node_mem_bytes[:] = np.uint64(int(inst.layer_mem_bytes.sum()) // 3 + 1)
+    want = oracle.dp_fact(inst, 8)
+    nseg, ends, nodes = W.random_plans(inst, 300, seed=L, invalid_fraction=0.2)
+    scored = oracle.eval_plans(inst, nseg, ends, nodes)
+    dev = [torch.from_numpy(a).cuda() for a in (nseg, ends, nodes)]
+    sol = torch.zeros(22, dtype=torch.float64, device="cuda")
+    beta = torch.zeros(300, dtype=torch.float64, device="cuda")
+    stat = torch.zeros(300, dtype=torch.uint8, device="cuda")
+
+    def check():
+        torch.cuda.synchronize()
+        got = record(sol)
+        assert got.status == want.status and got.beta_ms == want.beta_ms
+        assert (got.m, tuple(got.cuts[: got.m - 1]), tuple(got.placement[: got.m])) == want.plan()
+        assert np.array_equal(beta.cpu().numpy(), scored[0]) and np.array_equal(stat.cpu().numpy(), scored[1])
+        for t in (sol, beta, stat):
+            t.zero_()
+        torch.cuda.synchronize()
+
+    def calls(p):
+        p.solve_exact_dev(sol.data_ptr())
+        p.eval_plans_dev(300, *(a.data_ptr() for a in dev), beta.data_ptr(), stat.data_ptr())
+
+    for first_elsewhere in (False, True):
+        with pp.Problem.from_instance(inst) as p:
+            p.force_generic(mode)
+            if workspace:
+                p.set_workspace(torch.empty(p.workspace_bytes(), dtype=torch.uint8, device="cuda"))
+            if first_elsewhere:
+                calls(p)
+                check()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g):
+                p.set_stream(torch.cuda.current_stream().cuda_stream)
+                calls(p)
+            for _ in range(3):
+                g.replay()
+                check()
+            del g
+            s = torch.cuda.Stream()
+            p.set_stream(s.cuda_stream)
+            calls(p)
+            check()
+            got = p.solve_exact()
+            assert got.beta_ms == want.beta_ms and got.plan() == want.plan()

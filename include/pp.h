@@ -417,6 +417,11 @@ pp_status pp_debug_fail_alloc(int32_t nth);
  * it is sound. */
 pp_status pp_debug_starve(int32_t polls);
 
+/* Test hook: how many accesses to their tables the kernels of one source have checked since the last call, in
+ * the bounds-checking build; 0 in the normal one.  kernel: 0 = bounded search, 1 = batched search with an
+ * instance to a block, 2 = placement stage, 3 = evaluator, 4 = random plans.  Synchronises the device. */
+pp_status pp_debug_bounds_checks(int32_t kernel, uint64_t *n);
+
 /* Force (1) or forbid (0) the generic sweep kernel; 2 = automatic choice among the kernels that
  * take one source mask per warp (the two-mask kernel is left out); 3 = the two-mask kernel on every
  * level it can run, however small; -1 restores the automatic choice.  Meant for tests that want

@@ -29,7 +29,7 @@ EXPORTS = (
     "pp_greedy_batch_dev", "pp_random_plans", "pp_random_plans_dev", "pp_debug_minmax_rate",
     "pp_problem_set_profiling", "pp_eval_plans_packed", "pp_eval_plans_packed_dev",
     "pp_partition_minsum_batch", "pp_partition_minsum_batch_dev",
-    "pp_kpath_colour_batch", "pp_kpath_colour_batch_dev", "pp_debug_fail_alloc", "pp_debug_starve",
+    "pp_kpath_colour_batch", "pp_kpath_colour_batch_dev", "pp_debug_fail_alloc", "pp_debug_starve", "pp_debug_bounds_checks",
     "pp_kpath_matching", "pp_solve_exact_compute",
 )
 
@@ -96,6 +96,7 @@ def lib() -> ctypes.CDLL:
         L.pp_kpath_colour_batch_dev.argtypes = [i32, vp, i64, i32] + [vp] * 8
         L.pp_debug_fail_alloc.argtypes = [i32]
         L.pp_debug_starve.argtypes = [i32]
+        L.pp_debug_bounds_checks.argtypes = [i32, ctypes.POINTER(u64)]
         L.pp_kpath_matching.argtypes = [i32, vp, i32, vp, i32, i32, vp, vp, vp, vp]
         L.pp_solve_exact_compute.argtypes = [i32, vp, vp, vp, i32] + [vp] * 7
         L.pp_status_str.argtypes = [ctypes.c_int]
@@ -445,6 +446,13 @@ def solve_exact_compute(inst, layer_work, node_speed) -> Solution:
 def debug_fail_alloc(nth: int):
     """pp_debug_fail_alloc: the nth device allocation from now on reports out of memory (0 clears)."""
     _check(lib().pp_debug_fail_alloc(int(nth)), "pp_debug_fail_alloc")
+
+
+def debug_bounds_checks(kernel: int) -> int:
+    """pp_debug_bounds_checks: accesses checked by the kernels of one source since the last call."""
+    n = ctypes.c_uint64()
+    _check(lib().pp_debug_bounds_checks(int(kernel), ctypes.byref(n)), "pp_debug_bounds_checks")
+    return int(n.value)
 
 
 def debug_starve(polls: int):

@@ -67,8 +67,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
 
 def build_debug(force: bool = False) -> str:
-    """The bounds-checking build of the same sources, libpp_dbg.so: every index into the state table
-    and the rank table is checked, a violation sets the device error word instead of trapping."""
+    """The bounds-checking build of the same sources, libpp_dbg.so: every index into the tables of the searches,
+    the placement stage and the scoring kernels is checked, a violation is recorded and reported instead of trapping."""
     return _build(LIB_DEBUG, "_dbg", ["-DPP_DEBUG_BOUNDS"], force, False)
 
 

@@ -1608,6 +1608,7 @@ static pp_status match_one_launch(int32_t n, const uint32_t *bw, int32_t n_cuts,
     d.stride = sms;
     d.out = &slot.match;
     slot.match.status = (int)PP_ERR_CUDA;
+    slot.match.bounds = 0;
     const size_t nn = (size_t)n * n, at = match_runs_at(n, trials), words = at + order.size() * (sizeof(MatchRun) / 4);
     std::unique_ptr<uint32_t[]> in(new uint32_t[words]);
     std::memcpy(in.get(), bw, nn * 4);
@@ -1632,6 +1633,7 @@ static pp_status match_one_launch(int32_t n, const uint32_t *bw, int32_t n_cuts,
         return e != cudaSuccess ? from_cuda(e) : e2 != cudaSuccess ? from_cuda(e2) : PP_ERR_CUDA;
     }
     const MatchOut &got = slot.match;
+    if (got.bounds) return PP_ERR_CUDA;
     std::copy(got.nodes, got.nodes + n_cuts + 1, nodes);
     if (cut_threshold) std::copy(got.threshold, got.threshold + n_cuts, cut_threshold);
     return static_cast<pp_status>(got.status);
@@ -1882,6 +1884,14 @@ pp_status pp_debug_starve(int32_t polls)
 {
     if (polls < 0) return PP_ERR_ARG;
     g_starved_polls.store(polls);
+    return PP_OK;
+}
+
+pp_status pp_debug_bounds_checks(int32_t kernel, uint64_t *n)
+{
+    unsigned long long (*const of[5])() = {prune_checks, batch_checks, match_checks, eval_checks, random_checks};
+    if (!n || kernel < 0 || kernel >= 5) return PP_ERR_ARG;
+    *n = of[kernel]();
     return PP_OK;
 }
 

@@ -91,6 +91,8 @@ __host__ __device__ inline BatchLayout batch_layout(int L, int k)
 
 }  // namespace
 
+PP_CHECKS_OF(batch)
+
 size_t batch_smem_bytes(int L, int k)
 {
     if (k > 12) return (size_t)1 << 40;  // compact rows are 16-bit numbers
@@ -142,6 +144,8 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
     const double kInf = __longlong_as_double(0x7FF0000000000000ll);
     const uint32_t FULL = 0xFFFFFFFFu;
     const int kk = k * k, jmax = k < L ? k : L;
+    PP_BLOCK_BOUNDS(chk);
+    [[maybe_unused]] const size_t n_dp = ((size_t)k << (k - 1)) * Ls, n_rank = (size_t)kk * Ls;  // entries of the tables
     for (uint32_t S = tid; S < (1u << k); S += kBatchThreads) rowoff[S] = (uint16_t)t_rowoff[S];
 
     for (int64_t inst = blockIdx.x; inst < B; inst += gridDim.x) {
@@ -165,6 +169,7 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
             s_fast = s_U = s_D = 0u;
             s_best = kNoBest;
             M[0] = 0ull;
+            PP_RESET(chk);
         }
         __syncthreads();
         bool bad = false;
@@ -286,9 +291,9 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
                 if (u >= 0 && c < L) {
                     uint32_t d = cls[c];
                     if (d & 0x8000u) d = cls[d & 0x7FFFu];
-                    r = rk[u * D + (int)d];
+                    if (PP_IN_BOUNDS(chk, u * D + (int)d, U * D)) r = rk[u * D + (int)d];
                 }
-                rank[pr * Ls + c] = (uint16_t)r;
+                if (PP_IN_BOUNDS(chk, pr * Ls + c, n_rank)) rank[pr * Ls + c] = (uint16_t)r;
             }
         }
         __syncthreads();  // the per-entry ranks share their bytes with the state table
@@ -296,7 +301,7 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
         for (int v = wid; v < k; v += kBatchWarps)
             for (int c = lane; c < Ls; c += 32) {
                 const bool fits = c < L && M[c + 1] <= cap[v];
-                dp[(size_t)rowoff[1u << v] * Ls + c] = (uint16_t)(fits ? 0u : kInf16);
+                if (PP_IN_BOUNDS(chk, (size_t)rowoff[1u << v] * Ls + c, n_dp)) dp[(size_t)rowoff[1u << v] * Ls + c] = (uint16_t)(fits ? 0u : kInf16);
                 if (fits && c == L - 1) atomicMin(&s_best, pack_best(0u, 1, 1u << v, v));
             }
         __syncthreads();
@@ -318,6 +323,7 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
 #pragma unroll
                         for (int i = 0; i < P / 2; i += 2) {
                             if (at + 2 * i >= Ls) break;
+                            if (!PP_IN_BOUNDS(chk, src - dp + 2 * i + 3, n_dp) || !PP_IN_BOUNDS(chk, rw - rank + v * k * Ls + 2 * i + 3, n_rank)) break;
                             const uint2 a = *reinterpret_cast<const uint2 *>(src + 2 * i);
                             const uint2 b = *reinterpret_cast<const uint2 *>(rw + v * k * Ls + 2 * i);
                             g2[i] = __vminu2(g2[i], __vmaxu2(a.x, b.x));
@@ -334,7 +340,7 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
                 uint16_t *dst = dp + (size_t)row * Ls + at;
 #pragma unroll
                 for (int i = 0; i < P; i += 4)
-                    if (at + i < Ls) {
+                    if (at + i < Ls && PP_IN_BOUNDS(chk, dst - dp + i + 3, n_dp)) {
                         *reinterpret_cast<uint2 *>(dst + i) = make_uint2(out[i] | (out[i + 1] << 16), out[i + 2] | (out[i + 3] << 16));
 #pragma unroll
                         for (int q = i; q < i + 4; ++q)
@@ -356,7 +362,7 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
             if (tid == 0) {
                 o_beta[inst] = kInf;
                 o_m[inst] = 0;
-                o_status[inst] = bad ? (int8_t)PP_ERR_LIMIT : (int8_t)PP_INFEASIBLE;
+                o_status[inst] = bad ? (int8_t)PP_ERR_LIMIT : PP_BROKEN(chk) ? (int8_t)PP_ERR_CUDA : (int8_t)PP_INFEASIBLE;
             }
             continue;
         }
@@ -382,7 +388,8 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
                 const uint16_t *row = dp + (size_t)rowoff[from] * Ls + c, *rw = rank + (size_t)w * Ls + c;
                 for (uint32_t rem = from; rem; rem &= rem - 1, row += Ls) {
                     const int v = __ffs(rem) - 1;
-                    if (max((uint32_t)*row, (uint32_t)rw[v * k * Ls]) <= rstar) pick = min(pick, ((unsigned)c << 5) | (unsigned)v);
+                    if (PP_IN_BOUNDS(chk, row - dp, n_dp) && PP_IN_BOUNDS(chk, rw - rank + v * k * Ls, n_rank) &&
+                        max((uint32_t)*row, (uint32_t)rw[v * k * Ls]) <= rstar) pick = min(pick, ((unsigned)c << 5) | (unsigned)v);
                 }
                 pick = __reduce_min_sync(FULL, pick);
             }
@@ -394,6 +401,7 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
             w = (int)(pick & 31u);
             c2 = (int)(pick >> 5);
         }
+        if (PP_BROKEN(chk)) status = (int)PP_ERR_CUDA;
         // beta* is the bottleneck of the plan: no link of it ranks above the optimum, and no plan is better
         const int next = __shfl_down_sync(FULL, my_node, 1);
         double x = 0.0;

@@ -19,6 +19,8 @@
 
 namespace pp {
 
+PP_CHECKS_OF(eval)
+
 namespace {
 
 constexpr int kEvalThreads = 256;
@@ -59,6 +61,8 @@ k_eval(const int L, const int k, const unsigned char *__restrict__ tables, const
     const uint16_t *s_fwd = reinterpret_cast<const uint16_t *>(smem_eval + tab.fwd);
     uint16_t *s_ends = reinterpret_cast<uint16_t *>(smem_eval + lay.ends);
     uint8_t *s_nodes = smem_eval + lay.nodes;
+    PP_BLOCK_BOUNDS(chk);
+    [[maybe_unused]] const size_t n_fwd = (size_t)k1 * L + 1, n_bw = (size_t)k1 * k1;  // entries of the tables
     __shared__ uint8_t s_order[kEvalThreads], s_m[kEvalThreads];
     __shared__ uint32_t s_start[kEvalThreads];  // PACKED: first entry of the row within the staged stretch, or kFar
     __shared__ uint32_t s_first[2][32];
@@ -178,6 +182,7 @@ k_eval(const int L, const int k, const unsigned char *__restrict__ tables, const
                 twice = twice || ((used >> n) & 1u);  // node n again, or no such node
                 used |= 1u << n;
                 late = late || (uint32_t)(e - first) >= (uint32_t)(L - 1 - first);
+                if (!PP_IN_BOUNDS(chk, n * L + first, n_fwd) || !PP_IN_BOUNDS(chk, n * k1 + next, n_bw) || !PP_IN_BOUNDS(chk, e, L)) break;
                 full = full || (uint32_t)(e - first) >= s_fwd[n * L + first];
                 const uint32_t link = s_bw[n * k1 + next];
                 dead = dead || link == 0u;
@@ -190,7 +195,7 @@ k_eval(const int L, const int k, const unsigned char *__restrict__ tables, const
                 n = next;
             }
             twice = twice || ((used >> n) & 1u);
-            full = full || (uint32_t)(L - 1 - first) >= s_fwd[n * L + first];
+            if (PP_IN_BOUNDS(chk, n * L + first, n_fwd)) full = full || (uint32_t)(L - 1 - first) >= s_fwd[n * L + first];
             flags = (twice ? PP_PLAN_BAD_NODE : 0) | (late ? PP_PLAN_BAD_ENDS : 0);
             if (!flags) flags = (full ? PP_PLAN_MEMORY : 0) | (dead ? PP_PLAN_DEAD_LINK : 0);
             if (!flags) bt = __ddiv_rn((double)num, (double)den);
@@ -204,6 +209,7 @@ k_eval(const int L, const int k, const unsigned char *__restrict__ tables, const
                 score([&](int j) { return (int)nodes[(size_t)far + j]; }, [&](int j) { return (int)ends[(size_t)far + j]; });
             }
         }
+        if (PP_BROKEN(chk)) flags = 255;
         beta[b] = bt;
         status[b] = (uint8_t)flags;
     }

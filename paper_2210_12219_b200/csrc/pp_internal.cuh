@@ -48,16 +48,51 @@ static constexpr unsigned long long kNoBest = ~0ull;
 static constexpr int32_t kErrBacktrack = 1;  // the backtrack found no predecessor (inconsistent table)
 static constexpr int32_t kErrBounds = 3;     // bounds-checking build: an index left its table
 
-// Bounds-checking build (-DPP_DEBUG_BOUNDS, libpp_dbg.so): every access to the state table and to
-// the rank table in global memory goes through PP_IN_BOUNDS, which records kErrBounds in the
-// device error word and makes the caller skip the access when the index is outside the table.
-// Nothing traps; the solve then returns PP_ERR_CUDA.  In the normal build the check is `true`.
+// Bounds-checking build (-DPP_DEBUG_BOUNDS, libpp_dbg.so): every access to a table of the searches (states and
+// ranks, the bounded search's rows, keys, maps and lists, the placement stage's table of bottlenecks) and every
+// look of the scoring kernels into their tables goes through PP_IN_BOUNDS, which counts it, records kErrBounds
+// in an error word and makes the caller skip the access when the index is outside the table.
+// Nothing traps; the solve then reports PP_ERR_CUDA, a scoring kernel the status 255 for the plans of the
+// block.  In the normal build the check is `true`.
+struct Bounds {
+    int32_t *err;
+};
 #ifdef PP_DEBUG_BOUNDS
-#define PP_IN_BOUNDS(d, index, limit) \
-    ((uint64_t)(index) < (uint64_t)(limit) ? true : (atomicCAS((d).err, 0, kErrBounds), false))
+static __device__ unsigned long long pp_checks;  // made by the kernels of this source
+__device__ __forceinline__ bool pp_check(int32_t *err, bool ok)
+{
+    atomicAdd(&pp_checks, 1ull);
+    if (!ok) atomicCAS(err, 0, kErrBounds);
+    return ok;
+}
+#define PP_IN_BOUNDS(d, index, limit) pp::pp_check((d).err, (uint64_t)(index) < (uint64_t)(limit))
+// an error word of the block; the block synchronises before the first check
+#define PP_BLOCK_BOUNDS(name)          \
+    __shared__ int32_t name##_word;    \
+    const Bounds name{&name##_word};   \
+    if (threadIdx.x == 0) name##_word = 0
+#define PP_RESET(name) *(name).err = 0
+#define PP_BROKEN(name) (*reinterpret_cast<volatile int32_t *>((name).err) != 0)
+#define PP_CHECKS_OF(name)                                              \
+    unsigned long long name##_checks()                                  \
+    {                                                                   \
+        unsigned long long n = 0, zero = 0;                             \
+        if (cudaMemcpyFromSymbol(&n, pp_checks, sizeof n) != cudaSuccess || cudaMemcpyToSymbol(pp_checks, &zero, sizeof n) != cudaSuccess) return 0; \
+        return n;                                                       \
+    }
 #else
 #define PP_IN_BOUNDS(d, index, limit) true
+#define PP_BLOCK_BOUNDS(name) [[maybe_unused]] const Bounds name{nullptr}
+#define PP_RESET(name) (void)0
+#define PP_BROKEN(name) false
+#define PP_CHECKS_OF(name) unsigned long long name##_checks() { return 0; }
 #endif
+// Checks made by the kernels of one source since the last call (pp_debug_bounds_checks); synchronises.
+unsigned long long prune_checks();
+unsigned long long batch_checks();
+unsigned long long match_checks();
+unsigned long long eval_checks();
+unsigned long long random_checks();
 
 // final-state key: smaller is better; rank in the high bits, then popcount, mask, node
 __host__ __device__ inline unsigned long long pack_best(uint32_t rank, int popc, uint32_t mask, int v)
@@ -149,6 +184,7 @@ struct PruneCtl {              // device; the kernel leaves it as it found it
                                // blocks that have arrived at the level's end
     uint32_t left;             // blocks that have left
     uint32_t failed;           // a barrier ran out of polls: the other blocks need not wait any longer
+    int32_t err;               // bounds-checking build: kErrBounds when an index left its table
 };
 struct PruneNote {             // what the host learns about a launch
     long long ns;              // duration on the device
@@ -238,6 +274,7 @@ struct MatchRun {
     int32_t first, cuts;       // a run of cuts of one class, in serving order
 };
 struct MatchOut {
+    int32_t bounds;            // bounds-checking build: 1 when an index left the table
     int32_t status, nodes[64];
     uint32_t threshold[64];
 };

@@ -91,6 +91,8 @@ __global__ void __launch_bounds__(kMatchThreads, 1) k_match(const __grid_constan
     __shared__ uint32_t s_thr[64];
     __shared__ MatchRun s_runs[kMaxRuns];
     __shared__ unsigned long long s_top[kMatchWarps], s_path[2];
+    PP_BLOCK_BOUNDS(chk);
+    [[maybe_unused]] const size_t n_w = (size_t)n << d.kk, n_bw = (size_t)n * n + kPadWords;  // entries of the tables
     const uint32_t *g_bw = d.bw, *g_draws = d.draws;
     const MatchRun *g_runs = d.runs;
     if constexpr (WORDS > 0) {
@@ -138,7 +140,8 @@ __global__ void __launch_bounds__(kMatchThreads, 1) k_match(const __grid_constan
     if (tid < n) s_bw[tid * n + tid] = 0u;
     // colours of a colouring for a path of `vertices`, and an empty table
     auto prepare = [&](uint32_t dr, int vertices) {
-        for (uint32_t e = tid; e < (uint32_t)n << vertices; e += kMatchThreads) W[e] = 0u;
+        for (uint32_t e = tid; e < (uint32_t)n << vertices; e += kMatchThreads)
+            if (PP_IN_BOUNDS(chk, e, n_w)) W[e] = 0u;
         if (tid < n) s_col[tid] = (uint8_t)__umulhi(dr, (uint32_t)vertices);
     };
     prepare(draw, s_runs[0].cuts + 1);
@@ -159,7 +162,7 @@ __global__ void __launch_bounds__(kMatchThreads, 1) k_match(const __grid_constan
                 prepare(tid < n ? g_draws[(size_t)t * n + tid] : 0u, kk);
             }
             __syncthreads();
-            if (tid < n && tid != uv && ((alive >> tid) & 1ull) && (sv < 0 || sv == tid)) W[(1u << s_col[tid]) * n + tid] = kFull;
+            if (tid < n && tid != uv && ((alive >> tid) & 1ull) && (sv < 0 || sv == tid) && PP_IN_BOUNDS(chk, (1u << s_col[tid]) * n + tid, n_w)) W[(1u << s_col[tid]) * n + tid] = kFull;
             // this lane's two vertices as path ends; a node that is not available has no colour
             const int v0 = lane, v1 = lane + 32;
             const int r0 = v0 < n ? v0 : 0, r1 = v1 < n ? v1 : 0;
@@ -181,6 +184,7 @@ __global__ void __launch_bounds__(kMatchThreads, 1) k_match(const __grid_constan
                     for (; u + kAhead <= to; u += kAhead) {
 #pragma unroll
                         for (int i = 0; i < kAhead; ++i) {
+                            if (!PP_IN_BOUNDS(chk, C * n + u + i, n_w) || !PP_IN_BOUNDS(chk, lane + (u + i) * n + 32, n_bw)) break;
                             const uint32_t x = row[u + i];
                             w0 = max(w0, min(x, bw[(u + i) * n]));
                             w1 = max(w1, min(x, bw[(u + i) * n + 32]));
@@ -190,6 +194,7 @@ __global__ void __launch_bounds__(kMatchThreads, 1) k_match(const __grid_constan
 #pragma unroll
                         for (int i = 0; i < kAhead - 1; ++i) {
                             const int ui = min(u + i, to - 1);  // the last one again where there are none left
+                            if (!PP_IN_BOUNDS(chk, C * n + ui, n_w) || !PP_IN_BOUNDS(chk, lane + ui * n + 32, n_bw)) break;
                             const uint32_t x = row[ui];
                             w0 = max(w0, min(x, bw[ui * n]));
                             w1 = max(w1, min(x, bw[ui * n + 32]));
@@ -197,19 +202,19 @@ __global__ void __launch_bounds__(kMatchThreads, 1) k_match(const __grid_constan
                     }
                     // one source set per entry: no other set writes it
                     if (cut == 0) {
-                        if (e0 & ~C) W[(C | e0) * n + v0] = w0;
-                        if (e1 & ~C) W[(C | e1) * n + v1] = w1;
+                        if ((e0 & ~C) && PP_IN_BOUNDS(chk, (C | e0) * n + v0, n_w)) W[(C | e0) * n + v0] = w0;
+                        if ((e1 & ~C) && PP_IN_BOUNDS(chk, (C | e1) * n + v1, n_w)) W[(C | e1) * n + v1] = w1;
                     } else {
-                        if ((e0 & ~C) && w0) atomicMax(&W[(C | e0) * n + v0], w0);
-                        if ((e1 & ~C) && w1) atomicMax(&W[(C | e1) * n + v1], w1);
+                        if ((e0 & ~C) && w0 && PP_IN_BOUNDS(chk, (C | e0) * n + v0, n_w)) atomicMax(&W[(C | e0) * n + v0], w0);
+                        if ((e1 & ~C) && w1 && PP_IN_BOUNDS(chk, (C | e1) * n + v1, n_w)) atomicMax(&W[(C | e1) * n + v1], w1);
                     }
                 }
             }
             __syncthreads();
             if (wid == 0) {
                 const uint32_t *row = W + all * n;
-                const uint32_t x0 = v0 < n && (uv < 0 || uv == v0) ? row[v0] : 0u;
-                const uint32_t x1 = v1 < n && (uv < 0 || uv == v1) ? row[v1] : 0u;
+                const uint32_t x0 = v0 < n && (uv < 0 || uv == v0) && PP_IN_BOUNDS(chk, all * n + v0, n_w) ? row[v0] : 0u;
+                const uint32_t x1 = v1 < n && (uv < 0 || uv == v1) && PP_IN_BOUNDS(chk, all * n + v1, n_w) ? row[v1] : 0u;
                 const uint32_t b = __reduce_max_sync(kFull, max(x0, x1));
                 const unsigned long long key = ((unsigned long long)b << 32) | (uint32_t)~t;
                 if (b != 0u && key > best) {
@@ -222,8 +227,9 @@ __global__ void __launch_bounds__(kMatchThreads, 1) k_match(const __grid_constan
                         if (i == 0) break;
                         C &= ~(1u << s_col[v]);
                         const uint32_t *prev = W + C * n;
-                        const bool h0 = (min(prev[r0], s_bw[r0 * n + v]) >= b) & in0;
-                        const bool h1 = (min(prev[r1], s_bw[r1 * n + v]) >= b) & in1;
+                        const bool ok = PP_IN_BOUNDS(chk, C * n + max(r0, r1), n_w) && PP_IN_BOUNDS(chk, max(r0, r1) * n + v, n_bw);
+                        const bool h0 = ok && (min(prev[r0], s_bw[r0 * n + v]) >= b) & in0;
+                        const bool h1 = ok && (min(prev[r1], s_bw[r1 * n + v]) >= b) & in1;
                         v = lowest(__ballot_sync(kFull, h0), __ballot_sync(kFull, h1));
                     }
                 }
@@ -291,6 +297,7 @@ __global__ void __launch_bounds__(kMatchThreads, 1) k_match(const __grid_constan
             __syncthreads();
         }
     }
+    if (PP_BROKEN(chk) && tid == 0) d.out->bounds = 1;
     if (blockIdx.x == 0) {
         for (int j = tid; j <= d.n_cuts; j += kMatchThreads) d.out->nodes[j] = fail ? -1 : s_nodes[j];
         for (int j = tid; j < d.n_cuts; j += kMatchThreads) d.out->threshold[j] = s_thr[j];
@@ -299,6 +306,8 @@ __global__ void __launch_bounds__(kMatchThreads, 1) k_match(const __grid_constan
 }
 
 }  // namespace
+
+PP_CHECKS_OF(match)
 
 size_t match_smem_bytes(int n, int kk) { return ((size_t)n * n + kPadWords + ((size_t)n << kk)) * 4 + ((size_t)2 << kk); }
 

@@ -172,6 +172,34 @@ __device__ __forceinline__ void store_row(uint32_t *p, const uint32_t (&x)[P])
     }
 }
 
+// The same at index i of a table of n entries: checked in the bounds-checking build, where a value from outside
+// reads as 0 and a row as +inf.
+template <bool SM, typename T>
+__device__ __forceinline__ T ld_at(const Bounds &chk, const T *table, size_t i, size_t n)
+{
+    return PP_IN_BOUNDS(chk, i, n) ? ld_now<SM>(table + i) : T(0);
+}
+template <typename T>
+__device__ __forceinline__ void st_at(const Bounds &chk, T *table, size_t i, size_t n, T x)
+{
+    if (PP_IN_BOUNDS(chk, i, n)) table[i] = x;
+}
+template <int P, bool CA>
+__device__ __forceinline__ void load_row_at(const Bounds &chk, const uint32_t *table, size_t i, size_t n, uint32_t (&x)[P])
+{
+    if (PP_IN_BOUNDS(chk, i, n) && PP_IN_BOUNDS(chk, i + P - 1, n)) {
+        load_row<P, CA>(table + i, x);
+    } else {
+#pragma unroll
+        for (int q = 0; q < P; ++q) x[q] = kInfKey;
+    }
+}
+template <int P>
+__device__ __forceinline__ void store_row_at(const Bounds &chk, uint32_t *table, size_t i, size_t n, const uint32_t (&x)[P])
+{
+    if (PP_IN_BOUNDS(chk, i, n) && PP_IN_BOUNDS(chk, i + P - 1, n)) store_row<P>(table + i, x);
+}
+
 // All blocks of the grid; false when the wait ran out, here or in another block (the caller reports it and
 // leaves by the end of the kernel, so that the counters are cleared).  A level's word holds the blocks
 // that have arrived above the node sets it added (32 bits each), so that the last poll brings both; *best,
@@ -260,6 +288,10 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
     uint32_t *t_gmin = SM ? reinterpret_cast<uint32_t *>(tables + tl.gmin) : d.gmin;
     uint32_t *t_rows = SM ? reinterpret_cast<uint32_t *>(tables + tl.rows) : d.rows;
     [[maybe_unused]] uint32_t *t_seg = SM ? t_rows + (((size_t)k << (k - 1)) * Lp) : d.seg;
+    // entries of the tables
+    [[maybe_unused]] const Bounds chk{&ctl->err};
+    [[maybe_unused]] const size_t n_sets = (size_t)1 << k, n_map = (size_t)k << k, n_gam = (size_t)k * k * Lp, n_rows = (size_t)d.row_cap * Lp,
+                                  n_seg = (size_t)k * L * Lp;
     const double kInf = __longlong_as_double(0x7FF0000000000000ll);
     const int top = k < L ? k : L;
     const uint32_t full = (1u << k) - 1u;
@@ -380,11 +412,11 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
             for (int i = 1; i < P; ++i) cur[i] = g[i - 1];
 #pragma unroll
             for (int i = 0; i < P; ++i) out[i] = kInfKey;
-            const uint32_t *seg = t_seg + (size_t)w * L * Lp + at0;
+            const size_t seg = (size_t)w * L * Lp + at0;
             for (int d0 = 0; d0 < L; d0 += kAhead) {  // the loads of kAhead steps are in flight together
                 uint32_t x[kAhead][P];
 #pragma unroll
-                for (int u = 0; u < kAhead; ++u) load_row<P, true>(seg + (size_t)min(d0 + u, L - 1) * Lp, x[u]);
+                for (int u = 0; u < kAhead; ++u) load_row_at<P, true>(chk, t_seg, seg + (size_t)min(d0 + u, L - 1) * Lp, n_seg, x[u]);
                 bool more = false;
 #pragma unroll
                 for (int u = 0; u < kAhead; ++u) {
@@ -465,7 +497,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
         const int slots = nblk * kWarps, my_slot = wid * nblk + (nblk == 1 ? 0 : (int)blockIdx.x);
         // node sets of three nodes and more start without rows (those of two nodes are all written below)
         for (uint32_t S = (nblk == 1 ? 0 : blockIdx.x) * kThreads + tid; S < (1u << k); S += nblk * kThreads)
-            if (__popc(S) > 2) t_live[S] = 0u;
+            if (__popc(S) > 2) st_at(chk, t_live, S, n_sets, 0u);
         if constexpr (CT) {
             // compute times of every run of layers: seg[(w * L + d) * Lp + c'] = layers c'-d .. c' on w
             const int n = k * L * Lp;
@@ -475,7 +507,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                 const uint32_t sp = s_speed[w];
                 if (c2 < L && first >= 0 && sp != 0 && s_M[c2 + 1] - s_M[first] <= s_cap[w])
                     key = key_of(__ddiv_rn((double)(s_Wp[c2 + 1] - s_Wp[first]), (double)sp));
-                t_seg[e] = key;
+                st_at(chk, t_seg, e, n_seg, key);
             }
             if (tid == 0)
                 for (int v = 0; v < k; ++v) {
@@ -516,7 +548,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                                 if (lo[q] < c) t[q] = 31 - __clz(c - lo[q]);
                             }
                             if (c < Lp) {
-                                t_gam[(size_t)(w * k + v) * Lp + c] = key;
+                                st_at(chk, t_gam, (size_t)(w * k + v) * Lp + c, n_gam, key);
                                 team_row[c] = x[q];
                             }
                         }
@@ -572,14 +604,14 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
 #pragma unroll
                             for (int q = 0; q < kOwn; ++q) {
                                 const int c = in_team + q * kTeam;
-                                if (c < Lp) t_rows[(size_t)id * Lp + c] = out[q];
+                                if (c < Lp) st_at(chk, t_rows, (size_t)id * Lp + c, n_rows, out[q]);
                             }
                         if (in_team == 0) {
-                            t_gmin[w * k + v] = gm;
-                            t_rowmap[(size_t)S2 * k + w] = ((unsigned long long)least << 32) | id;
+                            st_at(chk, t_gmin, w * k + v, k * k, gm);
+                            st_at(chk, t_rowmap, (size_t)S2 * k + w, n_map, ((unsigned long long)least << 32) | id);
                             if (w == b) {
-                                t_list[pr] = S2;
-                                t_live[S2] = S2;
+                                st_at(chk, t_list, pr, n_sets, S2);
+                                st_at(chk, t_live, S2, n_sets, S2);
                             }
                         }
                     }
@@ -598,9 +630,9 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                     g[i] = (link != 0 && c < L) ? key_of(__ddiv_rn(s_bits[c], div)) : kInfKey;
                     if (c < L - 1) gm = min(gm, g[i]);
                 }
-                if (on && in_row) store_row<P>(t_gam + (size_t)(w * k + v) * Lp + at, g);
+                if (on && in_row) store_row_at<P>(chk, t_gam, (size_t)(w * k + v) * Lp + at, n_gam, g);
                 gm = group_min<G>(gm);
-                if (on && sl == 0) t_gmin[w * k + v] = gm;
+                if (on && sl == 0) st_at(chk, t_gmin, w * k + v, k * k, gm);
 #pragma unroll
                 for (int i = 0; i < P; ++i) {
                     const int c = at + i;
@@ -612,12 +644,12 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                 const int a = v < w ? v : w, b = v < w ? w : v;
                 const int pr = a * (2 * k - a - 1) / 2 + (b - a - 1);
                 const uint32_t id = 2u * (uint32_t)pr + (w == b ? 1u : 0u);
-                if (keep && in_row) store_row<P>(t_rows + (size_t)id * Lp + at, out);
+                if (keep && in_row) store_row_at<P>(chk, t_rows, (size_t)id * Lp + at, n_rows, out);
                 if (on && sl == 0) {
-                    t_rowmap[(size_t)S2 * k + w] = ((unsigned long long)rmin << 32) | id;
+                    st_at(chk, t_rowmap, (size_t)S2 * k + w, n_map, ((unsigned long long)rmin << 32) | id);
                     if (w == b) {
-                        t_list[pr] = S2;
-                        t_live[S2] = S2;
+                        st_at(chk, t_list, pr, n_sets, S2);
+                        st_at(chk, t_live, S2, n_sets, S2);
                     }
                 }
                 __syncwarp();
@@ -626,7 +658,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                 status = (int)PP_ERR_CUDA;
                 break;
             }
-            for (int e = tid; e < k * k; e += kThreads) s_gmin[e] = (e / k != e % k) ? ld_now<SM>(t_gmin + e) : kInfKey;
+            for (int e = tid; e < k * k; e += kThreads) s_gmin[e] = (e / k != e % k) ? ld_at<SM>(chk, t_gmin, e, k * k) : kInfKey;
             __syncthreads();
         }
 
@@ -653,9 +685,9 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                 const unsigned long long it = base + lane / G;
                 const bool on = it < items;
                 const uint32_t li = on ? (nw > 1 ? __umulhi((uint32_t)it, recip_nw) : (uint32_t)it) : 0u;
-                const uint32_t S = ld_now<SM>(t_list + beg + li);
+                const uint32_t S = ld_at<SM>(chk, t_list, beg + li, n_sets);
                 const int w = select_bit(full & ~S, on ? (int)((uint32_t)it - li * (uint32_t)nw) : 0);
-                const uint32_t rows_of_S = ld_now<SM>(t_live + S);
+                const uint32_t rows_of_S = ld_at<SM>(chk, t_live, S, n_sets);
                 const uint32_t lim = limit_of(*reinterpret_cast<volatile unsigned long long *>(&s_best), level);
                 // source rows that can still matter: their smallest value and the link's smallest key
                 uint32_t src = 0;
@@ -665,7 +697,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                     const int v = v0 + sl;
                     bool ok = false;
                     if (v < k && ((S >> v) & 1u)) {
-                        const unsigned long long e = ld_now<SM>(t_rowmap + (size_t)S * k + v);
+                        const unsigned long long e = ld_at<SM>(chk, t_rowmap, (size_t)S * k + v, n_map);
                         s_ids[v] = (uint32_t)e;
                         ok = on && ((rows_of_S >> v) & 1u) && max((uint32_t)(e >> 32), s_gmin[w * k + v]) < lim;
                     }
@@ -684,10 +716,10 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                     src &= src - 1;
                     if (in_row) {
                         uint32_t a[P], b[P], a2[P], b2[P];
-                        load_row<P, SM>(t_rows + (size_t)s_ids[v] * Lp + at, a);
-                        load_row<P, SM>(t_gam + (size_t)(w * k + v) * Lp + at, b);
-                        load_row<P, SM>(t_rows + (size_t)s_ids[v2] * Lp + at, a2);
-                        load_row<P, SM>(t_gam + (size_t)(w * k + v2) * Lp + at, b2);
+                        load_row_at<P, SM>(chk, t_rows, (size_t)s_ids[v] * Lp + at, n_rows, a);
+                        load_row_at<P, SM>(chk, t_gam, (size_t)(w * k + v) * Lp + at, n_gam, b);
+                        load_row_at<P, SM>(chk, t_rows, (size_t)s_ids[v2] * Lp + at, n_rows, a2);
+                        load_row_at<P, SM>(chk, t_gam, (size_t)(w * k + v2) * Lp + at, n_gam, b2);
 #pragma unroll
                         for (int i = 0; i < P; ++i) g[i] = min(g[i], min(max(a[i], b[i]), max(a2[i], b2[i])));
                     }
@@ -699,11 +731,11 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                 const uint32_t S2 = S | (1u << w);
                 if (make_row(g, out, S2, w, level, lim, on, rmin)) {
                     const uint32_t id = (uint32_t)(used + it);
-                    if (in_row) store_row<P>(t_rows + (size_t)id * Lp + at, out);
+                    if (in_row) store_row_at<P>(chk, t_rows, (size_t)id * Lp + at, n_rows, out);
                     if (sl == 0) {
-                        t_rowmap[(size_t)S2 * k + w] = ((unsigned long long)rmin << 32) | id;
-                        if (atomicOr(t_live + S2, 1u << w) == 0u)
-                            t_list[beg + cnt + next_place(level)] = S2;
+                        st_at(chk, t_rowmap, (size_t)S2 * k + w, n_map, ((unsigned long long)rmin << 32) | id);
+                        if (PP_IN_BOUNDS(chk, S2, n_sets) && atomicOr(t_live + S2, 1u << w) == 0u)
+                            st_at(chk, t_list, beg + cnt + next_place(level), n_sets, S2);
                     }
                 }
                 __syncwarp();
@@ -747,27 +779,27 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                 if (j == 0) break;
                 const uint32_t from = S & ~(1u << w);
                 const int lo = s_lo[(size_t)w * Lp + c2], np = __popc(from);
-                const uint32_t rows_of = np > 1 ? ld_now<SM>(t_live + from) : from;
+                const uint32_t rows_of = np > 1 ? ld_at<SM>(chk, t_live, from, n_sets) : from;
                 unsigned int pick = 0xFFFFFFFFu;
                 if constexpr (SM)
                     for (int c0 = lo; c0 < c2 && pick == 0xFFFFFFFFu; c0 += 32) {
                         const int c = min(c0 + lane, c2 - 1);
                         for (uint32_t rem = from; rem; rem &= rem - 1) {
                             const int v = __ffs(rem) - 1;
-                            const unsigned long long e = np > 1 ? t_rowmap[(size_t)from * k + v] : 0ull;
+                            const unsigned long long e = np > 1 ? ld_at<SM>(chk, t_rowmap, (size_t)from * k + v, n_map) : 0ull;
                             const bool ok = ((rows_of >> v) & 1u) && (uint32_t)(e >> 32) <= vstar;
-                            uint32_t x = max(np > 1 ? t_rows[(size_t)(ok ? (uint32_t)e : 0u) * Lp + c] : base_key(v, c),
-                                             t_gam[(size_t)(w * k + v) * Lp + c]);
-                            if constexpr (CT) x = max(x, t_seg[(size_t)(w * L + c2 - c - 1) * Lp + c2]);
+                            uint32_t x = max(np > 1 ? ld_at<SM>(chk, t_rows, (size_t)(ok ? (uint32_t)e : 0u) * Lp + c, n_rows) : base_key(v, c),
+                                             ld_at<SM>(chk, t_gam, (size_t)(w * k + v) * Lp + c, n_gam));
+                            if constexpr (CT) x = max(x, ld_at<SM>(chk, t_seg, (size_t)(w * L + c2 - c - 1) * Lp + c2, n_seg));
                             if (ok && x <= vstar) pick = min(pick, ((unsigned)c << 5) | (unsigned)v);
                         }
                         pick = __reduce_min_sync(kFull, pick);
                     }
                 for (int vi = wid; !SM && vi < np; vi += kBack) {
                     const int v = select_bit(from, vi);
-                    const unsigned long long e = np > 1 ? ld_now<SM>(t_rowmap + (size_t)from * k + v) : 0ull;
+                    const unsigned long long e = np > 1 ? ld_at<SM>(chk, t_rowmap, (size_t)from * k + v, n_map) : 0ull;
                     if (!((rows_of >> v) & 1u) || (uint32_t)(e >> 32) > vstar) continue;
-                    const uint32_t *row = t_rows + (size_t)(uint32_t)e * Lp, *gm = t_gam + (size_t)(w * k + v) * Lp;
+                    const size_t row = (size_t)(uint32_t)e * Lp, gm = (size_t)(w * k + v) * Lp;
                     constexpr int kChunks = 4;  // of 32 positions, their loads in flight together
                     bool hit_one = false;
                     for (int c0 = lo; c0 < c2 && !hit_one; c0 += 32 * kChunks) {
@@ -777,8 +809,8 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
                             const int c = c0 + 32 * u + lane;
                             x[u] = kInfKey;
                             if (c < c2) {
-                                x[u] = max(np > 1 ? ld_now<SM>(row + c) : base_key(v, c), ld_now<SM>(gm + c));
-                                if constexpr (CT) x[u] = max(x[u], ld_now<SM>(t_seg + (size_t)(w * L + c2 - c - 1) * Lp + c2));
+                                x[u] = max(np > 1 ? ld_at<SM>(chk, t_rows, row + c, n_rows) : base_key(v, c), ld_at<SM>(chk, t_gam, gm + c, n_gam));
+                                if constexpr (CT) x[u] = max(x[u], ld_at<SM>(chk, t_seg, (size_t)(w * L + c2 - c - 1) * Lp + c2, n_seg));
                             }
                         }
 #pragma unroll
@@ -879,6 +911,15 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
 
     // ---- result ----
     __syncthreads();
+#ifdef PP_DEBUG_BOUNDS
+    if (blockIdx.x == 0 && __ldcg(&ctl->err) != 0) {
+        status = (int)PP_ERR_CUDA;
+        beta = kInf;
+        m = 0;
+    }
+    __syncthreads();
+    if (SM && tid == 0) ctl->err = 0;
+#endif
     if (blockIdx.x == 0) {
         if (!dense && tid < PP_MAX_K) {
             d.out->cuts[tid] = m ? s_cut[tid] : -1;
@@ -911,6 +952,7 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
         if (tid == 0) {
             ctl->best = kNoBest;
             ctl->left = ctl->failed = 0u;
+            ctl->err = 0;
         }
     }
 }
@@ -1014,6 +1056,8 @@ cudaError_t launch_shape(const PruneDev &d, const PruneHost &h, int sms, cudaStr
 }
 
 }  // namespace
+
+PP_CHECKS_OF(prune)
 
 int prune_row_pad(int L, int k)
 {

@@ -17,6 +17,8 @@
 
 namespace pp {
 
+PP_CHECKS_OF(random)
+
 constexpr int kRandomThreads = 128;
 
 // Rows travel through shared memory so that global memory sees whole contiguous blocks: the draws
@@ -32,6 +34,7 @@ k_random_plans(const int L, const int k, const uint16_t *__restrict__ fwd, const
     const int stride = k | 1, tid = threadIdx.x;
     uint2 *sd = smem_pairs;  // [threads][stride]: draws in, (cut, node) pairs out
     uint16_t *s_fwd = reinterpret_cast<uint16_t *>(smem_pairs + kRandomThreads * stride);  // [k][L]
+    PP_BLOCK_BOUNDS(chk);
     for (int i = tid; i < k * L; i += kRandomThreads) s_fwd[i] = fwd[i];
     // whatever wrote the draws, or reads or writes the plans, is complete (fwd is older, see launch_eval)
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -61,6 +64,7 @@ k_random_plans(const int L, const int k, const uint16_t *__restrict__ fwd, const
         for (int step = 0; step < k; ++step) {
             const uint2 draw = row[step];
             const int node = select_bit(free_nodes, (int)__umulhi(draw.x, (unsigned)(k - step)));
+            if (!PP_IN_BOUNDS(chk, node * L + first, k * L)) break;
             const uint32_t count = s_fwd[node * L + first];  // segments [first, e] that fit
             if (count == 0) break;
             const int last = first + (int)__umulhi(draw.y, count);
@@ -72,7 +76,7 @@ k_random_plans(const int L, const int k, const uint16_t *__restrict__ fwd, const
             first = last + 1;
         }
         if (!done) n = 0;
-        nseg[p0 + tid] = (uint8_t)n;
+        nseg[p0 + tid] = PP_BROKEN(chk) ? (uint8_t)255 : (uint8_t)n;
         for (int i = n; i < k; ++i) row[i] = make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
     }
     __syncthreads();

@@ -2,14 +2,16 @@
 """Benchmark of the exact partition-and-placement path on B200.
 
 One step = one pass of the whole hot path over one batch of synthetic input:
-  1. exact search on the Large instance (k = 18 nodes, L = 200 layers): gamma/rank tables,
-     base frontier, every popcount level of the (min,max) sweep, final choice, backtrack;
-  2. the batched many-instance search on 4096 instances (k = 8, L = 24);
+  1. exact search on the Large instance (k = 18 nodes, L = 200 layers): the bounded search, one launch
+     from the inputs to the result record;
+  2. the batched many-instance search on 4096 instances (k = 8, L = 24), which does sweep every state;
   3. the batched beta evaluator on 262144 candidate plans of the Large instance (compressed rows:
      16-bit cuts, 8-bit nodes, one offset per plan).
 The headline number is DP relaxations per second, where one relaxation is
 g = min(g, max(dp, gamma)) and an instance has k(k-1)2^(k-2) L of them (a closed form of
-the sizes, not of the data).
+the sizes, not of the data).  The bounded search performs few of those of the Large instance, which
+are most of a step's: the number says how fast exact plans come, it is no rate of executed
+operations.  The rates of what is executed stand under `roofline`.
 
 `value` is measured with the inputs resident in device memory; `e2e` goes through the
 host-pointer C entry points, host<->device copies inside the timed region.
@@ -253,9 +255,9 @@ def run_ours(args):
             return
 
         # per-part device times (same launch configuration, measured after the timed region): the
-        # whole solve as the timed step runs it, then its phases with events between them (which
-        # cost a few microseconds: a phase's kernels are then no longer launched under the tail of
-        # the previous phase)
+        # whole solve as the timed step runs it (the bounded search), then the phases of the dense
+        # search, which the step does not run, with events between them (which cost a few
+        # microseconds: a phase's kernels are then no longer launched under the tail of the previous)
         sweep_ms, rank_ms, fin_ms, solve_ms = [], [], [], []
         for _ in range(9):
             prob.solve_exact_dev(d_sol.data_ptr())
@@ -296,7 +298,7 @@ def run_ours(args):
             eval32_cold_ms.append(e0.elapsed_time(e1))
 
         # sustained leg: the Large solve back to back for about two seconds, clocks sampled meanwhile
-        # (the sweep is bound by an ALU pipe, so its time follows the SM clock the part settles at)
+        # (bound by latencies of the SM and of L2, so its time follows the clock the part settles at)
         n_sus = max(50, int(2000.0 / statistics.median(solve_ms)))
         with ClockSampler(local) as sus_clocks:
             e0.record(stream)
@@ -311,7 +313,8 @@ def run_ours(args):
                      "ms_times_mhz": sus_ms * sus_clk["sm_mhz"] if sus_clk else None,
                      "reasons": sus_clk["reasons"] if sus_clk else None}
 
-        # issue rate of the packed min/max forms the sweep is made of, measured now on this part
+        # issue rate of the packed min/max forms the dense sweep and the batched search are made of,
+        # measured now on this part
         rates = {"minmax_u16x2": pp.debug_minmax_rate(0), "min3_u16x2": pp.debug_minmax_rate(1),
                  "max3_u16x2": pp.debug_minmax_rate(2)}
 
@@ -384,10 +387,11 @@ def run_ours(args):
                     ts.append(q.last_solve_profile().ms_total)
                 qp = q.last_solve_profile()
                 other[name] = {"solve_ms": min(ts[2:]), "relaxations_per_s": n_relax(inst.k, inst.L) / (min(ts[2:]) * 1e-3),
-                               "state_bytes": qp.state_bytes, "fast_path": qp.fast_path, "pair_levels": qp.pair_levels}
+                               # of the dense sweep of this problem, which such a solve does not run
+                               "dense_state_bytes": qp.state_bytes, "fast_path": qp.fast_path, "pair_levels": qp.pair_levels}
 
         # the exact search under the paper's full objective, Eq. 1 (compute times of the partitions in the
-        # bottleneck): host-pointer call, fp64 states, wall clock of the whole call; for context
+        # bottleneck): host-pointer call, wall clock of the whole call; for context
         ct_inst = W.config_geometric(12, 64, 1)
         ct_work = (ct_inst.layer_mem_bytes // np.uint64(1024)).astype(np.uint64)
         ct_speed = (1000 + 37 * np.arange(ct_inst.k)).astype(np.uint32)
@@ -398,7 +402,7 @@ def run_ours(args):
             ct_ts.append((time.perf_counter() - t_ct) * 1e3)
         other["eq1_compute_term_geometric_k12_L50"] = {
             "call_ms": min(ct_ts[1:]), "relaxations_per_s": n_relax(ct_inst.k, ct_inst.L) / (min(ct_ts[1:]) * 1e-3),
-            "state_bytes": 8, "status": int(ct_sol.status), "m": int(ct_sol.m)}
+            "state_bytes": 4, "status": int(ct_sol.status), "m": int(ct_sol.m)}
 
         # the paper's own two-stage heuristic (Algorithm 1, then Algorithms 2 and 3) against the exact
         # optimum on the evaluation setting of its Section 4: 14 devices of 32 MB on a random geometric
@@ -524,11 +528,12 @@ def run_ours(args):
     assert host_out[0].beta_ms == sol_rec.beta_ms and host_out[0].m == sol_rec.m
 
     # ---- roofline ----
-    # The dense programme's roofline; sweep_ms and the kernel figures are those of the dense sweep, timed with
-    # its phases apart (the plain solve runs the bounded search).  It is the slower of (state bytes at HBM
-    # bandwidth) and (min/max element-ops at the ALU rate): every state is written once and read once (2 * states * element bytes); a
-    # relaxation is one max and one min, the window step about three more ops per state.  The ALU
-    # rate is the packed min/max issue rate measured above x 32 lanes x 2 elements x SMs x max clock.
+    # `roofline` is that of the kernels which take most of the timed step: the lane kernels of the batched search.
+    # They sweep densely, so the dense programme's operations are theirs: a relaxation is one max and one
+    # min, the window step about three more operations per state; the rate is the packed min/max issue rate
+    # measured above x 32 lanes x 2 elements x SMs x max clock.  The Large solve of the step is bound by
+    # latencies and has no such figure; what the dense programme would take at the peaks is listed beside its
+    # time, and the dense sweep (not run by the step) with its own figures.
     peaks, which = measured_peaks()
     med = statistics.median
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
@@ -546,36 +551,35 @@ def run_ours(args):
                 "t_mem_ms_at_8TBps": t_mem_nom, "bound": "hbm" if t_mem >= t_alu else "alu",
                 "solve_ms": solve_ms_, "frac": max(t_mem, t_alu) / solve_ms_,
                 "frac_at_8TBps": max(t_mem_nom, t_alu) / solve_ms_,
-                "note": "time of the dense programme's bytes and operations at the peaks over the solve's time: above 1 "
-                        "because the bounded search drops the states that cannot beat the best plan known and forms "
-                        "a small part of the dense table's rows"}
+                "note": "time of the dense programme's bytes and operations at the peaks over the solve's time, no "
+                        "utilisation: above 1 because the bounded search drops the states that cannot beat the best "
+                        "plan known and forms a small part of the dense table's rows"}
 
     elem = prof.state_bytes
     sweep_t = med(sweep_ms) * 1e-3
     whole = dp_roofline(k, L, elem, med(solve_ms))
     alg_bytes = whole["algorithmic_bytes"]
     alu_ops = whole["algorithmic_ops"]
-    n_launch = prof.sweep_launches
-    if whole["bound"] == "hbm":
-        achieved, peak, unit = alg_bytes / sweep_t / 1e9, peaks["hbm_gbs"], "GB/s"
-    else:
-        achieved, peak, unit = alu_ops / sweep_t / 1e12, alu_peak / 1e12, "Tops/s"
-    roofline = {"bound": whole["bound"], "achieved": achieved, "peak": peak, "unit": unit,
-                "frac": achieved / peak,
-                "traffic": SWEEP_DRAM_BYTES_PER_LAUNCH if prof.fast_path else None,
-                "peak_source": (which + " (burst copy figure; the sweep is timed alone)") if whole["bound"] == "hbm"
-                               else "measured in this run (packed min/max issue rate x max SM clock)",
-                "kernel": "k_sweep_pair + k_sweep_fast (%d launches per solve, one per popcount level)" % n_launch,
-                "algorithmic_bytes_per_launch": alg_bytes / n_launch,
-                "ms_per_launch": sweep_t * 1e3 / n_launch,
-                "algorithmic_bytes_per_solve": alg_bytes, "sweep_ms": sweep_t * 1e3,
-                "hbm": {"achieved_GBps": alg_bytes / sweep_t / 1e9, "peak_GBps": peaks["hbm_gbs"],
-                        "frac": alg_bytes / sweep_t / 1e9 / peaks["hbm_gbs"], "peak_source": which},
-                "alu": {"ops_per_solve": alu_ops, "achieved_ops_per_s": alu_ops / sweep_t,
-                        "peak_ops_per_s": alu_peak, "frac": alu_ops / sweep_t / alu_peak,
-                        "warp_instr_per_clk_per_sm": rates, "lanes_per_clk_per_sm": minmax_rate * 32,
-                        "peak_source": "measured in this run"},
-                "whole_solve": whole,
+    n_levels = min(k, L) - 1  # sweep launches of the dense search: one per popcount level from 2 up
+    batch_ops = N_BATCH * (2 * n_relax(BATCH_K, BATCH_L) + 3 * n_states(BATCH_K, BATCH_L))
+    batch_s = med(batch_ms) * 1e-3
+    dense_sweep = {"in_timed_step": False, "kernel": "k_sweep_pair + k_sweep_fast (%d launches per solve)" % n_levels,
+                   "state_bytes": elem, "sweep_ms": sweep_t * 1e3, "rank_build_ms": med(rank_ms), "finalize_ms": med(fin_ms),
+                   "ms_per_launch": sweep_t * 1e3 / n_levels, "algorithmic_bytes_per_launch": alg_bytes / n_levels,
+                   "dram_bytes_per_launch_ncu": SWEEP_DRAM_BYTES_PER_LAUNCH if prof.fast_path else None,
+                   "hbm": {"achieved_GBps": alg_bytes / sweep_t / 1e9, "peak_GBps": peaks["hbm_gbs"],
+                           "frac": alg_bytes / sweep_t / 1e9 / peaks["hbm_gbs"], "peak_source": which},
+                   "alu": {"ops_per_solve": alu_ops, "achieved_ops_per_s": alu_ops / sweep_t,
+                           "peak_ops_per_s": alu_peak, "frac": alu_ops / sweep_t / alu_peak}}
+    roofline = {"bound": "alu", "achieved": batch_ops / batch_s / 1e12, "peak": alu_peak / 1e12, "unit": "Tops/s",
+                "frac": batch_ops / batch_s / alu_peak, "traffic": None,
+                "peak_source": "measured in this run (packed min/max issue rate x max SM clock)",
+                "kernel": "k_lanes_prep + k_lanes_level + k_lanes_back (%d launches per batched solve)" % batch_launches,
+                "ms": batch_s * 1e3, "share_of_step": batch_s * 1e3 / ms_per_step, "algorithmic_ops": batch_ops,
+                "warp_instr_per_clk_per_sm": rates,
+                "large_solve": {"kernel": "k_prune (%d launch per solve)" % prof.total_launches, "ms": med(solve_ms),
+                                "bound": "latency of a dozen dependent steps", "dense_programme": whole},
+                "dense_sweep": dense_sweep,
                 "sustained": sustained}
     # the other parts of the step against their own bounds
     c3 = W.config_deeper_cnn()
@@ -584,10 +588,9 @@ def run_ours(args):
     # per plan: nseg, its offset, nseg - 1 cuts of 2 bytes, nseg nodes of 1 byte in; beta and flags out
     plan_bytes = 5 * N_PLANS + 3 * n_entries - 2 * int((np.diff(p_off.astype(np.int64)) > 0).sum()) + 9 * N_PLANS
     ev_cold = med(eval_cold_ms) * 1e-3
-    batch_ops = N_BATCH * (2 * n_relax(BATCH_K, BATCH_L) + 3 * n_states(BATCH_K, BATCH_L))
     part_rooflines = {
-        "deeper_cnn_k14_L100": dp_roofline(c3.k, c3.L, o3["state_bytes"], o3["solve_ms"]),
-        "large_unequal_layer_memory_k18_L200": dp_roofline(k, L, unl["state_bytes"], unl["solve_ms"]),
+        "deeper_cnn_k14_L100": dp_roofline(c3.k, c3.L, o3["dense_state_bytes"], o3["solve_ms"]),
+        "large_unequal_layer_memory_k18_L200": dp_roofline(k, L, unl["dense_state_bytes"], unl["solve_ms"]),
         "evaluator": {"bound": "hbm", "algorithmic_bytes": plan_bytes, "bytes_per_plan": plan_bytes / N_PLANS,
                       "ms_cold": ev_cold * 1e3, "achieved_GBps": plan_bytes / ev_cold / 1e9,
                       "frac": plan_bytes / ev_cold / 1e9 / peaks["hbm_gbs"],
@@ -600,14 +603,15 @@ def run_ours(args):
     out = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": warmup, "ms_per_step": ms_per_step, "higher_is_better": True,
-        "scaling": "weak", "vs_baseline": None, "dtype": "u16" if elem == 2 else "u32",
+        "scaling": "weak", "vs_baseline": None, "dtype": "u32 keys + u16 ranks",
         "data": "synthetic",
         "config": {"workload": WORKLOAD,
                    "relaxations_per_step": relax_step, "states_large": n_states(k, L),
                    "l2": "a step writes and reads 219 MB of tables of the batched search between two solves, more than "
                          "the 126 MB L2; no explicit flush (the dense sweep's state table is %.2f GB)" % (alg_bytes / 2 / 1e9),
                    "relaxations": "those of the dense programme (every node set, last node, next node and cut position), "
-                                  "whether the search visits them or not",
+                                  "whether the search visits them or not: the Large solve performs few of its 4.0e9, so "
+                                  "ms_per_step is the figure to compare, not a rate of executed operations",
                    "parallelism": "replicas only" if world > 1 else "single GPU"},
         "gpu_launches": launches_per_step * args.steps,
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": int(h2d),
@@ -618,8 +622,7 @@ def run_ours(args):
         "clocks": clk,
         "roofline": roofline,
         "breakdown": {
-            "large_solve_ms": med(solve_ms), "rank_build_ms": med(rank_ms),
-            "sweep_ms": med(sweep_ms), "finalize_ms": med(fin_ms),
+            "large_solve_ms": med(solve_ms),
             "large_relaxations_per_s": relax_large / (med(solve_ms) * 1e-3),
             "batch_ms": med(batch_ms), "instances_per_s": N_BATCH / (med(batch_ms) * 1e-3),
             "eval_ms": med(eval_ms), "plans_per_s": N_PLANS / (med(eval_ms) * 1e-3),
@@ -700,9 +703,9 @@ def run_reference(args):
 
 def run_only(args):
     """Small single-part runs for profilers (no timing, no JSON line): the Large instance restricted
-    to its first --k nodes (k = 16: a 0.44 GB state table, far above the L2 and small enough for a
-    multi-pass counter capture of single sweep launches), the batched solve, or one of the two
-    comparison baselines."""
+    to its first --k nodes (by the bounded search, with --mode by a dense sweep; k = 16: a 0.44 GB state
+    table, far above the L2 and small enough for a multi-pass counter capture of single sweep launches),
+    the batched solve, or one of the two comparison baselines."""
     import torch
 
     import paper_2210_12219_b200 as pp

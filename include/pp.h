@@ -154,7 +154,14 @@ pp_status pp_solve_exact(pp_problem *p, double *beta_ms, int32_t *m, int32_t *cu
 
 /* Same search; the result record is written to device memory `solution_dev` (device,
  * sizeof(pp_solution), 8-byte aligned) by work queued on the problem's stream.  Returns as
- * soon as the work is queued; feasibility is in solution_dev->status. */
+ * soon as the work is queued; feasibility is in solution_dev->status.
+ * The choice of the dense sweep where too many states remain is the synchronous call's only: it looks at the
+ * outcome of the bounded search, which this call cannot.  An instance in which no bound ever applies
+ * (no plan exists, or all plans are alike) therefore takes longer here from 16 nodes on: at k = 18, L = 200
+ * 2.6 ms without a plan and 5.9 ms with all plans alike, against 1.4 and 0.7 ms of the dense sweep and 1.7 and
+ * 0.9 ms of the synchronous call (k = 16, L = 100: 0.46 against 0.33).  A program that expects such
+ * instances can ask for the dense sweep with pp_problem_force_generic(p, 0); an ordinary instance of that
+ * size takes 0.03 to 0.06 ms here. */
 pp_status pp_solve_exact_dev(pp_problem *p, pp_solution *solution_dev);
 
 /*
@@ -425,7 +432,8 @@ pp_status pp_debug_bounds_checks(int32_t kernel, uint64_t *n);
 /* Force (1) or forbid (0) the generic sweep kernel; 2 = automatic choice among the kernels that
  * take one source mask per warp (the two-mask kernel is left out); 3 = the two-mask kernel on every
  * level it can run, however small; -1 restores the automatic choice.  Meant for tests that want
- * every kernel checked on the same instance; any mode but -1 takes the dense sweep. */
+ * every kernel checked on the same instance, and for asynchronous solves of instances that cannot be
+ * pruned (see pp_solve_exact_dev); any mode but -1 takes the dense sweep. */
 pp_status pp_problem_force_generic(pp_problem *p, int32_t mode);
 
 /*

@@ -223,7 +223,7 @@ cudaError_t launch(const Dev &d, const unsigned char *tables, int64_t B, int64_t
     cudaError_t e = cudaFuncSetAttribute(k_eval<PACKED, E, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
     if (e != cudaSuccess) return e;  // 68 KB at k = 20, L = 1024
     int64_t blocks = (B + kEvalThreads - 1) / kEvalThreads;
-    const int64_t cap = 148 * 12;  // resident at a time; a block's tables are staged once for all its plans
+    const int64_t cap = 148 * 12;  // five of them fit an SM at a time; a block's tables are staged once for all its plans
     if (blocks > cap) blocks = cap;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)blocks);

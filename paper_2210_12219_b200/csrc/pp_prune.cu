@@ -50,7 +50,9 @@ constexpr size_t kSharedBytes = 220 * 1024;
 constexpr int kAhead = 8;             // steps of a window scan whose compute times are asked for at a time
 constexpr int kSpinLimit = 1 << 22;  // polls of a barrier before the kernel gives up
 constexpr int kAloneRounds = 2;      // a level of at most this many rounds of one block is done by block 0 alone
-// P = 8 (up to 256 layers): 20 warps, so that the 2448 targets of the node sets of two of 18 nodes are one round
+// P = 8 (129 to 256 layers): 20 warps, more of a level's targets in a round.  Against 16 warps, mean of nine
+// instances each at L = 135, 200, 240: k = 18 34.0, 32.1, 29.1 -> 31.5, 28.9, 26.1 us a solve, k = 17 33.7, 29.1, 28.6 ->
+// 32.4, 28.0, 26.3, k = 13 and 15 within 2 %; k = 11 26.8, 25.9, 25.4 -> 27.4, 26.7, 25.7, where 16 would do.
 __host__ __device__ constexpr int prune_threads(int P) { return P == 8 ? 640 : P <= 16 ? 512 : 256; }
 
 // Which class of doubles a key stands for.

@@ -123,7 +123,8 @@ void pp_problem_destroy(pp_problem *p);
  * the problem on the stream it used before; the first call copies the inputs to the device, complete
  * when it returns (on the legacy stream in order).  May be called while `cuda_stream` is recorded
  * into a graph: nothing the handle keeps becomes part of the graph, and the caller sees to it that the
- * graph runs after the work the handle has queued elsewhere and before the handle is destroyed. */
+ * graph runs before the handle is destroyed.  Not waited for are a stream that is itself recorded, and, while
+ * `cuda_stream` is recorded, the legacy stream: its work has to be done before the graph runs. */
 pp_status pp_problem_set_stream(pp_problem *p, void *cuda_stream);
 
 /* Bytes of device scratch the exact search needs (state table, gamma and rank tables).  Without a

@@ -966,9 +966,12 @@ pp_status pp_problem_set_stream(pp_problem *p, void *cuda_stream)
 {
     if (!p) return PP_ERR_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    if (s != p->stream && (p->uploaded || p->d_sparse) && !recording(s)) {  // copies and scratch are ordered there
-        PP_CUDA(cudaStreamSynchronize(p->stream));
-        p->tables_ready = p->uploaded;
+    if (s != p->stream && (p->uploaded || p->d_sparse) && !recording(p->stream)) {  // copies and scratch are ordered there
+        if (p->stream || !recording(s)) {  // waiting for the legacy stream would end the recording
+            OutsideCapture outside;
+            PP_CUDA(cudaStreamSynchronize(p->stream));
+            p->tables_ready = p->uploaded;
+        }
     }
     p->stream = s;
     return upload_inputs(p, s != nullptr);  // the legacy stream, on which the buffer was allocated, has it in order

@@ -139,14 +139,17 @@ def test_handle_that_meets_its_stream_in_a_recording(L, k, mode, workspace):
         p.solve_exact_dev(sol.data_ptr())
         p.eval_plans_dev(300, *(a.data_ptr() for a in dev), beta.data_ptr(), stat.data_ptr())
 
-    for first_elsewhere in (False, True):
+    other = torch.cuda.Stream()
+    for first_on in (None, 0, other.cuda_stream):
         with pp.Problem.from_instance(inst) as p:
             p.force_generic(mode)
             if workspace:
                 p.set_workspace(torch.empty(p.workspace_bytes(), dtype=torch.uint8, device="cuda"))
-            if first_elsewhere:
+            if first_on is not None:  # and the recording begins while these calls may still be running
+                p.set_stream(first_on)
                 calls(p)
-                check()
+                if first_on == 0:
+                    torch.cuda.synchronize()
             g = torch.cuda.CUDAGraph()
             with torch.cuda.graph(g):
                 p.set_stream(torch.cuda.current_stream().cuda_stream)

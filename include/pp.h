@@ -160,7 +160,9 @@ pp_status pp_solve_exact(pp_problem *p, double *beta_ms, int32_t *m, int32_t *cu
  * outcome of the bounded search, which this call cannot.  An instance in which no bound ever applies
  * (no plan exists, or all plans are alike) therefore takes longer here from 16 nodes on: at k = 18, L = 200
  * 2.6 ms without a plan and 5.9 ms with all plans alike, against 1.4 and 0.7 ms of the dense sweep and 1.7 and
- * 0.9 ms of the synchronous call (k = 16, L = 100: 0.46 against 0.33).  A program that expects such
+ * 0.9 ms of the synchronous call (k = 16, L = 100: 0.46 against 0.33).  Where the quotients that decide lie closer
+ * together than about 2^-28 of their value as well, a second search by one block follows (k = 12, L = 60: 2.4
+ * ms, k = 14, L = 100: 26 ms), which the synchronous call leaves to the dense sweep too.  A program that expects such
  * instances can ask for the dense sweep with pp_problem_force_generic(p, 0); an ordinary instance of that
  * size takes 0.03 to 0.06 ms here. */
 pp_status pp_solve_exact_dev(pp_problem *p, pp_solution *solution_dev);

@@ -870,6 +870,7 @@ pp_status queue_sparse(pp_problem *p, PruneCtl *ctl, pp_solution *sol, PruneNote
     q.out = sol;
     q.note = note;
     q.row_cap = std::min(q.row_cap, row_limit);
+    q.fallback = row_limit != ~0ull;
     const PruneHost h{p->bits.data(), p->M.data(), p->cap.data(), p->bw.data(), nullptr, nullptr};
     PP_CUDA(launch_prune(q, h, p->sms, p->stream));
     p->total_launches = 1;

@@ -188,7 +188,7 @@ struct PruneCtl {              // device; the kernel leaves it as it found it
 };
 struct PruneNote {             // what the host learns about a launch
     long long ns;              // duration on the device
-    int32_t dense;             // 1 = the frontier outgrew its rows
+    int32_t dense;             // 1 = the frontier outgrew its rows, or is too large to resolve a class in
 };
 struct PruneDev {
     int L, k, Lp;              // Lp: row stride in keys
@@ -197,6 +197,7 @@ struct PruneDev {
     int polls;                 // the launch)
     int key_shift;             // keys: 1 + (bits of the double - key_base) >> key_shift
     unsigned long long key_base;
+    uint32_t fallback;         // 1 = the caller has another search (note->dense asks for it)
     uint32_t whole;            // nodes that hold the whole chain
     uint32_t tight_levels;     // bit j: some rest of the chain may not fit the nodes that j used ones leave
     const int16_t *lo;         // [k*L] window starts (see Dev), or null: the kernel works them out

@@ -49,6 +49,10 @@ constexpr int kSharedRounds = 3;  // k = 6, L = 12: 17 -> 12 us a solve; k = 7 (
 constexpr size_t kSharedBytes = 220 * 1024;
 constexpr int kAhead = 8;             // steps of a window scan whose compute times are asked for at a time
 constexpr int kSpinLimit = 1 << 22;  // polls of a barrier before the kernel gives up
+// The second search is block 0's alone, at 0.2 us a row it keeps.  After a first one of more node sets than this a
+// caller that has the dense search, which is exact at once, gets to run that (k = 14, L = 100, every state kept:
+// 25.6 -> 0.3 ms on the device; a search that a bound thins out has a few hundred sets at k = 18).
+constexpr uint32_t kAloneSets = 1024;
 constexpr int kAloneRounds = 2;      // a level of at most this many rounds of one block is done by block 0 alone
 // P = 8 (129 to 256 layers): 20 warps, more of a level's targets in a round.  Against 16 warps, mean of nine
 // instances each at L = 135, 200, 240: k = 18 34.0, 32.1, 29.1 -> 31.5, 28.9, 26.1 us a solve, k = 17 33.7, 29.1, 28.6 ->
@@ -896,6 +900,10 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
         beta = __longlong_as_double((long long)worst);
         // exact unless the class of the optimum holds a quotient smaller than the plan's own bottleneck
         if (key_of.zoom || s_low >= worst) break;
+        if (d.fallback && beg + cnt > kAloneSets) {
+            dense = true;
+            break;
+        }
         key_of.zoom = vstar;  // once more, this class resolved
         nblk = 1;
         if (tid == 0) s_best = kNoBest;

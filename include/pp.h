@@ -142,8 +142,9 @@ pp_status pp_problem_set_workspace(pp_problem *p, void *device_buffer, uint64_t 
  * Exact search (Eq. 2 minimised over every cut set and every injective placement) by a
  * (min,max) dynamic programme over (used-node mask, last node, last cut layer), swept by
  * popcount of the mask; then the canonical plan by backtracking.  States that provably lie on no
- * better plan than one already found are not expanded; where too many remain (a synchronous solve of
- * 15 nodes and more), the programme is swept densely instead.  The result is the same bit for bit.
+ * better plan than one already found are not expanded; where too many remain (160 000 rows, or many
+ * node sets and an optimum that has to be resolved among quotients closer than the search's keys), a
+ * synchronous solve sweeps the programme densely instead.  The result is the same bit for bit.
  *   beta_ms   host [1]    beta* in milliseconds, +inf if infeasible
  *   m         host [1]    number of segments, 0 if infeasible
  *   cuts      host [k-1]  e_1..e_{m-1}, rest -1   (may be NULL when k == 1)

@@ -279,7 +279,7 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
         const int U = (int)s_U, D = (int)s_D;
         // ---- 2. ranks of the quotients, spread out as rank[v][w][c] ----
         rank_quotients<kBatchThreads, unsigned long long, 16>(
-            dbits, ubw, U, D, __ddiv_rd((double)__uint_as_float(s_least), (double)s_fast),
+            dbits, ubw, U, D, [&](int u, int d) { return __ddiv_rn((double)dbits[d], (double)ubw[u]); }, __ddiv_rd((double)__uint_as_float(s_least), (double)s_fast),
             __ddiv_ru((double)__uint_as_float(s_most), (double)s_slow),
             reinterpret_cast<uint32_t *>(smem + lay.key), reinterpret_cast<unsigned long long *>(smem + lay.val),
             reinterpret_cast<uint32_t *>(smem + lay.hist), rk, s_sum);

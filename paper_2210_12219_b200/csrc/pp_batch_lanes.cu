@@ -82,7 +82,19 @@ __device__ __forceinline__ void st_piece(const BatchLanes &t, uint32_t *p, const
     if (PP_IN_BOUNDS(t, (size_t)(p - base), words)) *reinterpret_cast<Piece *>(p) = v;
 }
 
+// The correctly rounded quotient x / b of integers 0 <= x < 2^40 and 0 < b < 2^24 held as doubles; r is b's correctly rounded
+// reciprocal.  x r lies within two units in the last place of x / b, so its remainder is below 2^26 such units and exact, and
+// what the last step rounds is off by less than 2^-50 of a unit.  No quotient comes that near to the middle m between two
+// doubles: x / b - m is a multiple of half a unit over b, hence at least 2^-25 of a unit, and zero never, since m has 54
+// bits, the last one set, and would have to divide x.
+__device__ __forceinline__ double quotient(double x, double b, double r)
+{
+    const double q = __dmul_rn(x, r);
+    return __fma_rn(__fma_rn(-q, b, x), r, q);
+}
+
 // Shared memory of an instance in the preparing kernel (byte offsets; every part 16-byte aligned).
+constexpr size_t kDoubles = 32 + 2 * 56;  // distinct sizes, distinct bandwidths and their reciprocals: where val[] goes later
 struct PrepLayout {
     size_t val, key, rk, M, bits, dbits, cap, bw, ubw, hist, pair_u, cls, total;
 };
@@ -93,7 +105,7 @@ __host__ __device__ inline PrepLayout prep_layout(int L, int k)
     const size_t n = (size_t)k * (k - 1) * L;  // quotients
     size_t o = 0;
     auto take = [&o](size_t bytes) { size_t at = o; o = (o + bytes + 15) & ~(size_t)15; return at; };
-    p.val = take(n * 4);
+    p.val = take(n * 4 > kDoubles * 8 ? n * 4 : kDoubles * 8);
     p.key = take(n * 4);
     p.rk = take(n * 2);
     p.M = take(33 * 8);
@@ -113,7 +125,9 @@ __host__ __device__ inline PrepLayout prep_layout(int L, int k)
 // ranking of gamma (Eq. 3), and the instance's column of the tables of BatchLanes.
 //   * distinct usable bandwidths and distinct transfer sizes listed in order of first appearance;
 //   * window start lo_w(c2) by a branch-free binary search over the memory prefix sums;
-//   * ranks by rank_quotients.
+//   * ranks by rank_quotients, the quotients of its first pass by the reciprocals of the distinct bandwidths, three fp64
+//     instructions each where a division and two conversions take some thirty (4096 x (k = 8, L = 24) 219.3 -> 218.1 us a
+//     call, L = 32 297.0 -> 295.1, k = 5 62.8 -> 62.2).
 // What is left is a chain of short dependent phases, a third as long with four warps to an instance as with
 // one; the SM's other instances hide it.
 __global__ void __launch_bounds__(kPrepThreads, kPrepBlocks)
@@ -125,6 +139,7 @@ k_lanes_prep(const BatchLanes t, const int64_t B, const int L, const int k, cons
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const PrepLayout lay = prep_layout(L, k);
     uint32_t *s_val = reinterpret_cast<uint32_t *>(smem_prep + lay.val);
+    double *s_size = reinterpret_cast<double *>(smem_prep + lay.val), *s_link = s_size + 32, *s_recip = s_link + 56;
     unsigned long long *M = reinterpret_cast<unsigned long long *>(smem_prep + lay.M);
     unsigned long long *s_bits = reinterpret_cast<unsigned long long *>(smem_prep + lay.bits);
     unsigned long long *s_cap = reinterpret_cast<unsigned long long *>(smem_prep + lay.cap);
@@ -196,7 +211,10 @@ k_lanes_prep(const BatchLanes t, const int64_t B, const int L, const int k, cons
             const uint32_t firsts = __ballot_sync(FULL, lane < L && f == lane);
             const int c = __popc(firsts & ((1u << f) - 1u));
             cls[lane] = (uint8_t)c;
-            if (lane < L && f == lane) dbits[c] = mine;
+            if (lane < L && f == lane) {
+                dbits[c] = mine;
+                s_size[c] = (double)mine;
+            }
             if (lane == 0) s_first[2] = firsts;
         }
         // ---- windows, base frontier ----
@@ -244,7 +262,11 @@ k_lanes_prep(const BatchLanes t, const int64_t B, const int L, const int k, cons
         if (wid < 2) {
             const int u = x == 0u ? -1 : f < 32 ? __popc(m0 & ((1u << f) - 1u)) : n0 + __popc(m1 & ((1u << (f - 32)) - 1u));
             pair_u[tid] = (int8_t)u;
-            if (x != 0u && f == tid) ubw[u] = x;
+            if (x != 0u && f == tid) {
+                ubw[u] = x;
+                s_link[u] = (double)x;
+                s_recip[u] = __drcp_rn((double)x);
+            }
         }
         if (tid == kPrepThreads - 1) {
             unsigned long long best = kNoBest;
@@ -262,6 +284,7 @@ k_lanes_prep(const BatchLanes t, const int64_t B, const int L, const int k, cons
             const uint32_t fast = __reduce_max_sync(FULL, max(p0, p1));
             const uint32_t slow = __reduce_min_sync(FULL, min(p0 ? p0 : FULL, p1 ? p1 : FULL));
             rank_quotients<kPrepThreads, uint32_t, 11>(dbits, ubw, U, __popc(s_first[2]),
+                                                       [&](int u, int d) { return quotient(s_size[d], s_link[u], s_recip[u]); },
                                                        __ddiv_rd((double)__uint_as_float(least), (double)fast),
                                                        __ddiv_ru((double)__uint_as_float(most), (double)slow), s_key, s_val,
                                                        hist, rk, s_sum);

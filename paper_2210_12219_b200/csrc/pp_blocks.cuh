@@ -157,10 +157,11 @@ constexpr int kRankBuckets = 1024;
 // (monotone), counters in shared memory, their prefix sums, the quotients scattered into the order of the
 // buckets, and each compared with the few that share its bucket.  Some 90 instructions per quotient where
 // a staircase walk over the sorted quotient matrix took U + L dependent steps, 350.
+// first(u, i) is the quotient as the first pass gets it, which may read what val[] held before.
 // V holds a key and an entry number of kIdBits; key[] and val[] have n entries, hist kRankBuckets counters.
 // lo_d, hi_d: bounds of all positive quotients.  Ends with the block in step.
-template <int kThreads, typename V, int kIdBits>
-__device__ __forceinline__ void rank_quotients(const unsigned long long *bits, const uint32_t *bw, int U, int D,
+template <int kThreads, typename V, int kIdBits, typename First>
+__device__ __forceinline__ void rank_quotients(const unsigned long long *bits, const uint32_t *bw, int U, int D, First first,
                                                double lo_d, double hi_d, uint32_t *key, V *val, uint32_t *hist,
                                                uint16_t *rk, uint32_t *s_sum)
 {
@@ -176,7 +177,8 @@ __device__ __forceinline__ void rank_quotients(const unsigned long long *bits, c
         return __ddiv_rn((double)bits[e - u * D], (double)bw[u]);
     };
     for (int e = tid; e < n; e += kThreads) {
-        const unsigned long long q = (unsigned long long)__double_as_longlong(quotient(e));
+        const int u = D > 1 ? (int)__umulhi((uint32_t)e, recip_D) : e;
+        const unsigned long long q = (unsigned long long)__double_as_longlong(first(u, e - u * D));
         const uint32_t y = (uint32_t)((q > lowest ? q - lowest : 0ull) >> shift);  // 0.0 counts as the lowest
         key[e] = y;
         atomicAdd(&hist[y >> 21], 1u);

@@ -100,6 +100,13 @@ size_t batch_smem_bytes(int L, int k)
     return batch_layout(L, k).total;
 }
 
+// Blocks that an SM holds at a time: as many as the registers are shared out for, or as fit its 228 KB.
+int batch_blocks_per_sm(int L, int k)
+{
+    const size_t fit = (size_t)(228 << 10) / (batch_smem_bytes(L, k) + 1024);
+    return (int)std::max<size_t>(1, std::min<size_t>(kBatchBlocksPerSm, fit));
+}
+
 namespace {
 
 // t_rowoff, t_rows, t_first: compact row of (S, lowest node of S), rows ordered by (popcount, mask, node);

@@ -33,7 +33,6 @@ constexpr int kLevelFourBlocks = 5;  // source masks of up to this many nodes: r
 constexpr int kPrepThreads = 128, kPrepBlocks = 12;  // 18 KB of shared memory a block at most
 constexpr int kFlagLimit = 1;     // BatchLanes::flag: an input beyond the limits
 constexpr int kBackWarps = 8;
-constexpr int kLanesMinB = 64;  // below this the block-per-instance kernel keeps more of the GPU busy
 constexpr int kLanesMaxK = 8;   // NV <= 7 rows of a source mask in registers
 constexpr int kLanesMaxL = 32;  // LH <= 16 words per row
 
@@ -629,9 +628,21 @@ cudaError_t launch_level(int nv, const BatchLanes &t, int64_t B, int k, int L, i
 
 }  // namespace
 
-bool batch_lanes_takes(int64_t B, int L, int k)
+// A batch that fits the GPU at once goes an instance to a block (pp_batch.cu), which then takes the time of one
+// instance; here every level is a launch, however few warps it has.  us a call, here and there: 64 x (k = 4, L = 24)
+// 21.9, 12.5, 444 of them 23.8, 14.5; 300 x (k = 6, L = 24) 35.0, 20.7; 148 x (k = 8, L = 24) 50.5, 35.0, 444 of
+// them 62.1, 53.5.  A second wave of blocks costs as much again: 600 x (k = 6, L = 24) 37.1, 33.3, 888 41.2, 39.1,
+// 888 x (k = 8, L = 16) 70.0, 67.6, 700 x (k = 7, L = 32) 59.8, 53.5; but 600 x (k = 7, L = 24) 49.3, 51.3, (k = 8,
+// L = 24) 72.2, 84.5, 450 x (k = 8, L = 28) 75.9, 78.0, 888 x (k = 2, L = 32) 17.1, 18.6: from 17 positions on a
+// block's rows are 32 long, the ones here 24 up to L = 24.  A third wave loses everywhere (1000 x (k = 6, L = 9) 35.1,
+// 39.1, 1000 x (k = 8, L = 24) 90, 117).
+bool batch_lanes_takes(int64_t B, int L, int k, int sms)
 {
-    return B >= kLanesMinB && k >= 2 && k <= kLanesMaxK && L <= kLanesMaxL;
+    if (k < 2 || k > kLanesMaxK || L > kLanesMaxL) return false;
+    const int64_t wave = (int64_t)sms * batch_blocks_per_sm(L, k);
+    if (B <= wave) return false;
+    const bool second = k >= 4 && (k <= 6 || L <= 16 || (k == 7 && L > 24));
+    return !(second && B <= 2 * wave);
 }
 
 int batch_lanes_words(int L)

@@ -138,6 +138,7 @@ cudaError_t launch_eval_packed(const Dev &d, const unsigned char *tables, int64_
                                const uint16_t *ends, const uint8_t *nodes, double *beta, uint8_t *status,
                                bool early, cudaStream_t s);
 size_t batch_smem_bytes(int L, int k);
+int batch_blocks_per_sm(int L, int k);
 // Row numbering of the batched search, per (device, k): rows ordered by (popcount, mask, node), the masks
 // listed by (popcount, value) with the first of each popcount, source mask | target node << 16 of every row
 // with the first row of each popcount.
@@ -167,7 +168,7 @@ struct BatchLanes {
     uint32_t rows;            // k * 2^(k-1)
     int LH;                   // words per row in these tables: 4, 8, 12 or 16
 };
-bool batch_lanes_takes(int64_t B, int L, int k);
+bool batch_lanes_takes(int64_t B, int L, int k, int sms);
 int batch_lanes_words(int L);
 // prep: one block per instance ranks gamma and writes the instance's column of the tables
 cudaError_t launch_batch_prep(int64_t B, int L, int k, const uint64_t *bits, const uint64_t *mem,

@@ -214,7 +214,7 @@ pp_status pp_eval_plans_packed_dev(pp_problem *p, int64_t B, int64_t total, cons
  *   beta_ms [B], m [B], cuts [B*(k-1)], placement [B*k], status [B] (PP_OK / PP_INFEASIBLE,
  *   or PP_ERR_LIMIT for an instance with a value above the limits)
  * Two device paths give the same results.  Batches of more than one or two waves of thread blocks (three blocks to
- * an SM: 444 or 888 instances on 148 SMs), with 2 <= k <= 8 and L <= 32: a
+ * an SM, six for k <= 6: 444 to 1776 instances on 148 SMs), with 2 <= k <= 8 and L <= 32: a
  * warp sweeps 32 instances at once (one per lane); the state, rank and window tables of up to 4096
  * instances at a time live in scratch memory that the call takes from the library's own memory pool
  * and gives back, both ordered on the stream (k = 8, L = 24: 53 KB per instance; PP_ERR_NOMEM if

@@ -1260,8 +1260,8 @@ pp_status pp_random_plans(pp_problem *p, int64_t P, const uint32_t *draws, uint8
     return from_cuda(e2);
 }
 
-// blocks: an instance to a block, else an instance to a lane.  early: behind another piece of the same batch.
-static pp_status queue_exact_batch(int64_t B, int32_t L, int32_t k, const uint64_t *out_bits, const uint64_t *mem,
+// all: instances of the whole batch, of which these may be a piece.  blocks: an instance to a block, else an instance to a lane.  early: behind another piece of the same batch.
+static pp_status queue_exact_batch(int64_t B, int64_t all, int32_t L, int32_t k, const uint64_t *out_bits, const uint64_t *mem,
                                    const uint64_t *node_mem, const uint32_t *bw, double *beta_ms, int32_t *m, int32_t *cuts,
                                    int32_t *placement, int8_t *status, bool blocks, bool early, cudaStream_t s)
 {
@@ -1273,7 +1273,7 @@ static pp_status queue_exact_batch(int64_t B, int32_t L, int32_t k, const uint64
     LaneTables lt;
     PP_CUDA(lane_tables(k, &lt));
     if (blocks) {
-        PP_CUDA(launch_batch(B, L, k, lt, sms, out_bits, mem, node_mem, bw, beta_ms, m, cuts, placement, status, early, s));
+        PP_CUDA(launch_batch(B, all, L, k, lt, sms, out_bits, mem, node_mem, bw, beta_ms, m, cuts, placement, status, early, s));
         return PP_OK;
     }
     // Instance-per-lane path: the tables of a chunk of instances live in scratch memory from the
@@ -1348,7 +1348,7 @@ pp_status pp_solve_exact_batch_dev(int64_t B, int32_t L, int32_t k, const uint64
         return PP_ERR_ARG;
     bool blocks = false;
     PP_CUDA(batch_in_blocks(B, L, k, &blocks));
-    return queue_exact_batch(B, L, k, out_bits, mem, node_mem, bw, beta_ms, m, cuts, placement, status, blocks, false,
+    return queue_exact_batch(B, B, L, k, out_bits, mem, node_mem, bw, beta_ms, m, cuts, placement, status, blocks, false,
                              static_cast<cudaStream_t>(cuda_stream));
 }
 
@@ -1402,7 +1402,7 @@ static pp_status batch_from_host(batch_dev_fn run_dev, bool in_place, int64_t B,
                 const size_t each = sz[i] / nB;
                 std::memcpy(h + off[i] + b0 * each, static_cast<const unsigned char *>(in[i]) + b0 * each, n * each);
             }
-            st = queue_exact_batch((int64_t)n, L, k, reinterpret_cast<uint64_t *>(h + off[0]) + b0 * L,
+            st = queue_exact_batch((int64_t)n, B, L, k, reinterpret_cast<uint64_t *>(h + off[0]) + b0 * L,
                          reinterpret_cast<uint64_t *>(h + off[1]) + b0 * L, reinterpret_cast<uint64_t *>(h + off[2]) + b0 * k,
                          reinterpret_cast<uint32_t *>(h + off[3]) + b0 * k * k, reinterpret_cast<double *>(h + off[4]) + b0,
                          reinterpret_cast<int32_t *>(h + off[5]) + b0, reinterpret_cast<int32_t *>(h + off[6]) + b0 * (k - 1),

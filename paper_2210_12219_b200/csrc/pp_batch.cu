@@ -26,9 +26,12 @@ namespace pp {
 
 namespace {
 
-constexpr int kBatchThreads = 384;
-constexpr int kBatchBlocksPerSm = 3;
-constexpr int kBatchWarps = kBatchThreads / 32;
+// Blocks of 384 threads, three to an SM.  Where the batch does not fit the GPU so and the instances are small (k <= 6, whose
+// levels do not fill twelve warps) blocks of 192, six to an SM: us a call, 888 x (k = 4, L = 24) 23.7 -> 16.6, (k = 6, L = 24)
+// 39.1 -> 30.9, 1616 x (k = 5, L = 53) 68.5 -> 54.2, 4000 x (k = 4, L = 45) 109 -> 74, 3000 x (k = 6, L = 60) 194 -> 170; 444 x (k = 6, L = 24) 20.9, 22.7, 1000 x (k = 7, L = 45) 112, 117.
+// (256 threads, four to an SM: 22.8, 38.7, 61.3 and 20.7, 125; 384, four to an SM: 24.8, 41.1, 63.4.)
+constexpr int kWideThreads = 384, kWideBlocks = 3;
+constexpr int kNarrowThreads = 192, kNarrowBlocks = 6, kNarrowMaxK = 6, kNarrowMaxP = 8;
 constexpr uint32_t kInf16 = 0xFFFFu;
 
 // Lanes and positions a lane of a row of L positions.
@@ -49,7 +52,7 @@ struct BatchLayout {
     int Lc;  // row stride of the window codes: a lane reads those of all its P positions
 };
 
-__host__ __device__ inline BatchLayout batch_layout(int L, int k)
+__host__ __device__ inline BatchLayout batch_layout(int L, int k, int threads)
 {
     BatchLayout b;
     const size_t rows = (size_t)k << (k - 1);
@@ -79,7 +82,7 @@ __host__ __device__ inline BatchLayout batch_layout(int L, int k)
     const size_t strip = (size_t)sh.G * (sh.P + 1) + (size_t)(log2i(sh.G) + 1) * sh.G + 1;
     b.dp = o;
     b.strips = o + table;
-    const size_t end = b.strips + up16((size_t)(kBatchThreads / sh.G) * strip * sizeof(uint16_t));
+    const size_t end = b.strips + up16((size_t)(threads / sh.G) * strip * sizeof(uint16_t));
     size_t q = b.dp;
     b.hist = q; q += up16((size_t)kRankBuckets * sizeof(uint32_t));
     b.val = q;  q += up16(U * L * sizeof(unsigned long long));
@@ -97,22 +100,28 @@ size_t batch_smem_bytes(int L, int k)
 {
     if (k > 12) return (size_t)1 << 40;  // compact rows are 16-bit numbers
     if ((size_t)k * (k - 1) * L + 1 > 65534) return (size_t)1 << 40;  // ranks must fit 16 bits
-    return batch_layout(L, k).total;
+    return batch_layout(L, k, kWideThreads).total;
 }
 
-// Blocks that an SM holds at a time: as many as the registers are shared out for, or as fit its 228 KB.
-int batch_blocks_per_sm(int L, int k)
+// Whether the instances of such a batch go to narrow blocks, and the blocks that an SM holds at a time: as many as the
+// registers are shared out for, or as fit its 228 KB.
+static bool batch_narrow(int64_t all, int L, int k, int sms)
 {
-    const size_t fit = (size_t)(228 << 10) / (batch_smem_bytes(L, k) + 1024);
-    return (int)std::max<size_t>(1, std::min<size_t>(kBatchBlocksPerSm, fit));
+    return k <= kNarrowMaxK && batch_shape(L).P <= kNarrowMaxP && all > (int64_t)sms * kWideBlocks;
+}
+int batch_blocks_per_sm(int64_t all, int L, int k, int sms)
+{
+    const bool narrow = batch_narrow(all, L, k, sms);
+    const size_t fit = (size_t)(228 << 10) / (batch_layout(L, k, narrow ? kNarrowThreads : kWideThreads).total + 1024);
+    return (int)std::max<size_t>(1, std::min<size_t>(narrow ? kNarrowBlocks : kWideBlocks, fit));
 }
 
 namespace {
 
 // t_rowoff, t_rows, t_first: compact row of (S, lowest node of S), rows ordered by (popcount, mask, node);
 // source mask and target node of every row; first row of each popcount
-template <int G, int P>
-__global__ void __launch_bounds__(kBatchThreads, P <= 8 ? kBatchBlocksPerSm : 1)
+template <int NT, int G, int P>
+__global__ void __launch_bounds__(NT, P > 8 ? 1 : NT == kWideThreads ? kWideBlocks : kNarrowBlocks)
 k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const uint32_t *__restrict__ t_rows,
         const uint32_t *__restrict__ t_first, const uint64_t *__restrict__ g_bits, const uint64_t *__restrict__ g_mem,
         const uint64_t *__restrict__ g_cap, const uint32_t *__restrict__ g_bw, double *__restrict__ o_beta,
@@ -120,9 +129,9 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
 {
     // The next piece of a batch that is launched in pieces shares nothing with this one and may start beside it.
     asm volatile("griddepcontrol.launch_dependents;");
-    constexpr int kGroups = kBatchThreads / G;
+    constexpr int kGroups = NT / G;
     extern __shared__ __align__(16) unsigned char smem[];
-    const BatchLayout lay = batch_layout(L, k);
+    const BatchLayout lay = batch_layout(L, k, NT);
     unsigned long long *M = reinterpret_cast<unsigned long long *>(smem + lay.M);
     unsigned long long *cap = reinterpret_cast<unsigned long long *>(smem + lay.cap);
     unsigned long long *s_bits = reinterpret_cast<unsigned long long *>(smem + lay.bits);
@@ -139,7 +148,7 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
     __shared__ unsigned long long s_best;
     __shared__ uint32_t s_least, s_most;  // sizes as floats, rounded down and up
     __shared__ uint32_t s_slow, s_fast, s_U, s_D;
-    __shared__ uint32_t s_sum[kBatchWarps];
+    __shared__ uint32_t s_sum[(NT / 32)];
 
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int sl = lane & (G - 1), at = sl * P;
@@ -153,7 +162,7 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
     const int kk = k * k, jmax = k < L ? k : L;
     PP_BLOCK_BOUNDS(chk);
     [[maybe_unused]] const size_t n_dp = ((size_t)k << (k - 1)) * Ls, n_rank = (size_t)kk * Ls;  // entries of the tables
-    for (uint32_t S = tid; S < (1u << k); S += kBatchThreads) rowoff[S] = (uint16_t)t_rowoff[S];
+    for (uint32_t S = tid; S < (1u << k); S += NT) rowoff[S] = (uint16_t)t_rowoff[S];
 
     for (int64_t inst = blockIdx.x; inst < B; inst += gridDim.x) {
         const uint64_t *bits = g_bits + inst * L, *mem = g_mem + inst * L;
@@ -182,8 +191,8 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
         bool bad = false;
         {
             uint32_t least = 0x7F800000u, most = 0u;
-            for (int i = tid; i < L; i += kBatchThreads) {
-                if (i >= kBatchThreads) {
+            for (int i = tid; i < L; i += NT) {
+                if (i >= NT) {
                     x_bits = bits[i];
                     x_mem = mem[i];
                 }
@@ -238,7 +247,7 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
         }
         // ---- distinct bandwidths and sizes: a value's class is that of its first appearance, and the first
         // appearances are numbered as they come ----
-        for (int p = tid - 32; p >= 0 && p < kk; p += kBatchThreads) {
+        for (int p = tid - 32; p >= 0 && p < kk; p += NT) {
             const uint32_t x = s_bw[p];
             int f = p;
             for (int q = p - 1; q >= 0; --q) f = s_bw[q] == x ? q : f;
@@ -249,7 +258,7 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
             }
             pair_u[p] = (int16_t)(x == 0u ? -1 : f == p ? u : -2 - f);  // -2 - f: as pair f
         }
-        for (int c = kBatchThreads - 1 - tid; wid > 0 && c < L; c += kBatchThreads - 32) {
+        for (int c = NT - 1 - tid; wid > 0 && c < L; c += NT - 32) {
             const unsigned long long x = s_bits[c];
             int f = c;
             for (int q = c - 1; q >= 0; --q) f = s_bits[q] == x ? q : f;
@@ -262,7 +271,7 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
         }
         bad = __syncthreads_or(bad);
         // windows: lo = max(c* - 1, 0), c* = first start layer from which the segment ending at layer c2 fits
-        for (int w = wid; w < k; w += kBatchWarps) {
+        for (int w = wid; w < k; w += NT / 32) {
             const unsigned long long capw = cap[w];
             for (int c2 = lane; c2 < Lc; c2 += 32) {
                 int a = 0, b = c2;
@@ -285,12 +294,12 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
         __syncthreads();
         const int U = (int)s_U, D = (int)s_D;
         // ---- 2. ranks of the quotients, spread out as rank[v][w][c] ----
-        rank_quotients<kBatchThreads, unsigned long long, 16>(
+        rank_quotients<NT, unsigned long long, 16>(
             dbits, ubw, U, D, [&](int u, int d) { return __ddiv_rn((double)dbits[d], (double)ubw[u]); }, __ddiv_rd((double)__uint_as_float(s_least), (double)s_fast),
             __ddiv_ru((double)__uint_as_float(s_most), (double)s_slow),
             reinterpret_cast<uint32_t *>(smem + lay.key), reinterpret_cast<unsigned long long *>(smem + lay.val),
             reinterpret_cast<uint32_t *>(smem + lay.hist), rk, s_sum);
-        for (int pr = wid; pr < kk; pr += kBatchWarps) {
+        for (int pr = wid; pr < kk; pr += (NT / 32)) {
             int u = pair_u[pr];
             if (u < -1) u = pair_u[-2 - u];
             for (int c = lane; c < Ls; c += 32) {
@@ -305,7 +314,7 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
         }
         __syncthreads();  // the per-entry ranks share their bytes with the state table
         // ---- base frontier ----
-        for (int v = wid; v < k; v += kBatchWarps)
+        for (int v = wid; v < k; v += (NT / 32))
             for (int c = lane; c < Ls; c += 32) {
                 const bool fits = c < L && M[c + 1] <= cap[v];
                 if (PP_IN_BOUNDS(chk, (size_t)rowoff[1u << v] * Ls + c, n_dp)) dp[(size_t)rowoff[1u << v] * Ls + c] = (uint16_t)(fits ? 0u : kInf16);
@@ -430,19 +439,19 @@ k_batch(int64_t B, int L, int k, const uint32_t *__restrict__ t_rowoff, const ui
     asm volatile("griddepcontrol.wait;" ::: "memory");  // no launch is complete before the one in front of it
 }
 
-template <int G, int P>
+template <int NT, int G, int P>
 cudaError_t launch_shape(int64_t B, int L, int k, const LaneTables &lt, int sms, const uint64_t *bits, const uint64_t *mem,
                          const uint64_t *cap, const uint32_t *bw, double *beta, int32_t *m, int32_t *cuts,
                          int32_t *placement, int8_t *status, bool early, cudaStream_t s)
 {
-    const size_t sm = batch_smem_bytes(L, k);
-    cudaError_t e = cudaFuncSetAttribute(k_batch<G, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const size_t sm = batch_layout(L, k, NT).total;
+    cudaError_t e = cudaFuncSetAttribute(k_batch<NT, G, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     // a block per instance while they fit a few rounds of the GPU; beyond that blocks take several in turn
     const int64_t grid = std::min<int64_t>(B, (int64_t)sms * 16);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kBatchThreads);
+    cfg.blockDim = dim3(NT);
     cfg.dynamicSmemBytes = sm;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -450,23 +459,28 @@ cudaError_t launch_shape(int64_t B, int L, int k, const LaneTables &lt, int sms,
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = early ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k_batch<G, P>, B, L, k, lt.rowoff, lt.rows, lt.first, bits, mem, cap, bw, beta, m, cuts,
+    return cudaLaunchKernelEx(&cfg, k_batch<NT, G, P>, B, L, k, lt.rowoff, lt.rows, lt.first, bits, mem, cap, bw, beta, m, cuts,
                               placement, status);
 }
 
 }  // namespace
 
-cudaError_t launch_batch(int64_t B, int L, int k, const LaneTables &lt, int sms, const uint64_t *bits, const uint64_t *mem,
+cudaError_t launch_batch(int64_t B, int64_t all, int L, int k, const LaneTables &lt, int sms, const uint64_t *bits, const uint64_t *mem,
                          const uint64_t *cap, const uint32_t *bw, double *beta, int32_t *m, int32_t *cuts,
                          int32_t *placement, int8_t *status, bool early, cudaStream_t s)
 {
     if (B <= 0) return cudaSuccess;
     const BatchShape sh = batch_shape(L);
+    const bool narrow = batch_narrow(all, L, k, sms);
     switch (sh.G * 100 + sh.P) {
+#define PP_LAUNCH(nt, g, p) launch_shape<nt, g, p>(B, L, k, lt, sms, bits, mem, cap, bw, beta, m, cuts, placement, status, early, s)
 #define PP_CASE(g, p) \
-    case g * 100 + p: return launch_shape<g, p>(B, L, k, lt, sms, bits, mem, cap, bw, beta, m, cuts, placement, status, early, s);
-        PP_CASE(4, 4) PP_CASE(8, 4) PP_CASE(16, 4) PP_CASE(32, 4) PP_CASE(32, 8) PP_CASE(32, 16) PP_CASE(32, 32)
+    case g * 100 + p: return narrow ? PP_LAUNCH(kNarrowThreads, g, p) : PP_LAUNCH(kWideThreads, g, p);
+        PP_CASE(4, 4) PP_CASE(8, 4) PP_CASE(16, 4) PP_CASE(32, 4) PP_CASE(32, 8)
 #undef PP_CASE
+        case 3216: return PP_LAUNCH(kWideThreads, 32, 16);
+        case 3232: return PP_LAUNCH(kWideThreads, 32, 32);
+#undef PP_LAUNCH
     }
     return cudaErrorInvalidValue;
 }

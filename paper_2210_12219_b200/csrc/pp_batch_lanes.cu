@@ -631,18 +631,19 @@ cudaError_t launch_level(int nv, const BatchLanes &t, int64_t B, int k, int L, i
 // A batch that fits the GPU at once goes an instance to a block (pp_batch.cu), which then takes the time of one
 // instance; here every level is a launch, however few warps it has.  us a call, here and there: 64 x (k = 4, L = 24)
 // 21.9, 12.5, 444 of them 23.8, 14.5; 300 x (k = 6, L = 24) 35.0, 20.7; 148 x (k = 8, L = 24) 50.5, 35.0, 444 of
-// them 62.1, 53.5.  A second wave of blocks costs as much again: 600 x (k = 6, L = 24) 37.1, 33.3, 888 41.2, 39.1,
-// 888 x (k = 8, L = 16) 70.0, 67.6, 700 x (k = 7, L = 32) 59.8, 53.5; but 600 x (k = 7, L = 24) 49.3, 51.3, (k = 8,
-// L = 24) 72.2, 84.5, 450 x (k = 8, L = 28) 75.9, 78.0, 888 x (k = 2, L = 32) 17.1, 18.6: from 17 positions on a
-// block's rows are 32 long, the ones here 24 up to L = 24.  A third wave loses everywhere (1000 x (k = 6, L = 9) 35.1,
-// 39.1, 1000 x (k = 8, L = 24) 90, 117).
+// them 62.1, 53.5; in narrow blocks 888 x (k = 6, L = 24) 41.8, 30.9.  A second wave costs as much again: 1300 x (k = 6,
+// L = 24) 48.6, 47.3, 1776 55.4, 56.7, 1776 x (k = 6, L = 32) 62.5, 59.6, (k = 4, L = 24) 31.8, 27.2, 888 x (k = 8, L = 16)
+// 70.0, 67.6, 700 x (k = 7, L = 32) 59.8, 53.5; but 600 x (k = 7, L = 24) 49.3, 51.3, (k = 8, L = 24) 72.2, 84.5, 450 x
+// (k = 8, L = 28) 75.9, 78.0: from 17 positions on a block's rows are 32 long, the ones here 24 up to L = 24.  A third
+// wave loses (1000 x (k = 7, L = 9) 47.4, 53.5, (k = 8, L = 24) 90, 117).
 bool batch_lanes_takes(int64_t B, int L, int k, int sms)
 {
     if (k < 2 || k > kLanesMaxK || L > kLanesMaxL) return false;
-    const int64_t wave = (int64_t)sms * batch_blocks_per_sm(L, k);
+    const int64_t wave = (int64_t)sms * batch_blocks_per_sm(B, L, k, sms);
     if (B <= wave) return false;
     const bool second = k >= 4 && (k <= 6 || L <= 16 || (k == 7 && L > 24));
-    return !(second && B <= 2 * wave);
+    const int64_t most = k == 6 && L > 16 && L <= 24 ? wave + wave / 2 : 2 * wave;
+    return !(second && B <= most);
 }
 
 int batch_lanes_words(int L)

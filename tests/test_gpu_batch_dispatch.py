@@ -46,9 +46,11 @@ def device_batch(L, k, arrays):
     return BatchSolution(*(t.cpu().numpy() for t in (beta, m, cuts[:, : k - 1], place, status)))
 
 
-# device batches of at most three (two for k = 8 from 29 layers on) blocks an SM of 148, of twice as many, and larger ones
+# device batches of at most three (two for k = 8 from 29 layers on) blocks an SM of 148, of up to twice as many, for k <= 6
+# in narrow blocks, of up to twice as many again, and larger ones; longer chains, which always go an instance to a block
 @pytest.mark.parametrize("L,k,debug", [(1, 4, False), (7, 8, False), (16, 3, False), (16, 8, False), (17, 6, False), (24, 7, False),
-                                       (25, 7, False), (24, 8, True), (32, 4, True), (32, 8, False)])
+                                       (25, 7, False), (24, 8, True), (32, 4, True), (32, 8, False), (45, 5, True),
+                                       (66, 4, False), (130, 3, False), (258, 2, False)])
 def test_every_path_gives_the_oracles_plans(L, k, debug):
     build.build()
     insts = pool(L, k)
@@ -56,12 +58,12 @@ def test_every_path_gives_the_oracles_plans(L, k, debug):
     beyond = 11  # this one has a transfer beyond the limits
     with library(build.build_debug()) if debug else contextlib.nullcontext():
         # the last one is more than the host variant works on in place: it goes an instance to a lane
-        for B in (63, 64, 296, 297, 444, 445, 888, 889, max(1400, (1 << 20) // (16 * L + 4 * k * (k + 3)) + 45)):
+        for B in (63, 64, 296, 297, 444, 445, 888, 889, 1332, 1333, max(1800, (1 << 20) // (16 * L + 4 * k * (k + 3)) + 45)):
             pick = np.arange(B) % len(insts)
             arrays = [np.stack([getattr(i, f) for i in insts])[pick].copy() for f in FIELDS]
             flagged = pick == beyond
             arrays[0][flagged, L - 1] = np.uint64(1) << np.uint64(41)
-            got = device_batch(L, k, arrays) if B < 1400 else pp.solve_exact_batch(L, k, *arrays)
+            got = device_batch(L, k, arrays) if B < 1800 else pp.solve_exact_batch(L, k, *arrays)
             if B in (64, 889):
                 host = pp.solve_exact_batch(L, k, *arrays)
                 for x, y in zip((got.beta_ms, got.m, got.cuts, got.placement, got.status),

@@ -445,7 +445,7 @@ cudaError_t launch_shape(int64_t B, int L, int k, const LaneTables &lt, int sms,
                          int32_t *placement, int8_t *status, bool early, cudaStream_t s)
 {
     const size_t sm = batch_layout(L, k, NT).total;
-    cudaError_t e = cudaFuncSetAttribute(k_batch<NT, G, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_shared(k_batch<NT, G, P>, 1024);
     if (e != cudaSuccess) return e;
     // a block per instance while they fit a few rounds of the GPU; beyond that blocks take several in turn
     const int64_t grid = std::min<int64_t>(B, (int64_t)sms * 16);

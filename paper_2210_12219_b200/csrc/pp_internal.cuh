@@ -44,6 +44,16 @@ struct Dev {
     const void *pair_meta;     // per-node window constants of the two-mask sweep, or null
 };
 
+// Lets a kernel be launched with any amount of dynamic shared memory a block can have beside `own` bytes (or more) of its
+// own.  The limit belongs to the kernel, not to a launch: set to what one call needs, it is lowered by another thread's
+// smaller call between the two steps of this one, whose launch then fails.
+constexpr size_t kBlockShared = (size_t)227 << 10;
+template <typename... Params>
+inline cudaError_t allow_shared(void (*kernel)(Params...), size_t own = 0)
+{
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kBlockShared - own));
+}
+
 static constexpr unsigned long long kNoBest = ~0ull;
 static constexpr int32_t kErrBacktrack = 1;  // the backtrack found no predecessor (inconsistent table)
 static constexpr int32_t kErrBounds = 3;     // bounds-checking build: an index left its table

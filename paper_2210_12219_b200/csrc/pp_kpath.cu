@@ -151,7 +151,7 @@ cudaError_t launch_kpath(int n, int kk, int64_t Q, const uint32_t *bw, const uin
 {
     if (Q <= 0) return cudaSuccess;
     const size_t sm = kpath_smem_bytes(kk);
-    cudaError_t e = cudaFuncSetAttribute(k_kpath_colour, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_shared(k_kpath_colour);
     if (e != cudaSuccess) return e;
     const int warps = kpath_warps_per_block(kk);
     int64_t blocks = (Q + warps - 1) / warps;

@@ -319,7 +319,7 @@ template <int THREADS, int WORDS>
 cudaError_t launch_match_of(const MatchDev &d, const MatchIn<WORDS> &in, cudaStream_t s)
 {
     const size_t sm = match_smem_bytes(d.n, d.kk);
-    cudaError_t e = cudaFuncSetAttribute(k_match<THREADS, WORDS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_shared(k_match<THREADS, WORDS>, 2048);
     if (e != cudaSuccess) return e;
     MatchDev q = d;
     cudaLaunchConfig_t cfg = {};

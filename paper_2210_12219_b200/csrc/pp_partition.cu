@@ -465,7 +465,7 @@ cudaError_t launch_partition_minsum(int64_t B, int L, int cap_seg, const uint64_
     if (B <= 0) return cudaSuccess;
     if (B >= kLaneMinB && L <= kLaneMaxL) {
         const size_t lsm = (size_t)kLaneWarps * (2 * (size_t)L + 1) * 32 * sizeof(unsigned long long);
-        cudaError_t el = cudaFuncSetAttribute(k_partition_lanes, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm);
+        cudaError_t el = allow_shared(k_partition_lanes);
         if (el != cudaSuccess) return el;
         const int64_t groups = (B + 31) / 32;
         int64_t lblocks = (groups + kLaneWarps - 1) / kLaneWarps;
@@ -482,7 +482,7 @@ cudaError_t launch_partition_minsum(int64_t B, int L, int cap_seg, const uint64_
         return cudaGetLastError();
     }
     const size_t sm = partition_smem_bytes(L);
-    cudaError_t e = cudaFuncSetAttribute(k_partition_minsum, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_shared(k_partition_minsum);
     if (e != cudaSuccess) return e;
     k_partition_minsum<<<(unsigned)blocks, kPartWarps * 32, sm, s>>>(B, L, cap_seg, weight, mem, kappa, cost, m, cuts,
                                                                      sizes, status);

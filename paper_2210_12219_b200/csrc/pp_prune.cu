@@ -1021,7 +1021,7 @@ cudaError_t launch_shape(const PruneDev &d, const PruneHost &h, int sms, cudaStr
     cfg.stream = s;
     cfg.attrs = attr;
     if (const size_t all = shared_bytes<G, P, CT>(d.L, d.k, d.Lp)) {
-        cudaError_t e = cudaFuncSetAttribute(k_prune<G, P, CT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)all);
+        cudaError_t e = allow_shared(k_prune<G, P, CT, true>, 4096);
         if (e != cudaSuccess) return e;
         q.row_cap = (unsigned long long)d.k << (d.k - 1);
         cfg.dynamicSmemBytes = all;
@@ -1037,7 +1037,7 @@ cudaError_t launch_shape(const PruneDev &d, const PruneHost &h, int sms, cudaStr
     const bool cluster = blocks > 1 && widest <= (unsigned long long)kClusterRounds * kClusterBlocks * groups;
     if (cluster) blocks = kClusterBlocks;
     const size_t sm = prune_layout(d.L, d.k, d.Lp, groups, kStripBytes<G, P>, kCodes<G, P, CT>, CT).total;
-    cudaError_t e = cudaFuncSetAttribute(k_prune<G, P, CT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_shared(k_prune<G, P, CT, false>, 4096);
     if (e != cudaSuccess) return e;
     cfg.gridDim = dim3((unsigned)blocks);
     cfg.dynamicSmemBytes = sm;

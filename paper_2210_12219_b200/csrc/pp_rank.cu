@@ -175,7 +175,7 @@ cudaError_t launch_rank_base(const Dev &d, cudaStream_t s, int *launches)
         if (tile_lists < 1) tile_lists = 1;
         if (tile_lists > d.U) tile_lists = d.U;
         const size_t sm = (size_t)tile_lists * d.L * sizeof(double);
-        cudaError_t e = cudaFuncSetAttribute(k_rank_count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaError_t e = allow_shared(k_rank_count, 1024);
         if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((n + kRankQueries - 1) / kRankQueries, (d.U + tile_lists - 1) / tile_lists);

@@ -85,13 +85,11 @@ cudaError_t launch_sweep_generic(const Dev &d, int level, cudaStream_t s)
     size_t sm = (size_t)nw * d.Lpad * d.elem;
     cudaError_t e;
     if (d.elem == 2) {
-        e = cudaFuncSetAttribute(k_sweep_generic<uint16_t>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        e = allow_shared(k_sweep_generic<uint16_t>);
         if (e != cudaSuccess) return e;
         k_sweep_generic<uint16_t><<<(unsigned)n, 128, sm, s>>>(d, level);
     } else {
-        e = cudaFuncSetAttribute(k_sweep_generic<uint32_t>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        e = allow_shared(k_sweep_generic<uint32_t>);
         if (e != cudaSuccess) return e;
         k_sweep_generic<uint32_t><<<(unsigned)n, 128, sm, s>>>(d, level);
     }

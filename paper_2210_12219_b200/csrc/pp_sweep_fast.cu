@@ -428,7 +428,7 @@ template <int NV, bool GEN>
 cudaError_t launch_nv(const Dev &d, int level, const FastMeta *meta, unsigned grid, int split, size_t sm, cudaStream_t s,
                       int first_level)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_sweep_fast<NV, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_shared(k_sweep_fast<NV, GEN>);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);

@@ -432,7 +432,7 @@ size_t pair_smem_bytes(const Dev &d, int nv)
 template <int NV, bool L8>
 cudaError_t launch_pair_nv(const Dev &d, int level, unsigned grid, size_t sm, cudaStream_t s, int first_level)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_sweep_pair<NV, L8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_shared(k_sweep_pair<NV, L8>);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);

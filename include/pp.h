@@ -434,6 +434,11 @@ pp_status pp_debug_starve(int32_t polls);
  * instance to a block, 2 = placement stage, 3 = evaluator, 4 = random plans.  Synchronises the device. */
 pp_status pp_debug_bounds_checks(int32_t kernel, uint64_t *n);
 
+/* Test hook (host only, needs no device): what solves a batch on a device of `sms` multiprocessors.  host: the
+ * batch comes from host arrays (pp_solve_exact_batch).  *threads receives the threads of the block that an
+ * instance goes to, 0 where an instance goes to a lane. */
+pp_status pp_debug_batch_route(int64_t B, int32_t L, int32_t k, int32_t sms, int32_t host, int32_t *threads);
+
 /* Force (1) or forbid (0) the generic sweep kernel; 2 = automatic choice among the kernels that
  * take one source mask per warp (the two-mask kernel is left out); 3 = the two-mask kernel on every
  * level it can run, however small; -1 restores the automatic choice.  Meant for tests that want

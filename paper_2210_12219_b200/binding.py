@@ -30,6 +30,7 @@ EXPORTS = (
     "pp_problem_set_profiling", "pp_eval_plans_packed", "pp_eval_plans_packed_dev",
     "pp_partition_minsum_batch", "pp_partition_minsum_batch_dev",
     "pp_kpath_colour_batch", "pp_kpath_colour_batch_dev", "pp_debug_fail_alloc", "pp_debug_starve", "pp_debug_bounds_checks",
+    "pp_debug_batch_route",
     "pp_kpath_matching", "pp_solve_exact_compute",
 )
 
@@ -97,6 +98,7 @@ def lib() -> ctypes.CDLL:
         L.pp_debug_fail_alloc.argtypes = [i32]
         L.pp_debug_starve.argtypes = [i32]
         L.pp_debug_bounds_checks.argtypes = [i32, ctypes.POINTER(u64)]
+        L.pp_debug_batch_route.argtypes = [i64, i32, i32, i32, i32, ctypes.POINTER(i32)]
         L.pp_kpath_matching.argtypes = [i32, vp, i32, vp, i32, i32, vp, vp, vp, vp]
         L.pp_solve_exact_compute.argtypes = [i32, vp, vp, vp, i32] + [vp] * 7
         L.pp_status_str.argtypes = [ctypes.c_int]
@@ -452,6 +454,13 @@ def debug_bounds_checks(kernel: int) -> int:
     """pp_debug_bounds_checks: accesses checked by the kernels of one source since the last call."""
     n = ctypes.c_uint64()
     _check(lib().pp_debug_bounds_checks(int(kernel), ctypes.byref(n)), "pp_debug_bounds_checks")
+    return int(n.value)
+
+
+def debug_batch_route(B: int, L: int, k: int, host: bool = False, sms: int = 148) -> int:
+    """pp_debug_batch_route: threads of the block an instance of the batch goes to, 0 for a lane; needs no device."""
+    n = ctypes.c_int32()
+    _check(lib().pp_debug_batch_route(int(B), int(L), int(k), int(sms), int(host), ctypes.byref(n)), "pp_debug_batch_route")
     return int(n.value)
 
 

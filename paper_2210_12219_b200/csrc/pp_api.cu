@@ -1260,20 +1260,28 @@ pp_status pp_random_plans(pp_problem *p, int64_t P, const uint32_t *draws, uint8
     return from_cuda(e2);
 }
 
-// all: instances of the whole batch, of which these may be a piece.  blocks: an instance to a block, else an instance to a lane.  early: behind another piece of the same batch.
-static pp_status queue_exact_batch(int64_t B, int64_t all, int32_t L, int32_t k, const uint64_t *out_bits, const uint64_t *mem,
-                                   const uint64_t *node_mem, const uint32_t *bw, double *beta_ms, int32_t *m, int32_t *cuts,
-                                   int32_t *placement, int8_t *status, bool blocks, bool early, cudaStream_t s)
+// What solves a batch: an instance to a lane, or to a block, and there to a narrow one or a wide one.
+struct BatchRoute {
+    bool lanes, narrow;
+};
+
+// in_place: the batch lies in page-locked host memory.
+static BatchRoute batch_route(int64_t B, int L, int k, int sms, bool in_place)
 {
-    int dev = 0, sms = 0, max_sm = 0;
-    PP_CUDA(cudaGetDevice(&dev));
-    PP_CUDA(multiprocessors(dev, &sms));
-    PP_CUDA(cudaDeviceGetAttribute(&max_sm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    if (batch_smem_bytes(L, k) + 1024 > (size_t)max_sm) return PP_ERR_LIMIT;
+    return {!in_place && batch_lanes_takes(B, L, k, sms), batch_narrow(B, L, k, sms)};
+}
+
+// These are the batch whose route it is, or a piece of it.  early: behind another piece of the same batch.
+static pp_status queue_exact_batch(int64_t B, int32_t L, int32_t k, const uint64_t *out_bits, const uint64_t *mem,
+                                   const uint64_t *node_mem, const uint32_t *bw, double *beta_ms, int32_t *m, int32_t *cuts,
+                                   int32_t *placement, int8_t *status, int sms, BatchRoute route, bool early, cudaStream_t s)
+{
+    if (batch_smem_bytes(L, k) + 1024 > kBlockShared) return PP_ERR_LIMIT;
     LaneTables lt;
     PP_CUDA(lane_tables(k, &lt));
-    if (blocks) {
-        PP_CUDA(launch_batch(B, all, L, k, lt, sms, out_bits, mem, node_mem, bw, beta_ms, m, cuts, placement, status, early, s));
+    if (!route.lanes) {
+        PP_CUDA(launch_batch(B, route.narrow, L, k, lt, sms, out_bits, mem, node_mem, bw, beta_ms, m, cuts, placement, status, early,
+                             s));
         return PP_OK;
     }
     // Instance-per-lane path: the tables of a chunk of instances live in scratch memory from the
@@ -1325,14 +1333,12 @@ static pp_status queue_exact_batch(int64_t B, int64_t all, int32_t L, int32_t k,
     return PP_OK;
 }
 
-// Whether a batch goes an instance to a block.
-static cudaError_t batch_in_blocks(int64_t B, int32_t L, int32_t k, bool *blocks)
+// Multiprocessors of the current device.
+static cudaError_t current_sms(int *sms)
 {
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = multiprocessors(dev, &sms);
-    if (e == cudaSuccess) *blocks = !batch_lanes_takes(B, L, k, sms);
-    return e;
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e == cudaSuccess ? multiprocessors(dev, sms) : e;
 }
 
 pp_status pp_solve_exact_batch_dev(int64_t B, int32_t L, int32_t k, const uint64_t *out_bits,
@@ -1346,10 +1352,10 @@ pp_status pp_solve_exact_batch_dev(int64_t B, int32_t L, int32_t k, const uint64
     if (!out_bits || !mem || !node_mem || !bw || !beta_ms || !m || !placement || !status ||
         (!cuts && k > 1))
         return PP_ERR_ARG;
-    bool blocks = false;
-    PP_CUDA(batch_in_blocks(B, L, k, &blocks));
-    return queue_exact_batch(B, B, L, k, out_bits, mem, node_mem, bw, beta_ms, m, cuts, placement, status, blocks, false,
-                             static_cast<cudaStream_t>(cuda_stream));
+    int sms = 0;
+    PP_CUDA(current_sms(&sms));
+    return queue_exact_batch(B, L, k, out_bits, mem, node_mem, bw, beta_ms, m, cuts, placement, status, sms,
+                             batch_route(B, L, k, sms, false), false, static_cast<cudaStream_t>(cuda_stream));
 }
 
 // Host-pointer form of a batched entry point: stage the inputs, run the device-pointer form on
@@ -1365,6 +1371,20 @@ typedef pp_status (*batch_dev_fn)(int64_t, int32_t, int32_t, const uint64_t *, c
 // (k = 4, L = 40) 68.0 -> 63.4; pieces of 64 KB 90.9 and 65.3: a launch costs the host what copying 80 KB does).
 constexpr int64_t kHostPieces = 4;
 constexpr size_t kHostPieceBytes = 128 << 10;
+
+// A host batch's four inputs and five results: bytes of each, and where they lie in one buffer.
+struct BatchArrays {
+    size_t sz[9], off[10];
+};
+static BatchArrays batch_arrays(int64_t B, int32_t L, int32_t k)
+{
+    const size_t nB = (size_t)B;
+    BatchArrays a = {{nB * L * 8, nB * L * 8, nB * k * 8, nB * k * k * 4, nB * 8, nB * 4, nB * (size_t)std::max(k - 1, 1) * 4,
+                      nB * k * 4, nB}, {}};
+    for (int i = 0; i < 9; ++i) a.off[i + 1] = align_up(a.off[i] + a.sz[i], 256);
+    return a;
+}
+
 static pp_status batch_from_host(batch_dev_fn run_dev, bool in_place, int64_t B, int32_t L, int32_t k,
                                  const uint64_t *out_bits, const uint64_t *mem, const uint64_t *node_mem,
                                  const uint32_t *bw, double *beta_ms, int32_t *m, int32_t *cuts,
@@ -1377,11 +1397,8 @@ static pp_status batch_from_host(batch_dev_fn run_dev, bool in_place, int64_t B,
         (!cuts && k > 1))
         return PP_ERR_ARG;
     const size_t nB = (size_t)B;
-    const size_t sz[9] = {nB * L * 8, nB * L * 8, nB * k * 8, nB * k * k * 4, nB * 8,
-                          nB * 4,     nB * (size_t)std::max(k - 1, 1) * 4, nB * k * 4, nB};
-    size_t off[10];
-    off[0] = 0;
-    for (int i = 0; i < 9; ++i) off[i + 1] = align_up(off[i] + sz[i], 256);
+    const BatchArrays arrays = batch_arrays(B, L, k);
+    const size_t *const sz = arrays.sz, *const off = arrays.off;
     if (in_place && off[9] <= kPinnedBytes) {
         struct Lease {
             unsigned char *b = g_pinned.take();
@@ -1389,6 +1406,9 @@ static pp_status batch_from_host(batch_dev_fn run_dev, bool in_place, int64_t B,
         } lease;
         unsigned char *h = lease.b;
         if (!h) return PP_ERR_NOMEM;
+        int sms = 0;
+        PP_CUDA(current_sms(&sms));
+        const BatchRoute route = batch_route(B, L, k, sms, true);
         const void *in[4] = {out_bits, mem, node_mem, bw};
         // An instance to a block: the batch goes in pieces, so that the host copies one while the GPU works on the
         // one before.  With that a batch of this size is faster so than an instance to a lane whatever its number of
@@ -1402,12 +1422,12 @@ static pp_status batch_from_host(batch_dev_fn run_dev, bool in_place, int64_t B,
                 const size_t each = sz[i] / nB;
                 std::memcpy(h + off[i] + b0 * each, static_cast<const unsigned char *>(in[i]) + b0 * each, n * each);
             }
-            st = queue_exact_batch((int64_t)n, B, L, k, reinterpret_cast<uint64_t *>(h + off[0]) + b0 * L,
+            st = queue_exact_batch((int64_t)n, L, k, reinterpret_cast<uint64_t *>(h + off[0]) + b0 * L,
                          reinterpret_cast<uint64_t *>(h + off[1]) + b0 * L, reinterpret_cast<uint64_t *>(h + off[2]) + b0 * k,
                          reinterpret_cast<uint32_t *>(h + off[3]) + b0 * k * k, reinterpret_cast<double *>(h + off[4]) + b0,
                          reinterpret_cast<int32_t *>(h + off[5]) + b0, reinterpret_cast<int32_t *>(h + off[6]) + b0 * (k - 1),
                          reinterpret_cast<int32_t *>(h + off[7]) + b0 * k, reinterpret_cast<int8_t *>(h + off[8]) + b0,
-                                   true, p > 0, nullptr);
+                                   sms, route, p > 0, nullptr);
         }
         const cudaError_t e = cudaStreamSynchronize(nullptr);
         if (st != PP_OK) return st;
@@ -1909,6 +1929,15 @@ pp_status pp_debug_bounds_checks(int32_t kernel, uint64_t *n)
     unsigned long long (*const of[5])() = {prune_checks, batch_checks, match_checks, eval_checks, random_checks};
     if (!n || kernel < 0 || kernel >= 5) return PP_ERR_ARG;
     *n = of[kernel]();
+    return PP_OK;
+}
+
+pp_status pp_debug_batch_route(int64_t B, int32_t L, int32_t k, int32_t sms, int32_t host, int32_t *threads)
+{
+    if (!threads || B < 1 || L < 1 || k < 1 || sms < 1) return PP_ERR_ARG;
+    if (L > PP_MAX_L || k > PP_MAX_K || batch_smem_bytes(L, k) + 1024 > kBlockShared) return PP_ERR_LIMIT;
+    const BatchRoute route = batch_route(B, L, k, sms, host && batch_arrays(B, L, k).off[9] <= kPinnedBytes);
+    *threads = route.lanes ? 0 : batch_block_threads(route.narrow);
     return PP_OK;
 }
 

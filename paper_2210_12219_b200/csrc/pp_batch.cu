@@ -27,7 +27,7 @@ namespace pp {
 namespace {
 
 // Blocks of 384 threads, three to an SM.  Where the batch does not fit the GPU so and the instances are small (k <= 6, whose
-// levels do not fill twelve warps) blocks of 192, six to an SM: us a call, 888 x (k = 4, L = 24) 23.7 -> 16.6, (k = 6, L = 24)
+// levels do not fill twelve warps) blocks of 192, up to six to an SM: us a call, 888 x (k = 4, L = 24) 23.7 -> 16.6, (k = 6, L = 24)
 // 39.1 -> 30.9, 1616 x (k = 5, L = 53) 68.5 -> 54.2, 4000 x (k = 4, L = 45) 109 -> 74, 3000 x (k = 6, L = 60) 194 -> 170; 444 x (k = 6, L = 24) 20.9, 22.7, 1000 x (k = 7, L = 45) 112, 117.
 // (256 threads, four to an SM: 22.8, 38.7, 61.3 and 20.7, 125; 384, four to an SM: 24.8, 41.1, 63.4.)
 constexpr int kWideThreads = 384, kWideBlocks = 3;
@@ -103,17 +103,32 @@ size_t batch_smem_bytes(int L, int k)
     return batch_layout(L, k, kWideThreads).total;
 }
 
-// Whether the instances of such a batch go to narrow blocks, and the blocks that an SM holds at a time: as many as the
-// registers are shared out for, or as fit its 228 KB.
-static bool batch_narrow(int64_t all, int L, int k, int sms)
+int batch_block_threads(bool narrow) { return narrow ? kNarrowThreads : kWideThreads; }
+
+// Blocks that an SM holds at a time: as many as the registers are shared out for, or as fit its 228 KB.
+int batch_blocks_per_sm(int L, int k, bool narrow)
 {
-    return k <= kNarrowMaxK && batch_shape(L).P <= kNarrowMaxP && all > (int64_t)sms * kWideBlocks;
-}
-int batch_blocks_per_sm(int64_t all, int L, int k, int sms)
-{
-    const bool narrow = batch_narrow(all, L, k, sms);
-    const size_t fit = (size_t)(228 << 10) / (batch_layout(L, k, narrow ? kNarrowThreads : kWideThreads).total + 1024);
+    const size_t fit = (size_t)(228 << 10) / (batch_layout(L, k, batch_block_threads(narrow)).total + 1024);
     return (int)std::max<size_t>(1, std::min<size_t>(narrow ? kNarrowBlocks : kWideBlocks, fit));
+}
+
+// Whether the instances of a batch go to narrow blocks: where these take fewer waves.  That is no matter of the batch's
+// size alone: the tables of a longer chain leave room for five narrow blocks, four, or no more than wide ones.  Four are 24
+// warps against 36, which the levels of k > 4 feel: there it has to be a third fewer.  Ratio of the times, narrow to wide,
+// at 500, 600, 900, 1500, 4000 instances (888 are two waves either way from five on, 1.07 to 1.15):
+//   six to an SM    (k = 6, L = 45) 0.82, 0.88, 0.91, 0.85, 0.83
+//   five            (k = 6, L = 60) 0.83, 0.86, 0.93, 0.94, 0.88
+//   four            (k = 6, L = 80) 0.91, 1.19, 1.01, 1.03, 1.03; (k = 5, L = 110) 0.87, 1.20, 0.98, 1.01, 1.00;
+//                   (k = 4, L = 160) 0.77, 1.11, 0.92, 0.93, 0.93
+//   as many as wide (k = 6, L = 100), three, 1.37, 1.26, 1.29, 1.20, 1.23; (k = 6, L = 140), two, 1.24 to 1.31;
+//                   (k = 6, L = 200), one, 1.48 to 1.50
+bool batch_narrow(int64_t B, int L, int k, int sms)
+{
+    if (k > kNarrowMaxK || batch_shape(L).P > kNarrowMaxP) return false;
+    const int held = batch_blocks_per_sm(L, k, true);
+    const auto waves = [&](int blocks) { return (B + (int64_t)sms * blocks - 1) / ((int64_t)sms * blocks); };
+    const int64_t wide = waves(batch_blocks_per_sm(L, k, false)), narrow = waves(held);
+    return held > 4 || k < 5 ? narrow < wide : 3 * narrow <= 2 * wide;
 }
 
 namespace {
@@ -465,13 +480,12 @@ cudaError_t launch_shape(int64_t B, int L, int k, const LaneTables &lt, int sms,
 
 }  // namespace
 
-cudaError_t launch_batch(int64_t B, int64_t all, int L, int k, const LaneTables &lt, int sms, const uint64_t *bits, const uint64_t *mem,
+cudaError_t launch_batch(int64_t B, bool narrow, int L, int k, const LaneTables &lt, int sms, const uint64_t *bits, const uint64_t *mem,
                          const uint64_t *cap, const uint32_t *bw, double *beta, int32_t *m, int32_t *cuts,
                          int32_t *placement, int8_t *status, bool early, cudaStream_t s)
 {
     if (B <= 0) return cudaSuccess;
     const BatchShape sh = batch_shape(L);
-    const bool narrow = batch_narrow(all, L, k, sms);
     switch (sh.G * 100 + sh.P) {
 #define PP_LAUNCH(nt, g, p) launch_shape<nt, g, p>(B, L, k, lt, sms, bits, mem, cap, bw, beta, m, cuts, placement, status, early, s)
 #define PP_CASE(g, p) \

@@ -639,7 +639,7 @@ cudaError_t launch_level(int nv, const BatchLanes &t, int64_t B, int k, int L, i
 bool batch_lanes_takes(int64_t B, int L, int k, int sms)
 {
     if (k < 2 || k > kLanesMaxK || L > kLanesMaxL) return false;
-    const int64_t wave = (int64_t)sms * batch_blocks_per_sm(B, L, k, sms);
+    const int64_t wave = (int64_t)sms * batch_blocks_per_sm(L, k, batch_narrow(B, L, k, sms));
     if (B <= wave) return false;
     const bool second = k >= 4 && (k <= 6 || L <= 16 || (k == 7 && L > 24));
     const int64_t most = k == 6 && L > 16 && L <= 24 ? wave + wave / 2 : 2 * wave;

@@ -148,16 +148,18 @@ cudaError_t launch_eval_packed(const Dev &d, const unsigned char *tables, int64_
                                const uint16_t *ends, const uint8_t *nodes, double *beta, uint8_t *status,
                                bool early, cudaStream_t s);
 size_t batch_smem_bytes(int L, int k);
-int batch_blocks_per_sm(int64_t all, int L, int k, int sms);
+int batch_block_threads(bool narrow);
+int batch_blocks_per_sm(int L, int k, bool narrow);
+bool batch_narrow(int64_t B, int L, int k, int sms);
 // Row numbering of the batched search, per (device, k): rows ordered by (popcount, mask, node), the masks
 // listed by (popcount, value) with the first of each popcount, source mask | target node << 16 of every row
 // with the first row of each popcount.
 struct LaneTables {
     const uint32_t *rowoff = nullptr, *mlist = nullptr, *moff = nullptr, *rows = nullptr, *first = nullptr;
 };
-// all: instances of the whole batch.  early: may start beside the launch in front of it on the stream, which is a piece
-// of the same batch.
-cudaError_t launch_batch(int64_t B, int64_t all, int L, int k, const LaneTables &lt, int sms, const uint64_t *bits, const uint64_t *mem,
+// narrow: blocks of few threads (batch_narrow).  early: may start beside the launch in front of it on the stream, which is a
+// piece of the same batch.
+cudaError_t launch_batch(int64_t B, bool narrow, int L, int k, const LaneTables &lt, int sms, const uint64_t *bits, const uint64_t *mem,
                          const uint64_t *cap, const uint32_t *bw, double *beta, int32_t *m,
                          int32_t *cuts, int32_t *placement, int8_t *status, bool early, cudaStream_t s);
 // Many-instance search with one instance per lane (pp_batch_lanes.cu): tables of a chunk of

@@ -1,0 +1,31 @@
+"""Which batches go an instance to a lane, which to blocks of 192 threads and which to blocks of 384, by the library's own rule
+(no device is needed).  Every line was measured on both sides; the times stand beside the rules."""
+from __future__ import annotations
+
+import pytest
+
+import paper_2210_12219_b200 as pp
+from paper_2210_12219_b200 import build
+
+LANES, NARROW, WIDE = 0, 192, 384
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    build.build()
+
+
+@pytest.mark.parametrize("L,k,held", [(45, 6, 6), (66, 6, 5), (80, 6, 4), (91, 6, 3), (125, 6, 2), (193, 6, 1), (80, 5, 6), (100, 5, 5),
+                                      (125, 5, 4), (140, 5, 3), (180, 5, 2), (125, 4, 6), (160, 4, 4), (200, 4, 3), (256, 3, 5),
+                                      (256, 2, 6), (257, 2, 0), (45, 7, 0)])
+def test_narrow_blocks_take_fewer_waves(L, k, held):
+    # held: narrow blocks an SM has room for; three wide ones, or as many as narrow ones where that is fewer
+    for B in (1, 64, 444, 445, 500, 592, 593, 740, 888, 889, 900, 1184, 1185, 1332, 1500, 1776, 1777, 2221, 4000, 100_000):
+        waves = lambda blocks: -(-B // (148 * blocks))
+        if held == 0:
+            want = False
+        elif held > 4 or k == 4:
+            want = waves(held) < waves(3)
+        else:
+            want = 3 * waves(held) <= 2 * waves(min(held, 3))
+        assert pp.debug_batch_route(B, L, k) == (NARROW if want else WIDE), B

@@ -1265,10 +1265,16 @@ struct BatchRoute {
     bool lanes, narrow;
 };
 
-// in_place: the batch lies in page-locked host memory.
-static BatchRoute batch_route(int64_t B, int L, int k, int sms, bool in_place)
+// pieces: of a batch that lies in page-locked host memory, 0 for one on the device.
+// The pieces of short chains run side by side, so that all the batch's instances count for the width of the blocks.  A
+// piece of chains of more than 32 layers holds few instances, and wide blocks are done with it when the host has copied the
+// next.  A call from host arrays, narrow to wide: 600 and 1000 x (k = 6, L = 20) 0.96, 0.94, L = 32 1.03, 0.96, L = 33 1.02, 0.97,
+// L = 40 1.05, 1.01, L = 60 1.05 (740), L = 100 1.15 (560); k = 5, L = 20 0.95, 0.95, L = 40 1.04, 1.00, L = 80 1.06 (700);
+// k = 3, L = 60 1.00.
+static BatchRoute batch_route(int64_t B, int L, int k, int sms, int64_t pieces)
 {
-    return {!in_place && batch_lanes_takes(B, L, k, sms), batch_narrow(B, L, k, sms)};
+    const int64_t together = pieces && L > 32 ? (B + pieces - 1) / pieces : B;
+    return {!pieces && batch_lanes_takes(B, L, k, sms), batch_narrow(together, L, k, sms)};
 }
 
 // These are the batch whose route it is, or a piece of it.  early: behind another piece of the same batch.
@@ -1355,7 +1361,7 @@ pp_status pp_solve_exact_batch_dev(int64_t B, int32_t L, int32_t k, const uint64
     int sms = 0;
     PP_CUDA(current_sms(&sms));
     return queue_exact_batch(B, L, k, out_bits, mem, node_mem, bw, beta_ms, m, cuts, placement, status, sms,
-                             batch_route(B, L, k, sms, false), false, static_cast<cudaStream_t>(cuda_stream));
+                             batch_route(B, L, k, sms, 0), false, static_cast<cudaStream_t>(cuda_stream));
 }
 
 // Host-pointer form of a batched entry point: stage the inputs, run the device-pointer form on
@@ -1384,6 +1390,10 @@ static BatchArrays batch_arrays(int64_t B, int32_t L, int32_t k)
     for (int i = 0; i < 9; ++i) a.off[i + 1] = align_up(a.off[i] + a.sz[i], 256);
     return a;
 }
+static int64_t host_pieces(const BatchArrays &a)
+{
+    return std::max<int64_t>(1, std::min<int64_t>(kHostPieces, (int64_t)(a.off[4] / kHostPieceBytes)));
+}
 
 static pp_status batch_from_host(batch_dev_fn run_dev, bool in_place, int64_t B, int32_t L, int32_t k,
                                  const uint64_t *out_bits, const uint64_t *mem, const uint64_t *node_mem,
@@ -1408,13 +1418,13 @@ static pp_status batch_from_host(batch_dev_fn run_dev, bool in_place, int64_t B,
         if (!h) return PP_ERR_NOMEM;
         int sms = 0;
         PP_CUDA(current_sms(&sms));
-        const BatchRoute route = batch_route(B, L, k, sms, true);
+        const int64_t pieces = host_pieces(arrays);
+        const BatchRoute route = batch_route(B, L, k, sms, pieces);
         const void *in[4] = {out_bits, mem, node_mem, bw};
         // An instance to a block: the batch goes in pieces, so that the host copies one while the GPU works on the
         // one before.  With that a batch of this size is faster so than an instance to a lane whatever its number of
         // waves, us a call: 300 x (k = 5, L = 24) 68.8 -> 47.5, 444 x (k = 8, L = 24) 110.4 -> 90.6, 1000 of them 182 -> 171,
         // 1400 x (k = 6, L = 18) 148 -> 107, 3600 x (k = 4, L = 9) 177 -> 157.
-        const int64_t pieces = std::max<int64_t>(1, std::min<int64_t>(kHostPieces, (int64_t)(off[4] / kHostPieceBytes)));
         pp_status st = PP_OK;
         for (int64_t p = 0; p < pieces && st == PP_OK; ++p) {
             const size_t b0 = (size_t)(B * p / pieces), n = (size_t)(B * (p + 1) / pieces) - b0;
@@ -1936,7 +1946,8 @@ pp_status pp_debug_batch_route(int64_t B, int32_t L, int32_t k, int32_t sms, int
 {
     if (!threads || B < 1 || L < 1 || k < 1 || sms < 1) return PP_ERR_ARG;
     if (L > PP_MAX_L || k > PP_MAX_K || batch_smem_bytes(L, k) + 1024 > kBlockShared) return PP_ERR_LIMIT;
-    const BatchRoute route = batch_route(B, L, k, sms, host && batch_arrays(B, L, k).off[9] <= kPinnedBytes);
+    const BatchArrays a = batch_arrays(B, L, k);
+    const BatchRoute route = batch_route(B, L, k, sms, host && a.off[9] <= kPinnedBytes ? host_pieces(a) : 0);
     *threads = route.lanes ? 0 : batch_block_threads(route.narrow);
     return PP_OK;
 }

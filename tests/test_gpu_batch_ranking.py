@@ -13,11 +13,8 @@ from paper_2210_12219_b200 import workloads as W
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("L,k", [(7, 3), (24, 8), (32, 8), (17, 5)])
-def test_extreme_and_close_quotients(L, k):
-    build.build()
+def extreme_instances(L, k, n=72):
     rng = np.random.default_rng(100 * L + k)
-    n = 72
     insts = []
     for i in range(n):
         base = W.random_small(95000 + 100 * L + i, L, k)
@@ -40,6 +37,13 @@ def test_extreme_and_close_quotients(L, k):
             bw[rng.random((k, k)) < 0.7] = 0
         np.fill_diagonal(bw, 0)
         insts.append(W.Instance(L, k, bits, base.layer_mem_bytes, base.node_mem_bytes, bw, f"ranking[{i}]"))
+    return insts
+
+
+@pytest.mark.parametrize("L,k", [(7, 3), (24, 8), (32, 8), (17, 5)])
+def test_extreme_and_close_quotients(L, k):
+    build.build()
+    insts = extreme_instances(L, k)
     got = pp.solve_exact_batch(L, k, *(np.stack([getattr(i, f) for i in insts]) for f in (
         "layer_out_bits", "layer_mem_bytes", "node_mem_bytes", "bw_kbps")))
     for b, inst in enumerate(insts):

@@ -48,8 +48,8 @@ def test_bounds_checking_build_runs_the_parity_cases_clean():
         nseg, ends, nodes = W.random_plans(inst, 500, seed=2)
         with pp.Problem.from_instance(inst) as p:
             assert np.array_equal(p.eval_plans(nseg, ends, nodes)[0], oracle.eval_plans(inst, nseg, ends, nodes)[0])
-        # the batched search, both device paths (64 instances and more take the instance-per-lane
-        # kernels); a recorded violation would come back as PP_ERR_CUDA in the instance's status
+        # the batched search, an instance to a block (test_gpu_batch_lanes.py runs this build an instance to a lane);
+        # a recorded violation would come back as PP_ERR_CUDA in the instance's status
         for L, k, n in ((24, 8, 70), (7, 8, 65), (32, 4, 66), (13, 5, 20)):
             insts = [W.random_small(82000 + 100 * L + i, L, k, tight=(i % 3 == 1), dead_links=0.25 if i % 4 == 3 else 0.0)
                      for i in range(n)]

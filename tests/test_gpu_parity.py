@@ -411,7 +411,7 @@ def test_batched_solve_full_config():
 
 
 def test_batched_solve_odd_shapes():
-    # batches too small for the instance-per-lane kernels: one block per instance, chains shorter and
+    # small batches: one block per instance, chains shorter and
     # longer than a warp, a power of two long, more nodes than layers
     for L, k, n in ((1, 1, 3), (2, 3, 6), (5, 2, 9), (13, 5, 40), (3, 6, 12), (16, 3, 8), (30, 7, 10),
                     (32, 4, 8), (33, 4, 8), (70, 3, 6)):
@@ -431,9 +431,9 @@ def test_batched_solve_odd_shapes():
 
 
 def test_batched_solve_instance_per_lane_shapes():
-    # from 64 instances on, chains of up to 32 layers on up to 8 nodes are solved 32 instances to a
-    # warp: every row width of that path (4, 8, 12, 16 words), batches that end inside a group of 32,
-    # more nodes than layers, and the degenerate inputs
+    # the shapes that larger batches solve 32 instances to a warp (every row width of that path: 4, 8, 12, 16 words; more
+    # nodes than layers, degenerate inputs) from host arrays, where batches of this size go an instance to a block;
+    # test_gpu_batch_lanes.py and test_gpu_batch_dispatch.py take them through the other path
     for L, k, n in ((1, 4, 64), (2, 3, 64), (5, 2, 97), (7, 8, 65), (13, 5, 130), (16, 3, 96), (17, 6, 71), (24, 8, 100),
                     (25, 4, 64), (30, 7, 70), (32, 4, 89)):
         insts = [W.random_small(61000 + 100 * L + i, L, k, tight=(i % 3 == 1), ties=(i % 3 == 2),
@@ -459,8 +459,7 @@ def test_batched_solve_instance_per_lane_shapes():
 
 
 def test_batched_solve_asymmetric_links_and_pieces():
-    # a network whose two directions differ has up to k (k - 1) distinct bandwidths: such instances are
-    # ranked by the second preparing pass, symmetric ones by the first, in one batch
+    # a network whose two directions differ has up to k (k - 1) distinct bandwidths; beside symmetric ones in one batch
     rng = np.random.Generator(np.random.PCG64(20240607))
     for L, k, n in ((11, 5, 96), (24, 8, 70), (32, 7, 65)):
         insts = [W.random_small(63000 + 100 * L + i, L, k, tight=(i % 5 == 1), dead_links=0.2 if i % 4 == 3 else 0.0)
@@ -478,7 +477,7 @@ def test_batched_solve_asymmetric_links_and_pieces():
             assert got.status[b] == want.status, (L, k, b)
             assert got.plan(b) == want.plan(), (L, k, b)
             assert got.beta_ms[b] == want.beta_ms or np.isinf(want.beta_ms)
-    # more instances than share the scratch tables at a time: worked off in pieces on the same stream
+    # a host batch of many short chains, worked on in place in pieces (test_gpu_batch_lanes.py has those of the other path)
     L, k, n = 5, 3, 4096 + 45
     insts = [W.random_small(64000 + i, L, k, tight=(i % 3 == 1), ties=(i % 7 == 2)) for i in range(n)]
     got = pp.solve_exact_batch(L, k, *_stack(insts))

@@ -434,6 +434,11 @@ pp_status pp_debug_starve(int32_t polls);
  * instance to a block, 2 = placement stage, 3 = evaluator, 4 = random plans.  Synchronises the device. */
 pp_status pp_debug_bounds_checks(int32_t kernel, uint64_t *n);
 
+/* Test hook: the quotients bits[i] / kbps[i] of n pairs (host arrays, bits below PP_MAX_BITS, 0 < kbps < PP_MAX_KBPS) as the
+ * batched search with an instance to a lane computes them before it ranks them, from reciprocals of the
+ * bandwidths, and by CUDA's correctly rounded division.  Both go to host arrays of n; they must not differ. */
+pp_status pp_debug_quotients(int64_t n, const uint64_t *bits, const uint32_t *kbps, double *by_reciprocal, double *divided);
+
 /* Test hook (host only, needs no device): what solves a batch on a device of `sms` multiprocessors.  host: the
  * batch comes from host arrays (pp_solve_exact_batch).  *threads receives the threads of the block that an
  * instance goes to, 0 where an instance goes to a lane. */

@@ -30,7 +30,7 @@ EXPORTS = (
     "pp_problem_set_profiling", "pp_eval_plans_packed", "pp_eval_plans_packed_dev",
     "pp_partition_minsum_batch", "pp_partition_minsum_batch_dev",
     "pp_kpath_colour_batch", "pp_kpath_colour_batch_dev", "pp_debug_fail_alloc", "pp_debug_starve", "pp_debug_bounds_checks",
-    "pp_debug_batch_route",
+    "pp_debug_batch_route", "pp_debug_quotients",
     "pp_kpath_matching", "pp_solve_exact_compute",
 )
 
@@ -98,6 +98,7 @@ def lib() -> ctypes.CDLL:
         L.pp_debug_fail_alloc.argtypes = [i32]
         L.pp_debug_starve.argtypes = [i32]
         L.pp_debug_bounds_checks.argtypes = [i32, ctypes.POINTER(u64)]
+        L.pp_debug_quotients.argtypes = [i64, vp, vp, vp, vp]
         L.pp_debug_batch_route.argtypes = [i64, i32, i32, i32, i32, ctypes.POINTER(i32)]
         L.pp_kpath_matching.argtypes = [i32, vp, i32, vp, i32, i32, vp, vp, vp, vp]
         L.pp_solve_exact_compute.argtypes = [i32, vp, vp, vp, i32] + [vp] * 7
@@ -462,6 +463,17 @@ def debug_batch_route(B: int, L: int, k: int, host: bool = False, sms: int = 148
     n = ctypes.c_int32()
     _check(lib().pp_debug_batch_route(int(B), int(L), int(k), int(sms), int(host), ctypes.byref(n)), "pp_debug_batch_route")
     return int(n.value)
+
+
+def debug_quotients(bits, kbps):
+    """pp_debug_quotients: bits / kbps as the batched search ranks them, and by CUDA's division."""
+    bits, kbps = np.ascontiguousarray(bits, np.uint64), np.ascontiguousarray(kbps, np.uint32)
+    if bits.ndim != 1 or bits.shape != kbps.shape:
+        raise ValueError("bits and kbps must be one-dimensional and of one length")
+    out = np.empty(bits.size), np.empty(bits.size)
+    _check(lib().pp_debug_quotients(bits.size, bits.ctypes.data, kbps.ctypes.data, out[0].ctypes.data, out[1].ctypes.data),
+           "pp_debug_quotients")
+    return out
 
 
 def debug_starve(polls: int):

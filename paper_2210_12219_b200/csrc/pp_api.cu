@@ -1942,6 +1942,29 @@ pp_status pp_debug_bounds_checks(int32_t kernel, uint64_t *n)
     return PP_OK;
 }
 
+pp_status pp_debug_quotients(int64_t n, const uint64_t *bits, const uint32_t *kbps, double *by_reciprocal, double *divided)
+{
+    if (n < 0 || n > (int64_t)1 << 28) return PP_ERR_ARG;
+    if (n == 0) return PP_OK;
+    if (!bits || !kbps || !by_reciprocal || !divided) return PP_ERR_ARG;
+    for (int64_t i = 0; i < n; ++i)
+        if (bits[i] >= PP_MAX_BITS || kbps[i] >= PP_MAX_KBPS || kbps[i] == 0) return PP_ERR_LIMIT;
+    const size_t each = (size_t)n * 8;
+    unsigned char *buf = nullptr;
+    PP_CUDA(staging_alloc(reinterpret_cast<void **>(&buf), 4 * each, nullptr));
+    uint64_t *d_bits = reinterpret_cast<uint64_t *>(buf);
+    double *d_out = reinterpret_cast<double *>(buf + each);
+    uint32_t *d_kbps = reinterpret_cast<uint32_t *>(buf + 3 * each);
+    cudaError_t e = cudaMemcpyAsync(d_bits, bits, each, cudaMemcpyHostToDevice, nullptr);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(d_kbps, kbps, each / 2, cudaMemcpyHostToDevice, nullptr);
+    if (e == cudaSuccess) e = launch_quotients(n, d_bits, d_kbps, d_out, d_out + n, nullptr);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(by_reciprocal, d_out, each, cudaMemcpyDeviceToHost, nullptr);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(divided, d_out + n, each, cudaMemcpyDeviceToHost, nullptr);
+    cudaFreeAsync(buf, nullptr);
+    const cudaError_t e2 = cudaStreamSynchronize(nullptr);
+    return from_cuda(e != cudaSuccess ? e : e2);
+}
+
 pp_status pp_debug_batch_route(int64_t B, int32_t L, int32_t k, int32_t sms, int32_t host, int32_t *threads)
 {
     if (!threads || B < 1 || L < 1 || k < 1 || sms < 1) return PP_ERR_ARG;

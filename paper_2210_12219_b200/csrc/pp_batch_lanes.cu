@@ -22,6 +22,8 @@
 //   3. k_lanes_back, one warp per instance: the backtrack by the
 //      threshold rule, lanes over the candidates.
 // Same recurrence, final choice and backtrack rule as the single-instance path (pp_sweep.cu).
+#include <algorithm>
+
 #include "pp_blocks.cuh"
 
 namespace pp {
@@ -30,7 +32,9 @@ namespace {
 
 constexpr int kLevelWarps = 4;
 constexpr int kLevelFourBlocks = 5;  // source masks of up to this many nodes: registers capped for four blocks per SM
-constexpr int kPrepThreads = 128, kPrepBlocks = 12;  // 18 KB of shared memory a block at most
+// Registers for twelve blocks an SM; shared memory leaves room for 11 at k = 8, L = 24 (19 KB a block) and for nine at
+// L = 32 (23 KB), the widest shape.
+constexpr int kPrepThreads = 128, kPrepBlocks = 12;
 constexpr int kFlagLimit = 1;     // BatchLanes::flag: an input beyond the limits
 constexpr int kBackWarps = 8;
 constexpr int kLanesMaxK = 8;   // NV <= 7 rows of a source mask in registers
@@ -85,15 +89,28 @@ __device__ __forceinline__ void st_piece(const BatchLanes &t, uint32_t *p, const
 // reciprocal.  x r lies within two units in the last place of x / b, so its remainder is below 2^26 such units and exact, and
 // what the last step rounds is off by less than 2^-50 of a unit.  No quotient comes that near to the middle m between two
 // doubles: x / b - m is a multiple of half a unit over b, hence at least 2^-25 of a unit, and zero never, since m has 54
-// bits, the last one set, and would have to divide x.
+// bits, the last one set, and would have to divide x.  (pp_debug_quotients holds it against __ddiv_rn.)
 __device__ __forceinline__ double quotient(double x, double b, double r)
 {
     const double q = __dmul_rn(x, r);
     return __fma_rn(__fma_rn(-q, b, x), r, q);
 }
 
+// Test hook: the quotients of n pairs, and the same by CUDA's division.
+__global__ void k_quotients(const int64_t n, const uint64_t *__restrict__ bits, const uint32_t *__restrict__ kbps,
+                            double *__restrict__ by_reciprocal, double *__restrict__ divided)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const double x = (double)bits[i], b = (double)kbps[i];
+        by_reciprocal[i] = quotient(x, b, __drcp_rn(b));
+        divided[i] = __ddiv_rn(x, b);
+    }
+}
+
 // Shared memory of an instance in the preparing kernel (byte offsets; every part 16-byte aligned).
-constexpr size_t kDoubles = 32 + 2 * 56;  // distinct sizes, distinct bandwidths and their reciprocals: where val[] goes later
+// Distinct sizes, distinct bandwidths and their reciprocals: where val[] goes later, which is the larger one from 288
+// quotients on (k = 4, L = 9 has 108: 720 bytes more a block).
+constexpr size_t kDoubles = 32 + 2 * 56;
 struct PrepLayout {
     size_t val, key, rk, M, bits, dbits, cap, bw, ubw, hist, pair_u, cls, total;
 };
@@ -125,8 +142,9 @@ __host__ __device__ inline PrepLayout prep_layout(int L, int k)
 //   * distinct usable bandwidths and distinct transfer sizes listed in order of first appearance;
 //   * window start lo_w(c2) by a branch-free binary search over the memory prefix sums;
 //   * ranks by rank_quotients, the quotients of its first pass by the reciprocals of the distinct bandwidths, three fp64
-//     instructions each where a division and two conversions take some thirty (4096 x (k = 8, L = 24) 219.3 -> 218.1 us a
-//     call, L = 32 297.0 -> 295.1, k = 5 62.8 -> 62.2).
+//     instructions each where a division and two conversions take some thirty (4096 x (k = 8, L = 24) 219.2 -> 217.0 us a
+//     call, L = 32 296.6 -> 294.2, L = 9 150.7 -> 149.6; 2048 x (8, 24) 137.2 -> 136.3; 4096 x (5, 24) 63.1 -> 62.6, (4, 12)
+//     42.1 -> 41.6; the runs of one side lie within 0.3 % of their median).
 // What is left is a chain of short dependent phases, a third as long with four warps to an instance as with
 // one; the SM's other instances hide it.
 __global__ void __launch_bounds__(kPrepThreads, kPrepBlocks)
@@ -644,6 +662,14 @@ bool batch_lanes_takes(int64_t B, int L, int k, int sms)
     const bool second = k >= 4 && (k <= 6 || L <= 16 || (k == 7 && L > 24));
     const int64_t most = k == 6 && L > 16 && L <= 24 ? wave + wave / 2 : 2 * wave;
     return !(second && B <= most);
+}
+
+cudaError_t launch_quotients(int64_t n, const uint64_t *bits, const uint32_t *kbps, double *by_reciprocal, double *divided,
+                             cudaStream_t s)
+{
+    if (n <= 0) return cudaSuccess;
+    k_quotients<<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, s>>>(n, bits, kbps, by_reciprocal, divided);
+    return cudaGetLastError();
 }
 
 int batch_lanes_words(int L)

@@ -183,6 +183,9 @@ struct BatchLanes {
 };
 bool batch_lanes_takes(int64_t B, int L, int k, int sms);
 int batch_lanes_words(int L);
+// test hook: n quotients as the preparing kernel ranks them, and by CUDA's division
+cudaError_t launch_quotients(int64_t n, const uint64_t *bits, const uint32_t *kbps, double *by_reciprocal, double *divided,
+                             cudaStream_t s);
 // prep: one block per instance ranks gamma and writes the instance's column of the tables
 cudaError_t launch_batch_prep(int64_t B, int L, int k, const uint64_t *bits, const uint64_t *mem,
                               const uint64_t *cap, const uint32_t *bw, const BatchLanes &t, cudaStream_t s);

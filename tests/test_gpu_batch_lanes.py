@@ -1,5 +1,5 @@
-"""The batched search an instance to a lane, at sizes that the library's own rule sends there: the ranking of extreme and
-close quotients, instances beyond the limits, and batches that are worked off in pieces which share the scratch tables."""
+"""The batched search an instance to a lane, at sizes that the library's own rule sends there: its quotients and the ranking
+of extreme and close ones, instances beyond the limits, and batches that are worked off in pieces which share the scratch tables."""
 from __future__ import annotations
 
 import contextlib
@@ -40,6 +40,43 @@ def check(got, b, want):
 @pytest.fixture(scope="module", autouse=True)
 def _built():
     build.build()
+
+
+def near_middles(n, rng):
+    """Pairs whose quotient lies as near to the middle of two doubles as one with this bandwidth can, on either side."""
+    bits, kbps = [], []
+    for b in rng.integers(1 << 12, 1 << 23, n) * 2 + 1:
+        b = int(b)
+        for sign in (1, -1):
+            x = int(rng.integers(1 << 38, 1 << 39))
+            shift = 52 - ((x // b).bit_length() - 1)  # the quotient times 2^shift has 53 bits before the point
+            x += (sign * pow(2, -(shift + 1), b) - x) % b  # 2^(shift + 1) x = sign modulo b: a middle and 1 / (2 b) of a unit
+            bits.append(x)
+            kbps.append(b)
+    return bits, kbps
+
+
+def test_quotients_are_correctly_rounded():
+    rng = np.random.default_rng(5)
+    edges = [0, 1, 2, 3, (1 << 24) - 1, 1 << 24, (1 << 24) + 1, (1 << 39) - 1, 1 << 39, (1 << 40) - 2, (1 << 40) - 1]
+    links = [1, 2, 3, 5, 7, (1 << 12) - 1, 1 << 12, (1 << 23) - 1, 1 << 23, (1 << 23) + 1, (1 << 24) - 2, (1 << 24) - 1]
+    edge = np.array([(x, b) for x in edges for b in links], dtype=np.uint64)
+    small = np.array([(x, b) for x in range(600) for b in range(1, 600)], dtype=np.uint64)
+    hard = np.array(near_middles(100_000, rng), dtype=np.uint64).T
+    n = 1 << 23
+    whole = np.stack([rng.integers(0, 1 << 40, n, dtype=np.uint64), rng.integers(1, 1 << 24, n, dtype=np.uint64)], axis=1)
+    spread = np.stack([np.exp2(rng.uniform(0, 40, n)).astype(np.uint64), np.exp2(rng.uniform(0, 24, n)).astype(np.uint64)], axis=1)
+    spread[:, 0] = np.minimum(spread[:, 0], (1 << 40) - 1)
+    spread[:, 1] = np.minimum(spread[:, 1], (1 << 24) - 1)
+    for pairs in (edge, small, hard, whole, spread):
+        by_reciprocal, divided = pp.debug_quotients(pairs[:, 0], pairs[:, 1])
+        want = pairs[:, 0].astype(np.float64) / pairs[:, 1].astype(np.float64)
+        assert np.array_equal(by_reciprocal.view(np.uint64), divided.view(np.uint64))
+        assert np.array_equal(by_reciprocal.view(np.uint64), want.view(np.uint64))
+    for x, b in ((1 << 40, 1), (1, 0), (1, 1 << 24)):
+        with pytest.raises(pp.PPError) as e:
+            pp.debug_quotients([x], [b])
+        assert e.value.status == pp.PP_ERR_LIMIT
 
 
 @pytest.mark.parametrize("debug", [False, True])

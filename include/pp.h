@@ -213,8 +213,9 @@ pp_status pp_eval_plans_packed_dev(pp_problem *p, int64_t B, int64_t total, cons
  *   out_bits [B*L], mem [B*L], node_mem [B*k], bw [B*k*k]   inputs, instance-major
  *   beta_ms [B], m [B], cuts [B*(k-1)], placement [B*k], status [B] (PP_OK / PP_INFEASIBLE,
  *   or PP_ERR_LIMIT for an instance with a value above the limits)
- * Two device paths give the same results.  Batches of more than one or two waves of thread blocks (three blocks to
- * an SM, six for k <= 6: 444 to 1776 instances on 148 SMs), with 2 <= k <= 8 and L <= 32: a
+ * Two device paths give the same results.  Batches of more than one wave of thread blocks (three blocks to an SM, two
+ * for k = 8 from 29 layers on, six for k <= 6: 444, 296, 888 instances on 148 SMs), or than two where blocks are the
+ * faster path that long, with 2 <= k <= 8 and L <= 32: a
  * warp sweeps 32 instances at once (one per lane); the state, rank and window tables of up to 4096
  * instances at a time live in scratch memory that the call takes from the library's own memory pool
  * and gives back, both ordered on the stream (k = 8, L = 24: 53 KB per instance; PP_ERR_NOMEM if
@@ -223,7 +224,8 @@ pp_status pp_eval_plans_packed_dev(pp_problem *p, int64_t B, int64_t total, cons
  * Returns PP_ERR_LIMIT without touching outputs when the instance shape does not fit one block:
  * k > 12, k*(k-1)*L + 1 > 65534 (ranks are 16-bit), or k * 2^(k-1) * L 16-bit states plus the
  * rank tables beyond the shared memory of a block (k = 8, L = 24 needs 62 KB).  The host variant works on a
- * batch of up to 1 MB where it lies in page-locked memory, larger ones go through device memory; it is
+ * batch of up to 1 MB where it lies in page-locked memory, always a thread block to an instance and so without scratch;
+ * larger ones go through device memory as device batches do; it is
  * synchronous and uses the legacy default stream; the _dev variant takes device pointers and a
  * stream and is asynchronous.  cuts may be NULL when k == 1.
  */

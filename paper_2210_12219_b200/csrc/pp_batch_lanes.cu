@@ -649,11 +649,17 @@ cudaError_t launch_level(int nv, const BatchLanes &t, int64_t B, int k, int L, i
 // A batch that fits the GPU at once goes an instance to a block (pp_batch.cu), which then takes the time of one
 // instance; here every level is a launch, however few warps it has.  us a call, here and there: 64 x (k = 4, L = 24)
 // 21.9, 12.5, 444 of them 23.8, 14.5; 300 x (k = 6, L = 24) 35.0, 20.7; 148 x (k = 8, L = 24) 50.5, 35.0, 444 of
-// them 62.1, 53.5; in narrow blocks 888 x (k = 6, L = 24) 41.8, 30.9.  A second wave costs as much again: 1300 x (k = 6,
-// L = 24) 48.6, 47.3, 1776 55.4, 56.7, 1776 x (k = 6, L = 32) 62.5, 59.6, (k = 4, L = 24) 31.8, 27.2, 888 x (k = 8, L = 16)
-// 70.0, 67.6, 700 x (k = 7, L = 32) 59.8, 53.5; but 600 x (k = 7, L = 24) 49.3, 51.3, (k = 8, L = 24) 72.2, 84.5, 450 x
-// (k = 8, L = 28) 75.9, 78.0: from 17 positions on a block's rows are 32 long, the ones here 24 up to L = 24.  A third
-// wave loses (1000 x (k = 7, L = 9) 47.4, 53.5, (k = 8, L = 24) 90, 117).
+// them 62.1, 53.5; in narrow blocks 888 x (k = 6, L = 24) 41.8, 30.9.  From there on blocks cost by the wave, lanes by the
+// instance (three seeds; the runs of one side lie within 1 %).  A second wave is the faster one
+//   for k = 4, 5                 1000 x (4, 17) 26.4, 22.8, 1776 30.1, 27.2; (5, 32) 37.3, 30.8 and 45.3, 39.2
+//   for k = 6, 7 up to 16 layers 1776 x (6, 16) 47.4, 43.3; 460 x (7, 16) 41.2, 36.8, 888 49.2, 45.3
+//       and from 25 on           1776 x (6, 25) 59.7, 57.6, (6, 32) 62.1, 59.7; 888 x (7, 25) 63.9, 60.6, (7, 32) 66.8, 61.7
+//   for k = 8 up to 16           460 x (8, 16) 54.5, 51.8, 888 67.9, 67.9; (8, 9) 51.5, 47.5 and 64.6, 63.8.
+// From 17 to 24 positions a block's rows are 32 long, the ones here 24.  With k = 6 the lines then cross in the middle of
+// that wave: 1000 x (6, 17) 41.3, 41.5, 1330 47.2, 45.8, 1500 49.5, 51.3, 1776 52.0, 55.6; (6, 24) 43.3, 43.2, 49.1, 47.4, 51.5,
+// 51.7, 54.5, 57.3; k = 7 hardly gains anywhere (460, 600, 888 x (7, 24) 46.1, 45.8, 49.6, 51.5, 56.1, 59.7) and k = 8 loses
+// (460 x (8, 24) 64.1, 74.1), with longer rows too (888 x (8, 28) 99.6, 104.8; two blocks to an SM from 29 on: 600 x (8, 32)
+// 84.4, 106.7).  A third wave loses (2200 x (6, 24) 60.2, 70.1, (4, 17) 32.6, 35.1) or gains 3 to 5 % ((5, 32) 50.5, 48.2).
 bool batch_lanes_takes(int64_t B, int L, int k, int sms)
 {
     if (k < 2 || k > kLanesMaxK || L > kLanesMaxL) return false;

@@ -39,3 +39,24 @@ def test_host_batches_count_a_piece_of_long_chains(L, k, B, want):
     assert pp.debug_batch_route(B, L, k, host=True) == want
     if L > 32 and k <= 6:
         assert pp.debug_batch_route(B, L, k) == (NARROW if B > 444 and L < 91 else WIDE)
+
+
+# batches of short chains: a wave of blocks (three to an SM, six narrow ones for k <= 6, two for k = 8 from 29 layers on), two waves, or
+# one and a half go an instance to a block, larger ones an instance to a lane; host batches of up to 1 MB never do
+@pytest.mark.parametrize("L,k,most", [(24, 2, 888), (16, 3, 888), (9, 4, 1776), (32, 4, 1776), (20, 5, 1776), (16, 6, 1776), (17, 6, 1332), (24, 6, 1332),
+                                      (25, 6, 1776), (32, 6, 1776), (16, 7, 888), (17, 7, 444), (24, 7, 444), (25, 7, 888), (32, 7, 888),
+                                      (16, 8, 888), (17, 8, 444), (28, 8, 444), (29, 8, 296), (32, 8, 296)])
+def test_larger_batches_of_short_chains_go_to_the_lanes(L, k, most):
+    for B in (1, 64, most):
+        assert pp.debug_batch_route(B, L, k) != LANES, B
+    for B in (most + 1, 2 * most, 4096, 100_000):
+        assert pp.debug_batch_route(B, L, k) == LANES, B
+        arrays = (8 * L, 8 * L, 8 * k, 4 * k * k, 8, 4, 4 * (k - 1), 4 * k, 1)  # bytes an instance
+        in_place = sum(-(-B * a // 256) * 256 for a in arrays) <= 1 << 20
+        assert (pp.debug_batch_route(B, L, k, host=True) != LANES) == in_place, B
+
+
+@pytest.mark.parametrize("L,k", [(33, 8), (24, 9), (24, 1)])
+def test_other_shapes_never_do(L, k):
+    for B in (1, 4096, 100_000):
+        assert pp.debug_batch_route(B, L, k) != LANES

@@ -78,3 +78,24 @@ def test_every_path_gives_the_oracles_plans(L, k, debug):
                 assert got.beta_ms[b] == w.beta_ms or np.isinf(w.beta_ms), (B, b)
             for x in (got.beta_ms, got.m, got.status):  # and all the others like the first of their kind
                 assert np.array_equal(x, x[pick])
+
+
+# narrow blocks on rows that take them two rounds to stage, and batches of more instances than blocks, which take several
+# in turn (narrow and wide ones)
+@pytest.mark.parametrize("L,k,B,threads", [(200, 3, 445, 192), (256, 2, 445, 192), (193, 3, 900, 192), (45, 6, 2401, 192), (45, 4, 4801, 192),
+                                           (45, 7, 2401, 384)])
+@pytest.mark.parametrize("debug", [False, True])
+def test_long_rows_and_blocks_of_several_instances(L, k, B, threads, debug):
+    import torch
+    build.build()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    insts = pool(L, k)
+    want = [oracle.dp_naive(i) for i in insts]
+    pick = np.random.default_rng(B).permutation(B) % len(insts)
+    with library(build.build_debug()) if debug else contextlib.nullcontext():
+        assert pp.debug_batch_route(B, L, k, sms=sms) == threads
+        got = device_batch(L, k, [np.stack([getattr(i, f) for i in insts])[pick] for f in FIELDS])
+    for b in range(B):
+        w = want[pick[b]]
+        assert got.status[b] == w.status and got.plan(b) == w.plan(), b
+        assert got.beta_ms[b] == w.beta_ms or np.isinf(w.beta_ms), b

@@ -1266,14 +1266,19 @@ struct BatchRoute {
 };
 
 // pieces: of a batch that lies in page-locked host memory, 0 for one on the device.
-// The pieces of short chains run side by side, so that all the batch's instances count for the width of the blocks.  A
-// piece of chains of more than 32 layers holds few instances, and wide blocks are done with it when the host has copied the
-// next.  A call from host arrays, narrow to wide: 600 and 1000 x (k = 6, L = 20) 0.96, 0.94, L = 32 1.03, 0.96, L = 33 1.02, 0.97,
-// L = 40 1.05, 1.01, L = 60 1.05 (740), L = 100 1.15 (560); k = 5, L = 20 0.95, 0.95, L = 40 1.04, 1.00, L = 80 1.06 (700);
-// k = 3, L = 60 1.00.
+// The pieces of short chains run side by side, so that all the batch's instances count for the width of the blocks.
+// Pieces of chains of more than 32 layers hold fewer instances: up to 36 layers two of them meet on the GPU, and beyond
+// that wide blocks are done with one when the host has copied the next.  A call from host arrays, narrow and wide, us
+// (three seeds; the runs of one side lie within 2 %):
+//   (k = 6, L = 33)  500 73.9, 75.7; 600 80.7, 79.0; 740 94.3, 90.7; 888 103.0, 99.3; 1000 110.1, 114.3; 1100 116.4, 119.5
+//   (6, 36)          500 75.2, 77.0; 600 83.3, 81.0; 740 97.7, 93.1; 888 106.7, 101.3; 1000 113.4, 115.2; 1100 120.9, 121.6
+//   (6, 40), (6, 50) 500 79.9, 75.8 and 87.8, 82.5; 740 100.8, 95.0 and 110.1, 105.3; 1000 x (6, 40) 118.0, 117.3
+//   (5, 33), (5, 50) 600 67.6, 64.1 and 84.1, 81.3; 1000 92.7, 93.0 and 113.7, 112.8; (4, 33) to (4, 60) within 2 %
+// (two pieces of 222 fill a wave of wide blocks, 500 and 1000 instances come in pieces of 250).
 static BatchRoute batch_route(int64_t B, int L, int k, int sms, int64_t pieces)
 {
-    const int64_t together = pieces && L > 32 ? (B + pieces - 1) / pieces : B;
+    const int64_t each = pieces ? (B + pieces - 1) / pieces : B;
+    const int64_t together = !pieces || L <= 32 ? B : L <= 36 ? std::min(B, 2 * each) : each;
     return {!pieces && batch_lanes_takes(B, L, k, sms), batch_narrow(together, L, k, sms)};
 }
 

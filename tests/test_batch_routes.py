@@ -32,10 +32,12 @@ def test_narrow_blocks_take_fewer_waves(L, k, held):
 
 
 @pytest.mark.parametrize("L,k,B,want", [(20, 6, 600, NARROW), (24, 6, 1000, NARROW), (32, 4, 1000, NARROW), (33, 6, 600, WIDE), (40, 5, 1000, WIDE),
+                                        (33, 6, 500, NARROW), (33, 6, 740, WIDE), (33, 6, 1000, NARROW), (36, 6, 1100, NARROW), (37, 6, 1000, WIDE),
                                         (60, 6, 740, WIDE), (100, 6, 560, WIDE), (33, 6, 100, WIDE), (60, 6, 2000, NARROW),
                                         (60, 7, 800, WIDE)])
 def test_host_batches_count_a_piece_of_long_chains(L, k, B, want):
-    # up to 1 MB a host batch goes in pieces; 2000 x (60, 6) is more and goes as a device batch does
+    # up to 1 MB a host batch goes in pieces, of which two count up to 36 layers and one beyond; 2000 x (60, 6) is more
+    # and goes as a device batch does
     assert pp.debug_batch_route(B, L, k, host=True) == want
     if L > 32 and k <= 6:
         assert pp.debug_batch_route(B, L, k) == (NARROW if B > 444 and L < 91 else WIDE)

@@ -1858,6 +1858,13 @@ pp_status pp_solve_exact_compute(int32_t L, const uint64_t *layer_out_bits, cons
     quotient_range(1, Wp + L, k, node_speed, &lo, &hi);       // longest: all of them
     prune_key_range(hi > 0.0 ? lo : 1.0, hi > 0.0 ? hi : 1.0, &q);
     prune_node_bounds(node_mem_bytes, M[L], &q);
+    // all nodes together cannot do all the work in less (the quotients' roundings are far below the margin)
+    double speeds = 0.0;
+    for (int v = 0; v < k; ++v) speeds += (double)node_speed[v];
+    if (speeds > 0.0) {
+        const double floor_ms = (double)Wp[L] / speeds * (1.0 - 1e-9);
+        std::memcpy(&q.key_floor, &floor_ms, sizeof floor_ms);
+    }
     int dev = 0, sms = 0;
     PP_CUDA(cudaGetDevice(&dev));
     PP_CUDA(multiprocessors(dev, &sms));

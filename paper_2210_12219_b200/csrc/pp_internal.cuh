@@ -213,7 +213,8 @@ struct PruneDev {
     uint32_t arrivals;         // blocks a barrier in global memory waits for, and polls before it gives up (set by
     int polls;                 // the launch)
     int key_shift;             // keys: 1 + (bits of the double - key_base) >> key_shift
-    unsigned long long key_base;
+    unsigned long long key_base, key_top;  // bits of the smallest and of the largest positive term
+    unsigned long long key_floor;  // bits of a value that no plan is below
     uint32_t fallback;         // 1 = the caller has another search (note->dense asks for it)
     uint32_t whole;            // nodes that hold the whole chain
     uint32_t tight_levels;     // bit j: some rest of the chain may not fit the nodes that j used ones leave

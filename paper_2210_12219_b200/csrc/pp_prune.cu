@@ -34,8 +34,9 @@
 // A group of G lanes holds a row, P consecutive cut positions per lane.
 #include <algorithm>
 #include <cstring>
+#include <functional>
 
-#include "pp_blocks.cuh"
+#include "pp_thresholds.cuh"
 
 namespace pp {
 
@@ -97,7 +98,7 @@ __device__ __forceinline__ uint32_t group_min(uint32_t u)
 
 // Shared memory: the part common to the block, then one strip per group of lanes.
 struct PruneLayout {
-    size_t bits, M, cap, bw, gmin, lo, code, Wp, speed, strips, total;
+    size_t bits, M, cap, bw, Wp, speed, gmin, lo, code, strips, total;
 };
 __host__ __device__ inline PruneLayout prune_layout(int L, int k, int Lp, int groups, size_t strip, bool codes, bool compute)
 {
@@ -108,11 +109,11 @@ __host__ __device__ inline PruneLayout prune_layout(int L, int k, int Lp, int gr
     p.M = take((size_t)(L + 1) * 8);
     p.cap = take((size_t)k * 8);
     p.bw = take((size_t)k * k * 4);
-    p.gmin = take((size_t)k * k * 4);
-    p.lo = take((size_t)k * Lp * 2);
-    p.code = take(codes ? (size_t)k * Lp * sizeof(WindowCode) : 0);
     p.Wp = take(compute ? (size_t)(L + 1) * 8 : 0);
     p.speed = take(compute ? (size_t)k * 4 : 0);
+    p.gmin = take((size_t)k * k * 4);  // the tables of the search by thresholds lie from here on, before the others do
+    p.lo = take((size_t)k * Lp * 2);
+    p.code = take(codes ? (size_t)k * Lp * sizeof(WindowCode) : 0);
     p.strips = o;
     p.total = o + (size_t)groups * strip;
     return p;
@@ -248,9 +249,11 @@ struct PruneIn<N, true> {
     unsigned long long Wp[N + 1];
 };
 
-// SM: the tables of the search in shared memory, one block (launch_prune)
-template <int G, int P, bool CT, bool SM>
-__global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d, const __grid_constant__ PruneIn<G * P, CT> params)
+// SM: the tables of the search in shared memory, one block (launch_prune).  TH: the search by thresholds first, with its tables
+// as tlay has them.
+template <int G, int P, bool CT, bool SM, bool TH>
+__global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d, const ThresholdLayout tlay,
+                                                               const __grid_constant__ PruneIn<G * P, CT> params)
 {
     constexpr int kThreads = prune_threads(P), kWarps = kThreads / 32, kGroups = kThreads / G, kPerWarp = 32 / G;
     extern __shared__ __align__(16) unsigned char smem_prune[];
@@ -304,18 +307,20 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
     const int npairs = k * (k - 1) / 2;
 
     unsigned long long t_start = 0;
-    if (blockIdx.x == 0 && tid == 0) asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t_start));
+    if ((TH || blockIdx.x == 0) && tid == 0) asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t_start));
     // ---- inputs ----
     // read through an address of their own: neighbouring threads read neighbouring words, which the constant
     // bank would serve one after another
     const PruneIn<G * P, CT> *in = &params;
     asm volatile("" : "+l"(in));
-    for (int c = tid; c < Lp; c += kThreads) s_bits[c] = c < L ? (double)in->bits[c] : 0.0;
-    for (int c = tid; c <= L; c += kThreads) s_M[c] = in->M[c];
-    for (int e = tid; e < k * k; e += kThreads) {
-        s_bw[e] = in->bw[e];
-        s_gmin[e] = kInfKey;
+    [[maybe_unused]] unsigned long long *s_raw = reinterpret_cast<unsigned long long *>(smem_prune + tlay.raw);
+    for (int c = tid; c < Lp; c += kThreads) {
+        const unsigned long long x = c < L ? in->bits[c] : 0ull;
+        s_bits[c] = (double)x;
+        if constexpr (TH) s_raw[c] = x << 10 | (unsigned)c;
     }
+    for (int c = tid; c <= L; c += kThreads) s_M[c] = in->M[c];
+    for (int e = tid; e < k * k; e += kThreads) s_bw[e] = in->bw[e];
     if (tid < k) s_cap[tid] = in->cap[tid];
     if (SM && tid < 64) s_count[tid] = 0u;
     if (tid == 0) s_best = kNoBest;
@@ -323,8 +328,27 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
         for (int c = tid; c <= L; c += kThreads) s_Wp[c] = in->Wp[c];
         if (tid < k) s_speed[tid] = in->speed[tid];
     }
-    if (sl == 0) s_strip[Strip<G, P>::kNone] = kInfKey;
     __syncthreads();
+    bool solved = false;  // by thresholds
+    int writer = 0;       // the block that has the result
+    int m = 0, w_end = 0, status = (int)PP_INFEASIBLE;
+    double beta = kInf;
+    if constexpr (TH) {
+        if (CT || d.whole == 0) {
+            const ThresholdIn tin{L, k, s_raw, s_M, s_cap, s_bw, CT ? s_Wp : nullptr, CT ? s_speed : nullptr};
+            const int outcome = threshold_search<(G * P + 31) / 32, CT, kThreads>(d, tin, tlay, smem_prune, chk, s_cut, s_node, &writer, &m, &beta);
+            solved = outcome != kThresholdOpen;
+            if (outcome == kThresholdSolved) status = m > 0 ? (int)PP_OK : (int)PP_ERR_CUDA;
+            if (outcome == kThresholdGaveUp) status = (int)PP_ERR_CUDA;
+            if (m < 0) {
+                m = 0;
+                beta = kInf;
+            }
+            __syncthreads();
+        }
+    }
+    for (int e = tid; e < k * k; e += kThreads) s_gmin[e] = kInfKey;
+    if (sl == 0) s_strip[Strip<G, P>::kNone] = kInfKey;
     auto set_window = [&](int w, int c, int l) {
         s_lo[w * Lp + c] = (int16_t)l;
         if constexpr (kCodes<G, P, CT>) s_code[w * Lp + c] = window_code<G, P, uint32_t>(c, l);
@@ -332,7 +356,8 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
     // window starts: lo[w][c'] = earliest previous cut c >= 0 such that layers c+1..c' fit on w, c' itself when
     // not even layer c' alone does; by bisection, a lane has four positions of a node in flight (runs of
     // neighbouring positions, found by stepping on from one to the next: 9300 cycles at k = 13, L = 337)
-    if (d.lo)  // a problem that is solved again and again has them on the device
+    if (solved) {
+    } else if (d.lo)  // a problem that is solved again and again has them on the device
         for (int w = wid; w < k; w += kWarps)
             for (int c = lane; c < Lp; c += 32) set_window(w, c, c < L ? (int)d.lo[w * L + c] : c);
     else
@@ -379,8 +404,6 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
     KeyMap key_of{d.key_base, d.key_shift, 0u};
     bool dense = false;
     int nblk = SM ? 1 : (int)gridDim.x;  // blocks that work on the search: 1 once block 0 goes on alone
-    int m = 0, w_end = 0, status = (int)PP_INFEASIBLE;
-    double beta = kInf;
 
     // base state of one node: layers 0..c on v
     auto base_key = [&](int v, int c) -> uint32_t {
@@ -483,8 +506,8 @@ __global__ void __launch_bounds__(prune_threads(P), 1) k_prune(const PruneDev d,
         return true;
     };
 
-    bool found = !CT && whole != 0;
-    if (found) {
+    bool found = solved || (!CT && whole != 0);
+    if (found && !solved) {
         m = 1;
         beta = 0.0;
         w_end = __ffs(whole) - 1;
@@ -917,7 +940,7 @@ gave_up:  // a jump: leaving the loops by a flag cost every solve 0.3 % (k = 18,
 result:
     __syncthreads();
 #ifdef PP_DEBUG_BOUNDS
-    if (blockIdx.x == 0 && __ldcg(&ctl->err) != 0) {
+    if ((int)blockIdx.x == writer && __ldcg(&ctl->err) != 0) {
         status = (int)PP_ERR_CUDA;
         beta = kInf;
         m = 0;
@@ -925,7 +948,7 @@ result:
     __syncthreads();
     if (SM && tid == 0) ctl->err = 0;
 #endif
-    if (blockIdx.x == 0) {
+    if ((int)blockIdx.x == writer) {
         if (!dense && tid < PP_MAX_K) {
             d.out->cuts[tid] = m ? s_cut[tid] : -1;
             d.out->placement[tid] = m ? s_node[tid] : -1;
@@ -999,6 +1022,38 @@ size_t shared_bytes(int L, int k, int Lp)
     return all <= kSharedBytes ? all : 0;
 }
 
+constexpr size_t kOwnShared = 8192;  // static shared memory of k_prune, at most
+// Whether the search by thresholds is tried first.  us a call, the bounded search / by thresholds, mean of five to 25 instances:
+//   Eq. 1    cnn chains (L = 50, k = 8) 59.6 / 45.6, (50, 12) 69.0 / 50.3, (30, 9) 56.7 / 44.0; geometric graphs (14, 8) 45.9 / 37.6, (50, 12)
+//            48.9 / 39.2, (60, 9) 45.1 / 38.5; blocks (50, 10) 67.8 / 56.5, (14, 11) 82.6 / 55.3; stages (30, 9) 43.8 / 34.8, (60, 8) 48 / 46
+//   Eq. 2    cnn (50, 7) 51.3 / 46.4, (50, 8) 47.3 / 42.5, (14, 8) 45.2 / 40.6; uniform (40, 8) 53.4 / 45.1; blocks (50, 8) 43.5 / 41.2
+// It runs in a block's shared memory and by one block a threshold, so that it loses where most rows of more than eight or
+// nine nodes live.  Under Eq. 2 that cannot be told beforehand: cnn (50, 10) is 54.8 / 54.0 in the mean of 60 instances, 42 / 39 for an easy one
+// and 73 / 95 for a hard one; there k <= 8, whose sets all have room.  Under Eq. 1, where the windows of the bounded search are scans, k
+// <= 12; three of 60 of (50, 12) lose, 98 / 117 the most.  Chains that two nodes can hold end on the second level of the bounded
+// search (Eq. 2, stages (64, 8) 32.4 / 33.9).  L <= 64: at 128 blocks lose (k = 8, 44.0 / 47.6).
+// kThresholdRows: rows of as many nodes as the chain takes at least; uniform chains, whose optimum takes 6 of 10 nodes, have 2500
+// and more and lose (Eq. 2, (50, 10) 51 / 78).
+constexpr unsigned kThresholdRows = 1500;
+bool threshold_takes(const uint64_t *cap, uint64_t total, int L, int k, bool compute)
+{
+    if (L > 32 * kThresholdW || k > (compute ? kThresholdK : 8)) return false;
+    uint64_t sorted[PP_MAX_K];
+    std::copy(cap, cap + k, sorted);
+    std::sort(sorted, sorted + k, std::greater<uint64_t>());
+    int need = 0;
+    for (uint64_t left = total; need < k && left > 0; ++need) left -= std::min(left, sorted[need]);
+    unsigned rows = 0, binom = 1;
+    for (int j = 1; j <= need; ++j) {
+        binom = binom * (unsigned)(k - j + 1) / (unsigned)j;  // C(k, j)
+        rows += binom * (unsigned)j;
+    }
+    return rows <= kThresholdRows && (compute || need > 2);
+}
+// Where it comes before the search in one block's shared memory: Eq. 1, k = 6, 35 layers 40 to 52 / 33 to 45, 25 layers 30 to 41 / 31 to 41;
+// k = 5, 50 layers 36.8 / 31.5 (and 2 for the scratch that the search behind it may need), 25 30.6 / 32.
+bool threshold_before_shared(int L, int k) { return L <= 32 * kThresholdW && k >= 5 && k * L >= 200; }
+
 template <int G, int P, bool CT>
 cudaError_t launch_shape(const PruneDev &d, const PruneHost &h, int sms, cudaStream_t s)
 {
@@ -1020,24 +1075,36 @@ cudaError_t launch_shape(const PruneDev &d, const PruneHost &h, int sms, cudaStr
     cfg.blockDim = dim3((unsigned)threads);
     cfg.stream = s;
     cfg.attrs = attr;
-    if (const size_t all = shared_bytes<G, P, CT>(d.L, d.k, d.Lp)) {
-        cudaError_t e = allow_shared(k_prune<G, P, CT, true>, 4096);
+    const size_t all = CT && threshold_before_shared(d.L, d.k) ? 0 : shared_bytes<G, P, CT>(d.L, d.k, d.Lp);
+    if (all) {
+        cudaError_t e = allow_shared(k_prune<G, P, CT, true, false>, 4096);
         if (e != cudaSuccess) return e;
         q.row_cap = (unsigned long long)d.k << (d.k - 1);
         cfg.dynamicSmemBytes = all;
-        return cudaLaunchKernelEx(&cfg, k_prune<G, P, CT, true>, q, in);
+        return cudaLaunchKernelEx(&cfg, k_prune<G, P, CT, true, false>, q, ThresholdLayout{}, in);
     }
     // blocks: one round over the targets of the widest level if it is kept whole; a single block where
     // two rounds of it do, its barrier costs next to nothing
     const unsigned long long widest = widest_level(d.k);
     int blocks = (int)std::min<unsigned long long>((widest + groups - 1) / groups, (unsigned long long)sms);
     if (blocks <= 2) blocks = 1;
+    const PruneLayout lay = prune_layout(d.L, d.k, d.Lp, groups, kStripBytes<G, P>, kCodes<G, P, CT>, CT);
+    size_t sm = lay.total;
+    ThresholdLayout tlay{};
+    auto kernel = k_prune<G, P, CT, false, false>;
+    if constexpr (G * P <= 32 * kThresholdW) {
+        if (threshold_takes(h.cap, h.M[d.L], d.L, d.k, CT) && (blocks > 1 || (CT && threshold_before_shared(d.L, d.k)))) {
+            tlay = threshold_layout(d.L, d.k, (G * P + 31) / 32, CT, lay.gmin, kBlockShared - kOwnShared);
+            sm = std::max(sm, tlay.total);
+            blocks = sms;
+            kernel = k_prune<G, P, CT, false, true>;
+        }
+    }
     // up to kClusterRounds rounds of 8 blocks: one cluster, whose barrier is the hardware's (0.3 us; one in
     // global memory 1.5 to 2)
-    const bool cluster = blocks > 1 && widest <= (unsigned long long)kClusterRounds * kClusterBlocks * groups;
+    const bool cluster = tlay.set_cap == 0 && blocks > 1 && widest <= (unsigned long long)kClusterRounds * kClusterBlocks * groups;
     if (cluster) blocks = kClusterBlocks;
-    const size_t sm = prune_layout(d.L, d.k, d.Lp, groups, kStripBytes<G, P>, kCodes<G, P, CT>, CT).total;
-    cudaError_t e = allow_shared(k_prune<G, P, CT, false>, 4096);
+    cudaError_t e = allow_shared(kernel, kOwnShared);
     if (e != cudaSuccess) return e;
     cfg.gridDim = dim3((unsigned)blocks);
     cfg.dynamicSmemBytes = sm;
@@ -1057,7 +1124,7 @@ cudaError_t launch_shape(const PruneDev &d, const PruneHost &h, int sms, cudaStr
         ++q.arrivals;
         q.polls = polls;
     }
-    return cudaLaunchKernelEx(&cfg, k_prune<G, P, CT, false>, q, in);
+    return cudaLaunchKernelEx(&cfg, kernel, q, tlay, in);
 }
 
 }  // namespace
@@ -1084,6 +1151,7 @@ void prune_key_range(double lo, double hi, PruneDev *d)
     std::memcpy(&a, &lo, 8);
     std::memcpy(&b, &hi, 8);
     d->key_base = a;
+    d->key_top = b;
     d->key_shift = 0;
     while (((b - a) >> d->key_shift) >= 0x80000000ull) ++d->key_shift;
 }
@@ -1112,6 +1180,7 @@ void prune_node_bounds(const uint64_t *cap, uint64_t total, PruneDev *d)
 
 bool prune_in_shared(int L, int k, bool compute)
 {
+    if (compute && threshold_before_shared(L, k)) return false;
     const PruneShape sh = prune_shape(L, k);
     const int Lp = prune_row_pad(L, k);
     switch (sh.G * 100 + sh.P) {

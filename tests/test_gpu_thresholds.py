@@ -1,0 +1,79 @@
+"""The search by thresholds at the sizes where it can go wrong: rows of one word and of two, both sides of every line of its
+dispatch, many equal terms, terms of nothing, no plan at all, and instances it has to hand over."""
+from __future__ import annotations
+
+import contextlib
+
+import numpy as np
+import pytest
+
+import oracle
+import paper_2210_12219_b200 as pp
+from oracle import compute_term as CT
+from paper_2210_12219_b200 import build
+from paper_2210_12219_b200 import workloads as W
+from tests.test_gpu_errors import library
+
+pytestmark = pytest.mark.gpu
+
+
+def network(seed, L, k, kind):
+    """Nodes that hold a fifth to two thirds of the chain each; every third kind with links of their own each way."""
+    inst = W.random_small(seed, L, k, ties=kind == 1, dead_links=0.3 if kind == 2 else 0.0)
+    rng = np.random.default_rng(seed)
+    total = float(inst.layer_mem_bytes.sum())
+    inst.node_mem_bytes[:] = (total * rng.uniform(0.2, 0.67, k)).astype(np.uint64)
+    if kind == 3:  # transfers of nothing, and directed links
+        inst.layer_out_bits[rng.random(L) < 0.5] = 0
+        inst.bw_kbps[:] = rng.integers(1000, 12000, (k, k)) * (1 - np.eye(k, dtype=np.int64))
+    if kind == 4:  # hardly room: most have no plan
+        inst.node_mem_bytes[:] = (total * rng.uniform(0.2, 2.2, k) / k).astype(np.uint64)
+    if kind == 5:  # one value everywhere
+        inst.layer_out_bits[:] = 12345
+        inst.bw_kbps[:] = 777 * (1 - np.eye(k, dtype=np.int64))
+    return inst
+
+
+def same(got, want):
+    assert got.status == want.status and got.plan() == want.plan()
+    assert got.beta_ms == want.beta_ms or np.isinf(want.beta_ms)
+
+
+@pytest.mark.parametrize("debug", [False, True])
+@pytest.mark.parametrize("L,k", [(2, 8), (8, 7), (17, 7), (31, 8), (32, 8), (33, 7), (33, 8), (63, 8), (64, 7), (64, 8), (65, 8), (40, 9)])
+def test_transfers_only(L, k, debug):
+    build.build()
+    with library(build.build_debug()) if debug else contextlib.nullcontext():
+        for i in range(18):
+            inst = network(120_000 + 100 * L + 10 * k + i, L, k, i % 6)
+            want = oracle.dp_fact(inst, 4)
+            with pp.Problem.from_instance(inst) as p:
+                same(p.solve_exact(), want)
+                if i < 6:  # the dense search, which takes every form
+                    p.force_generic(1)
+                    same(p.solve_exact(), want)
+
+
+@pytest.mark.parametrize("debug", [False, True])
+@pytest.mark.parametrize("L,k", [(39, 5), (40, 5), (33, 6), (34, 6), (28, 7), (29, 7), (2, 8), (31, 8), (32, 8), (33, 8), (64, 5), (65, 5)])
+def test_compute_times(L, k, debug):
+    build.build()
+    with library(build.build_debug()) if debug else contextlib.nullcontext():
+        for i in range(6 if k < 7 else 3):
+            inst = network(130_000 + 100 * L + 10 * k + i, L, k, i % 6)
+            rng = np.random.default_rng(i)
+            work = rng.integers(0, 10**6, L).astype(np.uint64) if i % 3 else np.full(L, 70_000, np.uint64)
+            speed = rng.integers(0 if i == 2 else 500, 4000, k).astype(np.uint32)
+            same(pp.solve_exact_compute(inst, work, speed), CT.dp(inst, work.tolist(), speed.tolist()))
+
+
+@pytest.mark.parametrize("L,k", [(24, 9), (33, 10), (64, 10), (50, 11), (20, 12), (50, 12), (64, 12)])
+def test_no_work_leaves_the_transfers(L, k):
+    """Nothing costs compute: the optimum of Eq. 2, also where a block's table of node sets runs out."""
+    build.build()
+    for i in range(8):
+        inst = network(140_000 + 100 * L + 10 * k + i, L, k, i % 6)
+        if i >= 6:  # many nodes to a plan, most sets alive
+            inst.node_mem_bytes[:] = (float(inst.layer_mem_bytes.sum()) * np.random.default_rng(i).uniform(0.12, 0.3, k)).astype(np.uint64)
+        want = oracle.dp_fact(inst, 8)
+        same(pp.solve_exact_compute(inst, np.zeros(L, np.uint64), np.full(k, 1000, np.uint32)), want)

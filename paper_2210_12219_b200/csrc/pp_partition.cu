@@ -165,14 +165,14 @@ k_partition_minsum(int64_t B, int L, int cap_seg, const uint64_t *__restrict__ w
 }
 
 // One warp per chain of at most 32 NQ points: lane l holds the points l, l + 32, ... in registers.  A step
-// of the recurrence drops the candidates beyond the window (for good: the ends descend), takes the
-// minimum of what is left by two 32-bit warp reductions and hands the new candidate to its lane; the
-// window ends and the weights come from the lanes' registers one step ahead, off the chain.  The cut list is
-// put together in registers too and leaves in one piece: the outputs may lie across the bus.
+// of the recurrence hands the value of one point to the lanes of the points in front of it, which keep the smallest of those
+// within their windows; the next point's value is then one shuffle away.  (Taking the
+// minimum over a point's window by two warp reductions: 600 chains of 128 points on the device 25.1 us, 8000 of 50 37.1, 8000 of
+// 100 98.5; so 21.0, 27.8, 72.1.)  The cut list is put together in registers too and leaves in one piece: the outputs may lie
+// across the bus.
 //
-// Bound by the chain of L steps.  A call with one chain of 50 points: 31.9 us with the queue and inputs read
-// across the bus, 21.2 us so (120 points: 67.6 -> 38.2; 600 chains of 128: 260 -> 224, 8000 of 50: 782 -> 754).
-// Up to four points a lane: the queue of one lane does not depend on the window, these scans do.
+// Bound by the chain of L steps.  A call with one chain of 50 points: 31.9 us with the queue and inputs read across the bus, 10
+// less with the inputs as parameters; 120 points 35.5 by reductions, 32.6 so.  Up to four points a lane.
 //
 // PARAMS: the inputs of all chains (weights, memory, capacities one after another) are the kernel's
 // parameters; nothing is read across the bus or copied in front of the kernel.
@@ -182,6 +182,8 @@ struct PartIn {
 };
 struct PartNone {};
 constexpr int kWarpMaxL = 128;
+// No suffix of these chains comes near it (weights are below 2^40), and it can take more weights without wrapping.
+constexpr unsigned long long kFar = 1ull << 62;
 
 template <int NQ, bool PARAMS>
 __global__ void __launch_bounds__(kPartWarps * 32)
@@ -247,33 +249,32 @@ k_partition_warp(const __grid_constant__ std::conditional_t<PARAMS, PartIn, Part
                 const int to = end[q] + step;
                 if (to <= L && M[to] - M[min(q * 32 + lane, L)] <= cap) end[q] = to;
             }
-        // backward recurrence
-        unsigned long long G[NQ], live[NQ], g = 1ull, F = kInfCost;  // g: of the next point; cost 0, one partition
+        // Backward recurrence: G of a point goes to all points in front of it whose window holds it, so that the optimum of
+        // the next suffix is complete when its turn comes.
+        unsigned long long G[NQ], best[NQ], g = 1ull;  // g: of the point at hand; cost 0, one partition
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) G[q] = live[q] = kInfCost;
+        for (int q = 0; q < NQ; ++q) {
+            G[q] = kInfCost;
+            best[q] = kFar;
+        }
 #pragma unroll
         for (int q = NQ - 1; q >= 0; --q) {
             const unsigned long long before = q > 0 ? __shfl_sync(kAll, wt[q > 0 ? q - 1 : 0], 31) : 0ull;
             unsigned long long wprev = __shfl_up_sync(kAll, wt[q], 1);  // lane i: weight of the point before i
             if (lane == 0) wprev = before;
-            wprev <<= kPartsBits;
+            wprev = (wprev << kPartsBits) + 1ull;
 #pragma unroll 4
             for (int i = min(L - 1 - q * 32, 31); i >= 0; --i) {
-                const int e = __shfl_sync(kAll, end[q], i);
-                const unsigned long long w = __shfl_sync(kAll, wprev, i);
-                if (lane == i) G[q] = live[q] = g;
-                unsigned long long least = kInfCost;
+                if (lane == i) G[q] = g;
 #pragma unroll
-                for (int p = q; p < NQ; ++p) {
-                    if (p * 32 + lane >= e) live[p] = kInfCost;
-                    least = live[p] < least ? live[p] : least;
+                for (int p = 0; p <= q; ++p) {
+                    const int ahead = (q - p) * 32 + i - lane;
+                    if ((unsigned)ahead < (unsigned)(end[p] - p * 32 - lane) && g < best[p]) best[p] = g;
                 }
-                const uint32_t hi = __reduce_min_sync(kAll, (uint32_t)(least >> 32));
-                const uint32_t lo = __reduce_min_sync(kAll, (uint32_t)(least >> 32) == hi ? (uint32_t)least : kAll);
-                F = (unsigned long long)hi << 32 | lo;
-                g = F == kInfCost ? kInfCost : F + w + 1ull;
+                g = __shfl_sync(kAll, best[q] + wprev, i);
             }
         }
+        const unsigned long long F0 = __shfl_sync(kAll, best[0], 0), F = F0 >= kFar ? kInfCost : F0;
         const int parts = bad || F == kInfCost ? 0 : (int)(F & ((1ull << kPartsBits) - 1ull));
         const bool fits = parts <= cap_seg + 1;  // the cuts fit the caller's rows
         // forward walk: the earliest point that attains the optimum of the suffix

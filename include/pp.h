@@ -437,13 +437,13 @@ pp_status pp_debug_starve(int32_t polls);
 pp_status pp_debug_bounds_checks(int32_t kernel, uint64_t *n);
 
 /* Test hook: the quotients bits[i] / kbps[i] of n pairs (host arrays, bits below PP_MAX_BITS, 0 < kbps < PP_MAX_KBPS) as the
- * batched search with an instance to a lane computes them before it ranks them, from reciprocals of the
+ * batched search with an instance to a lane or a warp computes them, from reciprocals of the
  * bandwidths, and by CUDA's correctly rounded division.  Both go to host arrays of n; they must not differ. */
 pp_status pp_debug_quotients(int64_t n, const uint64_t *bits, const uint32_t *kbps, double *by_reciprocal, double *divided);
 
 /* Test hook (host only, needs no device): what solves a batch on a device of `sms` multiprocessors.  host: the
  * batch comes from host arrays (pp_solve_exact_batch).  *threads receives the threads of the block that an
- * instance goes to, 0 where an instance goes to a lane. */
+ * instance goes to, 0 where an instance shares a block with others and goes to one of its lanes or warps. */
 pp_status pp_debug_batch_route(int64_t B, int32_t L, int32_t k, int32_t sms, int32_t host, int32_t *threads);
 
 /* Force (1) or forbid (0) the generic sweep kernel; 2 = automatic choice among the kernels that

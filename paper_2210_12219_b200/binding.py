@@ -459,14 +459,14 @@ def debug_bounds_checks(kernel: int) -> int:
 
 
 def debug_batch_route(B: int, L: int, k: int, host: bool = False, sms: int = 148) -> int:
-    """pp_debug_batch_route: threads of the block an instance of the batch goes to, 0 for a lane; needs no device."""
+    """pp_debug_batch_route: threads of the block an instance of the batch goes to, 0 where it shares a block; needs no device."""
     n = ctypes.c_int32()
     _check(lib().pp_debug_batch_route(int(B), int(L), int(k), int(sms), int(host), ctypes.byref(n)), "pp_debug_batch_route")
     return int(n.value)
 
 
 def debug_quotients(bits, kbps):
-    """pp_debug_quotients: bits / kbps as the batched search ranks them, and by CUDA's division."""
+    """pp_debug_quotients: bits / kbps as the batched search computes them, and by CUDA's division."""
     bits, kbps = np.ascontiguousarray(bits, np.uint64), np.ascontiguousarray(kbps, np.uint32)
     if bits.ndim != 1 or bits.shape != kbps.shape:
         raise ValueError("bits and kbps must be one-dimensional and of one length")

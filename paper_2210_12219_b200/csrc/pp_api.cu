@@ -1260,7 +1260,7 @@ pp_status pp_random_plans(pp_problem *p, int64_t P, const uint32_t *draws, uint8
     return from_cuda(e2);
 }
 
-// What solves a batch: an instance to a lane, or to a block, and there to a narrow one or a wide one.
+// What solves a batch: an instance to a lane (or a warp, batch_warps_takes), or to a block, and there to a narrow one or a wide one.
 struct BatchRoute {
     bool lanes, narrow;
 };
@@ -1289,6 +1289,11 @@ static pp_status queue_exact_batch(int64_t B, int32_t L, int32_t k, const uint64
 {
     if (batch_smem_bytes(L, k) + 1024 > kBlockShared) return PP_ERR_LIMIT;
     LaneTables lt;
+    if (route.lanes && batch_warps_takes(B, L, k)) {
+        PP_CUDA(lane_tables(k - 1, &lt));
+        PP_CUDA(launch_batch_warps(B, L, k, lt, sms, out_bits, mem, node_mem, bw, beta_ms, m, cuts, placement, status, s));
+        return PP_OK;
+    }
     PP_CUDA(lane_tables(k, &lt));
     if (!route.lanes) {
         PP_CUDA(launch_batch(B, route.narrow, L, k, lt, sms, out_bits, mem, node_mem, bw, beta_ms, m, cuts, placement, status, early,

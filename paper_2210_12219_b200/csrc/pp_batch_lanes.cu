@@ -5,8 +5,8 @@
 // 32 instances at once, lane <-> instance.  Every lane then walks the same masks, nodes and cut
 // positions, so all of that is uniform and unrolled, and the only per-lane data are the states, the
 // gamma ranks and the window lengths.  Those live in global memory, instance-minor: the 32 lanes of a
-// warp read 32 neighbouring pieces of two words.  The tables of a chunk of 4096 instances are larger than L2
-// (k = 8, L = 24: 219 MB against 126; a level hits it for 20 to 45 % of its sectors).
+// warp read 32 neighbouring pieces of two words.  Batches whose tables are larger than L2 (4096 x (k = 8, L = 24): 219 MB
+// against 126) go an instance to a warp (batch_warps_takes).
 //
 // Per chunk of instances:
 //   1. k_lanes_prep, one block per instance: staging, windows, the ranking of gamma (Eq. 3); writes
@@ -83,17 +83,6 @@ __device__ __forceinline__ Piece ld_piece(const BatchLanes &t, const uint32_t *p
 __device__ __forceinline__ void st_piece(const BatchLanes &t, uint32_t *p, const uint32_t *base, size_t words, const Piece &v)
 {
     if (PP_IN_BOUNDS(t, (size_t)(p - base), words)) *reinterpret_cast<Piece *>(p) = v;
-}
-
-// The correctly rounded quotient x / b of integers 0 <= x < 2^40 and 0 < b < 2^24 held as doubles; r is b's correctly rounded
-// reciprocal.  x r lies within two units in the last place of x / b, so its remainder is below 2^26 such units and exact, and
-// what the last step rounds is off by less than 2^-50 of a unit.  No quotient comes that near to the middle m between two
-// doubles: x / b - m is a multiple of half a unit over b, hence at least 2^-25 of a unit, and zero never, since m has 54
-// bits, the last one set, and would have to divide x.  (pp_debug_quotients holds it against __ddiv_rn.)
-__device__ __forceinline__ double quotient(double x, double b, double r)
-{
-    const double q = __dmul_rn(x, r);
-    return __fma_rn(__fma_rn(-q, b, x), r, q);
 }
 
 // Test hook: the quotients of n pairs, and the same by CUDA's division.
@@ -630,18 +619,21 @@ template <int LH>
 cudaError_t launch_level(int nv, const BatchLanes &t, int64_t B, int k, int L, int split, unsigned grid, cudaStream_t s)
 {
     switch (nv) {
-#define PP_CASE(N) \
-    case N: {                                                                                                  \
-        const size_t sm = win_bytes_per_warp(LH) * kLevelWarps;                                                \
-        cudaError_t e = cudaFuncSetAttribute(k_lanes_level<N, LH>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                             (int)sm);                                                          \
-        if (e != cudaSuccess) return e;                                                                        \
-        return launch_dependent(k_lanes_level<N, LH>, grid, kLevelWarps * 32, sm, s, t, B, k, L, split);       \
-    }
+#define PP_CASE(N)                                                                                                     \
+    case N:                                                                                                            \
+        if constexpr (LH != 4 || N <= 5) { /* up to eight layers k = 7 and 8 go an instance to a warp */               \
+            const size_t sm = win_bytes_per_warp(LH) * kLevelWarps;                                                    \
+            cudaError_t e = cudaFuncSetAttribute(k_lanes_level<N, LH>, cudaFuncAttributeMaxDynamicSharedMemorySize,    \
+                                                 (int)sm);                                                             \
+            if (e != cudaSuccess) return e;                                                                            \
+            return launch_dependent(k_lanes_level<N, LH>, grid, kLevelWarps * 32, sm, s, t, B, k, L, split);           \
+        }                                                                                                              \
+        break;
         PP_CASE(1) PP_CASE(2) PP_CASE(3) PP_CASE(4) PP_CASE(5) PP_CASE(6) PP_CASE(7)
 #undef PP_CASE
-        default: return cudaErrorInvalidValue;
+        default: break;
     }
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace

@@ -7,6 +7,17 @@ namespace pp {
 
 __host__ __device__ constexpr int log2i(int x) { return x <= 1 ? 0 : 1 + log2i(x / 2); }
 
+// The correctly rounded quotient x / b of integers 0 <= x < 2^40 and 0 < b < 2^24 held as doubles; r is b's correctly rounded
+// reciprocal.  x r lies within two units in the last place of x / b, so its remainder is below 2^26 such units and exact, and
+// what the last step rounds is off by less than 2^-50 of a unit.  No quotient comes that near to the middle m between two
+// doubles: x / b - m is a multiple of half a unit over b, hence at least 2^-25 of a unit, and zero never, since m has 54
+// bits, the last one set, and would have to divide x.  (pp_debug_quotients holds it against __ddiv_rn.)
+__device__ __forceinline__ double quotient(double x, double b, double r)
+{
+    const double q = __dmul_rn(x, r);
+    return __fma_rn(__fma_rn(-q, b, x), r, q);
+}
+
 // The window minimum of a row that a group of G lanes holds, P consecutive positions a lane: out at
 // position c2 = min of g over [lo, c2 - 1].  The window is the tail of the block (= lane) that holds its
 // start (suffix minima, through shared memory), whole blocks in between (a sparse table over the G block

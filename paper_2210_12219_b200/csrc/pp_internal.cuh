@@ -193,6 +193,11 @@ cudaError_t launch_batch_prep(int64_t B, int L, int k, const uint64_t *bits, con
 cudaError_t launch_batch_lanes(int64_t B, int L, int k, const uint64_t *bits, const uint32_t *bw,
                                const BatchLanes &t, double *beta, int32_t *m, int32_t *cuts,
                                int32_t *placement, int8_t *status, cudaStream_t s);
+// The same with an instance to a warp (pp_batch_warps.cu).  others: the tables of k - 1 nodes
+bool batch_warps_takes(int64_t B, int L, int k);
+cudaError_t launch_batch_warps(int64_t B, int L, int k, const LaneTables &others, int sms, const uint64_t *bits, const uint64_t *mem,
+                               const uint64_t *cap, const uint32_t *bw, double *beta, int32_t *m, int32_t *cuts,
+                               int32_t *placement, int8_t *status, cudaStream_t s);
 // The search as a bounded sparse frontier (pp_prune.cu), one launch per solve.
 struct PruneCtl {              // device; the kernel leaves it as it found it
     unsigned long long best;   // best final state of the levels done: pack_best of its key

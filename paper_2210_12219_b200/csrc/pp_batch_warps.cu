@@ -15,7 +15,7 @@
 // lanes walk the list of node sets of the other nodes, eight sets a trip.  No barriers but the warp's own.
 // What bounds it: 16 000 warp instructions an instance (3500 the bound, 1400 the staging, a trip 92, of which the windows
 // 54) at 55 % of the issue slots while an SM has work (chains of dependent instructions), and then the longest instances, up
-// to 17 probes of 7 us: 2000 instances take 131, 4096 157, 20000 475, and an SM has work 60 % of the time at 4096.
+// to 17 probes of 7 us: 2000 instances take 131, 4096 156 to 172 by seed, 20000 475, and an SM has work 60 % of the time at 4096.
 // Not kept: teams of two to twelve warps for the instances that are not at their bound (187); one queue of instances for two
 // blocks (159) or four (215: the clusters leave SMs idle); states that cannot reach the last layer dropped (193).
 #include <algorithm>

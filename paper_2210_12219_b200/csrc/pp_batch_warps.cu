@@ -8,14 +8,14 @@
 // what the backtrack's threshold rule asks for: no ranking of the quotients.  It starts from a lower bound, the optimum
 // over the plans that may use a node again, which is one word a node; in 58 % of the instances of k = 8, L = 24 that is
 // beta* and one probe confirms it, the others take eight more (4096 of them, us a call: 243 by bisection alone, 172 with the
-// bound, 163 with values instead of ranks bisected; by lanes 218).
+// bound, 161 with values instead of ranks bisected, 150 with longer steps in front of that; by lanes 218).
 //
 // A warp keeps an instance's table in shared memory, reach[S] a row of eight words.  Lane (w, q) takes the rows of
 // target node w: the links into w and the windows of w are registers, a source set is two 16-byte loads, and all
 // lanes walk the list of node sets of the other nodes, eight sets a trip.  No barriers but the warp's own.
 // What bounds it: 16 000 warp instructions an instance (3500 the bound, 1400 the staging, a trip 92, of which the windows
 // 54) at 55 % of the issue slots while an SM has work (chains of dependent instructions), and then the longest instances, up
-// to 17 probes of 7 us: 2000 instances take 131, 4096 156 to 172 by seed, 20000 475, and an SM has work 60 % of the time at 4096.
+// to 15 probes or so of 7 us: 2000 instances take 119, 4096 150, 8000 235, and an SM has work 60 % of the time at 4096.
 // Not kept: teams of two to twelve warps for the instances that are not at their bound (187); one queue of instances for two
 // blocks (159) or four (215: the clusters leave SMs idle); states that cannot reach the last layer dropped (193).
 #include <algorithm>
@@ -471,12 +471,17 @@ k_batch_warps(const int64_t B, const int L, const int k, const uint32_t *__restr
         for (;;) {
             extremes();
             if (least == ~0ull || (m > 0 && least == most)) break;
-            // The smallest candidate; most optima that are not there lie little above it: 10 %, 35 %, twice as far, then whether
-            // there is a plan at all.  Between a threshold without and one with a plan the middle of their bits.
+            // The smallest candidate; most optima that are not there lie little above it: steps that grow, up to ten times as far,
+            // then whether there is a plan at all.  What counts is the longest instance, not the mean: with 1.1, 1.35, 2 and the
+            // largest candidate 4096 x (k = 8, L = 24) took 161 us (six seeds; 2000 131), with 1.07, 1.2, 1.6, 3 164, with 1.15, 1.5, 2.5, 6 155,
+            // with these 150 (2000 119).  Between a threshold without and one with a plan the middle of their bits.
             unsigned long long key = least;
             if (m > 0) key = least + ((most - least) >> 1);
-            else if (tries > 3) key = most;
-            else if (tries > 0) key = (unsigned long long)__double_as_longlong(__dmul_rn(first_t, tries == 1 ? 1.1 : tries == 2 ? 1.35 : 2.0));
+            else if (tries > 5) key = most;
+            else if (tries > 0) {
+                const double far_off = tries == 1 ? 1.2 : tries == 2 ? 1.7 : tries == 3 ? 2.8 : tries == 4 ? 5.0 : 10.0;
+                key = (unsigned long long)__double_as_longlong(__dmul_rn(first_t, far_off));
+            }
             const double t = __longlong_as_double((long long)min(max(key, least), most));
             within(t);
             int got = 0;
@@ -509,20 +514,20 @@ k_batch_warps(const int64_t B, const int L, const int k, const uint32_t *__restr
 }  // namespace
 
 // Whether the batches that do not go an instance to a block (batch_lanes_takes) go an instance to a warp rather than to a lane.
-// A warp takes as long as its instance's probes, 24 instances to an SM; lanes cost by the instance and by the layer.  us a call,
-// in lanes and in warps:
-//   k = 8  900 x L = 5 40.9, 19.1; 900 x 9 68.1, 42.8; 900 x 12 70.2, 60.2; 4096 x 9 150.5, 58.6
-//          1000 x 16 76.0, 90.3; 1400 89.2, 85.0; 4096 161.6, 114.0
-//          1800 x 24 131.0, 129.5; 2200 145.5, 136.1; 4096 218.2, 162.6; 20000 1072, 475; 1400 x 20 109.3, 111.5
-//          1000 x 32 114.6, 131.6; 1400 144.4, 131.1; 4096 295.9, 169.6; 1400 x 28 137.5, 127.6
-//   k = 7  900 x 9 45.7, 41.5; 4096 100.3, 49.7; 1800 x 16 69.7, 73.2; 2600 84.5, 74.8
-//          2200 x 24 92.6, 95.9; 2600 102.9, 97.6; 4096 135.8, 122.0; 1400 x 32 81.6, 89.4; 1800 101.3, 94.0; 4096 171.7, 128.0
-//   k = 6  4096 x 24 89.7, 96.0; 6000 146.2, 122.6 (two rounds of the lanes' tables); 12000 259.9, 211.6
+// A warp takes as long as its instance's probes, 24 instances to an SM; lanes cost by the instance, by the layer and, beyond 4096,
+// by rounds of their tables.  us a call (mean of four seeds), in lanes and in warps:
+//   k = 8  900 x L = 14 71.4, 68.5; 900 x 16 72.5, 75.7; 1200 81.6, 80.0; 1300 84.7, 82.0
+//          1400 x 20 109.2, 100.4; 1400 x 24 111.5, 113.6; 1600 121.6, 120.9; 1800 130.4, 118.5; 4096 219, 150
+//          1000 x 28 113.7, 114.7; 1100 119.9, 113.7; 1000 x 32 115.4, 117.1; 1100 121.5, 117.7; 4096 296, 161
+//   k = 7  900 x 9 45.9, 36.4; 900 x 12 48.0, 46.0; 900 x 13 49.0, 50.3; 1700 x 16 65.5, 66.0; 2000 72.8, 65.1
+//          1800 x 24 82.6, 83.3; 2000 86.6, 82.0; 1400 x 28 79.4, 80.2; 1600 86.8, 82.7; 1400 x 32 81.2, 83.0; 1600 88.7, 85.8
+//   k = 6  1780 x 5 34.0, 24.0; 1780 x 11 46.8, 45.0; 2500 x 13 55.9, 56.2; 4096 x 16 75.6, 81.7; 4200 105.3, 81.7
+//          4096 x 24 89.2, 91.2; 4200 121.0, 94.9; 2500 x 28 74.6, 74.9; 3000 83.8, 77.7; 3000 x 32 85.1, 80.7
 bool batch_warps_takes(int64_t B, int L, int k)
 {
-    if (k == 8) return B >= (L <= 12 ? 0 : L > 16 && L <= 24 ? 2000 : 1400);
-    if (k == 7) return B >= (L <= 10 ? 0 : L <= 24 ? 2600 : 1800);
-    return k == 6 && B >= 6000;
+    if (k == 8) return B >= (L <= 14 ? 0 : L <= 16 ? 1300 : L <= 24 ? 1700 : 1100);
+    if (k == 7) return B >= (L <= 12 ? 0 : L <= 24 ? 2000 : 1600);
+    return k == 6 && B >= (L <= 11 ? 0 : L <= 24 ? 4097 : 3000);
 }
 
 cudaError_t launch_batch_warps(int64_t B, int L, int k, const LaneTables &others, int sms, const uint64_t *bits, const uint64_t *mem,

@@ -14,8 +14,8 @@
 // target node w: the links into w and the windows of w are registers, a source set is two 16-byte loads, and all
 // lanes walk the list of node sets of the other nodes, eight sets a trip.  No barriers but the warp's own.
 // What bounds it: 16 000 warp instructions an instance (3500 the bound, 1400 the staging, a trip 92, of which the windows
-// 54) at 55 % of the issue slots while an SM has work (chains of dependent instructions), and then the longest instances, up
-// to 15 probes or so of 7 us: 2000 instances take 119, 4096 150, 8000 235, and an SM has work 60 % of the time at 4096.
+// 54) at 56 % of the issue slots while an SM has work (chains of dependent instructions), and then the longest instances, up
+// to 15 probes or so of 7 us: 2000 instances take 119, 4096 150, 8000 235, and an SM has work 66 % of the time at 4096.
 // Not kept: teams of two to twelve warps for the instances that are not at their bound (187); one queue of instances for two
 // blocks (159) or four (215: the clusters leave SMs idle); states that cannot reach the last layer dropped (193).
 #include <algorithm>

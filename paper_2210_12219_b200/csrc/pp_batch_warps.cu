@@ -8,14 +8,14 @@
 // what the backtrack's threshold rule asks for: no ranking of the quotients.  It starts from a lower bound, the optimum
 // over the plans that may use a node again, which is one word a node; in 58 % of the instances of k = 8, L = 24 that is
 // beta* and one probe confirms it, the others take eight more (4096 of them, us a call: 243 by bisection alone, 172 with the
-// bound, 161 with values instead of ranks bisected, 150 with longer steps in front of that; by lanes 218).
+// bound, 161 with values instead of ranks bisected, 148 with longer steps in front of that; by lanes 218).
 //
 // A warp keeps an instance's table in shared memory, reach[S] a row of eight words.  Lane (w, q) takes the rows of
 // target node w: the links into w and the windows of w are registers, a source set is two 16-byte loads, and all
 // lanes walk the list of node sets of the other nodes, eight sets a trip.  No barriers but the warp's own.
 // What bounds it: 16 000 warp instructions an instance (3500 the bound, 1400 the staging, a trip 92, of which the windows
 // 54) at 56 % of the issue slots while an SM has work (chains of dependent instructions), and then the longest instances, up
-// to 15 probes or so of 7 us: 2000 instances take 119, 4096 150, 8000 235, and an SM has work 66 % of the time at 4096.
+// to 15 probes or so of 7 us: 2000 instances take 119, 4096 148, 8000 231, and an SM has work 66 % of the time at 4096.
 // Not kept: teams of two to twelve warps for the instances that are not at their bound (187); one queue of instances for two
 // blocks (159) or four (215: the clusters leave SMs idle); states that cannot reach the last layer dropped (193).
 #include <algorithm>
@@ -272,6 +272,8 @@ k_batch_warps(const int64_t B, const int L, const int k, const uint32_t *__restr
     // A lower bound by the plans that may use a node again: one word a node instead of one a (set, node), so that the groups
     // of lanes take a threshold each.  It is beta* itself in 58 % of the instances of k = 8, L = 24 (median distance of the others
     // 16 of 650 quotients).  Returns the largest threshold found to be too small, or -1.
+    // Rounds, each a fifth of the range: four (4096 x (8, 24) with 2, 3, 4, 5, 6 of them 203, 154, 148, 150, 154; 900 x (8, 9) 46.0, 43.7,
+    // 44.5, 46.0, 47.3).
     auto lower_bound = [&]() -> float {
         float beaten = -1.0f, slow = __uint_as_float(0x7F800000u), fast = 0.0f;
 #pragma unroll
@@ -291,7 +293,7 @@ k_batch_warps(const int64_t B, const int L, const int k, const uint32_t *__restr
 #pragma unroll
         for (int v = 0; v < KW; ++v) mine_f[v] = __shfl_sync(kAll, (float)link[v % kPairs], (v / kPairs) * KW + w);
 #pragma unroll 1
-        for (int r = 0; r < 5; ++r) {
+        for (int r = 0; r < 4; ++r) {
             const float t = exp2f(from + (to - from) * ((float)(q + 1) / (float)(QW + 1)));
             uint32_t ok[KW];
 #pragma unroll

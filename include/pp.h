@@ -431,6 +431,11 @@ pp_status pp_debug_fail_alloc(int32_t nth);
  * it is sound. */
 pp_status pp_debug_starve(int32_t polls);
 
+/* Test hook of the bounds-checking build (the normal one returns PP_ERR_LIMIT): in the next search whose blocks decide a
+ * threshold each, block `block` comes to the vote on the optimum only after another one has given up waiting for it,
+ * which the others do after `polls` polls; 0 polls clears a pending request. */
+pp_status pp_debug_late(int32_t block, int32_t polls);
+
 /* Test hook: how many accesses to their tables the kernels of one source have checked since the last call, in
  * the bounds-checking build; 0 in the normal one.  kernel: 0 = bounded search, 1 = batched search with an
  * instance to a block, 2 = placement stage, 3 = evaluator, 4 = random plans.  Synchronises the device. */

@@ -29,7 +29,7 @@ EXPORTS = (
     "pp_greedy_batch_dev", "pp_random_plans", "pp_random_plans_dev", "pp_debug_minmax_rate",
     "pp_problem_set_profiling", "pp_eval_plans_packed", "pp_eval_plans_packed_dev",
     "pp_partition_minsum_batch", "pp_partition_minsum_batch_dev",
-    "pp_kpath_colour_batch", "pp_kpath_colour_batch_dev", "pp_debug_fail_alloc", "pp_debug_starve", "pp_debug_bounds_checks",
+    "pp_kpath_colour_batch", "pp_kpath_colour_batch_dev", "pp_debug_fail_alloc", "pp_debug_starve", "pp_debug_late", "pp_debug_bounds_checks",
     "pp_debug_batch_route", "pp_debug_quotients",
     "pp_kpath_matching", "pp_solve_exact_compute",
 )
@@ -97,6 +97,7 @@ def lib() -> ctypes.CDLL:
         L.pp_kpath_colour_batch_dev.argtypes = [i32, vp, i64, i32] + [vp] * 8
         L.pp_debug_fail_alloc.argtypes = [i32]
         L.pp_debug_starve.argtypes = [i32]
+        L.pp_debug_late.argtypes = [i32, i32]
         L.pp_debug_bounds_checks.argtypes = [i32, ctypes.POINTER(u64)]
         L.pp_debug_quotients.argtypes = [i64, vp, vp, vp, vp]
         L.pp_debug_batch_route.argtypes = [i64, i32, i32, i32, i32, ctypes.POINTER(i32)]
@@ -479,6 +480,11 @@ def debug_quotients(bits, kbps):
 def debug_starve(polls: int):
     """pp_debug_starve: the next launch whose blocks meet waits for a block too many, `polls` polls long (0 clears)."""
     _check(lib().pp_debug_starve(int(polls)), "pp_debug_starve")
+
+
+def debug_late(block: int, polls: int):
+    """pp_debug_late: a block of the next search by thresholds comes when the others have given up (bounds-checking build)."""
+    _check(lib().pp_debug_late(int(block), int(polls)), "pp_debug_late")
 
 
 def debug_minmax_rate(op: int, iters: int = 2048) -> float:

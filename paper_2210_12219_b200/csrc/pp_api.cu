@@ -117,6 +117,8 @@ bool alloc_should_fail()
 
 // Test hook (pp_debug_starve).
 std::atomic<int> g_starved_polls{0};
+// Test hook (pp_debug_late): block << 32 | polls.
+std::atomic<uint64_t> g_late{0};
 
 // Whether the stream is being recorded into a graph (the legacy stream cannot be).
 bool recording(cudaStream_t s)
@@ -885,6 +887,12 @@ pp_status queue_sparse(pp_problem *p, PruneCtl *ctl, pp_solution *sol, PruneNote
 }  // namespace
 
 int pp::starved_polls() { return g_starved_polls.load(std::memory_order_relaxed) ? g_starved_polls.exchange(0) : 0; }
+int pp::late_polls(int *block)
+{
+    const uint64_t late = g_late.load(std::memory_order_relaxed) ? g_late.exchange(0) : 0;
+    *block = (int)(late >> 32);
+    return (int)(uint32_t)late;
+}
 
 extern "C" {
 
@@ -1951,6 +1959,17 @@ pp_status pp_debug_starve(int32_t polls)
     if (polls < 0) return PP_ERR_ARG;
     g_starved_polls.store(polls);
     return PP_OK;
+}
+
+pp_status pp_debug_late(int32_t block, int32_t polls)
+{
+    if (block < 0 || polls < 0) return PP_ERR_ARG;
+#ifdef PP_DEBUG_BOUNDS
+    g_late.store(polls ? (uint64_t)block << 32 | (uint32_t)polls : 0);
+    return PP_OK;
+#else
+    return PP_ERR_LIMIT;
+#endif
 }
 
 pp_status pp_debug_bounds_checks(int32_t kernel, uint64_t *n)

@@ -217,6 +217,7 @@ struct PruneDev {
     int clustered;             // the blocks are one cluster (set by the launch)
     uint32_t arrivals;         // blocks a barrier in global memory waits for, and polls before it gives up (set by
     int polls;                 // the launch)
+    uint32_t late;             // bounds-checking build: number + 1 of the block that pp_debug_late holds up, or 0
     int key_shift;             // keys: 1 + (bits of the double - key_base) >> key_shift
     unsigned long long key_base, key_top;  // bits of the smallest and of the largest positive term
     unsigned long long key_floor;  // bits of a value that no plan is below
@@ -239,6 +240,8 @@ struct PruneDev {
 // Test hook (pp_debug_starve): polls of the next launch whose blocks meet, which then waits for one block
 // more than it has; 0 = an ordinary launch.  Asking for it uses it up.
 int starved_polls();
+// Test hook (pp_debug_late): polls of the next search by thresholds, in which block *block comes late; 0 = an ordinary one.
+int late_polls(int *block);
 void prune_key_range(double lo, double hi, PruneDev *d);
 void prune_node_bounds(const uint64_t *cap, uint64_t total, PruneDev *d);
 int prune_row_pad(int L, int k);

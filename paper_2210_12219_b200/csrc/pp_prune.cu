@@ -1124,6 +1124,13 @@ cudaError_t launch_shape(const PruneDev &d, const PruneHost &h, int sms, cudaStr
         ++q.arrivals;
         q.polls = polls;
     }
+#ifdef PP_DEBUG_BOUNDS
+    int late = 0;
+    if (const int polls = tlay.set_cap ? late_polls(&late) : 0) {
+        q.late = (uint32_t)late + 1u;
+        q.polls = polls;
+    }
+#endif
     return cudaLaunchKernelEx(&cfg, kernel, q, tlay, in);
 }
 

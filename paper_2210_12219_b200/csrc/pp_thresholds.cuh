@@ -30,6 +30,7 @@ constexpr size_t kThresholdSets = 640;
 constexpr int kCandidates = 512;  // terms that are ranked at a time
 constexpr int kThresholdRounds = 4;
 constexpr int kThresholdWords = 56;  // PruneCtl::count from here on: the votes of the rounds
+constexpr int kLatePolls = 1 << 20;  // test hook (pp_debug_late): after so many the late block comes in any case
 
 // Shared memory of the search.  W: words of a row.
 struct ThresholdLayout {
@@ -76,24 +77,32 @@ enum ThresholdOutcome { kThresholdOpen, kThresholdSolved, kThresholdNoPlan, kThr
 
 // The votes of a round: every block adds one arrival, whether its threshold is not known to be too small, and whether it
 // ran out of rows on it.  Nothing but this word passes between the blocks, so that it needs no fence (1100 cycles; the barrier
-// of the bounded search, which hands rows on, 3500).  False when the wait ran out, here or in another block.
-__device__ __forceinline__ bool threshold_vote(const PruneDev &d, unsigned long long *word, uint32_t open, uint32_t over, uint32_t *opens, uint32_t *overs)
+// of the bounded search, which hands rows on, 3500).  False when a wait ran out, and then for all blocks: one that gives up
+// marks the word in the same step in which it sees that arrivals are missing, and a block that comes after it reads the mark.
+constexpr unsigned long long kVoteLeft = 1ull << 63;
+__device__ __forceinline__ bool threshold_vote(const PruneDev &d, unsigned long long *word, uint32_t open, uint32_t over, [[maybe_unused]] bool terms, uint32_t *opens,
+                                               uint32_t *overs)
 {
     __shared__ unsigned long long s_seen;
-    PruneCtl *ctl = d.ctl;
     __syncthreads();
     if (threadIdx.x == 0) {
         unsigned long long seen;
+        auto waiting = [&] { return !(seen & kVoteLeft) && (uint32_t)(seen >> 40) < d.arrivals; };
+        auto look = [&] { asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(seen) : "l"(word) : "memory"); };
+#ifdef PP_DEBUG_BOUNDS
+        if (terms && d.late == blockIdx.x + 1) {  // test hook: behind a block that gave up
+            int i = 0;
+            do look();
+            while (!(seen & kVoteLeft) && ++i < kLatePolls);
+        }
+#endif
         asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(word), "l"((1ull << 40) | ((unsigned long long)open << 20) | over) : "memory");
         int spins = 0;
-        uint32_t failed = 0;
-        do {
-            asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(seen) : "l"(word) : "memory");
-            if ((++spins & 1023) == 0) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(failed) : "l"(&ctl->failed) : "memory");
-        } while ((uint32_t)(seen >> 40) < d.arrivals && spins < d.polls && !failed);
-        if ((uint32_t)(seen >> 40) < d.arrivals) {
-            asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(&ctl->failed), "r"(1u) : "memory");
-            seen = ~0ull;
+        do look();
+        while (waiting() && ++spins < d.polls);
+        while (waiting()) {  // as often as other blocks change the word, at most
+            const unsigned long long now = atomicCAS(word, seen, seen | kVoteLeft);
+            seen = now == seen ? seen | kVoteLeft : now;
         }
         s_seen = seen;
     }
@@ -101,7 +110,7 @@ __device__ __forceinline__ bool threshold_vote(const PruneDev &d, unsigned long 
     const unsigned long long seen = s_seen;
     *opens = (uint32_t)(seen >> 20) & 0xFFFFFu;
     *overs = (uint32_t)seen & 0xFFFFFu;
-    return seen != ~0ull;
+    return !(seen & kVoteLeft);
 }
 
 // W: words of a row; NT: threads of the block.  Ends with the block in step.  Solved: *winner is the block that has the
@@ -391,11 +400,11 @@ __device__ __forceinline__ int threshold_search(const PruneDev &d, const Thresho
             }
         }
         uint32_t opens, overs;
-        if (!threshold_vote(d, d.ctl->count + kThresholdWords + 2 * round, vote != 0, vote == 2, &opens, &overs)) return kThresholdGaveUp;
+        if (!threshold_vote(d, d.ctl->count + kThresholdWords + 2 * round, vote != 0, vote == 2, n != 0, &opens, &overs)) return kThresholdGaveUp;
         const int first = nblk - (int)opens;  // block of the smallest threshold that may have a plan
         if (round == 0 && opens == 0u) return kThresholdNoPlan;
         if (overs) {  // is it this one that ran out of rows?  Then the others near the optimum will, too
-            if (!threshold_vote(d, d.ctl->count + kThresholdWords + 2 * round + 1, (int)blockIdx.x == first && vote == 2, 0u, &opens, &overs))
+            if (!threshold_vote(d, d.ctl->count + kThresholdWords + 2 * round + 1, (int)blockIdx.x == first && vote == 2, 0u, false, &opens, &overs))
                 return kThresholdGaveUp;
             if (opens) return kThresholdOpen;
         }

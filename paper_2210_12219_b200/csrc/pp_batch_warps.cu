@@ -29,6 +29,7 @@ namespace {
 constexpr uint32_t kAll = 0xFFFFFFFFu;
 constexpr int KW = 8;  // words of a row, one a node: k <= 8
 constexpr int kWarpMaxL = 32;
+constexpr int kSingly = 4;       // candidates above the bound that are tried one after another
 constexpr int kWindowRegs = 15;  // distances of a window held in registers; longer ones come from shared memory
 
 // Shared memory of a warp, in bytes.
@@ -468,7 +469,7 @@ k_batch_warps(const int64_t B, const int L, const int k, const uint32_t *__restr
             hi[i] = link[i] > 0.0 ? cuts : 0;
         }
         double first_t = 0.0;
-        int m = 0, tries = 0;  // m: nodes of the plan of the smallest threshold that has one
+        int m = 0, tries = 0;  // m: nodes of the plan of the smallest threshold that has one; tries: probes, from 0 down walks
         bool fresh = false;    // the table is still that one's
         for (;;) {
             extremes();
@@ -483,20 +484,36 @@ k_batch_warps(const int64_t B, const int L, const int k, const uint32_t *__restr
             else if (tries > 0) {
                 const double far_off = tries == 1 ? 1.2 : tries == 2 ? 1.7 : tries == 3 ? 2.8 : tries == 4 ? 5.0 : 10.0;
                 key = (unsigned long long)__double_as_longlong(__dmul_rn(first_t, far_off));
+            } else if (tries <= -kSingly) {
+                key = least + min((most - least) >> 1, 1ull << min(36 - 4 * (tries + kSingly), 60));
             }
             const double t = __longlong_as_double((long long)min(max(key, least), most));
             within(t);
-            int got = 0;
-            // the smallest candidate may still lie below the bound, of which the last few per mille are not worked out
-            if (tries > 0 || __any_sync(kAll, (walks(ok) & last_bit) != 0u)) {
-                if (tries++ == 0) first_t = t;
-                got = probe();
+            bool probing = tries > 0, yes = false;
+            if (!probing) {
+                // The smallest candidates may still lie below the bound, which is worked out to a 625th of the range of all on its
+                // logarithm.  Where quotients are close together that is hundreds of them: a few are tried one after another, then by
+                // steps that grow sixteenfold and by the middle of what is left below the first that a walk gets through, as many walks
+                // as bits tell them apart (1700 x (8, 24) of near-equal layers and links with one link far slower 345 -> 154 us a
+                // call, spread ones 115.4 -> 116.2).
+                yes = __any_sync(kAll, (walks(ok) & last_bit) != 0u);
+                probing = yes && (tries > -kSingly || least == most);
+                if (probing) {
+                    tries = 0;
+                    first_t = t;
+#pragma unroll
+                    for (int i = 0; i < kPairs; ++i) hi[i] = link[i] > 0.0 ? cuts : 0;
+                } else --tries;
             }
-            fresh = got > 0;
-            if (got > 0) m = got;
+            if (probing) {
+                const int got = probe();
+                ++tries;
+                yes = fresh = got > 0;
+                if (yes) m = got;
+            }
 #pragma unroll
             for (int i = 0; i < kPairs; ++i) {
-                if (got > 0) hi[i] = max(lo[i], min(hi[i], upto[i]));
+                if (yes) hi[i] = max(lo[i], min(hi[i], upto[i]));
                 else lo[i] = min(hi[i], max(lo[i], upto[i]));
             }
         }

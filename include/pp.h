@@ -448,7 +448,7 @@ pp_status pp_debug_quotients(int64_t n, const uint64_t *bits, const uint32_t *kb
 
 /* Test hook (host only, needs no device): what solves a batch on a device of `sms` multiprocessors.  host: the
  * batch comes from host arrays (pp_solve_exact_batch).  *threads receives the threads of the block that an
- * instance goes to, 0 where an instance shares a block with others and goes to one of its lanes or warps. */
+ * instance goes to, 32 where it shares a block with others and goes to one of its warps, 0 where it goes to a lane. */
 pp_status pp_debug_batch_route(int64_t B, int32_t L, int32_t k, int32_t sms, int32_t host, int32_t *threads);
 
 /* Force (1) or forbid (0) the generic sweep kernel; 2 = automatic choice among the kernels that

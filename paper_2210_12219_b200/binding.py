@@ -460,7 +460,7 @@ def debug_bounds_checks(kernel: int) -> int:
 
 
 def debug_batch_route(B: int, L: int, k: int, host: bool = False, sms: int = 148) -> int:
-    """pp_debug_batch_route: threads of the block an instance of the batch goes to, 0 where it shares a block; needs no device."""
+    """pp_debug_batch_route: threads of the block an instance of the batch goes to, 32 for a warp, 0 for a lane; needs no device."""
     n = ctypes.c_int32()
     _check(lib().pp_debug_batch_route(int(B), int(L), int(k), int(sms), int(host), ctypes.byref(n)), "pp_debug_batch_route")
     return int(n.value)

@@ -1268,9 +1268,9 @@ pp_status pp_random_plans(pp_problem *p, int64_t P, const uint32_t *draws, uint8
     return from_cuda(e2);
 }
 
-// What solves a batch: an instance to a lane (or a warp, batch_warps_takes), or to a block, and there to a narrow one or a wide one.
+// What solves a batch: an instance to a lane, to a warp, or to a block, and there to a narrow one or a wide one.
 struct BatchRoute {
-    bool lanes, narrow;
+    bool lanes, warps, narrow;
 };
 
 // pieces: of a batch that lies in page-locked host memory, 0 for one on the device.
@@ -1287,7 +1287,8 @@ static BatchRoute batch_route(int64_t B, int L, int k, int sms, int64_t pieces)
 {
     const int64_t each = pieces ? (B + pieces - 1) / pieces : B;
     const int64_t together = !pieces || L <= 32 ? B : L <= 36 ? std::min(B, 2 * each) : each;
-    return {!pieces && batch_lanes_takes(B, L, k, sms), batch_narrow(together, L, k, sms)};
+    const bool shared = !pieces && batch_lanes_takes(B, L, k, sms), warps = shared && batch_warps_takes(B, L, k);
+    return {shared && !warps, warps, batch_narrow(together, L, k, sms)};
 }
 
 // These are the batch whose route it is, or a piece of it.  early: behind another piece of the same batch.
@@ -1297,7 +1298,7 @@ static pp_status queue_exact_batch(int64_t B, int32_t L, int32_t k, const uint64
 {
     if (batch_smem_bytes(L, k) + 1024 > kBlockShared) return PP_ERR_LIMIT;
     LaneTables lt;
-    if (route.lanes && batch_warps_takes(B, L, k)) {
+    if (route.warps) {
         PP_CUDA(lane_tables(k - 1, &lt));
         PP_CUDA(launch_batch_warps(B, L, k, lt, sms, out_bits, mem, node_mem, bw, beta_ms, m, cuts, placement, status, s));
         return PP_OK;
@@ -2009,7 +2010,7 @@ pp_status pp_debug_batch_route(int64_t B, int32_t L, int32_t k, int32_t sms, int
     if (L > PP_MAX_L || k > PP_MAX_K || batch_smem_bytes(L, k) + 1024 > kBlockShared) return PP_ERR_LIMIT;
     const BatchArrays a = batch_arrays(B, L, k);
     const BatchRoute route = batch_route(B, L, k, sms, host && a.off[9] <= kPinnedBytes ? host_pieces(a) : 0);
-    *threads = route.lanes ? 0 : batch_block_threads(route.narrow);
+    *threads = route.lanes ? 0 : route.warps ? 32 : batch_block_threads(route.narrow);
     return PP_OK;
 }
 

@@ -621,7 +621,7 @@ cudaError_t launch_level(int nv, const BatchLanes &t, int64_t B, int k, int L, i
     switch (nv) {
 #define PP_CASE(N)                                                                                                     \
     case N:                                                                                                            \
-        if constexpr (LH != 4 || N <= 4) { /* up to eight layers k >= 6 goes an instance to a warp */                  \
+        if constexpr (LH != 4 || N < kLanesShortK) { /* nodes in front: one less than the problem has */               \
             const size_t sm = win_bytes_per_warp(LH) * kLevelWarps;                                                    \
             cudaError_t e = cudaFuncSetAttribute(k_lanes_level<N, LH>, cudaFuncAttributeMaxDynamicSharedMemorySize,    \
                                                  (int)sm);                                                             \

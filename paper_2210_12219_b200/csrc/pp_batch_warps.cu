@@ -544,6 +544,7 @@ k_batch_warps(const int64_t B, const int L, const int k, const uint32_t *__restr
 //          4096 x 24 89.2, 91.2; 4200 121.0, 94.9; 2500 x 28 74.6, 74.9; 3000 83.8, 77.7; 3000 x 32 85.1, 80.7
 bool batch_warps_takes(int64_t B, int L, int k)
 {
+    if (L <= 8 && k > kLanesShortK) return true;
     if (k == 8) return B >= (L <= 14 ? 0 : L <= 16 ? 1300 : L <= 24 ? 1700 : 1100);
     if (k == 7) return B >= (L <= 12 ? 0 : L <= 24 ? 2000 : 1600);
     return k == 6 && B >= (L <= 11 ? 0 : L <= 24 ? 4097 : 3000);

@@ -1,4 +1,4 @@
-"""Which batches go an instance to a lane, which to blocks of 192 threads and which to blocks of 384, by the library's own rule
+"""Which batches go an instance to a lane, which to a warp, which to blocks of 192 threads and which to blocks of 384, by the library's own rule
 (no device is needed).  Every line was measured on both sides; the times stand beside the rules."""
 from __future__ import annotations
 
@@ -7,7 +7,7 @@ import pytest
 import paper_2210_12219_b200 as pp
 from paper_2210_12219_b200 import build
 
-LANES, NARROW, WIDE = 0, 192, 384
+LANES, WARPS, NARROW, WIDE = 0, 32, 192, 384
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -44,21 +44,41 @@ def test_host_batches_count_a_piece_of_long_chains(L, k, B, want):
 
 
 # batches of short chains: a wave of blocks (three to an SM, six narrow ones for k <= 6, two for k = 8 from 29 layers on), two waves, or
-# one and a half go an instance to a block, larger ones an instance to a lane; host batches of up to 1 MB never do
+# one and a half go an instance to a block, larger ones an instance to a lane or a warp; host batches of up to 1 MB never do
 @pytest.mark.parametrize("L,k,most", [(24, 2, 888), (16, 3, 888), (9, 4, 1776), (32, 4, 1776), (20, 5, 1776), (16, 6, 1776), (17, 6, 1332), (24, 6, 1332),
                                       (25, 6, 1776), (32, 6, 1776), (16, 7, 888), (17, 7, 444), (24, 7, 444), (25, 7, 888), (32, 7, 888),
                                       (16, 8, 888), (17, 8, 444), (28, 8, 444), (29, 8, 296), (32, 8, 296)])
-def test_larger_batches_of_short_chains_go_to_the_lanes(L, k, most):
+def test_larger_batches_of_short_chains_share_blocks(L, k, most):
     for B in (1, 64, most):
-        assert pp.debug_batch_route(B, L, k) != LANES, B
+        assert pp.debug_batch_route(B, L, k) in (NARROW, WIDE), B
     for B in (most + 1, 2 * most, 4096, 100_000):
-        assert pp.debug_batch_route(B, L, k) == LANES, B
+        assert pp.debug_batch_route(B, L, k) in (LANES, WARPS), B
+        assert pp.debug_batch_route(B, L, k) == LANES or k >= 6, B
         arrays = (8 * L, 8 * L, 8 * k, 4 * k * k, 8, 4, 4 * (k - 1), 4 * k, 1)  # bytes an instance
         in_place = sum(-(-B * a // 256) * 256 for a in arrays) <= 1 << 20
-        assert (pp.debug_batch_route(B, L, k, host=True) != LANES) == in_place, B
+        assert (pp.debug_batch_route(B, L, k, host=True) in (NARROW, WIDE)) == in_place, B
+
+
+# the smallest batch of a shape that goes an instance to a warp; one that is smaller by one goes to a lane, or to a block where
+# that is as far as the blocks go
+@pytest.mark.parametrize("L,k,B", [(1, 8, 889), (14, 8, 889), (15, 8, 1300), (16, 8, 1300), (17, 8, 1700), (24, 8, 1700), (25, 8, 1100), (32, 8, 1100),
+                                   (1, 7, 889), (12, 7, 889), (13, 7, 2000), (24, 7, 2000), (25, 7, 1600), (32, 7, 1600),
+                                   (1, 6, 1777), (11, 6, 1777), (12, 6, 4097), (24, 6, 4097), (25, 6, 3000), (32, 6, 3000)])
+def test_batches_an_instance_to_a_warp(L, k, B):
+    for n in (B, B + 1, 2 * B, 100_000):
+        assert pp.debug_batch_route(n, L, k) == WARPS, n
+    assert pp.debug_batch_route(B - 1, L, k) in ((NARROW, WIDE) if B in (889, 1777) else (LANES,))
+
+
+def test_the_lanes_are_asked_for_no_level_that_is_not_there():
+    # rows of four words have levels of five nodes and fewer (kLanesShortK)
+    for k in (6, 7, 8):
+        for L in range(1, 9):
+            for B in (*range(1, 2200, 7), *range(2200, 9000, 97), 4095, 4096, 4097, 100_000):
+                assert pp.debug_batch_route(B, L, k) != LANES, (B, L, k)
 
 
 @pytest.mark.parametrize("L,k", [(33, 8), (24, 9), (24, 1)])
 def test_other_shapes_never_do(L, k):
     for B in (1, 4096, 100_000):
-        assert pp.debug_batch_route(B, L, k) != LANES
+        assert pp.debug_batch_route(B, L, k) in (NARROW, WIDE)

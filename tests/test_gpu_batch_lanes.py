@@ -20,7 +20,7 @@ pytestmark = pytest.mark.gpu
 
 def lanes(B, L, k):
     import torch
-    return pp.debug_batch_route(B, L, k, sms=torch.cuda.get_device_properties(0).multi_processor_count) == 0
+    return pp.debug_batch_route(B, L, k, sms=torch.cuda.get_device_properties(0).multi_processor_count) == 0  # 32: to a warp
 
 
 def smallest_for_lanes(L, k):
@@ -80,7 +80,7 @@ def test_quotients_are_correctly_rounded():
 
 
 @pytest.mark.parametrize("debug", [False, True])
-@pytest.mark.parametrize("L,k", [(7, 3), (7, 8), (9, 2), (17, 5), (24, 8), (31, 6), (32, 8)])
+@pytest.mark.parametrize("L,k", [(7, 3), (7, 5), (9, 2), (17, 5), (24, 8), (31, 6), (32, 8)])
 def test_extreme_and_close_quotients(L, k, debug):
     insts = extreme_instances(L, k)
     want = [oracle.dp_naive(i) for i in insts]
@@ -93,7 +93,7 @@ def test_extreme_and_close_quotients(L, k, debug):
 
 
 @pytest.mark.parametrize("debug", [False, True])
-@pytest.mark.parametrize("L,k", [(12, 4), (5, 7), (32, 8)])
+@pytest.mark.parametrize("L,k", [(12, 4), (5, 5), (32, 8)])
 def test_instances_beyond_the_limits(L, k, debug):
     insts = [W.random_small(62000 + 100 * L + i, L, k) for i in range(80)]
     want = [oracle.dp_naive(i) for i in insts]
@@ -114,8 +114,10 @@ def test_instances_beyond_the_limits(L, k, debug):
             check(got, b, want[pick[b]])
 
 
-# 4096 instances share the scratch tables at a time: whole pieces, and a last one of a few instances or of one
-@pytest.mark.parametrize("L,k,B,debug", [(9, 4, 4096 + 45, False), (8, 5, 2 * 4096 + 1, True), (24, 6, 4097, False), (5, 8, 4096, False)])
+# 4096 instances share the scratch tables at a time: whole pieces, and a last one of a few instances or of one, over all widths
+# of a row (with six nodes and more the lanes take one piece at most)
+@pytest.mark.parametrize("L,k,B,debug", [(9, 4, 4096 + 45, False), (8, 5, 2 * 4096 + 1, True), (24, 5, 4097, False), (32, 5, 4097, True),
+                                         (24, 6, 4096, False), (5, 5, 4096, False)])
 def test_pieces_one_after_another(L, k, B, debug):
     insts = [W.random_small(66000 + i, L, k, tight=(i % 3 == 1), ties=(i % 7 == 2), dead_links=0.25 if i % 4 == 3 else 0.0)
              for i in range(B)]

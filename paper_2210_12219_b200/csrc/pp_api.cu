@@ -310,9 +310,6 @@ cudaError_t multiprocessors(int dev, int *sms)
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// instances whose tables share the scratch memory of the instance-per-lane batch path at a time
-constexpr int64_t kBatchLanesChunk = 4096;
-
 struct WorkLayout {
     size_t pos, order, gu, cnt, rk, inv, rank, table, total;
 };

@@ -533,21 +533,33 @@ k_batch_warps(const int64_t B, const int L, const int k, const uint32_t *__restr
 }  // namespace
 
 // Whether the batches that do not go an instance to a block (batch_lanes_takes) go an instance to a warp rather than to a lane.
-// A warp takes as long as its instance's probes, 24 instances to an SM; lanes cost by the instance, by the layer and, beyond 4096,
-// by rounds of their tables.  us a call (mean of four seeds), in lanes and in warps:
-//   k = 8  900 x L = 14 71.4, 68.5; 900 x 16 72.5, 75.7; 1200 81.6, 80.0; 1300 84.7, 82.0
-//          1400 x 20 109.2, 100.4; 1400 x 24 111.5, 113.6; 1600 121.6, 120.9; 1800 130.4, 118.5; 4096 219, 150
-//          1000 x 28 113.7, 114.7; 1100 119.9, 113.7; 1000 x 32 115.4, 117.1; 1100 121.5, 117.7; 4096 296, 161
-//   k = 7  900 x 9 45.9, 36.4; 900 x 12 48.0, 46.0; 900 x 13 49.0, 50.3; 1700 x 16 65.5, 66.0; 2000 72.8, 65.1
-//          1800 x 24 82.6, 83.3; 2000 86.6, 82.0; 1400 x 28 79.4, 80.2; 1600 86.8, 82.7; 1400 x 32 81.2, 83.0; 1600 88.7, 85.8
-//   k = 6  1780 x 5 34.0, 24.0; 1780 x 11 46.8, 45.0; 2500 x 13 55.9, 56.2; 4096 x 16 75.6, 81.7; 4200 105.3, 81.7
-//          4096 x 24 89.2, 91.2; 4200 121.0, 94.9; 2500 x 28 74.6, 74.9; 3000 83.8, 77.7; 3000 x 32 85.1, 80.7
+// A lane's time is that of its shape and, beyond kBatchLanesChunk instances, of rounds of their tables; a warp's is that of its
+// instance's probes, 24 instances to an SM, and depends on the values.  The lines were therefore drawn over five families: sizes and links
+// uniform, log-normal ones under rising memory, identical blocks under links of 1 to 50 Mbit/s, two groups of nodes with slow links
+// between them, and chains that hardly fit.  A warp is taken where it is faster in their geometric mean and loses a tenth at most in
+// any one; chains of few layers have no such line (identical blocks at a layer a node are slower in warps at all sizes up to 8000), there
+// the mean decides.  us a call in lanes / in warps, uniform, log-normal, blocks, groups, tight (mean of four seeds):
+//   k = 8   900 x L = 4  33 30 33 33 35 / 18 18 50 19 42        889 x 9   67 65 68 66 69 / 41 67 79 45 80
+//          1300 x 14     84 83 85 84 83 / 69 86 81 79 100       1500      92 91 92 92 92 / 73 91 85 81 100
+//          1500 x 16     94 92 93 93 92 / 89 90 86 90 104       1800     103 101 102 102 101 / 82 92 89 99 110
+//          1700 x 24     127 125 126 126 121 / 116 122 105 144 111   2000   141 138 140 139 133 / 121 129 104 142 104
+//          1300 x 32     133 131 132 132 127 / 121 158 102 140 116   1500   152 150 152 151 146 / 123 160 102 142 115
+//   k = 7   900 x 6      35 35 37 35 37 / 25 39 53 28 45        900 x 9   47 47 49 47 49 / 37 51 57 40 60
+//          1500 x 12     60 59 61 60 61 / 51 61 65 57 68        1700      64 63 65 64 65 / 50 63 66 58 70
+//          1800 x 20     83 81 83 83 79 / 77 75 73 91 76        2100      89 87 89 88 85 / 81 77 76 93 75
+//          2200 x 24     94 93 94 94 90 / 88 91 81 99 79        2500     102 100 102 102 98 / 86 94 84 104 78
+//          1700 x 32     98 95 97 97 94 / 88 111 84 99 86       2000     108 106 107 106 104 / 89 111 83 100 82
+//   k = 6  1777 x 6      38 38 39 37 40 / 28 36 49 28 44        1777 x 7  38 38 40 38 40 / 30 41 51 36 49
+//          4000 x 11     73 73 74 73 73 / 55 74 91 69 77        4097      97 97 101 98 98 / 62 77 91 67 83
+//          4096 x 24     91 90 91 91 88 / 91 104 108 120 75     4097     119 117 119 118 111 / 91 110 111 120 75
+// What lies closer together than any of these families is slow in the lanes, whose ranking it makes long (1700 x (8, 24) of near-equal
+// layers and links 350 / 153).
 bool batch_warps_takes(int64_t B, int L, int k)
 {
     if (L <= 8 && k > kLanesShortK) return true;
-    if (k == 8) return B >= (L <= 14 ? 0 : L <= 16 ? 1300 : L <= 24 ? 1700 : 1100);
-    if (k == 7) return B >= (L <= 12 ? 0 : L <= 24 ? 2000 : 1600);
-    return k == 6 && B >= (L <= 11 ? 0 : L <= 24 ? 4097 : 3000);
+    if (k == 8) return B >= (L <= 9 ? 0 : L <= 14 ? 1500 : L <= 16 ? 1800 : L <= 24 ? 2000 : 1500);
+    if (k == 7) return B >= (L <= 6 ? 0 : L <= 12 ? 1700 : L <= 20 ? 2100 : L <= 24 ? 2500 : 2000);
+    return k == 6 && B > (L <= 6 ? 0 : kBatchLanesChunk);
 }
 
 cudaError_t launch_batch_warps(int64_t B, int L, int k, const LaneTables &others, int sms, const uint64_t *bits, const uint64_t *mem,

@@ -181,9 +181,11 @@ struct BatchLanes {
     uint32_t rows;            // k * 2^(k-1)
     int LH;                   // words per row in these tables: 4, 8, 12 or 16
 };
+// Instances whose tables share its scratch memory at a time.
+constexpr int64_t kBatchLanesChunk = 4096;
 // Nodes up to which chains of up to eight layers (four words a row) go an instance to a lane; with more they go to a warp,
 // whatever the size of the batch, and the levels of more nodes are not there.
-constexpr int kLanesShortK = 5;
+constexpr int kLanesShortK = 7;
 bool batch_lanes_takes(int64_t B, int L, int k, int sms);
 int batch_lanes_words(int L);
 // test hook: n quotients as the preparing kernel ranks them, and by CUDA's division

@@ -61,9 +61,10 @@ def test_larger_batches_of_short_chains_share_blocks(L, k, most):
 
 # the smallest batch of a shape that goes an instance to a warp; one that is smaller by one goes to a lane, or to a block where
 # that is as far as the blocks go
-@pytest.mark.parametrize("L,k,B", [(1, 8, 889), (14, 8, 889), (15, 8, 1300), (16, 8, 1300), (17, 8, 1700), (24, 8, 1700), (25, 8, 1100), (32, 8, 1100),
-                                   (1, 7, 889), (12, 7, 889), (13, 7, 2000), (24, 7, 2000), (25, 7, 1600), (32, 7, 1600),
-                                   (1, 6, 1777), (11, 6, 1777), (12, 6, 4097), (24, 6, 4097), (25, 6, 3000), (32, 6, 3000)])
+@pytest.mark.parametrize("L,k,B", [(1, 8, 889), (9, 8, 889), (10, 8, 1500), (14, 8, 1500), (15, 8, 1800), (16, 8, 1800), (17, 8, 2000), (24, 8, 2000),
+                                   (25, 8, 1500), (32, 8, 1500), (1, 7, 889), (6, 7, 889), (7, 7, 1700), (12, 7, 1700), (13, 7, 2100), (20, 7, 2100),
+                                   (21, 7, 2500), (24, 7, 2500), (25, 7, 2000), (32, 7, 2000), (1, 6, 1777), (6, 6, 1777), (7, 6, 4097),
+                                   (32, 6, 4097)])
 def test_batches_an_instance_to_a_warp(L, k, B):
     for n in (B, B + 1, 2 * B, 100_000):
         assert pp.debug_batch_route(n, L, k) == WARPS, n
@@ -71,11 +72,10 @@ def test_batches_an_instance_to_a_warp(L, k, B):
 
 
 def test_the_lanes_are_asked_for_no_level_that_is_not_there():
-    # rows of four words have levels of five nodes and fewer (kLanesShortK)
-    for k in (6, 7, 8):
-        for L in range(1, 9):
-            for B in (*range(1, 2200, 7), *range(2200, 9000, 97), 4095, 4096, 4097, 100_000):
-                assert pp.debug_batch_route(B, L, k) != LANES, (B, L, k)
+    # rows of four words have the levels of seven nodes and fewer (kLanesShortK)
+    for L in range(1, 9):
+        for B in (*range(1, 2200, 7), *range(2200, 9000, 97), 4095, 4096, 4097, 100_000):
+            assert pp.debug_batch_route(B, L, 8) != LANES, (B, L)
 
 
 @pytest.mark.parametrize("L,k", [(33, 8), (24, 9), (24, 1)])

@@ -80,7 +80,7 @@ def test_quotients_are_correctly_rounded():
 
 
 @pytest.mark.parametrize("debug", [False, True])
-@pytest.mark.parametrize("L,k", [(7, 3), (7, 5), (9, 2), (17, 5), (24, 8), (31, 6), (32, 8)])
+@pytest.mark.parametrize("L,k", [(7, 3), (8, 7), (9, 2), (17, 5), (24, 8), (31, 6), (32, 8)])
 def test_extreme_and_close_quotients(L, k, debug):
     insts = extreme_instances(L, k)
     want = [oracle.dp_naive(i) for i in insts]
@@ -93,7 +93,7 @@ def test_extreme_and_close_quotients(L, k, debug):
 
 
 @pytest.mark.parametrize("debug", [False, True])
-@pytest.mark.parametrize("L,k", [(12, 4), (5, 5), (32, 8)])
+@pytest.mark.parametrize("L,k", [(12, 4), (7, 6), (32, 8)])
 def test_instances_beyond_the_limits(L, k, debug):
     insts = [W.random_small(62000 + 100 * L + i, L, k) for i in range(80)]
     want = [oracle.dp_naive(i) for i in insts]

@@ -436,6 +436,10 @@ pp_status pp_debug_starve(int32_t polls);
  * which the others do after `polls` polls; 0 polls clears a pending request. */
 pp_status pp_debug_late(int32_t block, int32_t polls);
 
+/* Test hook (host only): how the calling thread's last pp_solve_exact or pp_solve_exact_compute came to its result: 1 = by
+ * thresholds that the blocks decided each for itself, 2 = that search was tried and left it to the bounded one, 0 = neither. */
+pp_status pp_debug_thresholds(int32_t *outcome);
+
 /* Test hook: how many accesses to their tables the kernels of one source have checked since the last call, in
  * the bounds-checking build; 0 in the normal one.  kernel: 0 = bounded search, 1 = batched search with an
  * instance to a block, 2 = placement stage, 3 = evaluator, 4 = random plans.  Synchronises the device. */

@@ -29,7 +29,7 @@ EXPORTS = (
     "pp_greedy_batch_dev", "pp_random_plans", "pp_random_plans_dev", "pp_debug_minmax_rate",
     "pp_problem_set_profiling", "pp_eval_plans_packed", "pp_eval_plans_packed_dev",
     "pp_partition_minsum_batch", "pp_partition_minsum_batch_dev",
-    "pp_kpath_colour_batch", "pp_kpath_colour_batch_dev", "pp_debug_fail_alloc", "pp_debug_starve", "pp_debug_late", "pp_debug_bounds_checks",
+    "pp_kpath_colour_batch", "pp_kpath_colour_batch_dev", "pp_debug_fail_alloc", "pp_debug_starve", "pp_debug_late", "pp_debug_thresholds", "pp_debug_bounds_checks",
     "pp_debug_batch_route", "pp_debug_quotients",
     "pp_kpath_matching", "pp_solve_exact_compute",
 )
@@ -98,6 +98,7 @@ def lib() -> ctypes.CDLL:
         L.pp_debug_fail_alloc.argtypes = [i32]
         L.pp_debug_starve.argtypes = [i32]
         L.pp_debug_late.argtypes = [i32, i32]
+        L.pp_debug_thresholds.argtypes = [ctypes.POINTER(i32)]
         L.pp_debug_bounds_checks.argtypes = [i32, ctypes.POINTER(u64)]
         L.pp_debug_quotients.argtypes = [i64, vp, vp, vp, vp]
         L.pp_debug_batch_route.argtypes = [i64, i32, i32, i32, i32, ctypes.POINTER(i32)]
@@ -450,6 +451,13 @@ def solve_exact_compute(inst, layer_work, node_speed) -> Solution:
 def debug_fail_alloc(nth: int):
     """pp_debug_fail_alloc: the nth device allocation from now on reports out of memory (0 clears)."""
     _check(lib().pp_debug_fail_alloc(int(nth)), "pp_debug_fail_alloc")
+
+
+def debug_thresholds() -> int:
+    """pp_debug_thresholds: 1 where the thread's last synchronous solve was decided by thresholds, 2 where they handed it on, 0 else."""
+    n = ctypes.c_int32()
+    _check(lib().pp_debug_thresholds(ctypes.byref(n)), "pp_debug_thresholds")
+    return int(n.value)
 
 
 def debug_bounds_checks(kernel: int) -> int:

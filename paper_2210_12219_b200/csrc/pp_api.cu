@@ -884,6 +884,8 @@ pp_status queue_sparse(pp_problem *p, PruneCtl *ctl, pp_solution *sol, PruneNote
 }  // namespace
 
 int pp::starved_polls() { return g_starved_polls.load(std::memory_order_relaxed) ? g_starved_polls.exchange(0) : 0; }
+// What the search by thresholds did in the calling thread's last synchronous solve (pp_debug_thresholds).
+static thread_local int32_t t_thresholds = 0;
 int pp::late_polls(int *block)
 {
     const uint64_t late = g_late.load(std::memory_order_relaxed) ? g_late.exchange(0) : 0;
@@ -1064,6 +1066,7 @@ static pp_status solve_sparse(pp_problem *p, pp_solution *sol)
     if (st == PP_OK) {
         p->note = slot->note;
         p->note_on_device = false;
+        t_thresholds = slot->note.thresholds;
         *sol = slot->sol;
         if (p->note.dense) st = PP_ERR_LIMIT;
         else if (sol->status != PP_OK && sol->status != PP_INFEASIBLE) st = PP_ERR_CUDA;
@@ -1080,6 +1083,7 @@ pp_status pp_solve_exact(pp_problem *p, double *beta_ms, int32_t *m, int32_t *cu
     try {
         p->total_launches = 0;
         p->sparse_ran = false;
+        t_thresholds = 0;
         pp_status st = takes_sparse(p) ? solve_sparse(p, &sol) : PP_ERR_LIMIT;
         if (st == PP_ERR_LIMIT) {
             int32_t err = 0;
@@ -1906,6 +1910,7 @@ pp_status pp_solve_exact_compute(int32_t L, const uint64_t *layer_out_bits, cons
     }
     const pp_solution sol = slot->sol;
     const int32_t dense = slot->note.dense;
+    t_thresholds = e == cudaSuccess ? slot->note.thresholds : 0;
     g_slots.give(slot);
     if (e != cudaSuccess) return from_cuda(e);
     if (dense != 0 || (sol.status != PP_OK && sol.status != PP_INFEASIBLE)) return PP_ERR_CUDA;
@@ -1968,6 +1973,13 @@ pp_status pp_debug_late(int32_t block, int32_t polls)
 #else
     return PP_ERR_LIMIT;
 #endif
+}
+
+pp_status pp_debug_thresholds(int32_t *outcome)
+{
+    if (!outcome) return PP_ERR_ARG;
+    *outcome = t_thresholds;
+    return PP_OK;
 }
 
 pp_status pp_debug_bounds_checks(int32_t kernel, uint64_t *n)

@@ -216,6 +216,7 @@ struct PruneCtl {              // device; the kernel leaves it as it found it
 struct PruneNote {             // what the host learns about a launch
     long long ns;              // duration on the device
     int32_t dense;             // 1 = the frontier outgrew its rows, or is too large to resolve a class in
+    int32_t thresholds;        // 1 = the result is that of the search by thresholds, 2 = it left the search to the frontier; 0: not asked
 };
 struct PruneDev {
     int L, k, Lp;              // Lp: row stride in keys

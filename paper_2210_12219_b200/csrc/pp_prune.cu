@@ -963,6 +963,7 @@ result:
             asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t_end));
             d.note->ns = (long long)(t_end - t_start);
             d.note->dense = dense ? 1 : 0;
+            d.note->thresholds = !TH || (!CT && d.whole != 0) ? 0 : solved ? 1 : 2;
         }
     }
     if constexpr (SM) return;  // the counters in global memory are as they were
@@ -1054,6 +1055,12 @@ bool threshold_takes(const uint64_t *cap, uint64_t total, int L, int k, bool com
 // k = 5, 50 layers 36.8 / 31.5 (and 2 for the scratch that the search behind it may need), 25 30.6 / 32.
 bool threshold_before_shared(int L, int k) { return L <= 32 * kThresholdW && k >= 5 && k * L >= 200; }
 
+// Eq. 2: a grid that takes every SM for itself gains 9 to 40 % a solve, and takes from solves on other streams what a cluster of eight
+// blocks leaves them.  us a solve, one, two, four, eight handles on streams of their own, the bounded search and by thresholds: uniform
+// (24, 7) 28.1, 14.4, 8.4, 7.7 and 20.8, 16.9, 18.2, 19.0; cnn (50, 8) 27.8, 15.3, 8.6, 4.8 and 22.2, 20.7, 20.9, 20.9 (by 24 and by 74 blocks
+// 25.7, 17.0, -, 5.4 and 22.8, 14.0, -, 11.1).  Solves on the legacy stream run one after another in any case; Eq. 1 knows no other.
+bool on_legacy_stream(cudaStream_t s) { return s == nullptr || s == cudaStreamLegacy; }
+
 template <int G, int P, bool CT>
 cudaError_t launch_shape(const PruneDev &d, const PruneHost &h, int sms, cudaStream_t s)
 {
@@ -1093,7 +1100,7 @@ cudaError_t launch_shape(const PruneDev &d, const PruneHost &h, int sms, cudaStr
     ThresholdLayout tlay{};
     auto kernel = k_prune<G, P, CT, false, false>;
     if constexpr (G * P <= 32 * kThresholdW) {
-        if (threshold_takes(h.cap, h.M[d.L], d.L, d.k, CT) && (blocks > 1 || (CT && threshold_before_shared(d.L, d.k)))) {
+        if (threshold_takes(h.cap, h.M[d.L], d.L, d.k, CT) && (CT ? blocks > 1 || threshold_before_shared(d.L, d.k) : blocks > 1 && on_legacy_stream(s))) {
             tlay = threshold_layout(d.L, d.k, (G * P + 31) / 32, CT, lay.gmin, kBlockShared - kOwnShared);
             sm = std::max(sm, tlay.total);
             blocks = sms;

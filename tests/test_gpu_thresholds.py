@@ -3,6 +3,7 @@ dispatch, many equal terms, terms of nothing, no plan at all, and instances it h
 from __future__ import annotations
 
 import contextlib
+import time
 
 import numpy as np
 import pytest
@@ -77,3 +78,42 @@ def test_no_work_leaves_the_transfers(L, k):
             inst.node_mem_bytes[:] = (float(inst.layer_mem_bytes.sum()) * np.random.default_rng(i).uniform(0.12, 0.3, k)).astype(np.uint64)
         want = oracle.dp_fact(inst, 8)
         same(pp.solve_exact_compute(inst, np.zeros(L, np.uint64), np.full(k, 1000, np.uint32)), want)
+
+
+def test_transfers_only_on_a_stream_of_its_own():
+    """A search that takes every SM is for the legacy stream, whose solves run one after another: handles on streams of their own
+    go on side by side (four of them took 1.2 times as long as one, by thresholds 3.5 times)."""
+    import torch
+    build.build()
+    insts = [W.config_geometric(8, 48, seed) for seed in range(2, 6)]
+    want = [oracle.dp_fact(i, 8) for i in insts]
+    streams = [torch.cuda.Stream() for _ in insts]
+    sols = [torch.zeros(22, dtype=torch.float64, device="cuda") for _ in insts]
+    with contextlib.ExitStack() as stack:
+        ps = [stack.enter_context(pp.Problem.from_instance(i)) for i in insts]
+        for p, w in zip(ps, want):
+            same(p.solve_exact(), w)
+            assert pp.debug_thresholds() == 1
+        for p, w, s in zip(ps, want, streams):
+            p.set_stream(s.cuda_stream)
+            same(p.solve_exact(), w)
+            assert pp.debug_thresholds() == 0
+
+        def seconds(n):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            for _ in range(100):
+                for p, sol in zip(ps[:n], sols):
+                    p.solve_exact_dev(sol.data_ptr())
+            torch.cuda.synchronize()
+            return time.perf_counter() - t0
+
+        times = [(seconds(1), seconds(4)) for _ in range(9)][2:]
+        assert np.median([t[1] for t in times]) < 2.5 * np.median([t[0] for t in times]), times
+        for sol, w in zip(sols, want):
+            got = pp.pp_solution.from_buffer_copy(sol.cpu().numpy().tobytes()[:176])
+            assert got.beta_ms == w.beta_ms and (got.m, tuple(got.cuts[: got.m - 1]), tuple(got.placement[: got.m])) == w.plan()
+        for p, w in zip(ps, want):
+            p.set_stream(0)
+            same(p.solve_exact(), w)
+            assert pp.debug_thresholds() == 1

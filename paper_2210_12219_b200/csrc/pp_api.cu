@@ -1892,7 +1892,7 @@ pp_status pp_solve_exact_compute(int32_t L, const uint64_t *layer_out_bits, cons
     const unsigned long long limits[2] = {kSparseScratchBytes, ~0ull};
     for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
         unsigned char *buf = nullptr;
-        if (!prune_in_shared(L, k, true)) {
+        if (!prune_in_shared(q, h)) {
             const size_t table = sparse_bytes(k, q.Lp, limits[pass]);
             e = staging_alloc(reinterpret_cast<void **>(&buf), head + table, s);
             if (e != cudaSuccess) break;

@@ -269,14 +269,15 @@ __host__ __device__ inline SparseLayout sparse_layout(int k, int Lp)
     w.rows = o;
     return w;
 }
-// whether the search of such a problem needs no scratch in global memory; compute: the one of Eq. 1
-bool prune_in_shared(int L, int k, bool compute);
 struct PruneHost {             // host arrays, read before launch_prune returns
     const uint64_t *bits, *M, *cap;  // [L], [L+1] memory prefix sums, [k]
     const uint32_t *bw;        // [k*k]
     const uint64_t *Wp;        // Eq. 1 only: [L+1] prefix sums of the layers' work, [k] speeds
     const uint32_t *speed;
 };
+// whether the search of such a problem needs no scratch in global memory; compute: the bounded one of Eq. 1
+bool prune_in_shared(int L, int k, bool compute);
+bool prune_in_shared(const PruneDev &d, const PruneHost &h);  // Eq. 1, by thresholds first or not
 cudaError_t launch_prune(const PruneDev &d, const PruneHost &h, int sms, cudaStream_t s);
 // Random comparison baseline (Section 4): P plans of problem d from 2 k draws each.
 cudaError_t launch_random_plans(const Dev &d, const unsigned char *tables, int64_t P, const uint32_t *draws, uint8_t *nseg,

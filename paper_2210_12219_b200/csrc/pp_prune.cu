@@ -1036,14 +1036,32 @@ constexpr size_t kOwnShared = 8192;  // static shared memory of k_prune, at most
 // kThresholdRows: rows of as many nodes as the chain takes at least; uniform chains, whose optimum takes 6 of 10 nodes, have 2500
 // and more and lose (Eq. 2, (50, 10) 51 / 78).
 constexpr unsigned kThresholdRows = 1500;
-bool threshold_takes(const uint64_t *cap, uint64_t total, int L, int k, bool compute)
+// Three kinds of input lose by it whatever their size, and are seen beforehand (mean of eight instances, the bounded search / by thresholds):
+//   no set of nodes holds the chain, which the bounded search sees on its first levels: Eq. 2 (50, 7) 30 / 36, (64, 8) 31 / 41, Eq. 1 (50, 8) 35 / 42
+//   terms over more than kThresholdOctaves powers of two, of which the first round leaves too many between two blocks' thresholds: Eq. 2 (50, 7)
+//     of near-equal layers and links with one far smaller layer and one far slower link 50 / 54 and, closer still, 51 / 58, (64, 8) 55 / 62 and
+//     55 / 67, Eq. 1 (50, 5) 44 / 47 and 44 / 48 (but six nodes 52 / 51, eight 64 / 58)
+//   stacks of identical layers, all of whose rows are alive at the optimum: Eq. 2 (50, 7) 42 / 48, (64, 8) 42 / 50 (24 layers 51 / 47 and 44 / 42),
+//     Eq. 1 (50, 5) 43 / 46, (50, 10) 62 / 65, (64, 12) 72 / 81 (but (50, 6) 55 / 52, (50, 8) 63 / 60, (24, 12) 70 / 60)
+constexpr int kThresholdOctaves = 20;
+bool threshold_takes(const PruneDev &d, const PruneHost &h, bool compute)
 {
+    const int L = d.L, k = d.k;
+    const uint64_t *cap = h.cap, total = h.M[L];
     if (L > 32 * kThresholdW || k > (compute ? kThresholdK : 8)) return false;
+    if ((!compute || k <= 5) && (d.key_top - d.key_base) >> 52 > (unsigned)kThresholdOctaves) return false;
+    if (L > 32 && (!compute || k <= 5 || k >= 10)) {
+        int alike = 0;
+        for (int c = 0; c + 2 < L; ++c) alike += h.bits[c] == h.bits[c + 1] ? 1 : 0;
+        if (2 * alike > L) return false;
+    }
     uint64_t sorted[PP_MAX_K];
     std::copy(cap, cap + k, sorted);
     std::sort(sorted, sorted + k, std::greater<uint64_t>());
     int need = 0;
-    for (uint64_t left = total; need < k && left > 0; ++need) left -= std::min(left, sorted[need]);
+    uint64_t left = total;
+    for (; need < k && left > 0; ++need) left -= std::min(left, sorted[need]);
+    if (left > 0) return false;
     unsigned rows = 0, binom = 1;
     for (int j = 1; j <= need; ++j) {
         binom = binom * (unsigned)(k - j + 1) / (unsigned)j;  // C(k, j)
@@ -1053,7 +1071,10 @@ bool threshold_takes(const uint64_t *cap, uint64_t total, int L, int k, bool com
 }
 // Where it comes before the search in one block's shared memory: Eq. 1, k = 6, 35 layers 40 to 52 / 33 to 45, 25 layers 30 to 41 / 31 to 41;
 // k = 5, 50 layers 36.8 / 31.5 (and 2 for the scratch that the search behind it may need), 25 30.6 / 32.
-bool threshold_before_shared(int L, int k) { return L <= 32 * kThresholdW && k >= 5 && k * L >= 200; }
+bool threshold_before_shared(const PruneDev &d, const PruneHost &h)
+{
+    return h.Wp && d.k >= 5 && d.k * d.L >= 200 && threshold_takes(d, h, true);
+}
 
 // Eq. 2: a grid that takes every SM for itself gains 9 to 40 % a solve, and takes from solves on other streams what a cluster of eight
 // blocks leaves them.  us a solve, one, two, four, eight handles on streams of their own, the bounded search and by thresholds: uniform
@@ -1082,7 +1103,8 @@ cudaError_t launch_shape(const PruneDev &d, const PruneHost &h, int sms, cudaStr
     cfg.blockDim = dim3((unsigned)threads);
     cfg.stream = s;
     cfg.attrs = attr;
-    const size_t all = CT && threshold_before_shared(d.L, d.k) ? 0 : shared_bytes<G, P, CT>(d.L, d.k, d.Lp);
+    const bool before_shared = threshold_before_shared(d, h);
+    const size_t all = before_shared ? 0 : shared_bytes<G, P, CT>(d.L, d.k, d.Lp);
     if (all) {
         cudaError_t e = allow_shared(k_prune<G, P, CT, true, false>, 4096);
         if (e != cudaSuccess) return e;
@@ -1100,7 +1122,7 @@ cudaError_t launch_shape(const PruneDev &d, const PruneHost &h, int sms, cudaStr
     ThresholdLayout tlay{};
     auto kernel = k_prune<G, P, CT, false, false>;
     if constexpr (G * P <= 32 * kThresholdW) {
-        if (threshold_takes(h.cap, h.M[d.L], d.L, d.k, CT) && (CT ? blocks > 1 || threshold_before_shared(d.L, d.k) : blocks > 1 && on_legacy_stream(s))) {
+        if (before_shared || (blocks > 1 && (CT || on_legacy_stream(s)) && threshold_takes(d, h, CT))) {
             tlay = threshold_layout(d.L, d.k, (G * P + 31) / 32, CT, lay.gmin, kBlockShared - kOwnShared);
             sm = std::max(sm, tlay.total);
             blocks = sms;
@@ -1192,9 +1214,10 @@ void prune_node_bounds(const uint64_t *cap, uint64_t total, PruneDev *d)
 // F<G, P, CT> of the shape of a row of L layers among k nodes; Eq. 1 stops at 256 layers
 #define PP_SHAPES(CASE) CASE(8, 2) CASE(16, 2) CASE(32, 2) CASE(4, 4) CASE(8, 4) CASE(16, 4) CASE(32, 4) CASE(32, 8)
 
+bool prune_in_shared(const PruneDev &d, const PruneHost &h) { return !threshold_before_shared(d, h) && prune_in_shared(d.L, d.k, true); }
+
 bool prune_in_shared(int L, int k, bool compute)
 {
-    if (compute && threshold_before_shared(L, k)) return false;
     const PruneShape sh = prune_shape(L, k);
     const int Lp = prune_row_pad(L, k);
     switch (sh.G * 100 + sh.P) {

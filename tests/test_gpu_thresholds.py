@@ -117,3 +117,39 @@ def test_transfers_only_on_a_stream_of_its_own():
             p.set_stream(0)
             same(p.solve_exact(), w)
             assert pp.debug_thresholds() == 1
+
+
+def no_room(inst):
+    inst.node_mem_bytes[:] = np.uint64(float(inst.layer_mem_bytes.sum()) * 0.98 / inst.k)
+
+
+def one_small_one_slow(inst):
+    rng = np.random.default_rng(inst.k)
+    inst.layer_out_bits[:] = rng.integers(7_900_000, 8_100_000, inst.L)
+    inst.layer_out_bits[inst.L // 2] = 1
+    inst.bw_kbps[:] = rng.integers(7800, 8200, (inst.k, inst.k)) * (1 - np.eye(inst.k, dtype=np.int64))
+    inst.bw_kbps[1, 3] = inst.bw_kbps[3, 1] = 1
+
+
+def stack(inst):
+    inst.layer_out_bits[: inst.L - 1] = 8_388_608
+
+
+# takes: whether the search by thresholds is the faster one for such inputs, and therefore asked
+@pytest.mark.parametrize("change,L,k,eq1,takes", [(no_room, 50, 7, False, False), (no_room, 50, 8, True, False), (no_room, 50, 5, True, False),
+                                                  (one_small_one_slow, 50, 7, False, False), (one_small_one_slow, 50, 5, True, False),
+                                                  (one_small_one_slow, 33, 8, True, True), (stack, 33, 7, False, False), (stack, 32, 7, False, True),
+                                                  (stack, 50, 5, True, False), (stack, 33, 8, True, True), (stack, 33, 10, True, False),
+                                                  (lambda inst: None, 50, 7, False, True), (lambda inst: None, 50, 5, True, True)])
+def test_inputs_that_lose_go_to_the_bounded_search(change, L, k, eq1, takes):
+    build.build()
+    inst = network(150_000 + 100 * L + k, L, k, 0)
+    inst.node_mem_bytes[:] = (float(inst.layer_mem_bytes.sum()) * np.random.default_rng(L).uniform(0.2, 0.45, k)).astype(np.uint64)  # three nodes at least
+    change(inst)
+    if eq1:
+        work, speed = (inst.layer_mem_bytes // np.uint64(1024)).astype(np.uint64), np.random.default_rng(k).integers(500, 1501, k).astype(np.uint32)
+        same(pp.solve_exact_compute(inst, work, speed), CT.dp(inst, work.tolist(), speed.tolist()))
+    else:
+        with pp.Problem.from_instance(inst) as p:
+            same(p.solve_exact(), oracle.dp_fact(inst, 4))
+    assert pp.debug_thresholds() == (1 if takes else 0)

@@ -35,6 +35,23 @@ def network(seed, L, k, kind):
     return inst
 
 
+def three_nodes(inst):
+    """No two nodes hold the chain: where two do, the bounded search is as fast and is the one that runs."""
+    total = float(inst.layer_mem_bytes.sum())
+    inst.node_mem_bytes[:] = (total * np.random.default_rng(inst.L).uniform(0.2, 0.45, inst.k)).astype(np.uint64)
+
+
+def rising(seed, L, k):
+    """A chain whose memory rises along it, log-normal sizes and links: its optimum takes six nodes and more now and then."""
+    rng = np.random.default_rng(seed)
+    mem = 64.0 ** (np.arange(L) / L) * (0.8 + 0.4 * rng.random(L))
+    bits = np.clip(np.exp(np.log(10.2e6) - 0.28 + 0.75 * rng.standard_normal(L)), 1e5, 1.2e8)
+    cap = rng.integers(24 * 10**6, 48 * 10**6, k)
+    bw = np.zeros((k, k), np.uint32)
+    bw[np.triu_indices(k, 1)] = np.clip(np.exp(np.log(6000) - 0.125 + 0.5 * rng.standard_normal(k * (k - 1) // 2)), 500, 50000)
+    return W.Instance(L, k, bits.astype(np.uint64), (mem / mem.sum() * 102_400_000).astype(np.uint64), cap.astype(np.uint64), bw + bw.T, "rising")
+
+
 def same(got, want):
     assert got.status == want.status and got.plan() == want.plan()
     assert got.beta_ms == want.beta_ms or np.isinf(want.beta_ms)
@@ -70,11 +87,11 @@ def test_compute_times(L, k, debug):
 
 @pytest.mark.parametrize("L,k", [(24, 9), (33, 10), (64, 10), (50, 11), (20, 12), (50, 12), (64, 12)])
 def test_no_work_leaves_the_transfers(L, k):
-    """Nothing costs compute: the optimum of Eq. 2, also where a block's table of node sets runs out."""
+    """Nothing costs compute: the optimum of Eq. 2."""
     build.build()
     for i in range(8):
         inst = network(140_000 + 100 * L + 10 * k + i, L, k, i % 6)
-        if i >= 6:  # many nodes to a plan, most sets alive
+        if i >= 6:  # many nodes to a plan: with eleven and more the bounded search from the start
             inst.node_mem_bytes[:] = (float(inst.layer_mem_bytes.sum()) * np.random.default_rng(i).uniform(0.12, 0.3, k)).astype(np.uint64)
         want = oracle.dp_fact(inst, 8)
         same(pp.solve_exact_compute(inst, np.zeros(L, np.uint64), np.full(k, 1000, np.uint32)), want)
@@ -119,6 +136,47 @@ def test_transfers_only_on_a_stream_of_its_own():
             assert pp.debug_thresholds() == 1
 
 
+# the lines of the dispatch under Eq. 2, on the legacy stream: up to 64 layers and eight nodes, more than a block's round
+@pytest.mark.parametrize("debug", [False, True])
+@pytest.mark.parametrize("L,k,takes", [(8, 6, 0), (17, 7, 1), (31, 8, 1), (32, 8, 1), (33, 7, 1), (33, 8, 1), (64, 7, 1), (64, 8, 1), (65, 8, 0),
+                                       (40, 9, 0)])
+def test_which_search_answers(L, k, takes, debug):
+    build.build()
+    with library(build.build_debug()) if debug else contextlib.nullcontext():
+        for kind in (0, 2, 3):
+            inst = network(160_000 + 100 * L + 10 * k + kind, L, k, kind)
+            three_nodes(inst)
+            with pp.Problem.from_instance(inst) as p:
+                same(p.solve_exact(), oracle.dp_fact(inst, 4))
+            assert pp.debug_thresholds() == takes, kind
+
+
+# rows of one word and of two
+@pytest.mark.parametrize("debug", [False, True])
+@pytest.mark.parametrize("L", [24, 50])
+def test_what_does_not_fit_is_handed_over(L, debug):
+    build.build()
+    with library(build.build_debug()) if debug else contextlib.nullcontext():
+        # the optimum needs more node sets than a block has room for, or does not
+        seen = set()
+        for seed in range(12):
+            inst = rising(seed, L, 12)
+            same(pp.solve_exact_compute(inst, np.zeros(L, np.uint64), np.full(12, 1000, np.uint32)), oracle.dp_fact(inst, 8))
+            seen.add(pp.debug_thresholds())
+        assert seen == {1, 2}
+        # hundreds of quotients within a millionth of each other, in a range that four rounds do not resolve
+        for seed in range(4):
+            inst = network(seed, L, 8, 0)
+            three_nodes(inst)
+            rng = np.random.default_rng(seed)
+            inst.layer_out_bits[:] = 2**38 + rng.permutation(L)
+            inst.layer_out_bits[L // 2] = 2**20
+            inst.bw_kbps[:] = (4_000_000 + rng.integers(0, 6, (8, 8))) * (1 - np.eye(8, dtype=np.int64))
+            with pp.Problem.from_instance(inst) as p:
+                same(p.solve_exact(), oracle.dp_fact(inst, 8))
+            assert pp.debug_thresholds() == 2, seed
+
+
 def no_room(inst):
     inst.node_mem_bytes[:] = np.uint64(float(inst.layer_mem_bytes.sum()) * 0.98 / inst.k)
 
@@ -144,7 +202,7 @@ def stack(inst):
 def test_inputs_that_lose_go_to_the_bounded_search(change, L, k, eq1, takes):
     build.build()
     inst = network(150_000 + 100 * L + k, L, k, 0)
-    inst.node_mem_bytes[:] = (float(inst.layer_mem_bytes.sum()) * np.random.default_rng(L).uniform(0.2, 0.45, k)).astype(np.uint64)  # three nodes at least
+    three_nodes(inst)
     change(inst)
     if eq1:
         work, speed = (inst.layer_mem_bytes // np.uint64(1024)).astype(np.uint64), np.random.default_rng(k).integers(500, 1501, k).astype(np.uint32)

@@ -1043,12 +1043,12 @@ constexpr unsigned kThresholdRows = 1500;
 //     55 / 67, Eq. 1 (50, 5) 44 / 47 and 44 / 48 (but six nodes 52 / 51, eight 64 / 58)
 //   stacks of identical layers, all of whose rows are alive at the optimum: Eq. 2 (50, 7) 42 / 48, (64, 8) 42 / 50 (24 layers 51 / 47 and 44 / 42),
 //     Eq. 1 (50, 5) 43 / 46, (50, 10) 62 / 65, (64, 12) 72 / 81 (but (50, 6) 55 / 52, (50, 8) 63 / 60, (24, 12) 70 / 60)
-constexpr int kThresholdOctaves = 20;
+constexpr int kThresholdOctaves = 20, kThresholdPlainK = 8;  // nodes under Eq. 2, at most
 bool threshold_takes(const PruneDev &d, const PruneHost &h, bool compute)
 {
     const int L = d.L, k = d.k;
     const uint64_t *cap = h.cap, total = h.M[L];
-    if (L > 32 * kThresholdW || k > (compute ? kThresholdK : 8)) return false;
+    if (L > 32 * kThresholdW || k > (compute ? kThresholdK : kThresholdPlainK)) return false;
     if ((!compute || k <= 5) && (d.key_top - d.key_base) >> 52 > (unsigned)kThresholdOctaves) return false;
     if (L > 32 && (!compute || k <= 5 || k >= 10)) {
         int alike = 0;
@@ -1121,7 +1121,8 @@ cudaError_t launch_shape(const PruneDev &d, const PruneHost &h, int sms, cudaStr
     size_t sm = lay.total;
     ThresholdLayout tlay{};
     auto kernel = k_prune<G, P, CT, false, false>;
-    if constexpr (G * P <= 32 * kThresholdW) {
+    static_assert(kWideK >= kThresholdPlainK, "Eq. 2 by thresholds has rows of two positions a lane");
+    if constexpr (G * P <= 32 * kThresholdW && (CT || P == 2)) {
         if (before_shared || (blocks > 1 && (CT || on_legacy_stream(s)) && threshold_takes(d, h, CT))) {
             tlay = threshold_layout(d.L, d.k, (G * P + 31) / 32, CT, lay.gmin, kBlockShared - kOwnShared);
             sm = std::max(sm, tlay.total);

@@ -1442,8 +1442,8 @@ static pp_status batch_from_host(batch_dev_fn run_dev, bool in_place, int64_t B,
         const BatchRoute route = batch_route(B, L, k, sms, pieces);
         const void *in[4] = {out_bits, mem, node_mem, bw};
         // An instance to a block: the batch goes in pieces, so that the host copies one while the GPU works on the
-        // one before.  With that a batch of this size is faster so than an instance to a lane, also in several waves, us
-        // a call in lanes and in blocks: 300 x (k = 5, L = 24) 68.8, 47.5, 3600 x (4, 9) 194, 130, 1400 x (7, 24) 199, 153; two
+        // one before.  With that a batch of this size is faster so than an instance to a lane (to a warp has not been tried from
+        // page-locked memory), also in several waves, us a call in lanes and in blocks: 300 x (k = 5, L = 24) 68.8, 47.5, 3600 x (4, 9) 194, 130, 1400 x (7, 24) 199, 153; two
         // blocks to an SM 600 x (8, 32) 158, 146, 1100 246, 214; 450 and 1200 x (8, 28) 128, 112, 252, 208; 1900 x (8, 9) 228, 195,
         // 2200 x (8, 4) 147, 140.  Only k = 8, L = 5 to 7 is not beyond four waves, where a piece is a wave and a bit (1800
         // and 2100 x (8, 5) 140, 144 and 158, 161, x (8, 6) 158, 162 and 178, 182; 1776 x (8, 5) 139, 130).

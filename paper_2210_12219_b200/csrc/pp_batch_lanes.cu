@@ -652,6 +652,8 @@ cudaError_t launch_level(int nv, const BatchLanes &t, int64_t B, int k, int L, i
 // 51.7, 54.5, 57.3; k = 7 hardly gains anywhere (460, 600, 888 x (7, 24) 46.1, 45.8, 49.6, 51.5, 56.1, 59.7) and k = 8 loses
 // (460 x (8, 24) 64.1, 74.1), with longer rows too (888 x (8, 28) 99.6, 104.8; two blocks to an SM from 29 on: 600 x (8, 32)
 // 84.4, 106.7).  A third wave loses (2200 x (6, 24) 60.2, 70.1, (4, 17) 32.6, 35.1) or gains 3 to 5 % ((5, 32) 50.5, 48.2).
+// These lines know blocks and lanes; a warp is asked for only beyond them (batch_warps_takes), although it is faster already in front
+// of some for uniform sizes and links (888 x (8, 9) 63.8 in blocks, 889 in warps 40.7; identical blocks 79).
 bool batch_lanes_takes(int64_t B, int L, int k, int sms)
 {
     if (k < 2 || k > kLanesMaxK || L > kLanesMaxL) return false;

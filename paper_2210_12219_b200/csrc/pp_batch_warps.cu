@@ -6,18 +6,16 @@
 // is a dozen logical instructions a row where the search on ranks works through a row of 16-bit values.  beta* is
 // one of the quotients, so that a bisection over them ends with it exactly, and the table of the last feasible probe is
 // what the backtrack's threshold rule asks for: no ranking of the quotients.  It starts from a lower bound, the optimum
-// over the plans that may use a node again, which is one word a node; in 58 % of the instances of k = 8, L = 24 that is
-// beta* and one probe confirms it, the others take eight more (4096 of them, us a call: 243 by bisection alone, 172 with the
-// bound, 161 with values instead of ranks bisected, 148 with longer steps in front of that; by lanes 218).
+// over the plans that may use a node again, which is one word a node.  Of k = 8, L = 24 with sizes and links drawn uniformly that is
+// beta* in six of ten instances, and one probe confirms it; of log-normal ones in a third, of identical blocks or of two groups of
+// nodes in one of twelve and fewer, and those take ten probes or so.
 //
 // A warp keeps an instance's table in shared memory, reach[S] a row of eight words.  Lane (w, q) takes the rows of
 // target node w: the links into w and the windows of w are registers, a source set is two 16-byte loads, and all
 // lanes walk the list of node sets of the other nodes, eight sets a trip.  No barriers but the warp's own.
-// What bounds it: 16 000 warp instructions an instance (3500 the bound, 1400 the staging, a trip 92, of which the windows
-// 54) at 56 % of the issue slots while an SM has work (chains of dependent instructions), and then the longest instances, up
-// to 15 probes or so of 7 us: 2000 instances take 119, 4096 148, 8000 231, and an SM has work 66 % of the time at 4096.
-// Not kept: teams of two to twelve warps for the instances that are not at their bound (187); one queue of instances for two
-// blocks (159) or four (215: the clusters leave SMs idle); states that cannot reach the last layer dropped (193).
+// What bounds it: 16 000 warp instructions an instance of the uniform kind (3500 the bound, 1400 the staging, a trip 92, of which
+// the windows 54) at 56 % of the issue slots while an SM has work (chains of dependent instructions), and then the longest instances, up
+// to 15 probes or so of 7 us: 2000 instances take 121, 4096 150, 20000 480, and an SM has work 66 % of the time at 4096.
 #include <algorithm>
 
 #include "pp_blocks.cuh"
@@ -271,10 +269,8 @@ k_batch_warps(const int64_t B, const int L, const int k, const uint32_t *__restr
         return A;
     };
     // A lower bound by the plans that may use a node again: one word a node instead of one a (set, node), so that the groups
-    // of lanes take a threshold each.  It is beta* itself in 58 % of the instances of k = 8, L = 24 (median distance of the others
-    // 16 of 650 quotients).  Returns the largest threshold found to be too small, or -1.
-    // Rounds, each a fifth of the range: four (4096 x (8, 24) with 2, 3, 4, 5, 6 of them 203, 154, 148, 150, 154; 900 x (8, 9) 46.0, 43.7,
-    // 44.5, 46.0, 47.3).
+    // of lanes take a threshold each.  Four rounds, each a fifth of the range (uniform, 4096 x (8, 24): three rounds take 4 % more, five 1 %).
+    // Returns the largest threshold found to be too small, or -1.
     auto lower_bound = [&]() -> float {
         float beaten = -1.0f, slow = __uint_as_float(0x7F800000u), fast = 0.0f;
 #pragma unroll
@@ -475,9 +471,8 @@ k_batch_warps(const int64_t B, const int L, const int k, const uint32_t *__restr
             extremes();
             if (least == ~0ull || (m > 0 && least == most)) break;
             // The smallest candidate; most optima that are not there lie little above it: steps that grow, up to ten times as far,
-            // then whether there is a plan at all.  What counts is the longest instance, not the mean: with 1.1, 1.35, 2 and the
-            // largest candidate 4096 x (k = 8, L = 24) took 161 us (six seeds; 2000 131), with 1.07, 1.2, 1.6, 3 164, with 1.15, 1.5, 2.5, 6 155,
-            // with these 150 (2000 119).  Between a threshold without and one with a plan the middle of their bits.
+            // then whether there is a plan at all.  What counts is the longest instance, not the mean: in steps of 1.1, 1.35, 2 and then the
+            // largest candidate 4096 x (k = 8, L = 24) took 7 % longer.  Between a threshold without and one with a plan the middle of their bits.
             unsigned long long key = least;
             if (m > 0) key = least + ((most - least) >> 1);
             else if (tries > 5) key = most;

@@ -1,5 +1,5 @@
 """The batched search on both sides of every line of its dispatch: batches of one and two waves of blocks, and the
-batches beyond them that go an instance to a lane, over the row widths of both paths."""
+batches beyond them that go an instance to a lane or to a warp, over the row widths of all paths."""
 from __future__ import annotations
 
 import contextlib
@@ -57,7 +57,7 @@ def test_every_path_gives_the_oracles_plans(L, k, debug):
     want = [oracle.dp_naive(i) for i in insts]
     beyond = 11  # this one has a transfer beyond the limits
     with library(build.build_debug()) if debug else contextlib.nullcontext():
-        # the last one is more than the host variant works on in place: it goes an instance to a lane
+        # the last one is more than the host variant works on in place: it goes an instance to a lane or to a warp
         for B in (63, 64, 296, 297, 444, 445, 888, 889, 1332, 1333, max(1800, (1 << 20) // (16 * L + 4 * k * (k + 3)) + 45)):
             pick = np.arange(B) % len(insts)
             arrays = [np.stack([getattr(i, f) for i in insts])[pick].copy() for f in FIELDS]

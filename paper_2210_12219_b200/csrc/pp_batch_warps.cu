@@ -13,9 +13,9 @@
 // A warp keeps an instance's table in shared memory, reach[S] a row of eight words.  Lane (w, q) takes the rows of
 // target node w: the links into w and the windows of w are registers, a source set is two 16-byte loads, and all
 // lanes walk the list of node sets of the other nodes, eight sets a trip.  No barriers but the warp's own.
-// What bounds it: 16 000 warp instructions an instance of the uniform kind (3500 the bound, 1400 the staging, a trip 92, of which
+// What bounds it: 15 300 warp instructions an instance of the uniform kind (3500 the bound, 1400 the staging, a trip 92, of which
 // the windows 54) at 56 % of the issue slots while an SM has work (chains of dependent instructions), and then the longest instances, up
-// to 15 probes or so of 7 us: 2000 instances take 121, 4096 150, 20000 480, and an SM has work 66 % of the time at 4096.
+// to 15 probes or so of 7 us: 2000 instances take 118, 4096 150, 20000 483, and an SM has work 66 % of the time at 4096.
 #include <algorithm>
 
 #include "pp_blocks.cuh"

@@ -322,16 +322,13 @@ k_batch_warps(const int64_t B, const int L, const int k, const uint32_t *__restr
     auto within = [&](double t) {
 #pragma unroll
         for (int i = 0; i < kPairs; ++i) {
-            // size <= t b is within t.  The largest size whose quotient rounds to no more than t lies below
-            // t b (1 + 2^-53): beyond the product, which is rounded down, by less than 2^-10 (sizes are below
-            // 2^40).  What lies there is settled by its quotient.
-            const double p = __dmul_rd(t, link[i]), edge = __dadd_rn(p, 1.0 / 1024.0);
+            const SizeBracket fits = sizes_within(t, link[i]);
             int c = 0;
 #pragma unroll
             for (int step = 16; step; step >>= 1)
-                if (sorted[c + step - 1] <= edge) c += step;
+                if (sorted[c + step - 1] <= fits.most) c += step;
             if (!(link[i] > 0.0)) c = 0;
-            while (c > 0 && sorted[c - 1] > p && quotient(sorted[c - 1], link[i], recip[i]) > t) --c;
+            while (c > 0 && sorted[c - 1] > fits.sure && quotient(sorted[c - 1], link[i], recip[i]) > t) --c;
             upto[i] = c;
             okp[i] = under[c];
         }

@@ -18,6 +18,18 @@ __device__ __forceinline__ double quotient(double x, double b, double r)
     return __fma_rn(__fma_rn(-q, b, x), r, q);
 }
 
+// What a link of bandwidth b moves within t: every size up to `sure`, none beyond `most`; one between them is settled by its
+// quotient.  The largest size whose quotient rounds to no more than t lies below t b (1 + 2^-53), which is beyond the product rounded
+// down by less than 2^-10, sizes being below 2^40.
+struct SizeBracket {
+    double sure, most;
+};
+__device__ __forceinline__ SizeBracket sizes_within(double t, double b)
+{
+    const double sure = __dmul_rd(t, b);
+    return {sure, __dadd_rn(sure, 1.0 / 1024.0)};
+}
+
 // The window minimum of a row that a group of G lanes holds, P consecutive positions a lane: out at
 // position c2 = min of g over [lo, c2 - 1].  The window is the tail of the block (= lane) that holds its
 // start (suffix minima, through shared memory), whole blocks in between (a sparse table over the G block

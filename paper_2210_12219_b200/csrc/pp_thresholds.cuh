@@ -227,12 +227,10 @@ __device__ __forceinline__ int threshold_search(const PruneDev &d, const Thresho
 
     // the largest size that a link of bandwidth b moves within t
     auto size_within = [&](double t, double b) -> unsigned long long {
-        // A size up to t b is within t; the largest one whose quotient rounds to no more than t lies below t b (1 + 2^-53),
-        // which is beyond the product rounded down by less than 2^-10 (sizes are below 2^40), and its quotient decides.
-        const double p = __dmul_rd(t, b), edge = __dadd_rn(p, 1.0 / 1024.0);
-        if (!(edge < 1099511627776.0)) return 1ull << 40;
-        const unsigned long long most = (unsigned long long)edge;
-        return (double)most > p && __ddiv_rn((double)most, b) > t ? most - 1ull : most;  // a size of 0 is within any t
+        const SizeBracket fits = sizes_within(t, b);
+        if (!(fits.most < 1099511627776.0)) return 1ull << 40;
+        const unsigned long long most = (unsigned long long)fits.most;
+        return (double)most > fits.sure && __ddiv_rn((double)most, b) > t ? most - 1ull : most;  // a size of 0 is within any t
     };
     auto places_within = [&](unsigned long long most) -> int {
         int c = 0;
